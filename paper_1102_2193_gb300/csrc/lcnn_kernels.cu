@@ -5,6 +5,7 @@
 // masters; every convolution accumulates in FP32 on the tensor cores
 // (mma.sync m16n8k16 bf16, implicit GEMM).  Boundaries are periodic, like the
 // boxes the fields come from.
+#include <cooperative_groups.h>
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
@@ -99,6 +100,240 @@ __global__ void __launch_bounds__(128) k_conv_fwd(const __nv_bfloat16* __restric
   }
 }
 
+__device__ __forceinline__ uint32_t smem_addr(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
+__device__ __forceinline__ void cp16(uint32_t dst, const void* src) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(dst), "l"(src) : "memory");
+}
+__device__ __forceinline__ void cp_wait_all() { asm volatile("cp.async.wait_all;\n" ::: "memory"); }
+__device__ __forceinline__ void ldm4(uint32_t r[4], uint32_t a) {
+  asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];\n"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(a) : "memory");
+}
+__device__ __forceinline__ void ldm2(uint32_t r[2], uint32_t a) {
+  asm volatile("ldmatrix.sync.aligned.m8n8.x2.shared.b16 {%0,%1}, [%2];\n" : "=r"(r[0]), "=r"(r[1]) : "r"(a) : "memory");
+}
+__device__ __forceinline__ void ldm4t(uint32_t r[4], uint32_t a) {
+  asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];\n"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(a) : "memory");
+}
+// Byte offset of half h (8 channels, 16 bytes) of row p in a tile of 32-byte
+// rows (16 channels): the halves swap every four rows, so the eight rows of
+// an 8x8 ldmatrix, consecutive from any start, fall in eight different 16-byte
+// bank groups.
+__device__ __forceinline__ uint32_t row32(int p, int h) {
+  return (uint32_t)(p << 5) + (uint32_t)(((h ^ (p >> 2)) & 1) << 4);
+}
+__device__ __forceinline__ int modn(int v, int n) {
+  const int r = v % n;
+  return r < 0 ? r + n : r;
+}
+
+// Periodic 3x3x3 convolution over a TX x TY x TZ box of positions per block:
+// for each 16 input channels the box with its one-node halo (32 bytes a
+// position) and the 27 x COUT x 16 weights go to shared memory once, and the
+// 27 taps read their A fragments there by ldmatrix at shifted row addresses.
+// k_conv_fwd, which this replaces for 3x3x3 kernels, read every position 27
+// times through L1 with 4-byte loads (16 -> 16 channels at 128^3: 740 us).
+// A warp holds MT 16-position tiles x NT 8-channel tiles, so one B fragment
+// serves MT products; MT and NT are bounded by the accumulator registers, the
+// tile by 2 blocks per SM.  FP32 accumulation in the order (16-channel group,
+// tap).  blockIdx.y picks the group of NT * 8 output channels.
+template <int NT, int MT, int NW, int TX, int TY, int TZ>
+__global__ void __launch_bounds__(32 * NW) k_conv_tile(const __nv_bfloat16* __restrict__ in,
+                                                       const __nv_bfloat16* __restrict__ w,
+                                                       const float* __restrict__ bias, float* __restrict__ out32,
+                                                       __nv_bfloat16* __restrict__ out16, int W, int H, int D, int cin,
+                                                       int cout, int relu, int ntx, int nty) {
+  static_assert(TX * TY * TZ == 16 * MT * NW, "one 16-position tile per (warp, MT)");
+  constexpr int HX = TX + 2, HY = TY + 2, HZ = TZ + 2, HP = HX * HY * HZ, NTHR = 32 * NW;
+  constexpr int NPT = (HP + NTHR - 1) / NTHR, NWR = 27 * NT * 8;
+  extern __shared__ __align__(128) unsigned char smem[];
+  const uint32_t sA = smem_addr(smem), sW = sA + HP * 32;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int bx = blockIdx.x % ntx, by = (blockIdx.x / ntx) % nty, bz = blockIdx.x / (ntx * nty);
+  const int x0 = bx * TX, y0 = by * TY, z0 = bz * TZ, co0 = blockIdx.y * NT * 8;
+  int pos[NPT];
+#pragma unroll
+  for (int k = 0; k < NPT; ++k) {
+    const int p = tid + k * NTHR;
+    pos[k] = modn(x0 + p % HX - 1, W) + W * (modn(y0 + (p / HX) % HY - 1, H) + H * modn(z0 + p / (HX * HY) - 1, D));
+  }
+  int rowp[MT];
+#pragma unroll
+  for (int i = 0; i < MT; ++i) {
+    const int m = (warp * MT + i) * 16 + (lane & 15);
+    rowp[i] = m % TX + HX * ((m / TX) % TY + HY * (m / (TX * TY)));
+  }
+  const int ahalf = lane >> 4;                                // A: rows lane & 15, channels 8 ahalf..
+  const int brow = ((lane >> 4) & 1) * 8 + (lane & 7);        // B: output channel within a pair of 8-tiles
+  const int bhalf = (lane >> 3) & 1;
+  float acc[MT][NT][4];
+#pragma unroll
+  for (int i = 0; i < MT; ++i)
+#pragma unroll
+    for (int j = 0; j < NT; ++j) acc[i][j][0] = acc[i][j][1] = acc[i][j][2] = acc[i][j][3] = 0.f;
+  for (int c0 = 0; c0 < cin; c0 += 16) {
+    if (c0) __syncthreads();
+#pragma unroll
+    for (int k = 0; k < NPT; ++k) {
+      const int p = tid + k * NTHR;
+      if (p < HP) {
+        const __nv_bfloat16* src = in + (size_t)pos[k] * cin + c0;
+        cp16(sA + row32(p, 0), src);
+        cp16(sA + row32(p, 1), src + 8);
+      }
+    }
+    for (int r = tid; r < NWR; r += NTHR) {
+      const int t = r / (NT * 8), co = r % (NT * 8);
+      const __nv_bfloat16* src = w + ((size_t)(co0 + co) * 27 + t) * cin + c0;
+      cp16(sW + row32(r, 0), src);
+      cp16(sW + row32(r, 1), src + 8);
+    }
+    cp_wait_all();
+    __syncthreads();
+#pragma unroll 1
+    for (int dz = 0; dz < 3; ++dz)
+#pragma unroll
+      for (int dyx = 0; dyx < 9; ++dyx) {
+        const int t = dz * 9 + dyx;
+        const int off = dyx % 3 + HX * (dyx / 3 + HY * dz);
+        uint32_t a[MT][4], b[NT][2];
+#pragma unroll
+        for (int i = 0; i < MT; ++i) ldm4(a[i], sA + row32(rowp[i] + off, ahalf));
+#pragma unroll
+        for (int j = 0; j + 1 < NT; j += 2) {
+          uint32_t q[4];
+          ldm4(q, sW + row32(t * NT * 8 + j * 8 + brow, bhalf));
+          b[j][0] = q[0];
+          b[j][1] = q[1];
+          b[j + 1][0] = q[2];
+          b[j + 1][1] = q[3];
+        }
+        if constexpr (NT & 1) ldm2(b[NT - 1], sW + row32(t * NT * 8 + (NT - 1) * 8 + (lane & 7), bhalf));
+#pragma unroll
+        for (int i = 0; i < MT; ++i)
+#pragma unroll
+          for (int j = 0; j < NT; ++j) mma_bf16(acc[i][j], a[i], b[j]);
+      }
+  }
+  const int g = lane >> 2, tg = lane & 3;
+#pragma unroll
+  for (int i = 0; i < MT; ++i)
+#pragma unroll
+    for (int r = 0; r < 2; ++r) {
+      const int m = (warp * MT + i) * 16 + g + 8 * r;
+      const int x = x0 + m % TX, y = y0 + (m / TX) % TY, z = z0 + m / (TX * TY);
+      if (x >= W || y >= H || z >= D) continue;
+      const size_t o = ((size_t)x + (size_t)W * (y + (size_t)H * z)) * cout + co0 + tg * 2;
+#pragma unroll
+      for (int j = 0; j < NT; ++j) {
+        float v0 = acc[i][j][2 * r], v1 = acc[i][j][2 * r + 1];
+        if (bias) {
+          v0 += bias[co0 + j * 8 + tg * 2];
+          v1 += bias[co0 + j * 8 + tg * 2 + 1];
+        }
+        if (relu) {
+          v0 = fmaxf(v0, 0.f);
+          v1 = fmaxf(v1, 0.f);
+        }
+        if (out32) {
+          out32[o + j * 8] = v0;
+          out32[o + j * 8 + 1] = v1;
+        }
+        if (out16) {
+          out16[o + j * 8] = __float2bfloat16_rn(v0);
+          out16[o + j * 8 + 1] = __float2bfloat16_rn(v1);
+        }
+      }
+    }
+}
+
+// Partial dW of the 3x3x3 kernel: block (chunk, 16 output channels x 16 input
+// channels, tap group) sums its boxes of 16 x TY x TZ positions (boxes chunk,
+// chunk + nchunk, ... in order) with the input box and its halo and the
+// output-gradient box in shared memory; nine warps take TPW taps each.  Both
+// operands are position-major, so A (dout^T) and B (shifted input) are read by
+// transposing ldmatrix, a tap being a shifted row address; one A fragment
+// serves TPW taps.  k_conv_wgrad read both through 2-byte global loads, once
+// per tap (16 x 16 channels at 64^3: 185 us).  Positions past the end of a
+// ragged box read a row of zeros on both sides.
+template <int TPW, int TY, int TZ>
+__global__ void __launch_bounds__(288) k_wgrad_tile(const __nv_bfloat16* __restrict__ dout,
+                                                    const __nv_bfloat16* __restrict__ in, float* __restrict__ part,
+                                                    int W, int H, int D, int cin, int cout, int ntx, int nty, int ntz,
+                                                    int nchunk) {
+  constexpr int TX = 16, HX = TX + 2, HY = TY + 2, HZ = TZ + 2, HP = HX * HY * HZ, NP = TX * TY * TZ, NTHR = 288;
+  extern __shared__ __align__(128) unsigned char smem[];
+  const uint32_t sI = smem_addr(smem), sD = sI + (HP + 1) * 32, zrow = sI + HP * 32;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int nci = cin / 16, co0 = (blockIdx.y / nci) * 16, ci0 = (blockIdx.y % nci) * 16;
+  const int t0 = (blockIdx.z * 9 + warp) * TPW;
+  float acc[TPW][2][4];
+#pragma unroll
+  for (int k = 0; k < TPW; ++k)
+#pragma unroll
+    for (int j = 0; j < 2; ++j) acc[k][j][0] = acc[k][j][1] = acc[k][j][2] = acc[k][j][3] = 0.f;
+  int off[TPW];
+#pragma unroll
+  for (int k = 0; k < TPW; ++k) {
+    const int t = t0 + k;
+    off[k] = t % 3 + HX * ((t / 3) % 3 + HY * (t / 9));
+  }
+  if (tid < 8) reinterpret_cast<uint32_t*>(smem)[HP * 8 + tid] = 0u;
+  const int ar = ((lane >> 4) & 1) * 8 + (lane & 7), ah = (lane >> 3) & 1;  // A: position, output-channel half
+  const int br = ((lane >> 3) & 1) * 8 + (lane & 7), bh = lane >> 4;        // B: position, input-channel half
+  for (int tile = blockIdx.x; tile < ntx * nty * ntz; tile += nchunk) {
+    const int x0 = (tile % ntx) * TX, y0 = ((tile / ntx) % nty) * TY, z0 = (tile / (ntx * nty)) * TZ;
+    __syncthreads();
+    for (int p = tid; p < HP; p += NTHR) {
+      const int q = modn(x0 + p % HX - 1, W) + W * (modn(y0 + (p / HX) % HY - 1, H) + H * modn(z0 + p / (HX * HY) - 1, D));
+      const __nv_bfloat16* src = in + (size_t)q * cin + ci0;
+      cp16(sI + row32(p, 0), src);
+      cp16(sI + row32(p, 1), src + 8);
+    }
+    for (int m = tid; m < NP; m += NTHR) {
+      const int x = x0 + m % TX, y = y0 + (m / TX) % TY, z = z0 + m / (TX * TY);
+      if (x < W && y < H && z < D) {
+        const __nv_bfloat16* src = dout + ((size_t)x + (size_t)W * (y + (size_t)H * z)) * cout + co0;
+        cp16(sD + row32(m, 0), src);
+        cp16(sD + row32(m, 1), src + 8);
+      } else {
+        uint4* d = reinterpret_cast<uint4*>(smem + (HP + 1) * 32 + m * 32);
+        d[0] = d[1] = make_uint4(0u, 0u, 0u, 0u);
+      }
+    }
+    cp_wait_all();
+    __syncthreads();
+    const bool xin = x0 + br < W;
+    for (int s = 0; s < TY * TZ; ++s) {
+      const int yy = s % TY, zz = s / TY;
+      if (y0 + yy >= H || z0 + zz >= D) continue;
+      const int base = br + HX * (yy + HY * zz);
+      uint32_t a[4];
+      ldm4t(a, sD + row32(s * 16 + ar, ah));
+#pragma unroll
+      for (int k = 0; k < TPW; ++k) {
+        uint32_t b[4];
+        ldm4t(b, xin ? sI + row32(base + off[k], bh) : zrow);
+        mma_bf16(acc[k][0], a, b);
+        mma_bf16(acc[k][1], a, b + 2);
+      }
+    }
+  }
+  const int g = lane >> 2, tg = lane & 3;
+  float* dw = part + (size_t)blockIdx.x * cout * 27 * cin;
+#pragma unroll
+  for (int k = 0; k < TPW; ++k)
+#pragma unroll
+    for (int j = 0; j < 2; ++j)
+#pragma unroll
+      for (int r = 0; r < 2; ++r) {
+        float* o = dw + ((size_t)(co0 + g + 8 * r) * 27 + t0 + k) * cin + ci0 + j * 8 + tg * 2;
+        o[0] = acc[k][j][2 * r];
+        o[1] = acc[k][j][2 * r + 1];
+      }
+}
+
 // Partial dW[co][t][ci] = sum_p dout[p][co] in[tap(p, t)][ci] over one chunk
 // of positions, stored for the chunk (part[chunk][co][t][ci]); one warp per
 // (chunk, tap, 16 output channels).  A = dout^T (16 C_out x 16 positions),
@@ -150,12 +385,22 @@ __global__ void __launch_bounds__(32) k_conv_wgrad(const __nv_bfloat16* __restri
   }
 }
 
-// dw[e] += sum over the chunks, in chunk order, of part[chunk][e].
-__global__ void k_wgrad_sum(const float* __restrict__ part, float* __restrict__ dw, int nchunk, size_t nw) {
-  for (size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x; e < nw; e += (size_t)gridDim.x * blockDim.x) {
-    float s = 0.f;
-    for (int c = 0; c < nchunk; ++c) s += part[(size_t)c * nw + e];
-    dw[e] += s;
+// dw[e] += sum over the chunks of part[chunk][e]: eight threads per element
+// take every eighth chunk each, in order, and their sums are added in order
+// (one thread per element left the sum of 256 chunks to a chain of dependent
+// adds in a few blocks: 15 us; now bound by the read of the partials).
+__global__ void __launch_bounds__(256) k_wgrad_sum(const float* __restrict__ part, float* __restrict__ dw, int nchunk,
+                                                   size_t nw) {
+  __shared__ float sp[8][32];
+  const size_t e = blockIdx.x * (size_t)32 + threadIdx.x;
+  float v = 0.f;
+  if (e < nw)
+    for (int c = threadIdx.y; c < nchunk; c += 8) v += part[(size_t)c * nw + e];
+  sp[threadIdx.y][threadIdx.x] = v;
+  __syncthreads();
+  if (threadIdx.y == 0 && e < nw) {
+    for (int k = 1; k < 8; ++k) v += sp[k][threadIdx.x];
+    dw[e] += v;
   }
 }
 
@@ -168,20 +413,44 @@ __global__ void k_flip_weights(const __nv_bfloat16* __restrict__ w, __nv_bfloat1
   wt[((size_t)ci * taps + (taps - 1 - t)) * cout + co] = w[i];
 }
 
-__global__ void k_bias_grad(const float* __restrict__ dout, float* __restrict__ db, int npos, int c) {
-  __shared__ float s[256];
-  for (int ch = blockIdx.x; ch < c; ch += gridDim.x) {
-    float v = 0.f;
-    for (int p = threadIdx.x; p < npos; p += blockDim.x) v += dout[(size_t)p * c + ch];
-    s[threadIdx.x] = v;
-    __syncthreads();
-    for (int d = blockDim.x / 2; d > 0; d >>= 1) {
-      if (threadIdx.x < d) s[threadIdx.x] += s[threadIdx.x + d];
-      __syncthreads();
-    }
-    if (threadIdx.x == 0) db[ch] += s[0];
+// db[ch] += sum_p dout[p][ch]: a cluster of eight blocks takes up to 16
+// channels; a thread adds every position of its residue class for its channel
+// (coalesced rows), the block sums go through distributed shared memory and
+// are added in block order, so the result is the same on every run.  One
+// block per channel, striding over whole rows, read each line c times from
+// too few SMs (16 channels at 64^3: 223 us).
+constexpr int BIAS_CLUSTER = 8, BIAS_THREADS = 512;
+__global__ void __cluster_dims__(BIAS_CLUSTER, 1, 1) __launch_bounds__(BIAS_THREADS)
+    k_bias_grad(const float* __restrict__ dout, float* __restrict__ db, int npos, int c) {
+  __shared__ float s[BIAS_THREADS];
+  __shared__ float tot[16];
+  const int tid = threadIdx.x, rank = blockIdx.x % BIAS_CLUSTER, c0 = (blockIdx.x / BIAS_CLUSTER) * 16;
+  const int ch = tid & 15, row = tid >> 4;
+  constexpr int ROWS = BIAS_THREADS / 16;
+  float v[4] = {0.f, 0.f, 0.f, 0.f};
+  if (c0 + ch < c) {
+    const size_t step = (size_t)ROWS * BIAS_CLUSTER;
+    size_t p = (size_t)rank * ROWS + row;
+    for (; p + 3 * step < (size_t)npos; p += 4 * step)
+#pragma unroll
+      for (int k = 0; k < 4; ++k) v[k] += dout[(p + k * step) * c + c0 + ch];
+    for (; p < (size_t)npos; p += step) v[0] += dout[p * c + c0 + ch];
+  }
+  s[tid] = (v[0] + v[1]) + (v[2] + v[3]);
+  __syncthreads();
+  for (int d = ROWS / 2; d > 0; d >>= 1) {
+    if (row < d) s[tid] += s[tid + d * 16];
     __syncthreads();
   }
+  if (tid < 16) tot[tid] = s[tid];
+  cooperative_groups::cluster_group cl = cooperative_groups::this_cluster();
+  cl.sync();
+  if (rank == 0 && tid < 16 && c0 + tid < c) {
+    float t = 0.f;
+    for (int r = 0; r < BIAS_CLUSTER; ++r) t += cl.map_shared_rank(tot, r)[tid];
+    db[c0 + tid] += t;
+  }
+  cl.sync();
 }
 
 // dz = dy * (y > 0) (ReLU backward from the stored activation); also to BF16.
@@ -230,19 +499,28 @@ __global__ void k_pool2_bwd(const float* __restrict__ dout, float* __restrict__ 
 // Nearest x2 upsampling of a (So^3, c1) tensor into channels [0, c1) of a
 // (2So)^3 tensor with c1 + c2 channels, and the copy of the skip tensor
 // (c2 channels) into channels [c1, c1 + c2).
+// VEC channels per thread (8 when c1, c2 and the pointers allow 16-byte moves,
+// else 1; element-wise at 128^3 x 48 channels: 357 us against the 45 us that
+// its bytes take).
+template <int VEC>
 __global__ void k_up2_concat(const __nv_bfloat16* __restrict__ lo, const __nv_bfloat16* __restrict__ skip,
                              __nv_bfloat16* __restrict__ out, int S, int c1, int c2) {
-  const int c = c1 + c2, So = S / 2;
-  const size_t n = (size_t)S * S * S * c;
+  const int cv = (c1 + c2) / VEC, So = S / 2;
+  const size_t n = (size_t)S * S * S * cv;
   for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
-    const int ch = (int)(i % c);
-    const size_t p = i / c;
+    const unsigned p = n >> 32 ? (unsigned)(i / (unsigned)cv) : (unsigned)i / (unsigned)cv;
+    const int ch = (int)(i - (size_t)p * cv) * VEC;
+    const __nv_bfloat16* src;
     if (ch < c1) {
-      const int x = (int)(p % S), y = (int)((p / S) % S), z = (int)(p / ((size_t)S * S));
-      out[i] = lo[((size_t)(x / 2) + (size_t)So * ((y / 2) + (size_t)So * (z / 2))) * c1 + ch];
+      const unsigned x = p % S, y = (p / S) % S, z = p / ((unsigned)S * S);
+      src = lo + ((size_t)(x / 2) + (size_t)So * ((y / 2) + (size_t)So * (z / 2))) * c1 + ch;
     } else {
-      out[i] = skip[p * c2 + (ch - c1)];
+      src = skip + (size_t)p * c2 + (ch - c1);
     }
+    if constexpr (VEC == 8)
+      reinterpret_cast<uint4*>(out)[i] = *reinterpret_cast<const uint4*>(src);
+    else
+      out[i] = *src;
   }
 }
 
@@ -363,7 +641,7 @@ __global__ void k_adam(float* __restrict__ p, const float* __restrict__ g, float
 // [solid indicator, Q xx,xy,xz,yy,yz, R/32, p/64, 20 w] from FP64 SoA fields.
 __global__ void k_pack_input(const double* __restrict__ solid, const double* __restrict__ q, float r, float pitch,
                              float w, __nv_bfloat16* __restrict__ x16, float* __restrict__ base, float* __restrict__ fluid,
-                             double* __restrict__ nfluid, int npos, int cpad) {
+                             double* __restrict__ nfluid, int npos, int cpad, bool vec) {
   int cnt = 0;
   for (int p = blockIdx.x * blockDim.x + threadIdx.x; p < npos; p += gridDim.x * blockDim.x) {
     cnt += solid[p] < 0.0;
@@ -373,7 +651,17 @@ __global__ void k_pack_input(const double* __restrict__ solid, const double* __r
       v[1 + c] = (float)q[(size_t)c * npos + p];
       if (base) base[(size_t)p * 5 + c] = v[1 + c];
     }
-    for (int c = 0; c < cpad; ++c) x16[(size_t)p * cpad + c] = __float2bfloat16_rn(c < 9 ? v[c] : 0.f);
+    if (vec) {  // cpad == 16: the position's 32 bytes in two stores
+      __nv_bfloat162 h[8];
+#pragma unroll
+      for (int k = 0; k < 8; ++k)
+        h[k] = __floats2bfloat162_rn(2 * k < 9 ? v[2 * k] : 0.f, 2 * k + 1 < 9 ? v[2 * k + 1] : 0.f);
+      uint4* d = reinterpret_cast<uint4*>(x16 + (size_t)p * 16);
+      d[0] = *reinterpret_cast<uint4*>(h);
+      d[1] = *reinterpret_cast<uint4*>(h + 4);
+    } else {
+      for (int c = 0; c < cpad; ++c) x16[(size_t)p * cpad + c] = __float2bfloat16_rn(c < 9 ? v[c] : 0.f);
+    }
     if (fluid) fluid[p] = sol ? 0.f : 1.f;
   }
   if (nfluid) {
@@ -430,6 +718,54 @@ static inline int grid_for(size_t n, int bs = 256) {
   return (int)(g > 65535 * 8 ? 65535 * 8 : (g < 1 ? 1 : g));
 }
 
+static inline bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15) == 0; }
+
+template <int NT, int MT, int NW, int TX, int TY, int TZ>
+static int launch_conv_tile(const __nv_bfloat16* in, const __nv_bfloat16* w, const float* bias, float* out32,
+                            __nv_bfloat16* out16, int W, int H, int D, int cin, int cout, int relu, cudaStream_t s) {
+  constexpr int smem = ((TX + 2) * (TY + 2) * (TZ + 2) + 27 * NT * 8) * 32;
+  auto* fn = k_conv_tile<NT, MT, NW, TX, TY, TZ>;
+  if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess) return LC_NN_ERR_CUDA;
+  const int ntx = (W + TX - 1) / TX, nty = (H + TY - 1) / TY, ntz = (D + TZ - 1) / TZ;
+  fn<<<dim3((unsigned)ntx * nty * ntz, cout / (NT * 8)), 32 * NW, smem, s>>>(in, w, bias, out32, out16, W, H, D, cin,
+                                                                            cout, relu, ntx, nty);
+  return cudaGetLastError() == cudaSuccess ? LC_NN_OK : LC_NN_ERR_CUDA;
+}
+
+// Boxes of 16 x 8 x 4 positions and all output channels per block while they
+// fill the GPU (152 SMs x 2 blocks), else boxes of 8 x 4 x 4 positions with
+// the output channels split in groups of 16 over the blocks.
+static int conv_tiled(const __nv_bfloat16* in, const __nv_bfloat16* w, const float* bias, float* out32,
+                      __nv_bfloat16* out16, int W, int H, int D, int cin, int cout, int relu, cudaStream_t s) {
+  if (cout != 8 && cout % 16) return LC_NN_ERR_ARG;
+  const long long big = (long long)((W + 15) / 16) * ((H + 7) / 8) * ((D + 3) / 4);
+#define LCNN_BIG(NT) return launch_conv_tile<NT, 4, 8, 16, 8, 4>(in, w, bias, out32, out16, W, H, D, cin, cout, relu, s)
+  if (big >= 256) {
+    switch (cout / 8) {
+      case 1: LCNN_BIG(1);
+      case 2: LCNN_BIG(2);
+      case 4: case 8: LCNN_BIG(4);
+      case 6: LCNN_BIG(6);
+      case 10: LCNN_BIG(5);
+      default: return LC_NN_ERR_ARG;
+    }
+  }
+#undef LCNN_BIG
+  if (cout == 8) return launch_conv_tile<1, 2, 4, 8, 4, 4>(in, w, bias, out32, out16, W, H, D, cin, cout, relu, s);
+  return launch_conv_tile<2, 2, 4, 8, 4, 4>(in, w, bias, out32, out16, W, H, D, cin, cout, relu, s);
+}
+
+template <int TPW, int TY, int TZ>
+static int launch_wgrad_tile(const __nv_bfloat16* dout, const __nv_bfloat16* in, float* part, int W, int H, int D,
+                             int cin, int cout, int nchunk, cudaStream_t s) {
+  constexpr int smem = (18 * (TY + 2) * (TZ + 2) + 1 + 16 * TY * TZ) * 32;
+  auto* fn = k_wgrad_tile<TPW, TY, TZ>;
+  if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess) return LC_NN_ERR_CUDA;
+  fn<<<dim3(nchunk, (cout / 16) * (cin / 16), 3 / TPW), 288, smem, s>>>(
+      dout, in, part, W, H, D, cin, cout, (W + 15) / 16, (H + TY - 1) / TY, (D + TZ - 1) / TZ, nchunk);
+  return cudaGetLastError() == cudaSuccess ? LC_NN_OK : LC_NN_ERR_CUDA;
+}
+
 }  // namespace lcnn
 
 using namespace lcnn;
@@ -447,6 +783,9 @@ int lc_nn_conv3d_fwd(const void* in, const void* w, const float* bias, float* ou
   auto* a = (const __nv_bfloat16*)in;
   auto* b = (const __nv_bfloat16*)w;
   auto* o16 = (__nv_bfloat16*)out16;
+  // 3x3x3: input tiles in shared memory (16-byte copies, so aligned tensors);
+  // 1x1x1 has no taps to share, and unaligned tensors take 4-byte loads
+  if (taps == 27 && aligned16(in) && aligned16(w)) return conv_tiled(a, b, bias, out32, o16, W, H, D, cin, cout, relu, s);
   switch (cout / 8) {
     case 1: k_conv_fwd<1><<<grid, 128, 0, s>>>(a, b, bias, out32, o16, npos, W, H, D, cin, taps, relu); break;
     case 2: k_conv_fwd<2><<<grid, 128, 0, s>>>(a, b, bias, out32, o16, npos, W, H, D, cin, taps, relu); break;
@@ -495,6 +834,19 @@ int lc_nn_conv3d_wgrad(const void* dout, const void* in, float* dw, float* parti
   cudaStream_t s = (cudaStream_t)stream;
   auto* a = (const __nv_bfloat16*)dout;
   auto* b = (const __nv_bfloat16*)in;
+  const size_t nw = (size_t)cout * taps * cin;
+  const dim3 sblk(32, 8);
+  const unsigned sgrid = (unsigned)((nw + 31) / 32);
+  if (taps == 27 && cin % 16 == 0 && aligned16(dout) && aligned16(in)) {
+    // the boxes of the chunks are summed in box order; the taps of one chunk
+    // go to three blocks where the chunks alone leave SMs idle
+    const int rc = nchunk * (cout / 16) * (cin / 16) >= 256
+                       ? launch_wgrad_tile<3, 8, 4>(a, b, partial, W, H, D, cin, cout, nchunk, s)
+                       : launch_wgrad_tile<1, 4, 4>(a, b, partial, W, H, D, cin, cout, nchunk, s);
+    if (rc != LC_NN_OK) return rc;
+    k_wgrad_sum<<<sgrid, sblk, 0, s>>>(partial, dw, nchunk, nw);
+    return cudaGetLastError() == cudaSuccess ? LC_NN_OK : LC_NN_ERR_CUDA;
+  }
   switch (cin / 8) {
     case 1: k_conv_wgrad<1><<<grid, 32, 0, s>>>(a, b, partial, npos, W, H, D, cin, cout, taps, chunk); break;
     case 2: k_conv_wgrad<2><<<grid, 32, 0, s>>>(a, b, partial, npos, W, H, D, cin, cout, taps, chunk); break;
@@ -503,13 +855,12 @@ int lc_nn_conv3d_wgrad(const void* dout, const void* in, float* dw, float* parti
     case 10: k_conv_wgrad<10><<<grid, 32, 0, s>>>(a, b, partial, npos, W, H, D, cin, cout, taps, chunk); break;
     default: return LC_NN_ERR_ARG;
   }
-  const size_t nw = (size_t)cout * taps * cin;
-  k_wgrad_sum<<<grid_for(nw), 256, 0, s>>>(partial, dw, nchunk, nw);
+  k_wgrad_sum<<<sgrid, sblk, 0, s>>>(partial, dw, nchunk, nw);
   return cudaGetLastError() == cudaSuccess ? LC_NN_OK : LC_NN_ERR_CUDA;
 }
 
 int lc_nn_bias_grad(const float* dout, float* db, int npos, int c, void* stream) {
-  k_bias_grad<<<c, 256, 0, (cudaStream_t)stream>>>(dout, db, npos, c);
+  k_bias_grad<<<(c + 15) / 16 * BIAS_CLUSTER, BIAS_THREADS, 0, (cudaStream_t)stream>>>(dout, db, npos, c);
   return cudaGetLastError() == cudaSuccess ? LC_NN_OK : LC_NN_ERR_CUDA;
 }
 
@@ -537,8 +888,13 @@ int lc_nn_pool2_bwd(const float* dout, float* din, int S, int c, void* stream) {
 
 int lc_nn_up2_concat(const void* lo, const void* skip, void* out, int S, int c1, int c2, void* stream) {
   if (S % 2) return LC_NN_ERR_ARG;
-  k_up2_concat<<<grid_for((size_t)S * S * S * (c1 + c2)), 256, 0, (cudaStream_t)stream>>>(
-      (const __nv_bfloat16*)lo, (const __nv_bfloat16*)skip, (__nv_bfloat16*)out, S, c1, c2);
+  const size_t n = (size_t)S * S * S * (c1 + c2);
+  if (c1 % 8 == 0 && c2 % 8 == 0 && aligned16(lo) && aligned16(skip) && aligned16(out))
+    k_up2_concat<8><<<grid_for(n / 8), 256, 0, (cudaStream_t)stream>>>(
+        (const __nv_bfloat16*)lo, (const __nv_bfloat16*)skip, (__nv_bfloat16*)out, S, c1, c2);
+  else
+    k_up2_concat<1><<<grid_for(n), 256, 0, (cudaStream_t)stream>>>(
+        (const __nv_bfloat16*)lo, (const __nv_bfloat16*)skip, (__nv_bfloat16*)out, S, c1, c2);
   return cudaGetLastError() == cudaSuccess ? LC_NN_OK : LC_NN_ERR_CUDA;
 }
 
@@ -575,7 +931,8 @@ int lc_nn_pack_input(const double* solid, const double* q, double R, double pitc
                      float* fluid, double* nfluid, int npos, int cpad, void* stream) {
   if (cpad < 9) return LC_NN_ERR_ARG;
   k_pack_input<<<grid_for(npos), 256, 0, (cudaStream_t)stream>>>(solid, q, (float)R, (float)pitch, (float)w,
-                                                                   (__nv_bfloat16*)x16, base, fluid, nfluid, npos, cpad);
+                                                                   (__nv_bfloat16*)x16, base, fluid, nfluid, npos, cpad,
+                                                                   cpad == 16 && aligned16(x16));
   return cudaGetLastError() == cudaSuccess ? LC_NN_OK : LC_NN_ERR_CUDA;
 }
 

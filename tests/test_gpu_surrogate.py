@@ -89,6 +89,36 @@ def test_conv_fwd_dgrad_wgrad(P, cin, cout, taps):
         assert rel((dw3 - 1.0).cpu().numpy(), dw_ref) < 1e-5  # accumulated onto dw
 
 
+@pytest.mark.parametrize("cin,cout,D,H,W", [(16, 16, 72, 36, 40), (48, 16, 72, 36, 40), (16, 80, 65, 34, 50),
+                                            (32, 48, 5, 7, 9), (16, 32, 1, 3, 17)])
+def test_conv_tiles(P, cin, cout, D, H, W):
+    """The tiled 3x3x3 kernels on both box sizes, ragged in every direction and smaller than a box: forward, input
+    gradient and weight gradient against the FP64 reference on BF16-exact inputs (error: FP32 accumulation)."""
+    L = P.lib()
+    rng = np.random.default_rng(cin + cout + D)
+    x, w = bf16_exact(rng.standard_normal((D, H, W, cin))), bf16_exact(rng.standard_normal((cout, 27, cin)) / 20)
+    dz = bf16_exact(rng.standard_normal((D, H, W, cout)))
+    out = torch.empty((D * H * W, cout), dtype=torch.float32, device="cuda")
+    din = torch.empty((D * H * W, cin), dtype=torch.float32, device="cuda")
+    wt = torch.empty(cout * 27 * cin, dtype=torch.bfloat16, device="cuda")
+    dw = torch.zeros((cout, 27, cin), dtype=torch.float32, device="cuda")
+    db = torch.zeros(cout, dtype=torch.float32, device="cuda")
+    part = torch.empty(L.lc_nn_wgrad_partial_floats(W, H, D, cin, cout, 27), dtype=torch.float32, device="cuda")
+    X, Wt, Z = dev16(x), dev16(w), dev16(dz)
+    assert L.lc_nn_conv3d_fwd(ptr(X), ptr(Wt), None, ptr(out), None, W, H, D, cin, cout, 27, 0, None) == 0
+    assert L.lc_nn_conv3d_dgrad(ptr(Z), ptr(Wt), ptr(wt), ptr(din), None, W, H, D, cin, cout, 27, None) == 0
+    assert L.lc_nn_conv3d_wgrad(ptr(Z), ptr(X), ptr(dw), ptr(part), W, H, D, cin, cout, 27, None) == 0
+    assert L.lc_nn_bias_grad(ptr(dev32(dz)), ptr(db), D * H * W, cout, None) == 0
+    torch.cuda.synchronize()
+    dx_ref, dw_ref, db_ref = nn.conv_bwd(x, w, dz)
+    assert rel(out.cpu().numpy().reshape(D, H, W, cout), nn.conv(x, w, np.zeros(cout))) < 1e-5
+    assert rel(din.cpu().numpy().reshape(D, H, W, cin), dx_ref) < 1e-5
+    assert rel(dw.cpu().numpy(), dw_ref) < 1e-5
+    assert rel(db.cpu().numpy(), db_ref) < 1e-5
+    # an output-channel count that has no kernel stays refused
+    assert L.lc_nn_conv3d_fwd(ptr(X), ptr(Wt), None, ptr(out), None, W, H, D, cin, 24, 27, 0, None) != 0
+
+
 def test_pool_upsample_kernels(P):
     L = P.lib()
     rng = np.random.default_rng(7)
