@@ -348,15 +348,18 @@ class Solver:
         """Components of the defect nodes (lc_lb_defects): counts, roots,
         sizes, centroids [n, 3] and gyration tensors [n, 6]."""
         nd, nc = C.c_longlong(), C.c_longlong()
-        self._check(self.L.lc_lb_defects(self.h, float(thr), 0, C.byref(nd), C.byref(nc), None, None, None, None))
-        k = nc.value
-        root = np.empty(k, np.int64)
-        size = np.empty(k, np.int64)
-        cen = np.empty((k, 3))
-        gyr = np.empty((k, 6))
         lp = C.POINTER(C.c_longlong)
-        self._check(self.L.lc_lb_defects(self.h, float(thr), k, C.byref(nd), C.byref(nc), root.ctypes.data_as(lp),
-                                         size.ctypes.data_as(lp), _dp(cen), _dp(gyr)))
+        cap = 1024  # most textures hold fewer loops; more take a second call with room for all
+        while True:
+            root, size = np.empty(cap, np.int64), np.empty(cap, np.int64)
+            cen, gyr = np.empty((cap, 3)), np.empty((cap, 6))
+            self._check(self.L.lc_lb_defects(self.h, float(thr), cap, C.byref(nd), C.byref(nc),
+                                             root.ctypes.data_as(lp), size.ctypes.data_as(lp), _dp(cen), _dp(gyr)))
+            k = nc.value
+            if k <= cap:
+                break
+            cap = k
+        root, size, cen, gyr = (a[:k].copy() for a in (root, size, cen, gyr))
         return dict(n_defect=nd.value, n_comp=nc.value, root=root, size=size, centroid=cen, gyration=gyr)
 
     def defect_labels(self, thr=0.435, out=None):

@@ -18,7 +18,7 @@ SOURCES = ["lclb_kernels.cu", "lclb_api.cu", "lclb_defects.cu", "lcnn_kernels.cu
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 NVCC_FLAGS = ["-O3", "-std=c++17", "-lineinfo", "-Xcompiler", "-fPIC", "-Xcompiler", "-O2",
               "-Xcompiler", "-ffp-contract=off",
-              "--expt-relaxed-constexpr", "-I", INCLUDE, "-I", CSRC]
+              "--split-compile", "0", "--expt-relaxed-constexpr", "-I", INCLUDE, "-I", CSRC]
 
 
 def nvcc() -> str:

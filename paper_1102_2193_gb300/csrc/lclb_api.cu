@@ -1698,7 +1698,7 @@ int lc_lb_defects(lc_lb* h, double thr, size_t cap, long long* n_defect, long lo
     double* gyr = cen + 3 * (size_t)nc;
     int rc = LC_OK;
     if (cudaMemsetAsync(tmp, 0, ib + sizeof(double) * 15 * (size_t)nc, g->stream) != cudaSuccess ||
-        launch_defects_stats(g->d_boxes, h->index, N, nc, h->def, h->def + N, dsz, circ, cen, gyr, g->stream) !=
+        launch_defects_stats(g->d_boxes, h->index, N, h->hb.nx + h->hb.ny + h->hb.nz, nc, h->def, h->def + N, dsz, circ, cen, gyr, g->stream) !=
             cudaSuccess ||
         cudaMemcpyAsync(hl.data(), h->def + 2 * (size_t)N, sizeof(int) * nc, cudaMemcpyDeviceToHost, g->stream) !=
             cudaSuccess ||
@@ -1871,7 +1871,7 @@ int lc_lb_diagnostics_noalloc(lc_lb* h, lc_diag* out) {
   if (int rc = h_check(h)) return rc;
   if (!out) return fail(&h->err, LC_ERR_ARG, "null output");
   const int nb = diag_state_blocks(h->hb.N);
-  if (nb > NOALLOC_MAX_BLOCKS)
+  if (h->hb.N > NOALLOC_MAX_BLOCKS * 256 || nb > NOALLOC_MAX_BLOCKS)
     return fail(&h->err, LC_ERR_ARG,
                 "box of %d nodes exceeds the %d-node limit of the allocation-free diagnostics", h->hb.N,
                 NOALLOC_MAX_BLOCKS * 256);

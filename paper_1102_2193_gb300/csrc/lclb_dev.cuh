@@ -196,6 +196,49 @@ __device__ __forceinline__ T qab(const T* q, int a, int b) {
   return -q[0] - q[3];
 }
 
+// Whether every eigenvalue of the symmetric traceless Q lies below t, decided
+// in FP32 where that is safe: 1 yes, 0 no, -1 too close to call.  t I - Q is
+// positive definite exactly when its three leading principal minors are
+// positive (Sylvester's criterion); with M the sum of |t| and the |entries|,
+// the FP32 evaluation (inputs rounded) of the minors is within 10 u M,
+// 40 u M^2 and 150 u M^3 of the exact ones (u = 6e-8), so a minor further than
+// the margins below from zero has its true sign.  FP64 runs at 1/64 of the
+// FP32 rate on this GPU, and almost every node is far from the threshold.
+__device__ __forceinline__ int below_f32(const float q[5], float t) {
+  const float m00 = t - q[0], m11 = t - q[3], m22 = t + q[0] + q[3];
+  const float M = fabsf(t) + fabsf(q[0]) + fabsf(q[1]) + fabsf(q[2]) + fabsf(q[3]) + fabsf(q[4]);
+  if (!(M < 1e9f)) return -1;
+  const float e1 = 1e-6f * M, e2 = 4e-6f * M * M, e3 = 1.6e-5f * M * M * M;
+  if (m00 < -e1) return 0;
+  if (!(m00 > e1)) return -1;
+  const float p2 = m00 * m11 - q[1] * q[1];
+  if (p2 < -e2) return 0;
+  if (!(p2 > e2)) return -1;
+  const float det = m00 * (m11 * m22 - q[4] * q[4]) - q[1] * (q[1] * m22 + q[4] * q[2]) - q[2] * (q[1] * q[4] + m11 * q[2]);
+  if (det < -e3) return 0;
+  return det > e3 ? 1 : -1;
+}
+
+// Sum and first moments of the 19 deviations in FP64, through the sums and
+// differences of opposite directions (39 additions instead of the 76 of the
+// 19 x 4 products; FP64 issue bounds the kernels that call it).
+template <typename T>
+__device__ __forceinline__ void moments_f64(const T df[NQ], double& drho, double m[3], bool want_m = true) {
+  drho = (double)df[0];
+  m[0] = m[1] = m[2] = 0.0;
+#pragma unroll
+  for (int q = 1; q < NQ; q += 2) {
+    const double a = (double)df[q], b = (double)df[q + 1];
+    drho += a + b;
+    if (want_m) {
+      const double d = a - b;
+      if (cx(q)) m[0] += cx(q) > 0 ? d : -d;
+      if (cy(q)) m[1] += cy(q) > 0 ? d : -d;
+      if (cz(q)) m[2] += cz(q) > 0 ? d : -d;
+    }
+  }
+}
+
 template <typename T>
 __device__ __forceinline__ T ldg(const T* p) { return __ldg(p); }
 

@@ -2133,48 +2133,56 @@ __global__ void k_export(const DevBox* __restrict__ boxes, int b, int which, dou
     for (int q = 0; q < NQ; ++q) out[(size_t)q * N + i] = wq(q) * B.p.rho0 + (double)df[q];
     return;
   }
-  double drho = 0.0, mm[3] = {0.0, 0.0, 0.0};
-  for (int q = 0; q < NQ; ++q) {
-    drho += (double)df[q];
-    mm[0] += cx(q) * (double)df[q];
-    mm[1] += cy(q) * (double)df[q];
-    mm[2] += cz(q) * (double)df[q];
-  }
+  double drho, mm[3];
+  moments_f64(df, drho, mm, which != EXP_RHO);
   const double rho = B.p.rho0 + drho;
   if (which == EXP_RHO) {
     out[i] = rho;
     return;
   }
   const T* F = static_cast<const T*>(B.F);
+  const double inv = 1.0 / rho;
   for (int a = 0; a < 3; ++a) {
     const double Fa = (B.p.lc_on ? (double)F[(size_t)a * N + i] : 0.0) + B.p.g[a];
-    out[(size_t)a * N + i] = (mm[a] + 0.5 * Fa) / rho;
+    out[(size_t)a * N + i] = (mm[a] + 0.5 * Fa) * inv;
   }
 }
 
 // Diagnostics per block: [0] sum(df), [1..3] sum(df c), [4] fluid nodes,
-// [5] defect nodes (3/2 lambda_max(Q) < 0.435).
+// [5] defect nodes (3/2 lambda_max(Q) < 0.435).  Bound by FP64 issue: the
+// moments take 39 FP64 additions per node, a thread sums DIAG_PER nodes before
+// the block reduction, and the defect test runs in FP32 except at nodes too
+// close to the threshold (with the closed-form eigenvalue in FP64 at every
+// node and 19 x 4 products: 1102 us at 128^3).
+constexpr int DIAG_PER = 4;
 template <typename T>
 __global__ void __launch_bounds__(256) k_diag_state(const DevBox* __restrict__ boxes, int b, double* __restrict__ part) {
   const DevBox& B = boxes[b];
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
   double v[6] = {0, 0, 0, 0, 0, 0};
   __shared__ double sred[32 * 6];
-  if (i < B.N) {
+  int nfl = 0, ndef = 0;
+  const int nx = B.nx, ny = B.ny, N = B.N;
+  for (int r = 0; r < DIAG_PER; ++r) {
+    const long long il = ((long long)blockIdx.x * DIAG_PER + r) * 256 + threadIdx.x;
+    if (il >= N) break;
+    const int i = (int)il;
     const uint8_t m = B.mask[i];
-    if (!(m & IDMASK)) {
-      const int x = i % B.nx, y = (i / B.nx) % B.ny, z = i / (B.nx * B.ny);
-      T df[NQ];
-      pull(B, static_cast<const T*>(B.f[B.st->fpar]), x, y, z, i, m, B.st->pre_valid != 0, df);
-      for (int q = 0; q < NQ; ++q) {
-        v[0] += (double)df[q];
-        v[1] += cx(q) * (double)df[q];
-        v[2] += cy(q) * (double)df[q];
-        v[3] += cz(q) * (double)df[q];
-      }
-      v[4] = 1.0;
-      double q[5];
-      for (int k = 0; k < 5; ++k) q[k] = load_q<T>(B, i, k);
+    if (m & IDMASK) continue;
+    const int x = i % nx, y = (i / nx) % ny, z = i / (nx * ny);
+    T df[NQ];
+    pull(B, static_cast<const T*>(B.f[B.st->fpar]), x, y, z, i, m, B.st->pre_valid != 0, df);
+    double drho, mom[3];
+    moments_f64(df, drho, mom);
+    v[0] += drho;
+    v[1] += mom[0];
+    v[2] += mom[1];
+    v[3] += mom[2];
+    ++nfl;
+    double q[5];
+    for (int k = 0; k < 5; ++k) q[k] = load_q<T>(B, i, k);
+    const float qf[5] = {(float)q[0], (float)q[1], (float)q[2], (float)q[3], (float)q[4]};
+    int low = below_f32(qf, 0.29f);
+    if (low < 0) {
       // largest eigenvalue of the traceless symmetric Q (closed form, as in principal_dir)
       double a00 = q[0], a01 = q[1], a02 = q[2], a11 = q[3], a12 = q[4], a22 = -q[0] - q[3];
       double p1 = a01 * a01 + a02 * a02 + a12 * a12;
@@ -2184,38 +2192,39 @@ __global__ void __launch_bounds__(256) k_diag_state(const DevBox* __restrict__ b
         double p = sqrt(p2 / 6.0);
         double b00 = a00 / p, b01 = a01 / p, b02 = a02 / p, b11 = a11 / p, b12 = a12 / p, b22 = a22 / p;
         double det = b00 * (b11 * b22 - b12 * b12) - b01 * (b01 * b22 - b12 * b02) + b02 * (b01 * b12 - b11 * b02);
-        double r = fmin(1.0, fmax(-1.0, det / 2.0));
-        lam = 2.0 * p * cos(acos(r) / 3.0);
+        double r3 = fmin(1.0, fmax(-1.0, det / 2.0));
+        lam = 2.0 * p * cos(acos(r3) / 3.0);
       }
-      v[5] = (1.5 * lam < 0.435) ? 1.0 : 0.0;
+      low = 1.5 * lam < 0.435;
     }
+    ndef += low;
   }
+  v[4] = (double)nfl;
+  v[5] = (double)ndef;
   block_sum<6>(v, sred);
   if (threadIdx.x == 0)
     for (int k = 0; k < 6; ++k) part[6 * blockIdx.x + k] = v[k];
 }
 
-// Deterministic sum of n records of width w (column k) starting at rec0;
-// out[k] = sum, or max for columns flagged in maxmask.
+// Deterministic sum of n records of width w starting at rec0, one block per
+// column k; out[k] = sum, or max for columns flagged in maxmask.
 __global__ void __launch_bounds__(256) k_reduce(const double* __restrict__ part, int rec0, int n, int w,
                                                 unsigned maxmask, double* __restrict__ out) {
   __shared__ double s[256];
-  for (int k = 0; k < w; ++k) {
-    const bool ismax = (maxmask >> k) & 1u;
-    double v = 0.0;
-    for (int r = threadIdx.x; r < n; r += 256) {
-      const double x = part[(size_t)(rec0 + r) * w + k];
-      v = ismax ? fmax(v, x) : v + x;
-    }
-    s[threadIdx.x] = v;
-    __syncthreads();
-    for (int d = 128; d > 0; d >>= 1) {
-      if (threadIdx.x < d) s[threadIdx.x] = ismax ? fmax(s[threadIdx.x], s[threadIdx.x + d]) : s[threadIdx.x] + s[threadIdx.x + d];
-      __syncthreads();
-    }
-    if (threadIdx.x == 0) out[k] = s[0];
+  const int k = blockIdx.x;
+  const bool ismax = (maxmask >> k) & 1u;
+  double v = 0.0;
+  for (int r = threadIdx.x; r < n; r += 256) {
+    const double x = part[(size_t)(rec0 + r) * w + k];
+    v = ismax ? fmax(v, x) : v + x;
+  }
+  s[threadIdx.x] = v;
+  __syncthreads();
+  for (int d = 128; d > 0; d >>= 1) {
+    if (threadIdx.x < d) s[threadIdx.x] = ismax ? fmax(s[threadIdx.x], s[threadIdx.x + d]) : s[threadIdx.x] + s[threadIdx.x + d];
     __syncthreads();
   }
+  if (threadIdx.x == 0) out[k] = s[0];
 }
 
 // ---------------------------------------------------------------------------
@@ -2692,16 +2701,16 @@ cudaError_t launch_rediscretise(int prec, DevBox* boxes, int nboxes, const int2*
   return cudaGetLastError();
 }
 
-int diag_state_blocks(int N) { return nblk(N, 256); }
+int diag_state_blocks(int N) { return (N - 1) / (256 * DIAG_PER) + 1; }
 
 cudaError_t launch_diag_state(int prec, const DevBox* boxes, int b, int N, double* part, cudaStream_t s) {
-  if (prec == 0) k_diag_state<float><<<nblk(N, 256), 256, 0, s>>>(boxes, b, part);
-  else k_diag_state<double><<<nblk(N, 256), 256, 0, s>>>(boxes, b, part);
+  if (prec == 0) k_diag_state<float><<<diag_state_blocks(N), 256, 0, s>>>(boxes, b, part);
+  else k_diag_state<double><<<diag_state_blocks(N), 256, 0, s>>>(boxes, b, part);
   return cudaGetLastError();
 }
 
 cudaError_t launch_reduce(const double* part, int rec0, int n, int w, unsigned maxmask, double* out, cudaStream_t s) {
-  k_reduce<<<1, 256, 0, s>>>(part, rec0, n, w, maxmask, out);
+  k_reduce<<<w, 256, 0, s>>>(part, rec0, n, w, maxmask, out);
   return cudaGetLastError();
 }
 
