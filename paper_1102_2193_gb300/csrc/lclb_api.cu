@@ -46,7 +46,6 @@ struct Phase {
   TileCfg cfg;
   int4* d_tiles = nullptr;
   int ntiles = 0;
-  int grid = 0;
   std::vector<int> start, count;  // per box
   double* d_part = nullptr;
   size_t part_cap = 0;
@@ -113,8 +112,12 @@ struct Group {
   // 0 force (diagnostics/export; split variant), 1 lb (split variant), 2 lc,
   // 3 fused force+lb (fused variant), 4 stress, 5 lb from stored stress (stored variant)
   Phase ph[NPHASE];
-  cudaStream_t side = nullptr;   // second stream: link momentum exchange runs beside the Q update
-  cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
+  int2* d_groups = nullptr;      // near-node groups (box, first entry), a multiple of NEAR_PAD per box
+  int ngroups = 0, group_cap = 0;
+  std::vector<int> gstart, gcount;  // groups of each box
+  double* d_npart = nullptr;     // residual record of each group
+  unsigned* d_done = nullptr;    // finished work units per box of k_lc, then the totals
+  unsigned* d_total = nullptr;
   // Step variant: 0 = fused stress/force/LB kernel; 1 = split: the stress/
   // force kernel and the LB kernel run concurrently in z slabs on two streams
   // (LB slab s waits for force slab s only); 2 = stored: H and P stored once
@@ -136,6 +139,8 @@ struct Group {
   std::vector<int2> chunk_f, chunk_lb;       // (first tile, count) per slab, force and LB phases
   int2* d_chunks = nullptr;
   int nchunks = 0, chunk_cap = 0;
+  int2* d_lchunks = nullptr;     // link chunks of the k_lc launch
+  int nlchunks = 0, lchunk_cap = 0;
   int2* d_mob = nullptr;        // (box, colloid) of every mobile colloid
   int nmob = 0, mob_cap = 0;
   double* d_scratch = nullptr;  // FP64 export buffer
@@ -218,15 +223,21 @@ int build_phase(Group* g, int k) {
     P.part_cap = need;
     CK(cudaMemsetAsync(P.d_part, 0, sizeof(double) * need, g->stream), &g->err);
   }
-  P.grid = P.cfg.persistent ? std::min(P.ntiles, g->nsm * P.cfg.persistent) : P.ntiles;
-  if (P.grid < 1) P.grid = 1;
   g->dirty = true;
   return LC_OK;
 }
 
-Launch phase_launch(Group* g, int k, int box = -1) {
+// Whether phase k's launch takes the near-node groups as well as its tiles.
+bool has_groups(int k) { return k == 2 || k == 4 || k == 5; }
+
+void set_grid(Group* g, Launch& L, const TileCfg& cfg, bool persistent, int extra) {
+  const int units = L.ntiles + L.ngroups / cfg.ty + extra;
+  L.grid = std::max(1, cfg.persistent && persistent ? std::min(units, g->nsm * cfg.persistent) : units);
+}
+
+Launch phase_launch(Group* g, int k, int mode, int box = -1) {
   Phase& P = g->ph[k];
-  Launch L;
+  Launch L{};
   L.boxes = g->d_boxes;
   L.zc = P.cfg.zc;
   L.ty = P.cfg.ty;
@@ -234,12 +245,19 @@ Launch phase_launch(Group* g, int k, int box = -1) {
   if (box < 0) {
     L.tiles = P.d_tiles;
     L.ntiles = P.ntiles;
-    L.grid = P.grid;
+    L.ngroups = has_groups(k) ? g->ngroups : 0;
   } else {
     L.tiles = P.d_tiles + P.start[box];
     L.ntiles = P.count[box];
-    L.grid = P.count[box];
+    L.ngroups = 0;
   }
+  L.groups = g->d_groups;
+  L.npart = g->d_npart;
+  L.chunks = g->d_lchunks;
+  L.nchunks = g->nlchunks;
+  L.done = g->d_done;
+  L.total = g->d_total;
+  set_grid(g, L, P.cfg, box < 0, (mode & LC_COMMIT) && k == 2 ? g->nlchunks : 0);
   return L;
 }
 
@@ -266,6 +284,98 @@ int build_chunks(Group* g) {
   if (!ch.empty())
     CK(cudaMemcpyAsync(g->d_chunks, ch.data(), sizeof(int2) * ch.size(), cudaMemcpyHostToDevice, g->stream), &g->err);
   g->dirty = true;
+  return LC_OK;
+}
+
+// Groups of 32 near nodes covering every box's near-list capacity.
+int build_groups(Group* g) {
+  std::vector<int2> gr;
+  g->gstart.assign(g->boxes.size(), 0);
+  g->gcount.assign(g->boxes.size(), 0);
+  for (size_t b = 0; b < g->boxes.size(); ++b) {
+    const int n = (g->boxes[b]->hb.near_cap + 32 * NEAR_PAD - 1) / (32 * NEAR_PAD) * NEAR_PAD;
+    g->gstart[b] = (int)gr.size();
+    g->gcount[b] = n;
+    for (int k = 0; k < n; ++k) gr.push_back(make_int2((int)b, 32 * k));
+  }
+  if ((int)gr.size() > g->group_cap) {
+    if (g->d_groups) g->mem.put(g->d_groups, g->al);
+    if (g->d_npart) g->mem.put(g->d_npart, g->al);
+    g->group_cap = (int)gr.size() + 64;
+    g->d_groups = (int2*)galloc(g, sizeof(int2) * g->group_cap);
+    g->d_npart = (double*)galloc(g, sizeof(double) * 2 * g->group_cap);
+    if (!g->d_groups || !g->d_npart) return fail(&g->err, LC_ERR_OOM, "near group allocation failed");
+    CK(cudaMemsetAsync(g->d_npart, 0, sizeof(double) * 2 * g->group_cap, g->stream), &g->err);
+  }
+  g->ngroups = (int)gr.size();
+  if (!gr.empty())
+    CK(cudaMemcpyAsync(g->d_groups, gr.data(), sizeof(int2) * gr.size(), cudaMemcpyHostToDevice, g->stream), &g->err);
+  g->dirty = true;
+  return LC_OK;
+}
+
+// Link chunks of the k_lc launch of a step (one link per thread; a box whose
+// links cannot change takes its count, else its capacity), and the work units
+// of each box in it: near groups in blocks of ty, link chunks, tiles.
+int build_totals(Group* g) {
+  const Phase& P = g->ph[2];
+  std::vector<unsigned> tot(g->boxes.size());
+  std::vector<int2> ch;
+  for (size_t b = 0; b < g->boxes.size(); ++b) {
+    const lc_lb* h = g->boxes[b];
+    const int step = 32 * P.cfg.ty, n = h->hb.nmobile > 0 ? h->hb.nlinks_cap : h->nlinks;
+    const size_t at = ch.size();
+    for (int s = 0; s < n; s += step) ch.push_back(make_int2((int)b, s));
+    tot[b] = (unsigned)(P.count[b] + g->gcount[b] / P.cfg.ty) + (unsigned)(ch.size() - at);
+  }
+  if ((int)ch.size() > g->lchunk_cap) {
+    if (g->d_lchunks) g->mem.put(g->d_lchunks, g->al);
+    g->lchunk_cap = (int)ch.size() + 64;
+    g->d_lchunks = (int2*)galloc(g, sizeof(int2) * g->lchunk_cap);
+    if (!g->d_lchunks) return fail(&g->err, LC_ERR_OOM, "link chunk allocation failed");
+  }
+  g->nlchunks = (int)ch.size();
+  if (!ch.empty())
+    CK(cudaMemcpyAsync(g->d_lchunks, ch.data(), sizeof(int2) * ch.size(), cudaMemcpyHostToDevice, g->stream), &g->err);
+  CK(cudaMemcpyAsync(g->d_total, tot.data(), sizeof(unsigned) * tot.size(), cudaMemcpyHostToDevice, g->stream), &g->err);
+  return LC_OK;
+}
+
+// Near-node list of box h after its geometry is built: static boxes get the
+// exact capacity, boxes with a mobile colloid a bound over its motion (near
+// nodes lie within sqrt 2 of the surface; a shell's nodes are at most the
+// volume of the shell widened by half a cell diagonal).
+int build_near(lc_lb* h) {
+  Group* g = h->g;
+  DevBox& B = h->hb;
+  cudaStream_t s = g->stream;
+  int n = 0;
+  CK(cudaMemsetAsync(B.nnear, 0, sizeof(int), s), &h->err);
+  CK(launch_near_list(g->d_boxes, h->index, B.N, s), &h->err);
+  CK(cudaMemcpyAsync(&n, B.nnear, sizeof(int), cudaMemcpyDeviceToHost, s), &h->err);
+  CK(cudaStreamSynchronize(s), &h->err);
+  double bound = n;
+  if (B.nmobile > 0) {
+    double m = B.wall_z ? 2.0 * B.nx * B.ny : 0.0;
+    for (const DevColloid& C : h->col) {
+      const double o = C.a0 + 2.4, i = std::max(0.0, C.a0 - 0.9);
+      m += 4.0 / 3.0 * M_PI * (o * o * o - i * i * i) + 64.0;
+    }
+    bound = std::min((double)B.N, std::max(bound, m));
+  }
+  const int need = (int)bound;
+  if (need > B.near_cap) {
+    if (B.near_node) g->mem.put(B.near_node, g->al);
+    B.near_cap = 0;
+    B.near_node = (int*)galloc(g, sizeof(int) * (size_t)need);
+    if (!B.near_node) return fail(&h->err, LC_ERR_OOM, "near list allocation failed");
+    B.near_cap = need;
+    int rc = upload_box(g, h);
+    if (rc) return rc;
+    CK(cudaMemsetAsync(B.nnear, 0, sizeof(int), s), &h->err);
+    CK(launch_near_list(g->d_boxes, h->index, B.N, s), &h->err);
+    if ((rc = build_groups(g))) return rc;
+  }
   return LC_OK;
 }
 
@@ -311,10 +421,24 @@ template <typename T>
 void fill_phys(PhysT<T>& o, const DevParams& p) {
   o.rho0 = (T)p.rho0;
   o.omega = (T)(1.0 / p.tau);
-  o.pref = (T)(1.0 - 0.5 / p.tau);
-  o.A0 = (T)p.A0; o.gamma = (T)p.gamma; o.K = (T)p.K; o.q0 = (T)p.q0; o.xi = (T)p.xi; o.Gamma = (T)p.Gamma;
+  o.ptau = (T)(p.tau - 0.5);
+  o.K = (T)p.K;
   o.S0 = (T)p.S0;
   for (int a = 0; a < 3; ++a) o.g[a] = (T)p.g[a];
+}
+
+template <typename T>
+void fill_lck(LcK<T>& o, const DevParams& p) {
+  const double A0g = p.A0 * p.gamma, lin = -p.A0 * (1.0 - p.gamma / 3.0) - 4.0 * p.K * p.q0 * p.q0;
+  o.A0g = (T)A0g; o.nA0g = (T)-A0g; o.nA3 = (T)(-A0g / 3.0); o.c_lin = (T)lin; o.c_lo = (T)(lin - 6.0 * p.K);
+  o.K = (T)p.K; o.nKq0 = (T)(-p.K * p.q0); o.n2Kq0 = (T)(-2.0 * p.K * p.q0); o.Kq0 = (T)(p.K * p.q0);
+  o.f2c = (T)(0.5 * p.A0 * (1.0 - p.gamma / 3.0) + 2.0 * p.K * p.q0 * p.q0);
+  o.f4c = (T)(0.25 * A0g); o.K8 = (T)(0.125 * p.K);
+  o.xi2 = (T)(2.0 * p.xi); o.nt = (T)(-2.0 * p.xi / 3.0); o.nK4 = (T)(-0.25 * p.K);
+  o.up = (T)(1.0 - p.xi); o.dn = (T)(-(1.0 + p.xi)); o.di = (T)(-2.0 * p.xi);
+  o.Gamma = (T)p.Gamma; o.g0 = (T)(0.5 * p.xi); o.g1 = (T)(0.25 * (p.xi + 1.0)); o.g2 = (T)(0.25 * (p.xi - 1.0));
+  o.A2 = (T)(2.0 * A0g); o.nA2 = (T)(-2.0 * A0g);
+  o.two = (T)2; o.ntwo = (T)-2; o.third = (T)(1.0 / 3.0); o.nthird = (T)(-1.0 / 3.0); o.nsix = (T)-6; o.nhalf = (T)-0.5;
 }
 
 // Allocate and initialise one box inside group g.
@@ -334,6 +458,8 @@ int make_box(Group* g, const lc_grid* G, const lc_params* p, lc_lb* h) {
   B.p.flow_on = p->flow_enabled ? 1 : 0;
   fill_phys(B.pf, B.p);
   fill_phys(B.pd, B.p);
+  fill_lck(B.kf, B.p);
+  fill_lck(B.kd, B.p);
   for (int k = 0; k < 2; ++k) {
     B.f[k] = galloc(g, NQ * N * ts);
     B.Q[k] = galloc(g, 5 * N * ts);
@@ -351,8 +477,9 @@ int make_box(Group* g, const lc_grid* G, const lc_params* p, lc_lb* h) {
   B.st = (DevState*)galloc(g, sizeof(DevState));
   B.gerr = g->d_err;
   B.nlinks = (int*)galloc(g, sizeof(int));
+  B.nnear = (int*)galloc(g, sizeof(int));
   if (!B.f[0] || !B.f[1] || !B.Q[0] || !B.Q[1] || !B.u || !B.F || !B.H || !B.P || !B.mask || !B.col || !B.st ||
-      !B.nlinks)
+      !B.nlinks || !B.nnear)
     return fail(&h->err, LC_ERR_OOM, "device allocation failed for a %dx%dx%d box", G->nx, G->ny, G->nz);
   cudaStream_t s = g->stream;
   for (int k = 0; k < 2; ++k) {
@@ -366,6 +493,7 @@ int make_box(Group* g, const lc_grid* G, const lc_params* p, lc_lb* h) {
   CK(cudaMemsetAsync(B.mask, 0, N, s), &h->err);
   CK(cudaMemsetAsync(B.col, 0, sizeof(DevColloid) * MAXCOL, s), &h->err);
   CK(cudaMemsetAsync(B.nlinks, 0, sizeof(int), s), &h->err);
+  CK(cudaMemsetAsync(B.nnear, 0, sizeof(int), s), &h->err);
   int rc = write_state(g, h, 1);
   if (rc) return rc;
   rc = upload_box(g, h);
@@ -393,11 +521,8 @@ Group* new_group(int prec, void* stream, int nboxes, std::string* err) {
     }
     g->own_stream = true;
   }
-  if (cudaStreamCreateWithFlags(&g->side, cudaStreamNonBlocking) != cudaSuccess ||
-      cudaStreamCreateWithFlags(&g->side2, cudaStreamNonBlocking) != cudaSuccess ||
-      cudaEventCreateWithFlags(&g->ev_lb, cudaEventDisableTiming) != cudaSuccess ||
-      cudaEventCreateWithFlags(&g->ev_fork, cudaEventDisableTiming) != cudaSuccess ||
-      cudaEventCreateWithFlags(&g->ev_join, cudaEventDisableTiming) != cudaSuccess) {
+  if (cudaStreamCreateWithFlags(&g->side2, cudaStreamNonBlocking) != cudaSuccess ||
+      cudaEventCreateWithFlags(&g->ev_lb, cudaEventDisableTiming) != cudaSuccess) {
     fail(err, LC_ERR_CUDA, "cannot create the side stream");
     delete g;
     return nullptr;
@@ -411,7 +536,10 @@ Group* new_group(int prec, void* stream, int nboxes, std::string* err) {
   g->d_red = (double*)galloc(g, sizeof(double) * 64);
   g->d_err = (int*)galloc(g, sizeof(int) * 4);
   if (g->d_err) cudaMemsetAsync(g->d_err, 0, sizeof(int) * 4, g->stream);
-  if (!g->d_boxes || !g->d_red || !g->d_err || cudaMallocHost(&g->h_red, sizeof(double) * 64) != cudaSuccess) {
+  g->d_done = (unsigned*)galloc(g, sizeof(unsigned) * 2 * std::max(1, nboxes));
+  if (g->d_done) cudaMemsetAsync(g->d_done, 0, sizeof(unsigned) * 2 * std::max(1, nboxes), g->stream);
+  g->d_total = g->d_done + std::max(1, nboxes);
+  if (!g->d_boxes || !g->d_red || !g->d_err || !g->d_done || cudaMallocHost(&g->h_red, sizeof(double) * 64) != cudaSuccess) {
     fail(err, LC_ERR_OOM, "group allocation failed");
     g->mem.release(g->al);
     if (g->own_stream) cudaStreamDestroy(g->stream);
@@ -428,12 +556,6 @@ void free_group(Group* g) {
   if (g->graph) cudaGraphDestroy(g->graph);
   g->mem.release(g->al);
   if (g->h_red) cudaFreeHost(g->h_red);
-  if (g->side) {
-    cudaStreamSynchronize(g->side);
-    cudaStreamDestroy(g->side);
-  }
-  if (g->ev_fork) cudaEventDestroy(g->ev_fork);
-  if (g->ev_join) cudaEventDestroy(g->ev_join);
   if (g->side2) {
     cudaStreamSynchronize(g->side2);
     cudaStreamDestroy(g->side2);
@@ -503,7 +625,7 @@ void tune_file_store(const TuneKey& key, const std::vector<TileCfg>& c) {
 }
 
 cudaError_t launch_phase(Group* g, int k, int mode, int box = -1) {
-  Launch L = phase_launch(g, k, box);
+  Launch L = phase_launch(g, k, mode, box);
   double* part = g->ph[k].d_part +
                  (box < 0 ? 0 : (size_t)g->ph[k].start[box] * PART_WIDTH[k] * part_records(g->ph[k], k));
   if (k == 0) return launch_force(g->prec, L, mode, part);
@@ -801,7 +923,7 @@ int build_chunks_slab(Group* g) {
 
 cudaError_t launch_range(Group* g, int k, int2 range, int mode, cudaStream_t st) {
   Phase& P = g->ph[k];
-  Launch L;
+  Launch L{};
   L.boxes = g->d_boxes;
   L.zc = P.cfg.zc;
   L.ty = P.cfg.ty;
@@ -1038,10 +1160,8 @@ int check_step_err(Group* g, std::string* err) {
               cbox, with);
 }
 
-// One coupled step: fused stress + body force + collide/stream, then the Q
-// update on the main stream and the link momentum exchange on the side
-// stream (both read only what the fused kernel wrote), joined before the
-// colloid update.
+// One coupled step: stress, body force and collide/stream, then one launch
+// for the Q update, the link momentum exchange and the colloid update.
 int enqueue_force_lb(Group* g) {
   if (g->variant == 1) return enqueue_split(g, FORCE_ACC);
   if (g->variant == 2) {
@@ -1062,15 +1182,7 @@ int enqueue_step(Group* g) {
     return LC_OK;
   }
   if (int rc = enqueue_force_lb(g)) return rc;
-  if (g->nchunks > 0) {
-    CK(cudaEventRecord(g->ev_fork, g->stream), &g->err);
-    CK(cudaStreamWaitEvent(g->side, g->ev_fork, 0), &g->err);
-    CK(launch_links(g->prec, g->d_boxes, g->d_chunks, g->nchunks, g->nchunks, g->side), &g->err);
-    CK(cudaEventRecord(g->ev_join, g->side), &g->err);
-  }
-  CK(launch_phase(g, 2, LC_RESID), &g->err);
-  if (g->nchunks > 0) CK(cudaStreamWaitEvent(g->stream, g->ev_join, 0), &g->err);
-  CK(launch_colloid(g->d_boxes, (int)g->boxes.size(), g->stream), &g->err);
+  CK(launch_phase(g, 2, LC_RESID | LC_COMMIT), &g->err);
   if (g->nmob > 0)
     CK(launch_rediscretise(g->prec, g->d_boxes, (int)g->boxes.size(), g->d_mob, g->nmob, g->nsm, g->stream), &g->err);
   return LC_OK;
@@ -1120,8 +1232,7 @@ int capture(Group* g) {
     cudaGraphDestroy(g->graph);
     g->graph = nullptr;
   }
-  if (g->variant == 3)
-    if (int rc = build_items(g)) return rc;
+  if (int rc = g->variant == 3 ? build_items(g) : build_totals(g)) return rc;
   CK(cudaStreamBeginCapture(g->stream, cudaStreamCaptureModeThreadLocal), &g->err);
   int rc = enqueue_step(g);
   cudaGraph_t gr = nullptr;
@@ -1221,8 +1332,12 @@ int group_step(Group* g, int n) {
   if (rc) return rc;
   const char* env = getenv("LCLB_NO_GRAPH");
   if (env && env[0] == '1') {
-    if (g->variant == 3 && g->dirty) {
-      if ((rc = build_items(g))) return rc;
+    if (g->dirty) {
+      if ((rc = g->variant == 3 ? build_items(g) : build_totals(g))) return rc;
+      if (g->gexec) {  // the graph of the old work lists
+        cudaGraphExecDestroy(g->gexec);
+        g->gexec = nullptr;
+      }
       g->dirty = false;
     }
     for (int s = 0; s < n; ++s)
@@ -1239,11 +1354,17 @@ int box_residual(Group* g, int b, double* rms, double* mx, long long nfluid) {
   Phase& P = g->ph[2];
   const int rec = part_records(P, 2);
   CK(launch_reduce(P.d_part, P.start[b] * rec, P.count[b] * rec, 2, 2u, g->d_red, g->stream), &g->err);
-  CK(cudaMemcpyAsync(g->h_red, g->d_red, 2 * sizeof(double), cudaMemcpyDeviceToHost, g->stream), &g->err);
+  // the near nodes' records are apart from the tiles' (k_step keeps them together)
+  const bool near = g->variant != 3 && g->gcount[b] > 0;
+  if (near)
+    CK(launch_reduce(g->d_npart, g->gstart[b], g->gcount[b], 2, 2u, g->d_red + 2, g->stream), &g->err);
+  CK(cudaMemcpyAsync(g->h_red, g->d_red, 4 * sizeof(double), cudaMemcpyDeviceToHost, g->stream), &g->err);
   CK(cudaStreamSynchronize(g->stream), &g->err);
-  *rms = nfluid > 0 ? std::sqrt(g->h_red[0] / (double)nfluid) : 0.0;
+  const double sum = g->h_red[0] + (near ? g->h_red[2] : 0.0);
+  const double top = near ? std::fmax(g->h_red[1], g->h_red[3]) : g->h_red[1];
+  *rms = nfluid > 0 ? std::sqrt(sum / (double)nfluid) : 0.0;
   if (int rc = check_step_err(g, &g->err)) return rc;
-  *mx = g->h_red[1];
+  *mx = top;
   return LC_OK;
 }
 
@@ -1268,6 +1389,7 @@ int rebuild_geometry(lc_lb* h) {
   int rc = upload_box(g, h);
   if (rc) return rc;
   CK(launch_geometry(g->d_boxes, h->index, h->hb.N, s), &h->err);
+  if ((rc = build_near(h))) return rc;
   // boundary links, colloid by colloid, in node order
   const int nb = (h->hb.N + 255) / 256;
   if ((rc = ensure_iwork(g, (size_t)nb + 8))) return rc;
@@ -1349,6 +1471,7 @@ int lc_lb_create(const lc_grid* grid, const lc_params* params, void* stream, lc_
   if (!rc) rc = rebuild_geometry(h);
   for (int k = 0; k < NPHASE && !rc; ++k) rc = build_phase(g, k);
   if (!rc) rc = build_chunks(g);
+  if (!rc) rc = build_groups(g);
   if (rc) {
     g_err = h->err.empty() ? g->err : h->err;
     free_group(g);
@@ -1926,6 +2049,7 @@ int lc_lb_batch_create(int n, const lc_grid* grids, const lc_params* params, voi
   }
   for (int k = 0; k < NPHASE && !rc; ++k) rc = build_phase(g, k);
   if (!rc) rc = build_chunks(g);
+  if (!rc) rc = build_groups(g);
   if (rc) {
     free_group(g);
     return rc;

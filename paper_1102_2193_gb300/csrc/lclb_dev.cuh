@@ -42,10 +42,26 @@ struct DevParams {
 // never convert from FP64 per node).
 template <typename T>
 struct PhysT {
-  T rho0, omega, pref;  // rho0, 1/tau, 1 - 1/(2 tau)
-  T A0, gamma, K, q0, xi, Gamma, S0;
+  T rho0, omega, ptau;  // rho0, 1/tau, (1 - 1/(2 tau)) tau = tau - 1/2
+  T K, S0;
   T g[3];
 };
+
+// Constants of the liquid-crystal algebra, every combination that the node
+// functions multiply by formed once per box (C the model's constants, in
+// FP64).  The two-node kernels keep a copy with each value twice in shared
+// memory (LcK<f2>), one 8-byte load per packed operand.
+template <typename T>
+struct LcK {
+  T A0g, nA0g, nA3, c_lin, c_lo;   // A0 g, its negative, -A0 g / 3, H: Q beyond -A0 g Tr(Q^2), the same - 6 K
+  T K, nKq0, n2Kq0, Kq0;           // K, -K q0, -2 K q0, K q0
+  T f2c, f4c, K8;                  // f': Tr Q^2, (Tr Q^2)^2, K / 8
+  T xi2, nt, nK4, up, dn, di;      // 2 xi, -2 xi / 3, -K / 4, 1 - xi, -(1 + xi), -2 xi
+  T Gamma, g0, g1, g2;             // xi / 2, (xi + 1) / 4, (xi - 1) / 4
+  T A2, nA2;                       // 2 A0 g, -2 A0 g
+  T two, ntwo, third, nthird, nsix, nhalf;
+};
+constexpr int LCK_N = sizeof(LcK<float>) / sizeof(float);
 
 // One colloid.  X, V, W: current state.  Xb, Vb, Wb: the state used when the
 // post-collision populations now in memory were produced; the bounce-back of
@@ -102,16 +118,26 @@ struct DevBox {
   DevState* st;
   int* gerr;            // error words of the box's group: [0] wait gave up, [1] contact in some box
   int* nlinks;          // device count of boundary links
+  // fluid nodes next to a solid or wall (mask bit NEAR), in no particular order:
+  // device count, capacity (a bound on the count over the box's motion)
+  int* nnear;
+  int* near_node;
+  int near_cap;
+  int pad1;
   int* link_node;       // boundary links of this box, sorted by (colloid, node, dir)
   int8_t* link_dir;
   int8_t* link_col;
   DevParams p;
   PhysT<float> pf;
   PhysT<double> pd;
+  LcK<float> kf;
+  LcK<double> kd;
 };
 
 // FP32 boxes of even width run the two-node paths of the stress kernel and
-// the Q update over tiles 64 nodes wide (those phases' tile lists step x by 64).
+// the Q update over tiles 64 nodes wide (those phases' tile lists step x by
+// 64): a lane holds two nodes, which the packed FP32x2 instructions evaluate
+// at once.
 __host__ __device__ __forceinline__ bool pair_width(int nx, bool fp32) { return fp32 && nx % 2 == 0; }
 __device__ __forceinline__ bool pair_box(const DevBox& B) { return B.pair != 0; }
 
@@ -121,6 +147,13 @@ template <>
 __device__ __forceinline__ const PhysT<float>& phys<float>(const DevBox& B) { return B.pf; }
 template <>
 __device__ __forceinline__ const PhysT<double>& phys<double>(const DevBox& B) { return B.pd; }
+
+template <typename T>
+__device__ __forceinline__ const LcK<T>& lck(const DevBox& B);
+template <>
+__device__ __forceinline__ const LcK<float>& lck<float>(const DevBox& B) { return B.kf; }
+template <>
+__device__ __forceinline__ const LcK<double>& lck<double>(const DevBox& B) { return B.kd; }
 
 // ---------------------------------------------------------------------------
 // Small helpers
@@ -500,20 +533,24 @@ __device__ __forceinline__ void gather_q(const DevBox& B, const T* __restrict__ 
   }
 }
 
-// 1/sqrt(v) in FP64 from the FP32 estimate and one Newton step (relative
-// error ~1e-14 for the unit vectors of the surface values).
+// 1/sqrt(v) in FP64 from the FP32 estimate and Newton steps (FP32 storage:
+// one, relative error ~1e-14; FP64 storage: two, to rounding).
+template <int STEPS>
 __device__ __forceinline__ double rsqrt_f64(double v) {
   double r = (double)rsqrtf((float)v);
-  return r * (1.5 - 0.5 * v * r * r);
+#pragma unroll
+  for (int k = 0; k < STEPS; ++k) r = r * (1.5 - 0.5 * v * r * r);
+  return r;
 }
 
-// Surface order Q0 (Eq. 7) for the nodes next to a solid in FP32 storage, in
-// FP64: the unit normal s at solid node (sx, sy, sz) of colloid c (c < 0: a z
-// wall, n0 = z); homeotropic n0 = s, planar n0 = nf projected on the plane
-// normal to s (nf: the node's director, computed once per node), the
-// tie-break s x e_k as surface_q0.
+// Surface order Q0 (Eq. 7) in FP64: the unit normal s at solid node
+// (sx, sy, sz) of colloid c (c < 0: a z wall, n0 = z); homeotropic n0 = s,
+// planar n0 = nf projected on the plane normal to s (nf: the fluid node's
+// director), the tie-break s x e_k as surface_q0.
+template <typename T>
 __device__ __forceinline__ void surface_q0_near(const DevBox& B, int c, int sx, int sy, int sz, const double nf[3],
                                                 double q0[5]) {
+  constexpr int ST = sizeof(T) == 8 ? 2 : 1;
   double n[3];
   if (c < 0) {
     n[0] = 0.0; n[1] = 0.0; n[2] = 1.0;
@@ -521,7 +558,7 @@ __device__ __forceinline__ void surface_q0_near(const DevBox& B, int c, int sx, 
     const DevColloid& C = B.col[c];
     double d[3];
     disp(B, (double)sx, (double)sy, (double)sz, C.X, d);
-    const double ri = rsqrt_f64(d[0] * d[0] + d[1] * d[1] + d[2] * d[2]);
+    const double ri = rsqrt_f64<ST>(d[0] * d[0] + d[1] * d[1] + d[2] * d[2]);
     const double sv[3] = {d[0] * ri, d[1] * ri, d[2] * ri};
     if (C.anchoring == 0) {
       n[0] = sv[0]; n[1] = sv[1]; n[2] = sv[2];
@@ -540,7 +577,7 @@ __device__ __forceinline__ void surface_q0_near(const DevBox& B, int c, int sx, 
         pv[2] = sv[0] * e[1] - sv[1] * e[0];
         p2 = pv[0] * pv[0] + pv[1] * pv[1] + pv[2] * pv[2];
       }
-      const double pi = rsqrt_f64(p2);
+      const double pi = rsqrt_f64<ST>(p2);
       n[0] = pv[0] * pi; n[1] = pv[1] * pi; n[2] = pv[2] * pi;
     }
   }
@@ -552,317 +589,231 @@ __device__ __forceinline__ void surface_q0_near(const DevBox& B, int c, int sx, 
   q0[4] = S0 * n[1] * n[2];
 }
 
-// FP32 storage, node next to a solid or wall: the derivatives from the
-// compensated values hi + lo of the node and of its face neighbours, each
-// neighbour difference formed as (hi_j - hi_i) + (lo_j - lo_i), and a solid
-// or wall neighbour's surface value as Q0 - Q_i scaled by w/(K + w) (1 for
-// strong anchoring), with Q0 and that difference in FP64.  With hi alone the
-// rounding of Q (~3e-8) enters the Laplacian of every node at the colloid
-// surface, and the colloid's LC force, a small sum of large face terms, would
-// carry it at ~1e-4 relative.  qi receives the node's Q (hi + lo in FP32).
-__device__ __forceinline__ void near_derivatives_f32(const DevBox& B, int x, int y, int z, int i, float qi[5],
-                                                     float dq[3][5], float lap[5]) {
-  const int N = B.N, qpar = B.st->qpar;
-  const float* __restrict__ Q = static_cast<const float*>(B.Q[qpar]);
-  const __nv_bfloat16* __restrict__ Lo = B.Qlo[qpar];
-  float qh[5], ql[5];
-#pragma unroll
-  for (int k = 0; k < 5; ++k) {
-    qh[k] = __ldg(Q + (size_t)k * N + i);
-    ql[k] = __bfloat162float(Lo[(size_t)k * N + i]);
-    qi[k] = qh[k] + ql[k];
-  }
-  int nb[6], zz[2], cf[6];
-  face_neighbours(B, x, y, z, nb, zz);
-  const int nx = B.nx, ny = B.ny;
-  bool planar = false;
-#pragma unroll
-  for (int d = 0; d < 6; ++d) {
-    const int j = nb[d];
-    cf[d] = j < 0 ? -1 : (int)(B.mask[j] & IDMASK) - 1;  // colloid of a solid neighbour, else -1
-    if (cf[d] >= 0 && B.col[cf[d]].anchoring != 0) planar = true;
-  }
-  double nf[3] = {1.0, 0.0, 0.0};
-  if (planar) {
-    double qid[5];
-#pragma unroll
-    for (int k = 0; k < 5; ++k) qid[k] = (double)qh[k] + (double)ql[k];
-    principal_dir<double>(qid, nf);
-  }
-  float dn[6][5];
-#pragma unroll
-  for (int d = 0; d < 6; ++d) {
-    const int j = nb[d];
-    if (j >= 0 && cf[d] < 0) {
-#pragma unroll
-      for (int k = 0; k < 5; ++k)
-        dn[d][k] = (__ldg(Q + (size_t)k * N + j) - qh[k]) + (__bfloat162float(Lo[(size_t)k * N + j]) - ql[k]);
-    } else {
-      int sx = x, sy = y, sz = z;
-      if (d == 0) sx = x + 1 == nx ? 0 : x + 1;
-      if (d == 1) sx = x == 0 ? nx - 1 : x - 1;
-      if (d == 2) sy = y + 1 == ny ? 0 : y + 1;
-      if (d == 3) sy = y == 0 ? ny - 1 : y - 1;
-      if (d == 4) sz = zz[0];
-      if (d == 5) sz = zz[1];
-      const int c = j < 0 ? -1 : cf[d];
-      double q0[5];
-      surface_q0_near(B, c, sx, sy, sz, nf, q0);
-      const double s = c < 0 ? 1.0 : B.col[c].wfac;
-#pragma unroll
-      for (int k = 0; k < 5; ++k) dn[d][k] = (float)(s * ((q0[k] - (double)qh[k]) - (double)ql[k]));
-    }
-  }
-#pragma unroll
-  for (int k = 0; k < 5; ++k) {
-    dq[0][k] = 0.5f * (dn[0][k] - dn[1][k]);
-    dq[1][k] = 0.5f * (dn[2][k] - dn[3][k]);
-    dq[2][k] = 0.5f * (dn[4][k] - dn[5][k]);
-    lap[k] = (dn[0][k] + dn[1][k]) + (dn[2][k] + dn[3][k]) + (dn[4][k] + dn[5][k]);
-  }
-}
-
-// Derivatives from the face-neighbour values: central first differences
-// dq[g][k] = d_g Q_k and the 7-point Laplacian (Sec. 2.2: one stencil at all
-// fluid nodes, surface values standing in for solid neighbours).
+// Derivatives from the face-neighbour values: twice the central first
+// differences, dq[g][k] = 2 d_g Q_k (the halves are taken into the constants
+// of lc_node_d), and the 7-point Laplacian (Sec. 2.2: one stencil at all fluid
+// nodes, surface values standing in for solid neighbours).
 template <typename T>
 __device__ __forceinline__ void derivatives(const T qi[5], const T qn[6][5], T dq[3][5], T lap[5]) {
 #pragma unroll
   for (int k = 0; k < 5; ++k) {
-    dq[0][k] = T(0.5) * (qn[0][k] - qn[1][k]);
-    dq[1][k] = T(0.5) * (qn[2][k] - qn[3][k]);
-    dq[2][k] = T(0.5) * (qn[4][k] - qn[5][k]);
-    lap[k] = (qn[0][k] + qn[1][k]) + (qn[2][k] + qn[3][k]) + (qn[4][k] + qn[5][k]) - T(6) * qi[k];
+    dq[0][k] = qn[0][k] - qn[1][k];
+    dq[1][k] = qn[2][k] - qn[3][k];
+    dq[2][k] = qn[4][k] - qn[5][k];
+    const T n6 = (qn[0][k] + qn[1][k]) + (qn[2][k] + qn[3][k]) + (qn[4][k] + qn[5][k]);
+    lap[k] = n6 + T(-6) * qi[k];
   }
 }
 
-// C_ab = eps_agd d_g Q_db (a "curl" of Q acting on the first index).
-template <typename T>
-__device__ __forceinline__ T curlq(const T dq[3][5], int a, int b) {
-  int a1 = (a + 1) % 3, a2 = (a + 2) % 3;
-  return qab(dq[a1], a2, b) - qab(dq[a2], a1, b);
-}
-
-// Molecular field H = -dF/dQ + Tr(dF/dQ) I/3 (Eq. 2) of the free energy of
-// Eq. 1:
-//   H = -A0(1-g/3) Q + A0 g (Q.Q - Tr(Q^2)/3 I) - A0 g Tr(Q^2) Q + K lap Q
-//       - 2 K q0 (C + C^T) - 4 K q0^2 Q,     C_ab = eps_agd d_g Q_db.
-template <typename T>
-__device__ __forceinline__ void molecular_field(const PhysT<T>& P, const T q[5], const T dq[3][5], const T lap[5],
-                                                T h[5]) {
-  const T A0 = P.A0, g = P.gamma, K = P.K, q0 = P.q0;
-  T trq2 = T(0);
-#pragma unroll
-  for (int a = 0; a < 3; ++a)
-#pragma unroll
-    for (int b = 0; b < 3; ++b) trq2 += qab(q, a, b) * qab(q, a, b);
-  const T cb = -A0 * (T(1) - g / T(3)) - A0 * g * trq2 - T(4) * K * q0 * q0;
-  const int ia[5] = {0, 0, 0, 1, 1}, ib[5] = {0, 1, 2, 1, 2};
-#pragma unroll
-  for (int k = 0; k < 5; ++k) {
-    const int a = ia[k], b = ib[k];
-    T q2 = qab(q, a, 0) * qab(q, 0, b) + qab(q, a, 1) * qab(q, 1, b) + qab(q, a, 2) * qab(q, 2, b);
-    if (a == b) q2 -= trq2 / T(3);
-    T chi = curlq(dq, a, b) + curlq(dq, b, a);
-    h[k] = cb * q[k] + A0 * g * q2 + K * lap[k] - T(2) * K * q0 * chi;
-  }
-}
-
-// Free energy density f' (Eq. 1 up to a total divergence):
-//   f_bulk + K/2 |dQ|^2 + 2 K q0 Q_ab C_ab + 2 K q0^2 Tr(Q^2).
-template <typename T>
-__device__ __forceinline__ T free_energy_density(const PhysT<T>& P, const T q[5], const T dq[3][5]) {
-  const T A0 = P.A0, g = P.gamma, K = P.K, q0 = P.q0;
-  T trq2 = T(0), trq3 = T(0), grad2 = T(0), chi = T(0);
-#pragma unroll
-  for (int a = 0; a < 3; ++a)
-#pragma unroll
-    for (int b = 0; b < 3; ++b) {
-      T qv = qab(q, a, b);
-      trq2 += qv * qv;
-      trq3 += qv * (qab(q, b, 0) * qab(q, 0, a) + qab(q, b, 1) * qab(q, 1, a) + qab(q, b, 2) * qab(q, 2, a));
-      chi += qv * curlq(dq, a, b);
-#pragma unroll
-      for (int gg = 0; gg < 3; ++gg) grad2 += qab(dq[gg], a, b) * qab(dq[gg], a, b);
-    }
-  T fb = T(0.5) * A0 * (T(1) - g / T(3)) * trq2 - A0 * g / T(3) * trq3 + T(0.25) * A0 * g * trq2 * trq2;
-  return fb + T(0.5) * K * grad2 + T(2) * K * q0 * chi + T(2) * K * q0 * q0 * trq2;
-}
-
-// Stress of Eq. 4 with P0 = rho cs^2 - f' (the LB carries rho cs^2):
-//   P_ab = f' d_ab + 2 xi (Q_ab + d_ab/3) Q:H - xi (A_ab + A_ba) - (2 xi/3) H_ab
-//          - E_ab + A_ab - A_ba,        A = Q H,
-//   E_ab = d_a Q_gn Pi_b,gn = K <d_a Q, d_b Q> + 2 K q0 sum_gn d_a Q_gn G^b_gn,
-//   G^b_gn = eps_mbg Q_mn.
-// p[3*a + b].
-template <typename T>
-__device__ __forceinline__ void stress(const PhysT<T>& P, const T q[5], const T dq[3][5], const T h[5], T fprime,
-                                       T p[9]) {
-  const T K = P.K, q0 = P.q0, xi = P.xi;
-  T A[3][3];
-#pragma unroll
-  for (int a = 0; a < 3; ++a)
-#pragma unroll
-    for (int b = 0; b < 3; ++b)
-      A[a][b] = qab(q, a, 0) * qab(h, 0, b) + qab(q, a, 1) * qab(h, 1, b) + qab(q, a, 2) * qab(h, 2, b);
-  T qh = A[0][0] + A[1][1] + A[2][2];
-#pragma unroll
-  for (int a = 0; a < 3; ++a)
-#pragma unroll
-    for (int b = 0; b < 3; ++b) {
-      T e1 = T(0), e2 = T(0);
-#pragma unroll
-      for (int gg = 0; gg < 3; ++gg)
-#pragma unroll
-        for (int n = 0; n < 3; ++n) {
-          T da = qab(dq[a], gg, n);
-          e1 += da * qab(dq[b], gg, n);
-          if (gg != b) {
-            int m = 3 - b - gg;  // eps(m, b, gg) != 0
-            T sgn = ((m - b + 3) % 3 == 2) ? T(1) : T(-1);  // eps(m,b,g) = +1 when (m,b,g) is cyclic
-            e2 += da * sgn * qab(q, m, n);
-          }
-        }
-      T v = -(K * e1 + T(2) * K * q0 * e2);
-      T dlt = a == b ? T(1) : T(0);
-      v += fprime * dlt + T(2) * xi * (qab(q, a, b) + dlt / T(3)) * qh - xi * (A[a][b] + A[b][a]) -
-           T(2) * xi / T(3) * qab(h, a, b) + A[a][b] - A[b][a];
-      p[3 * a + b] = v;
-    }
-}
-
-// All liquid-crystal quantities of one fluid node from its Q and its face-
-// neighbour values, sharing intermediates: Q.Q (for H and Tr Q^3), the curl
-// C_ab = eps_agd d_g Q_db (for the chiral part of H and of f'), and
-// <d_a Q, d_b Q> for the 6 symmetric pairs (its trace is |grad Q|^2).
+// All liquid-crystal quantities of one fluid node from its Q, the doubled
+// first derivatives dq[g][k] = 2 d_g Q_k and the Laplacian lap[k]:
 //   H   = cb Q + A0 g (Q.Q - Tr(Q^2) I/3) + K lap Q - 2 K q0 (C + C^T),
-//         cb = -A0(1 - g/3) - A0 g Tr(Q^2) - 4 K q0^2                       (Eqs. 1, 2)
+//         cb = -A0(1 - g/3) - A0 g Tr(Q^2) - 4 K q0^2, C_ab = eps_agd d_g Q_db  (Eqs. 1, 2)
 //   f'  = A0/2 (1-g/3) Tr Q^2 - A0 g/3 Tr Q^3 + A0 g/4 (Tr Q^2)^2
-//         + K/2 |grad Q|^2 + 2 K q0 Q:C + 2 K q0^2 Tr Q^2                    (Eq. 1)
+//         + K/2 |grad Q|^2 + 2 K q0 Q:C + 2 K q0^2 Tr Q^2                        (Eq. 1)
 //   P   = f' I + 2 xi (Q + I/3) Q:H - xi (A + A^T) - (2 xi/3) H - E + A - A^T,
 //         A = Q H,  E_ab = K <d_a Q, d_b Q> + 2 K q0 sum_gn d_a Q_gn eps_mbg Q_mn  (Eq. 4)
-// The same expressions as molecular_field / free_energy_density / stress.
-// lc_node_d: the same from the derivatives dq[g][k] = d_g Q_k and the
-// Laplacian lap[k].  T is the arithmetic type of the node values (float,
-// double, or f2: two nodes at once); C that of the constants (float for f2).
-// Every constant factor is formed in C first, so that for f2 each term is one
-// packed multiply or fused multiply-add.
-template <typename T, bool NEED_P, typename C>
-__device__ __forceinline__ void lc_node_d(const PhysT<C>& P, const T qi[5], const T dq[3][5], const T lap[5], T h[5],
-                                          T p[9], T* fprime);
+// The algebra is written out in the five stored components with what
+// tracelessness gives (off-diagonal Q.Q from two products each, H_zz from H_xx
+// and H_yy, the commutator and anticommutator of Q and H from the nine entries
+// of Q H): about 290 operations a node against 470 for the 3x3 loops it
+// replaces, which matters where FP64 issue bounds the step (k_stress FP64,
+// 64^3: 84-87 % of the FP64 pipe).  The chiral stress term is skipped when
+// q0 = 0 (uniform over a box).  Products are added, never subtracted, with the
+// sign on a factor that is reused: the packed f2 form has no negated multiply.
+// T is the arithmetic type (float, double, or f2: two nodes at once); chiral:
+// q0 != 0.
+template <typename T>
+__device__ __forceinline__ void lc_node_d(const LcK<T>& P, bool chiral, const T qi[5], const T dq[3][5],
+                                          const T lap[5], T h[5], T p[9], T* fprime) {
+  const T a = qi[0], b = qi[1], c = qi[2], d = qi[3], e = qi[4];
+  const T f = -a - d;
+  const T nb = -b, nc = -c, ne = -e;
+  // Q.Q: (xx, xy, xz, yy, yz, zz)
+  const T bb = b * b, cc = c * c, ee = e * e;
+  const T s0 = a * a + (bb + cc), s3 = d * d + (bb + ee), s5 = f * f + (cc + ee);
+  const T s1 = c * e + nb * f, s2 = b * e + nc * d, s4 = b * c + ne * a;
+  const T trq2 = s0 + s3 + s5;
+  // 2 (C_ab + C_ba) off the diagonal, 2 C_aa on it
+  const T* X = dq[0];
+  const T* Y = dq[1];
+  const T* Z = dq[2];
+  const T tx = X[0] + X[3], ty = Y[0] + Y[3], tz = Z[0] + Z[3];  // minus the zz components
+  const T c0 = Y[2] - Z[1], c3 = Z[1] - X[4], c5 = X[4] - Y[2];
+  const T c1 = (Y[4] - Z[3]) + (Z[0] - X[2]);
+  const T c2 = (X[1] - Z[4]) - (Y[0] + ty);
+  const T c4 = (Z[2] - Y[1]) + (X[3] + tx);
+  const T cb = P.c_lin + P.nA0g * trq2;
+  // the bulk terms are O(A0 q^2) and cancel near equilibrium: they are summed
+  // among themselves first, each product but one unrounded, so that the small
+  // gradient terms are not rounded at their size
+  h[0] = T(P.nA3 * trq2 + T(cb * a + P.A0g * s0)) + T(P.K * lap[0] + P.n2Kq0 * c0);
+  h[1] = T(cb * b + P.A0g * s1) + T(P.K * lap[1] + P.nKq0 * c1);
+  h[2] = T(cb * c + P.A0g * s2) + T(P.K * lap[2] + P.nKq0 * c2);
+  h[3] = T(P.nA3 * trq2 + T(cb * d + P.A0g * s3)) + T(P.K * lap[3] + P.n2Kq0 * c3);
+  h[4] = T(cb * e + P.A0g * s4) + T(P.K * lap[4] + P.nKq0 * c4);
+  const T hz = -h[0] - h[3];
+  // <2 d_a Q, 2 d_b Q> for the six pairs (double contraction over the five
+  // stored components of two traceless symmetric tensors)
+  auto dd = [&](const T* u, const T* v, T tu, T tv) {
+    const T on = u[0] * v[0] + (u[3] * v[3] + tu * tv);
+    return T(on + P.two * T(u[1] * v[1] + (u[2] * v[2] + u[4] * v[4])));
+  };
+  const T e0 = dd(X, X, tx, tx), e1 = dd(X, Y, tx, ty), e2 = dd(X, Z, tx, tz);
+  const T e3 = dd(Y, Y, ty, ty), e4 = dd(Y, Z, ty, tz), e5 = dd(Z, Z, tz, tz);
+  const T qc = a * c0 + (d * c3 + (f * c5 + (b * c1 + (c * c2 + e * c4))));  // 2 Q:C
+  const T trq3 = a * s0 + (d * s3 + (f * s5 + P.two * T(b * s1 + (c * s2 + e * s4))));
+  const T fp = P.f2c * trq2 + (P.nA3 * trq3 + (P.f4c * T(trq2 * trq2) + (P.K8 * (e0 + e3 + e5) + P.Kq0 * qc)));
+  // A = Q H
+  const T h0 = h[0], h1 = h[1], h2 = h[2], h3 = h[3], h4 = h[4];
+  const T a00 = a * h0 + (b * h1 + c * h2), a01 = a * h1 + (b * h3 + c * h4), a02 = a * h2 + (b * h4 + c * hz);
+  const T a10 = b * h0 + (d * h1 + e * h2), a11 = b * h1 + (d * h3 + e * h4), a12 = b * h2 + (d * h4 + e * hz);
+  const T a20 = c * h0 + (e * h1 + f * h2), a21 = c * h1 + (e * h3 + f * h4), a22 = c * h2 + (e * h4 + f * hz);
+  const T qh2 = P.xi2 * (a00 + a11 + a22);
+  const T nt = P.nt, nK4 = P.nK4, up = P.up, dn = P.dn, di = P.di;
+  const T dg = fp + P.third * qh2;
+  const T z1 = qh2 * b + (nt * h1 + nK4 * e1), z2 = qh2 * c + (nt * h2 + nK4 * e2), z4 = qh2 * e + (nt * h4 + nK4 * e4);
+  p[0] = qh2 * a + (nt * h0 + (nK4 * e0 + (di * a00 + dg)));
+  p[4] = qh2 * d + (nt * h3 + (nK4 * e3 + (di * a11 + dg)));
+  p[8] = qh2 * f + (nt * hz + (nK4 * e5 + (di * a22 + dg)));
+  p[1] = up * a01 + (dn * a10 + z1);
+  p[3] = up * a10 + (dn * a01 + z1);
+  p[2] = up * a02 + (dn * a20 + z2);
+  p[6] = up * a20 + (dn * a02 + z2);
+  p[5] = up * a12 + (dn * a21 + z4);
+  p[7] = up * a21 + (dn * a12 + z4);
+  if (chiral) {
+    // chiral part of E: twice the axial vector of (d_a Q) Q
+    const T fd = f - d, af = a - f, da = d - a;
+    auto chi = [&](const T* D, T tD, T& p0, T& p1, T& p2) {
+      const T m0 = D[3] + tD, m1 = D[0] + tD, m2 = D[0] - D[3];
+      p0 = p0 + P.nKq0 * T(D[1] * c + (D[2] * nb + (D[4] * fd + e * m0)));
+      p1 = p1 + P.nKq0 * T(D[2] * af + (D[4] * b + (D[1] * ne + nc * m1)));
+      p2 = p2 + P.nKq0 * T(b * m2 + (D[1] * da + (D[2] * e + D[4] * nc)));
+    };
+    chi(X, tx, p[0], p[1], p[2]);
+    chi(Y, ty, p[3], p[4], p[5]);
+    chi(Z, tz, p[6], p[7], p[8]);
+  }
+  *fprime = fp;
+}
 
-template <typename T, bool NEED_P>
-__device__ __forceinline__ void lc_node(const PhysT<T>& P, const T qi[5], const T qn[6][5], T h[5], T p[9],
+template <typename T>
+__device__ __forceinline__ void lc_node(const DevBox& B, const T qi[5], const T qn[6][5], T h[5], T p[9],
                                         T* fprime) {
   T dq[3][5], lap[5];
   derivatives(qi, qn, dq, lap);
-  lc_node_d<T, NEED_P, T>(P, qi, dq, lap, h, p, fprime);
+  lc_node_d<T>(lck<T>(B), B.p.q0 != 0.0, qi, dq, lap, h, p, fprime);
 }
 
-template <typename T, bool NEED_P, typename C>
-__device__ __forceinline__ void lc_node_d(const PhysT<C>& P, const T qi[5], const T dq[3][5], const T lap[5], T h[5],
-                                          T p[9], T* fprime) {
-  const C A0 = P.A0, g = P.gamma, K = P.K, q0 = P.q0, xi = P.xi;
-  const C third = C(1) / C(3);
-  const C A0g = A0 * g, twoKq0 = C(2) * K * q0;
-  const C c_lin = -A0 * (C(1) - g * third) - C(4) * K * q0 * q0;  // H: coefficient of Q beyond -A0 g Tr(Q^2)
-  const C A0g3 = A0g * third;
-  // Q (3x3), D[g] = d_g Q (3x3 each) from the 5 stored components
-  T Q[3][3], D[3][3][3], S2[3][3], Cm[3][3];
+// Per-node choice ca ? a : b (f2: per lane value).
+template <typename T>
+__device__ __forceinline__ T pos_part(T v) {
+  return v > T(0) ? v : T(0);
+}
+
+// Increment of Q in one step (Eq. 2) at one node (or, T = f2, two):
+//   co-rotation S = X + X^T - 2 xi (Q + I/3) Tr(QW), X = G (Q + I/3),
+//     G = xi D + Omega: 27 products for X instead of 72 for its four factors;
+//   upwind fluxes: with the positive and negative parts of the face velocity
+//     the six fluxes are one product per neighbour and component plus one
+//     with the node's own Q, adv = (self Q_i + sum_d cd[d] Q_d) / 2 (35
+//     multiply-adds and 6 selects instead of 30 and 30);
+//   FP32 storage (COMP): H was evaluated at hi, the stored Q is hi + lo: the
+//     local part of H(hi + lo) - H(hi) to first order (the bulk terms'
+//     derivative at hi applied to lo, and lo's own term -6 K lo of the
+//     Laplacian; the neighbours' lo enter at the ~1e-9 level).  Without it the
+//     relaxation stalls where A0 lo ~ the residual.
+// flow_terms: G (row-major), cd and self from the velocities ui and un of the
+// node and its six face neighbours; open[d] = false closes face d (solid or
+// wall) to the flux.
+template <typename T>
+__device__ __forceinline__ void flow_terms(const LcK<T>& P, const T ui[3], const T un[6][3], const bool open[6],
+                                           T G[9], T cd[6], T& self) {
+  // w[a][b] = 2 d_b u_a
+  T w[3][3];
 #pragma unroll
-  for (int a = 0; a < 3; ++a)
+  for (int i = 0; i < 3; ++i)
 #pragma unroll
-    for (int b = 0; b < 3; ++b) {
-      Q[a][b] = qab(qi, a, b);
+    for (int j = 0; j < 3; ++j) w[i][j] = un[2 * j][i] - un[2 * j + 1][i];
 #pragma unroll
-      for (int gg = 0; gg < 3; ++gg) D[gg][a][b] = qab(dq[gg], a, b);
-    }
+  for (int k = 0; k < 6; ++k) {
+    const T uf = ui[k >> 1] + un[k][k >> 1];
+    T up = pos_part(uf);
+    T dn = uf - up;
+    if (!open[k]) up = dn = T(0);
+    // + face: outflow up Q_i + dn Q_d; - face: minus (up Q_d + dn Q_i)
+    cd[k] = (k & 1) ? T(-up) : dn;
+    const T own = (k & 1) ? T(-dn) : up;
+    self = k ? T(self + own) : own;
+  }
+  const T g0 = P.g0, g1 = P.g1, g2 = P.g2;
+  G[0] = g0 * w[0][0];
+  G[4] = g0 * w[1][1];
+  G[8] = g0 * w[2][2];
+  G[1] = g1 * w[0][1] + g2 * w[1][0];
+  G[3] = g1 * w[1][0] + g2 * w[0][1];
+  G[2] = g1 * w[0][2] + g2 * w[2][0];
+  G[6] = g1 * w[2][0] + g2 * w[0][2];
+  G[5] = g1 * w[1][2] + g2 * w[2][1];
+  G[7] = g1 * w[2][1] + g2 * w[1][2];
+}
+
+// Twice the advective flux divergence of one component.
+template <typename T>
+__device__ __forceinline__ T advect(const T cd[6], T self, T q, const T n[6]) {
+  T v = self * q;
 #pragma unroll
-  for (int a = 0; a < 3; ++a)
+  for (int d = 0; d < 6; ++d) v = v + cd[d] * n[d];
+  return v;
+}
+
+// FLOW = false: the flow is frozen (u = 0), G and adv are not read.
+template <bool COMP, bool FLOW, typename T>
+__device__ __forceinline__ void q_increment(const LcK<T>& P, const T qi[5], const T adv[5], const T G[9],
+                                            const T hin[5], const T lo[5], T d5[5]) {
+  const T a = qi[0], b = qi[1], c = qi[2], d = qi[3], e = qi[4];
+  const T f = -a - d;
+  T h[5];
 #pragma unroll
-    for (int b = a; b < 3; ++b) {
-      S2[a][b] = Q[a][0] * Q[0][b] + Q[a][1] * Q[1][b] + Q[a][2] * Q[2][b];
-      S2[b][a] = S2[a][b];
-    }
+  for (int k = 0; k < 5; ++k) h[k] = hin[k];
+  if constexpr (COMP) {
+    const T A0g = P.A0g;
+    const T la = lo[0], lb = lo[1], lc = lo[2], ld = lo[3], le = lo[4];
+    const T lf = -la - ld;
+    const T ta = a * la, tb = b * lb, tc = c * lc, td = d * ld, te = e * le;
+    const T trl = (ta + td + f * lf) + P.two * (tb + tc + te);
+    const T trq2 = (a * a + (d * d + f * f)) + P.two * T(b * b + (c * c + e * e));
+    const T cb = P.c_lo + P.nA0g * trq2;
+    const T m = P.nA2 * trl;
+    const T nf = a + d, nd = -d, na = -a, l3 = P.nthird * trl, A2 = P.A2;
+    h[0] = h[0] + (cb * la + (A2 * (ta + tb + tc + l3) + m * a));
+    h[3] = h[3] + (cb * ld + (A2 * (tb + td + te + l3) + m * d));
+    h[1] = h[1] + (cb * lb + (A0g * T(nf * lb + (b * (la + ld) + (c * le + e * lc))) + m * b));
+    h[2] = h[2] + (cb * lc + (A0g * T(nd * lc + (b * le + (e * lb + c * (la + lf)))) + m * c));
+    h[4] = h[4] + (cb * le + (A0g * T(na * le + (b * lc + (c * lb + e * (ld + lf)))) + m * e));
+  }
+  if constexpr (!FLOW) {
 #pragma unroll
-  for (int a = 0; a < 3; ++a)
+    for (int k = 0; k < 5; ++k) d5[k] = P.Gamma * h[k];
+    return;
+  }
+  const T at = a + P.third, dt = d + P.third, ft = f + P.third;
+  const T tm = P.ntwo * T(a * G[0] + (d * G[4] + (f * G[8] + (b * (G[1] + G[3]) + (c * (G[2] + G[6]) + e * (G[5] + G[7]))))));
+  const T x00 = G[0] * at + (G[1] * b + G[2] * c), x11 = G[3] * b + (G[4] * dt + G[5] * e);
+  const T x22 = G[6] * c + (G[7] * e + G[8] * ft);
+  T S[5];
+  S[0] = P.two * x00 + tm * at;
+  S[3] = P.two * x11 + tm * dt;
+  const T s5 = P.two * x22 + tm * ft;
+  S[1] = (G[0] * b + (G[1] * dt + G[2] * e)) + (G[3] * at + (G[4] * b + (G[5] * c + tm * b)));
+  S[2] = (G[0] * c + (G[1] * e + G[2] * ft)) + (G[6] * at + (G[7] * b + (G[8] * c + tm * c)));
+  S[4] = (G[3] * c + (G[4] * e + G[5] * ft)) + (G[6] * b + (G[7] * dt + (G[8] * e + tm * e)));
+  const T tr3 = P.nthird * (S[0] + S[3] + s5);
+  S[0] = S[0] + tr3;
+  S[3] = S[3] + tr3;
 #pragma unroll
-    for (int b = 0; b < 3; ++b) Cm[a][b] = D[(a + 1) % 3][(a + 2) % 3][b] - D[(a + 2) % 3][(a + 1) % 3][b];
-  const T trq2 = S2[0][0] + S2[1][1] + S2[2][2];
-  const T cb = c_lin - A0g * trq2;
-  const T tq3 = A0g3 * trq2;
-  T H[3][3];
-#pragma unroll
-  for (int a = 0; a < 3; ++a)
-#pragma unroll
-    for (int b = a; b < 3; ++b) {
-      const int k = a == 0 ? b : (a == 1 ? 2 + b : 5);
-      const T lp = k < 5 ? lap[k] : -(lap[0] + lap[3]);
-      T v = cb * Q[a][b] + A0g * S2[a][b] + K * lp - twoKq0 * (Cm[a][b] + Cm[b][a]);
-      if (a == b) v = v - tq3;
-      H[a][b] = v;
-      H[b][a] = v;
-    }
-  h[0] = H[0][0]; h[1] = H[0][1]; h[2] = H[0][2]; h[3] = H[1][1]; h[4] = H[1][2];
-  if (!NEED_P) return;
-  // E_ab = K d_aQ : d_bQ; both factors are symmetric and traceless, so the
-  // double contraction over the 5 stored components is
-  // A_xx B_xx + A_yy B_yy + A_zz B_zz + 2 (A_xy B_xy + A_xz B_xz + A_yz B_yz)
-  // with A_zz = -(A_xx + A_yy)
-  T E[3][3], tz[3];
-#pragma unroll
-  for (int a = 0; a < 3; ++a) tz[a] = dq[a][0] + dq[a][3];
-  const C twoK = C(2) * K;
-#pragma unroll
-  for (int a = 0; a < 3; ++a)
-#pragma unroll
-    for (int b = a; b < 3; ++b) {
-      const T e = K * (dq[a][0] * dq[b][0] + dq[a][3] * dq[b][3] + tz[a] * tz[b]) +
-                  twoK * (dq[a][1] * dq[b][1] + dq[a][2] * dq[b][2] + dq[a][4] * dq[b][4]);
-      E[a][b] = e;
-      E[b][a] = e;
-    }
-  const T Kgrad2 = E[0][0] + E[1][1] + E[2][2];  // K |grad Q|^2
-#pragma unroll
-  for (int a = 0; a < 3; ++a)
-#pragma unroll
-    for (int b = 0; b < 3; ++b) {
-      // the chiral part: sum over g != b of eps(m, b, g) d_a Q_g. . Q_m. (m = 3 - b - g);
-      // eps(m, b, g) = +1 for g = b + 1, m = b + 2 and -1 for g = b + 2, m = b + 1 (mod 3)
-      const int g1 = (b + 1) % 3, g2 = (b + 2) % 3;
-      const T e2 = (D[a][g1][0] * Q[g2][0] + D[a][g1][1] * Q[g2][1] + D[a][g1][2] * Q[g2][2]) -
-                   (D[a][g2][0] * Q[g1][0] + D[a][g2][1] * Q[g1][1] + D[a][g2][2] * Q[g1][2]);
-      E[a][b] = E[a][b] + twoKq0 * e2;
-    }
-  T trq3 = T(0), qc = T(0);
-#pragma unroll
-  for (int a = 0; a < 3; ++a)
-#pragma unroll
-    for (int b = 0; b < 3; ++b) {
-      trq3 = trq3 + Q[a][b] * S2[a][b];
-      qc = qc + Q[a][b] * Cm[a][b];
-    }
-  const C fb2 = C(0.5) * A0 * (C(1) - g * third), fb4 = C(0.25) * A0g;
-  const T fp = (fb2 * trq2 - A0g3 * trq3) + fb4 * (trq2 * trq2) + C(0.5) * Kgrad2 + twoKq0 * qc +
-               (C(2) * K * q0 * q0) * trq2;
-  T Am[3][3];
-#pragma unroll
-  for (int a = 0; a < 3; ++a)
-#pragma unroll
-    for (int b = 0; b < 3; ++b) Am[a][b] = Q[a][0] * H[0][b] + Q[a][1] * H[1][b] + Q[a][2] * H[2][b];
-  const T qh = Am[0][0] + Am[1][1] + Am[2][2];
-  const C twoxi = C(2) * xi, twoxi3 = twoxi * third;
-  const T qh2 = twoxi * qh;
-#pragma unroll
-  for (int a = 0; a < 3; ++a)
-#pragma unroll
-    for (int b = 0; b < 3; ++b) {
-      // 2 xi (Q + I/3) Q:H - xi (A + A^T) - (2 xi/3) H - E + A - A^T, plus f' on the diagonal
-      T v = qh2 * Q[a][b] - xi * (Am[a][b] + Am[b][a]) - twoxi3 * H[a][b] - E[a][b] + (Am[a][b] - Am[b][a]);
-      if (a == b) v = v + (fp + third * qh2);
-      p[3 * a + b] = v;
-    }
-  *fprime = fp;
+  for (int k = 0; k < 5; ++k) d5[k] = S[k] + (P.Gamma * h[k] + P.nhalf * adv[k]);
 }
 
 }  // namespace lclb

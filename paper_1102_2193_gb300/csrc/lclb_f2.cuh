@@ -16,6 +16,7 @@ struct f2 {
   float2 v;
   f2() = default;
   __device__ __forceinline__ f2(float a) : v(make_float2(a, a)) {}
+  __device__ __forceinline__ explicit f2(int a) : v(make_float2((float)a, (float)a)) {}
   __device__ __forceinline__ f2(float a, float b) : v(make_float2(a, b)) {}
   __device__ __forceinline__ explicit f2(float2 w) : v(w) {}
 };
@@ -55,5 +56,7 @@ __device__ __forceinline__ f2 operator-(f2 a, float b) { return a - f2(b); }
 __device__ __forceinline__ f2 operator-(float a, f2 b) { return f2(a) - b; }
 __device__ __forceinline__ f2 operator-(f2mul m, float c) { return m - f2(c); }
 __device__ __forceinline__ f2 operator-(float c, f2mul m) { return f2(c) - m; }
+
+__device__ __forceinline__ f2 pos_part(f2 v) { return f2(fmaxf(v.v.x, 0.f), fmaxf(v.v.y, 0.f)); }
 
 }  // namespace lclb

@@ -12,9 +12,10 @@ constexpr int FORCE_ACC = 1;  // accumulate colloid LC force/torque
 constexpr int FORCE_FE = 2;   // write free-energy partials (one double per tile)
 constexpr int LB_MOM = 1;     // write mass/momentum partials (4 doubles per tile)
 constexpr int LC_RESID = 1;   // write residual partials (sum of squares, max; 2 doubles per tile)
+constexpr int LC_COMMIT = 2;  // k_lc also runs the link exchange and, when a box is done, its colloid update and parity flip
 
 // boundary links per link-exchange work unit
-constexpr int LINK_CHUNK = 256;
+constexpr int LINK_CHUNK = 64;
 
 // One work item of the persistent step kernel k_step: a tile (32 x ty x zc)
 // of one phase of one box, a chunk of a box's boundary links, or a box's
@@ -38,9 +39,20 @@ struct Launch {
   int ntiles;
   int zc;             // tile depth in z
   int ty;             // tile height in y (tile width in x is 32)
-  int grid;           // blocks (persistent: tiles are strided over blocks)
+  int grid;           // blocks (persistent: work units are strided over blocks)
   cudaStream_t stream;
+  // nodes next to a solid or wall, in groups (box, first entry of its near
+  // list) of 32, one per warp; a box's groups are a multiple of NEAR_PAD, so
+  // the warps of a block share a box
+  const int2* groups;
+  int ngroups;
+  double* npart;      // k_lc: residual record (sum of squares, max) of each group
+  const int2* chunks; // k_lc with LC_COMMIT: link chunks (box, first link)
+  int nchunks;
+  unsigned* done;       // k_lc with LC_COMMIT: finished work units per box (zero between launches)
+  const unsigned* total;  // work units of each box in this launch
 };
+constexpr int NEAR_PAD = 8;  // the largest tile height
 
 cudaError_t launch_force(int prec, const Launch& L, int mode, double* part);
 cudaError_t launch_lb(int prec, const Launch& L, int mode, double* part);
@@ -62,6 +74,9 @@ int step_blocks_per_sm(int prec, int ty);
 // Re-discretisation after the colloid update; mob lists (box, colloid) of mobile colloids.
 cudaError_t launch_rediscretise(int prec, DevBox* boxes, int nboxes, const int2* mob, int nmob, int nsm,
                                 cudaStream_t s);
+// Fills box b's list of near nodes (up to its capacity) and its count, which
+// the caller has zeroed.
+cudaError_t launch_near_list(DevBox* boxes, int b, int N, cudaStream_t s);
 cudaError_t launch_geometry(DevBox* boxes, int b, int N, cudaStream_t s);
 cudaError_t launch_link_build(DevBox* boxes, int b, int N, int c, int* blocksum, int base, int* total,
                               cudaStream_t s);

@@ -12,8 +12,8 @@
 // launch serves one box or a batch of boxes of different sizes.
 #include <cstdio>
 
-#include "lclb_dev.cuh"
 #include "lclb_f2.cuh"
+#include "lclb_dev.cuh"
 #include "lclb_internal.h"
 
 namespace lclb {
@@ -143,11 +143,26 @@ __device__ __forceinline__ void load_box(DevBox& sb, const DevBox* boxes, int b)
   __syncthreads();
 }
 
+// The constants of the two-node paths, twice each, from the shared record.
+__device__ __forceinline__ void load_k2(LcK<f2>& k2, const DevBox& B) {
+  const float* src = reinterpret_cast<const float*>(&B.kf);
+  f2* dst = reinterpret_cast<f2*>(&k2);
+  const int nthr = blockDim.x * blockDim.y;
+  for (int k = threadIdx.x + blockDim.x * threadIdx.y; k < LCK_N; k += nthr) dst[k] = f2(src[k]);
+  __syncthreads();
+}
+
 // Tile loops: reload the shared box record only when the tile's box changes
 // (b is uniform over the block, so the barriers are too).
 __device__ __forceinline__ void load_box(DevBox& sb, const DevBox* boxes, int b, int& cur) {
   if (b == cur) return;
   load_box(sb, boxes, b);
+  cur = b;
+}
+__device__ __forceinline__ void load_box(DevBox& sb, LcK<f2>& k2, const DevBox* boxes, int b, int& cur) {
+  if (b == cur) return;
+  load_box(sb, boxes, b);
+  load_k2(k2, sb);
   cur = b;
 }
 
@@ -169,7 +184,7 @@ __device__ __forceinline__ uint8_t stress_at(const DevBox& B, const PhysT<T>& PP
   T qi[5], qn[6][5], h[5], p[9], fp;
   double surf = 0.0;
   gather_q(B, Q, gx, gy, kk, i, m, qi, qn, fe ? &surf : nullptr);
-  lc_node<T, true>(PP, qi, qn, h, p, &fp);
+  lc_node<T>(B, qi, qn, h, p, &fp);
 #pragma unroll
   for (int c = 0; c < 9; ++c) sP[c * HP] = p[c];
   if (hout) {
@@ -343,30 +358,32 @@ __device__ __forceinline__ void pull(const DevBox& B, const T* __restrict__ fin,
     }
     return;
   }
+  // near node: the 18 mask bytes, then the 19 populations, each in one round of
+  // independent loads (taken direction by direction, the dependent pairs of
+  // loads were most of the time of a small box's LB kernel)
   const T rho0 = phys<T>(B).rho0;
+  int s[NQ];
+  uint8_t ms[NQ];
+  s[0] = i;
+  ms[0] = 0;
 #pragma unroll
-  for (int q = 0; q < NQ; ++q) {
+  for (int q = 1; q < NQ; ++q) {
     const int zsrc = zs[1 - cz(q)];
-    int s = -1;
-    uint8_t ms = WALLFLAG;
-    if (zsrc >= 0 && zsrc < nz) {
-      s = xs[1 - cx(q)] + nx * (ys[1 - cy(q)] + ny * zsrc);
-      ms = B.mask[s] & IDMASK;
-    }
-    if (ms == 0) {
-      df[q] = ldg(fin + (size_t)q * N + s);
-    } else {
-      T corr = T(0);
-      if (ms != WALLFLAG) {
-        const DevColloid& C = B.col[ms - 1];
-        T ub[3];
-        rigid_velocity_t<T>(B, T(x) - T(0.5 * cx(q)), T(y) - T(0.5 * cy(q)), T(z) - T(0.5 * cz(q)), C.Xb, C.Vb, C.Wb,
-                            ub);
-        const T cub = T(cx(q)) * ub[0] + T(cy(q)) * ub[1] + T(cz(q)) * ub[2];
-        corr = T(6.0 * wq(q)) * rho0 * cub;
-      }
-      df[q] = ldg(fin + (size_t)opp(q) * N + i) + corr;
-    }
+    const bool in = zsrc >= 0 && zsrc < nz;
+    s[q] = in ? xs[1 - cx(q)] + nx * (ys[1 - cy(q)] + ny * zsrc) : i;
+    ms[q] = B.mask[s[q]] & IDMASK;
+    if (!in) ms[q] = WALLFLAG;
+  }
+#pragma unroll
+  for (int q = 0; q < NQ; ++q) df[q] = ldg(fin + (ms[q] == 0 ? (size_t)q * N + s[q] : (size_t)opp(q) * N + i));
+#pragma unroll
+  for (int q = 1; q < NQ; ++q) {
+    if (ms[q] == 0 || ms[q] == WALLFLAG) continue;
+    const DevColloid& C = B.col[ms[q] - 1];
+    T ub[3];
+    rigid_velocity_t<T>(B, T(x) - T(0.5 * cx(q)), T(y) - T(0.5 * cy(q)), T(z) - T(0.5 * cz(q)), C.Xb, C.Vb, C.Wb, ub);
+    const T cub = T(cx(q)) * ub[0] + T(cy(q)) * ub[1] + T(cz(q)) * ub[2];
+    df[q] += T(6.0 * wq(q)) * rho0 * cub;
   }
 }
 
@@ -377,29 +394,43 @@ __device__ __forceinline__ void pull(const DevBox& B, const T* __restrict__ fin,
 template <typename T>
 __device__ __forceinline__ void collide_store(const PhysT<T>& PP, T* __restrict__ fout, T* __restrict__ ub, int N,
                                               int i, const T df[NQ], T Fx, T Fy, T Fz) {
-  T drho = T(0), mx = T(0), my = T(0), mz = T(0);
+  // Opposite directions share all but a sign: with c.j the odd part (j = 3 rho u +
+  // 3 (tau - 1/2) F) and an even part base + (c.u)(c.g) (g = 1.5 j + 4.5 (tau - 1/2) F),
+  // df*_q = df_q + omega (w_q (even + c.j) - df_q), the bracket small near
+  // equilibrium so that df_q is rounded once.  About 150 operations a node instead
+  // of 420 direction by direction: FP64 issue bounds the FP64 kernel (k_lbp,
+  // 64^3: 229 -> 109 us), and the FP32 one issued 767 instructions per warp of nodes.
+  T drho = df[0], mx = T(0), my = T(0), mz = T(0);
 #pragma unroll
-  for (int q = 0; q < NQ; ++q) {
-    drho += df[q];
-    if (cx(q)) mx += cx(q) > 0 ? df[q] : -df[q];
-    if (cy(q)) my += cy(q) > 0 ? df[q] : -df[q];
-    if (cz(q)) mz += cz(q) > 0 ? df[q] : -df[q];
+  for (int q = 1; q < NQ; q += 2) {
+    const T s = df[q] + df[q + 1], d = df[q] - df[q + 1];
+    drho += s;
+    if (cx(q)) mx += cx(q) > 0 ? d : -d;
+    if (cy(q)) my += cy(q) > 0 ? d : -d;
+    if (cz(q)) mz += cz(q) > 0 ? d : -d;
   }
+  const T omega = PP.omega, pt = PP.ptau;
   const T rho = PP.rho0 + drho;
   const T inv = T(1) / rho;
   const T ux = (mx + T(0.5) * Fx) * inv, uy = (my + T(0.5) * Fy) * inv, uz = (mz + T(0.5) * Fz) * inv;
   const T usq = ux * ux + uy * uy + uz * uz;
   const T uF = ux * Fx + uy * Fy + uz * Fz;
-  const T omega = PP.omega, pref = PP.pref;
+  const T r3 = T(3) * rho, p3 = T(3) * pt, p45 = T(4.5) * pt;
+  const T jx = r3 * ux + p3 * Fx, jy = r3 * uy + p3 * Fy, jz = r3 * uz + p3 * Fz;
+  const T gx = T(1.5) * jx + p45 * Fx, gy = T(1.5) * jy + p45 * Fy, gz = T(1.5) * jz + p45 * Fz;
+  const T base = drho - (T(0.5) * r3 * usq + p3 * uF);
   const uint64_t pol_stream = l2_stream(), pol_keep = l2_keep();
+  st_hint(fout + i, df[0] + omega * (T(wq(0)) * base - df[0]), pol_stream);
 #pragma unroll
-  for (int q = 0; q < NQ; ++q) {
+  for (int q = 1; q < NQ; q += 2) {
     const T w = T(wq(q));
-    const T cu = T(cx(q)) * ux + T(cy(q)) * uy + T(cz(q)) * uz;
-    const T cF = T(cx(q)) * Fx + T(cy(q)) * Fy + T(cz(q)) * Fz;
-    const T eq = w * (drho + rho * (T(3) * cu + T(4.5) * cu * cu - T(1.5) * usq));
-    const T src = pref * w * (T(3) * (cF - uF) + T(9) * cu * cF);
-    st_hint(fout + (size_t)q * N + i, df[q] - omega * (df[q] - eq) + src, pol_stream);
+    T cu = T(0), cg = T(0), cj = T(0);
+    if (cx(q)) { cu += cx(q) > 0 ? ux : -ux; cg += cx(q) > 0 ? gx : -gx; cj += cx(q) > 0 ? jx : -jx; }
+    if (cy(q)) { cu += cy(q) > 0 ? uy : -uy; cg += cy(q) > 0 ? gy : -gy; cj += cy(q) > 0 ? jy : -jy; }
+    if (cz(q)) { cu += cz(q) > 0 ? uz : -uz; cg += cz(q) > 0 ? gz : -gz; cj += cz(q) > 0 ? jz : -jz; }
+    const T even = base + cu * cg;
+    st_hint(fout + (size_t)q * N + i, df[q] + omega * (w * (even + cj) - df[q]), pol_stream);
+    st_hint(fout + (size_t)(q + 1) * N + i, df[q + 1] + omega * (w * (even - cj) - df[q + 1]), pol_stream);
   }
   st_hint(ub + i, ux, pol_keep);
   st_hint(ub + (size_t)N + i, uy, pol_keep);
@@ -538,88 +569,195 @@ __device__ __forceinline__ void column_roll(T cz[2][K], const T pc[5][K]) {
 // A plain node (NEAR_NODE false) takes its own Q and that of its x- and
 // z-neighbours from pq (self, x + 1, x - 1, z + 1, z - 1: gathered by the warp
 // and rolled down the thread's column) and loads the y-neighbours.
-// FP32 node next to a solid or wall: derivatives from the compensated Q
-// (near_derivatives_f32), H and P stored, colloid faces summed.  Every node
-// of the shell around a colloid or along a wall takes this path: the
-// colloid's LC force is a small sum of large face terms, and the body force
-// at the boundary links, which sets the hydrodynamic force, is the face
-// divergence of the stress of these nodes.  Not inlined, so that the wider
-// arithmetic of this rare path does not raise the register count of the
-// plain path of the stress kernels.
-__device__ __noinline__ void near_stress_f32(const DevBox& B, float* __restrict__ Hb, float* __restrict__ Pb, int x,
-                                             int y, int z, int i, int mode, int& my_c, double my_acc[6]) {
-  const int N = B.N;
-  float qi[5], dq[3][5], lap[5], h[5], p[9], fp;
-  near_derivatives_f32(B, x, y, z, i, qi, dq, lap);
-  lc_node_d<float, true>(B.pf, qi, dq, lap, h, p, &fp);
-#pragma unroll
-  for (int c = 0; c < 5; ++c) Hb[(size_t)c * N + i] = h[c];
-#pragma unroll
-  for (int c = 0; c < 9; ++c) Pb[(size_t)c * N + i] = p[c];
-  if (mode & FORCE_ACC) {
-    int nb[6], zz[2];
-    face_neighbours(B, x, y, z, nb, zz);
-    for (int d = 0; d < 6; ++d) {
-      const int j = nb[d];
-      if (j < 0) continue;
-      const uint8_t fj = B.mask[j] & IDMASK;
-      if (fj == 0) continue;
-      const int ax = d >> 1;
-      const float sgn = (d & 1) ? -1.f : 1.f;
-      const float pcv[3] = {p[ax], p[3 + ax], p[6 + ax]};
-      colloid_face(B, fj - 1, ax, sgn, pcv, x, y, z, my_c, my_acc);
-    }
-  }
-}
+//
+// Near node: derivatives from the differences to the six neighbours, the
+// difference to a solid or wall neighbour being w/(K + w) (Q0 - Q) (1 for
+// strong anchoring) with Q0 in FP64.  FP32 storage takes the compensated
+// values, (hi_j - hi_i) + (lo_j - lo_i), and the surface difference in FP64:
+// with hi alone the rounding of Q (~3e-8) enters the Laplacian of every node at
+// the colloid surface, and the colloid's LC force, a small sum of large face
+// terms, would carry it at ~1e-4 relative.
+//
+// A warp evaluates 32 near nodes.  Their solid faces (one or two per node of
+// the six) are packed into a queue and shared out over the lanes, once for the
+// surface values and once for the colloid force, because the FP64 arithmetic
+// of a face is a chain of some 60 dependent operations that every lane of the
+// warp would otherwise run through six times.  scratch: shared memory of the
+// warp (NearScratch<T>).
+template <typename T>
+struct NearScratch {
+  uint16_t face[192];  // lane | d << 8 of each solid face
+  T dn[192][5];        // Qs - Q of each solid face
+};
 
-template <typename T, bool NEAR_NODE>
-__device__ __forceinline__ void stress_node(const DevBox& B, const PhysT<T>& PP, const T* __restrict__ Q,
-                                            T* __restrict__ Hb, T* __restrict__ Pb, int x, int y, int z, int i,
-                                            uint8_t m, int mode, int& my_c, double my_acc[6],
-                                            const T (*pq)[5] = nullptr) {
-  if constexpr (NEAR_NODE && sizeof(T) == 4) {
-    near_stress_f32(B, Hb, Pb, x, y, z, i, mode, my_c, my_acc);
-    return;
+template <typename T>
+__device__ __noinline__ void near_stress(const DevBox& B, int i, int mode, NearScratch<T>& sc) {
+  const unsigned full = 0xffffffffu;
+  const int lane = threadIdx.x & 31;
+  const bool valid = i >= 0;
+  if (!__ballot_sync(full, valid)) return;
+  const int N = B.N, nx = B.nx, ny = B.ny, qpar = B.st->qpar;
+  const int j0 = valid ? i : 0;
+  const int x = j0 % nx, y = (j0 / nx) % ny, z = j0 / (nx * ny);
+  const T* __restrict__ Q = static_cast<const T*>(B.Q[qpar]);
+  const __nv_bfloat16* __restrict__ Lo = B.Qlo[qpar];
+  constexpr bool comp = sizeof(T) == 4;
+  T qh[5];
+  float ql[5];
+#pragma unroll
+  for (int k = 0; k < 5; ++k) {
+    qh[k] = ldg(Q + (size_t)k * N + j0);
+    ql[k] = 0.f;
+    if constexpr (comp) ql[k] = __bfloat162float(Lo[(size_t)k * N + j0]);
   }
-  const int N = B.N;
-  T qi[5], qn[6][5], h[5], p[9], fp;
-  if (NEAR_NODE) {
-    gather_q(B, Q, x, y, z, i, m, qi, qn, nullptr);
-  } else {
-    int nb[6], zz[2];
-    face_neighbours(B, x, y, z, nb, zz);
+  int nb[6], zz[2], cf[6];
+  face_neighbours(B, x, y, z, nb, zz);
+#pragma unroll
+  for (int d = 0; d < 6; ++d) cf[d] = (int)(B.mask[nb[d] < 0 ? j0 : nb[d]] & IDMASK);
+  unsigned solid = 0;  // solid faces of the node
+  bool planar = false;
+#pragma unroll
+  for (int d = 0; d < 6; ++d) {
+    const int c = nb[d] < 0 ? -1 : cf[d] - 1;
+    if (valid && (nb[d] < 0 || c >= 0)) solid |= 1u << d;
+    if (valid && c >= 0 && B.col[c].anchoring != 0) planar = true;
+  }
+  double nf[3] = {1.0, 0.0, 0.0};
+  if (planar) {
+    double qid[5];
+#pragma unroll
+    for (int k = 0; k < 5; ++k) qid[k] = (double)qh[k] + (double)ql[k];
+    principal_dir<double>(qid, nf);
+  }
+  // queue of solid faces; slot[d]: position of this node's face d
+  int slot[6], nface = 0;
+#pragma unroll
+  for (int d = 0; d < 6; ++d) {
+    const unsigned m = __ballot_sync(full, (solid >> d) & 1u);
+    slot[d] = nface + __popc(m & ((1u << lane) - 1u));
+    if ((solid >> d) & 1u) sc.face[slot[d]] = (uint16_t)(lane | (d << 8));
+    nface += __popc(m);
+  }
+  __syncwarp();
+  // node, direction and colloid (-1: wall) of face t on this lane
+  auto face_of = [&](int t, int& own, int& d, int& c, int s[3]) {
+    const int e = t < nface ? sc.face[t] : lane;
+    own = e & 31;
+    d = e >> 8;
+    const int o = __shfl_sync(full, j0, own);
+    s[0] = o % nx; s[1] = (o / nx) % ny; s[2] = o / (nx * ny);
+    const int ax = d >> 1, v = s[ax] + ((d & 1) ? -1 : 1);
+    const int L = ax == 0 ? nx : (ax == 1 ? ny : B.nz);
+    const bool out = ax == 2 && B.wall_z && (v < 0 || v >= L);
+    s[ax] = out ? v : wrap1(v, L);
+    c = t < nface && !out ? (int)(B.mask[s[0] + nx * (s[1] + ny * s[2])] & IDMASK) - 1 : -1;
+  };
+  for (int t0 = 0; t0 < nface; t0 += 32) {
+    const int t = t0 + lane;
+    int own, d, c, s[3];
+    face_of(t, own, d, c, s);
+    double nfo[3], qo[5];
+    float lo[5];
+#pragma unroll
+    for (int a = 0; a < 3; ++a) nfo[a] = __shfl_sync(full, nf[a], own);
 #pragma unroll
     for (int k = 0; k < 5; ++k) {
-      qi[k] = pq[0][k];
-      qn[0][k] = pq[1][k];
-      qn[1][k] = pq[2][k];
-      qn[4][k] = pq[3][k];
-      qn[5][k] = pq[4][k];
+      qo[k] = (double)__shfl_sync(full, qh[k], own);
+      lo[k] = __shfl_sync(full, ql[k], own);
     }
+    if (t < nface) {
+      double q0[5];
+      surface_q0_near<T>(B, c, s[0], s[1], s[2], nfo, q0);
+      const double w = c < 0 ? 1.0 : B.col[c].wfac;
 #pragma unroll
-    for (int d = 2; d < 4; ++d)
-#pragma unroll
-      for (int k = 0; k < 5; ++k) qn[d][k] = ldg(Q + (size_t)k * N + nb[d]);
+      for (int k = 0; k < 5; ++k) sc.dn[t][k] = (T)(w * ((q0[k] - qo[k]) - (double)lo[k]));
+    }
   }
-  lc_node<T, true>(PP, qi, qn, h, p, &fp);
+  __syncwarp();
+  T dn[6][5];
 #pragma unroll
-  for (int c = 0; c < 5; ++c) Hb[(size_t)c * N + i] = h[c];
+  for (int d = 0; d < 6; ++d) {
+    const bool so = (solid >> d) & 1u;
+    const size_t j = so || nb[d] < 0 ? j0 : nb[d];
 #pragma unroll
-  for (int c = 0; c < 9; ++c) Pb[(size_t)c * N + i] = p[c];
-  if (NEAR_NODE && (mode & FORCE_ACC)) {
-    int nb[6], zz[2];
-    face_neighbours(B, x, y, z, nb, zz);
+    for (int k = 0; k < 5; ++k) {
+      T v = ldg(Q + (size_t)k * N + j) - qh[k];
+      if constexpr (comp) v += __bfloat162float(Lo[(size_t)k * N + j]) - ql[k];
+      dn[d][k] = so ? sc.dn[slot[d]][k] : v;
+    }
+  }
+  T qi[5], dq[3][5], lap[5], h[5], p[9], fp;
 #pragma unroll
-    for (int d = 0; d < 6; ++d) {
-      const int j = nb[d];
-      if (j < 0) continue;
-      const uint8_t fj = B.mask[j] & IDMASK;
-      if (fj == 0) continue;
+  for (int k = 0; k < 5; ++k) {
+    qi[k] = qh[k] + (T)ql[k];
+    dq[0][k] = dn[0][k] - dn[1][k];  // doubled, as derivatives()
+    dq[1][k] = dn[2][k] - dn[3][k];
+    dq[2][k] = dn[4][k] - dn[5][k];
+    lap[k] = (dn[0][k] + dn[1][k]) + (dn[2][k] + dn[3][k]) + (dn[4][k] + dn[5][k]);
+  }
+  lc_node_d<T>(lck<T>(B), B.p.q0 != 0.0, qi, dq, lap, h, p, &fp);
+  if (valid) {
+    T* Hb = static_cast<T*>(B.H);
+    T* Pb = static_cast<T*>(B.P);
+#pragma unroll
+    for (int c = 0; c < 5; ++c) Hb[(size_t)c * N + i] = h[c];
+    if (B.p.flow_on) {  // with the flow frozen nothing reads the stress
+#pragma unroll
+      for (int c = 0; c < 9; ++c) Pb[(size_t)c * N + i] = p[c];
+    }
+  }
+  if (!(mode & FORCE_ACC)) return;
+  int my_c = -1;
+  double my_acc[6] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
+  for (int t0 = 0; t0 < nface; t0 += 32) {
+    const int t = t0 + lane;
+    int own, d, c, s[3];
+    face_of(t, own, d, c, s);
+    T po[9];
+#pragma unroll
+    for (int k = 0; k < 9; ++k) po[k] = __shfl_sync(full, p[k], own);
+    if (t < nface && c >= 0) {
       const int ax = d >> 1;
       const T sgn = (d & 1) ? T(-1) : T(1);
-      const T pcv[3] = {p[ax], p[3 + ax], p[6 + ax]};
-      colloid_face(B, fj - 1, ax, sgn, pcv, x, y, z, my_c, my_acc);
+      const T pcv[3] = {ax == 0 ? po[0] : (ax == 1 ? po[1] : po[2]), ax == 0 ? po[3] : (ax == 1 ? po[4] : po[5]),
+                        ax == 0 ? po[6] : (ax == 1 ? po[7] : po[8])};
+      // the fluid node: one step back from the solid node
+      const int L = ax == 0 ? nx : (ax == 1 ? ny : B.nz);
+      s[ax] = wrap1(s[ax] + ((d & 1) ? 1 : -1), L);
+      colloid_face(B, c, ax, sgn, pcv, s[0], s[1], s[2], my_c, my_acc);
     }
+  }
+  __syncwarp();
+  warp_flush_colloid(B.col, my_c, my_acc, 6);
+}
+
+// Plain node, one per lane: own Q and that of the x- and z-neighbours from pq.
+template <typename T>
+__device__ __forceinline__ void stress_node(const DevBox& B, const PhysT<T>& PP, const T* __restrict__ Q,
+                                            T* __restrict__ Hb, T* __restrict__ Pb, int x, int y, int z, int i,
+                                            const T (*pq)[5]) {
+  const int N = B.N;
+  T qi[5], qn[6][5], h[5], p[9], fp;
+  int nb[6], zz[2];
+  face_neighbours(B, x, y, z, nb, zz);
+#pragma unroll
+  for (int k = 0; k < 5; ++k) {
+    qi[k] = pq[0][k];
+    qn[0][k] = pq[1][k];
+    qn[1][k] = pq[2][k];
+    qn[4][k] = pq[3][k];
+    qn[5][k] = pq[4][k];
+  }
+#pragma unroll
+  for (int d = 2; d < 4; ++d)
+#pragma unroll
+    for (int k = 0; k < 5; ++k) qn[d][k] = ldg(Q + (size_t)k * N + nb[d]);
+  lc_node<T>(B, qi, qn, h, p, &fp);
+#pragma unroll
+  for (int c = 0; c < 5; ++c) Hb[(size_t)c * N + i] = h[c];
+  if (B.p.flow_on) {  // with the flow frozen nothing reads the stress
+#pragma unroll
+    for (int c = 0; c < 9; ++c) Pb[(size_t)c * N + i] = p[c];
   }
 }
 
@@ -629,7 +767,8 @@ __device__ __forceinline__ void stress_node(const DevBox& B, const PhysT<T>& PP,
 // time, so a row that crosses a colloid does not run the surface path with
 // most of its lanes idle.
 template <typename T, int TY>
-__device__ __forceinline__ void stress_tile(const DevBox& B, const int4 td, int zc, int mode, int (*sq)[2 * TX]) {
+__device__ __forceinline__ void stress_tile(const DevBox& B, const int4 td, int zc, int mode, int (*sq)[2 * TX],
+                                            NearScratch<T>& sc) {
   if (!B.p.lc_on) return;
   const int lane = threadIdx.x, wy = threadIdx.y;
   const PhysT<T>& PP = phys<T>(B);
@@ -640,8 +779,6 @@ __device__ __forceinline__ void stress_tile(const DevBox& B, const int4 td, int 
   const int x = td.y + lane, y = td.z + wy;
   const int zend = min(td.w + zc, B.nz);
   const bool valid = x < nx && y < ny;
-  int my_c = -1;
-  double my_acc[6] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
   int nq = 0;  // queued near nodes of this warp (warp-uniform)
   T qz[2][5];  // Q of the thread's own column at z - 1 and z, rolled down the z march
   column_start<T, 5>(B, Q, x, y, td.w, valid, qz);
@@ -653,16 +790,14 @@ __device__ __forceinline__ void stress_tile(const DevBox& B, const int4 td, int 
     T pq[5][5];
     column_next<T, 5>(B, Q, x, y, z, valid, qz, pq);
     x_neighbours<T, 5>(Q, (size_t)B.N, pq[0], lane, x, nx, nx * (y + ny * z), valid, &pq[1]);
-    if (fluid && !near) stress_node<T, false>(B, PP, Q, Hb, Pb, x, y, z, i, m, mode, my_c, my_acc, pq);
+    if (fluid && !near) stress_node<T>(B, PP, Q, Hb, Pb, x, y, z, i, pq);
     const unsigned nb = __ballot_sync(0xffffffffu, near);
     if (nb) {
       if (near) sq[wy][nq + __popc(nb & ((1u << lane) - 1u))] = i;
       nq += __popc(nb);
       __syncwarp();
       if (nq >= TX) {
-        const int j = sq[wy][lane];
-        const int jx = j % nx, jy = (j / nx) % ny, jz = j / (nx * ny);
-        stress_node<T, true>(B, PP, Q, Hb, Pb, jx, jy, jz, j, B.mask[j], mode, my_c, my_acc);
+        near_stress<T>(B, sq[wy][lane], mode, sc);
         __syncwarp();
         nq -= TX;
         if (lane < nq) sq[wy][lane] = sq[wy][TX + lane];
@@ -671,13 +806,8 @@ __device__ __forceinline__ void stress_tile(const DevBox& B, const int4 td, int 
     }
     column_roll<T, 5>(qz, pq);
   }
-  if (lane < nq) {
-    const int j = sq[wy][lane];
-    const int jx = j % nx, jy = (j / nx) % ny, jz = j / (nx * ny);
-    stress_node<T, true>(B, PP, Q, Hb, Pb, jx, jy, jz, j, B.mask[j], mode, my_c, my_acc);
-  }
+  near_stress<T>(B, lane < nq ? sq[wy][lane] : -1, mode, sc);
   __syncwarp();
-  if (mode & FORCE_ACC) warp_flush_colloid(B.col, my_c, my_acc, 6);
 }
 
 // ---------------------------------------------------------------------------
@@ -744,8 +874,8 @@ __device__ __forceinline__ void queue_push(int (*sq)[2 * TX], int wy, int lane, 
 // are issued before the current plane is evaluated, so their latency is
 // covered by that plane's arithmetic rather than by other warps.
 template <int TY>
-__device__ __forceinline__ void stress_tile_pair(const DevBox& B, const int4 td, int zc, int mode,
-                                                 int (*sq)[2 * TX]) {
+__device__ __forceinline__ void stress_tile_pair(const DevBox& B, const LcK<f2>& K2, const int4 td, int zc, int mode,
+                                                 int (*sq)[2 * TX], NearScratch<float>& sc) {
   if (!B.p.lc_on) return;
   const int lane = threadIdx.x, wy = threadIdx.y;
   const float* __restrict__ Q = static_cast<const float*>(B.Q[B.st->qpar]);
@@ -757,13 +887,8 @@ __device__ __forceinline__ void stress_tile_pair(const DevBox& B, const int4 td,
   const int zend = min(td.w + zc, nz);
   const bool valid = x < nx && y < ny;
   const int yp = y + 1 == ny ? 0 : y + 1, ym = y == 0 ? ny - 1 : y - 1;
-  int my_c = -1;
-  double my_acc[6] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
   int nq = 0;
-  auto near_fn = [&](int j) {
-    stress_node<float, true>(B, B.pf, Q, Hb, Pb, j % nx, (j / nx) % ny, j / (nx * ny), j, B.mask[j], mode, my_c,
-                             my_acc);
-  };
+  auto near_fn = [&](int j) { near_stress<float>(B, j, mode, sc); };
   f2 qz[2][5];  // the pair's Q at z - 1 and z, rolled down the z march
   f2 pz[5], pyp[5], pym[5];  // next plane's loads: the pair's Q at z + 1, the rows y + 1 and y - 1 at z
   unsigned pm2;              // and the pair's mask bytes at z
@@ -810,7 +935,7 @@ __device__ __forceinline__ void stress_tile_pair(const DevBox& B, const int4 td,
     if (plain) {
       f2 dq[3][5], lap[5], h[5], p[9], fp;
       derivatives(qz[1], qn, dq, lap);
-      lc_node_d<f2, true, float>(B.pf, qz[1], dq, lap, h, p, &fp);
+      lc_node_d<f2>(K2, B.p.q0 != 0.0, qz[1], dq, lap, h, p, &fp);
       const uint64_t keep = l2_keep();
 #pragma unroll
       for (int c = 0; c < 5; ++c) st2_keep(Hb + c * N + i, h[c], keep);
@@ -825,28 +950,233 @@ __device__ __forceinline__ void stress_tile_pair(const DevBox& B, const int4 td,
       qz[1][k] = qn[4][k];
     }
   }
-  if (lane < nq) near_fn(sq[wy][lane]);
+  near_fn(lane < nq ? sq[wy][lane] : -1);
   __syncwarp();
-  if (mode & FORCE_ACC) warp_flush_colloid(B.col, my_c, my_acc, 6);
 }
 
+// ---------------------------------------------------------------------------
+// nodes next to a solid or wall, and the plain tiles of the step kernels
+// ---------------------------------------------------------------------------
+// k_stress, k_lbp and k_lc take two kinds of work units: groups of 32 near
+// nodes from the box's list, one per warp, and tiles, which leave the near
+// nodes out.  The groups come first in the launch and spread over all SMs.  (With
+// the near nodes queued by the warp that meets them, the warps whose column
+// crosses a colloid ran batch after batch of the long surface path while the
+// rest of the GPU had finished: 38 us for the stress of a 37 x 29 x 23 box with
+// two colloids.)  Calls fn(B, node) for the group's node of this lane, or
+// fn(B, -1).
+template <int TY, typename Fn>
+__device__ __forceinline__ void near_group(const DevBox& B, const int2* __restrict__ groups, int block, Fn fn) {
+  const int e = groups[block * TY + threadIdx.y].y + (int)threadIdx.x;
+  const int n = min(*B.nnear, B.near_cap);
+  fn(e < n ? B.near_node[e] : -1);
+}
+
+// Planes of NC float components over a tile of 64 x TY columns and the rows
+// y0 - 1 .. y0 + TY, four z planes in a ring in shared memory.  Per row: the 64
+// columns, then the columns x0 - 1 and x0 + 64 (wrapped; the tile's own rows
+// only).  A plane is copied by cp.async one plane of arithmetic ahead, so the
+// march waits neither for memory nor holds prefetched values in registers;
+// one barrier per plane separates the copies into a slot from its last reads.
+template <int NC, int TY>
+struct Ring {
+  static constexpr int PW = 68, RY = TY + 2, PLANE = NC * RY * PW, SLOTS = 4;
+  static constexpr size_t BYTES = sizeof(float) * PLANE * SLOTS;
+};
+
+__device__ __forceinline__ void cp_async8(float* dst, const float* src) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src)
+               : "memory");
+}
+__device__ __forceinline__ void cp_async4(float* dst, const float* src) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src)
+               : "memory");
+}
+__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
+__device__ __forceinline__ void cp_async_wait0() { asm volatile("cp.async.wait_group 0;\n" ::: "memory"); }
+
+// Columns of the tile at (td.y, td.z): what a lane copies and where it finds
+// its neighbours.
+struct RingLane {
+  int x, y, row, rowm, rowp, rowe;  // node column; row starts of y, y - 1, y + vy, and of the edge column (node index)
+  int vx, vy, li, ri;               // valid columns and rows of the tile; ring columns of x - 1 and x + 2
+  bool valid, edge;                 // the lane's pair is a node pair; the lane copies an edge column
+};
+template <int TY>
+__device__ __forceinline__ RingLane ring_lane(const DevBox& B, const int4 td) {
+  RingLane R;
+  const int lane = threadIdx.x, nx = B.nx, ny = B.ny;
+  R.vx = min(64, nx - td.y);
+  R.vy = min(TY, ny - td.z);
+  R.x = td.y + 2 * lane;
+  R.y = td.z + (int)threadIdx.y;
+  R.valid = R.x < nx && R.y < ny;
+  R.row = nx * R.y;
+  R.rowm = nx * (td.z == 0 ? ny - 1 : td.z - 1);
+  R.rowp = nx * (td.z + R.vy >= ny ? 0 : td.z + R.vy);
+  R.edge = lane < 2 && R.y < ny;
+  R.rowe = R.row + (lane == 0 ? (td.y == 0 ? nx - 1 : td.y - 1) : (td.y + R.vx >= nx ? 0 : td.y + R.vx));
+  R.li = lane == 0 ? 64 : 2 * lane - 1;
+  R.ri = 2 * lane + 2 >= R.vx ? 65 : 2 * lane + 2;
+  return R;
+}
+
+// Copies plane z (-1 .. nz; wrapped, or nothing beyond a wall) of components
+// k0 .. k0 + NF - 1 (field F, component stride N) into the ring.
+template <int NC, int TY, int NF>
+__device__ __forceinline__ void ring_load(float* ring, const DevBox& B, const RingLane& R, const float* __restrict__ F,
+                                          int k0, int z, int slot) {
+  using Rg = Ring<NC, TY>;
+  const int nz = B.nz, lane = threadIdx.x, wy = threadIdx.y;
+  if (B.wall_z && (z < 0 || z >= nz)) return;
+  const size_t base = (size_t)B.nx * B.ny * (z < 0 ? z + nz : (z >= nz ? z - nz : z));
+  float* dst = ring + slot * Rg::PLANE + k0 * Rg::RY * Rg::PW;
+  const bool xin = R.x < B.nx;
+#pragma unroll
+  for (int k = 0; k < NF; ++k) {
+    const float* src = F + (size_t)k * B.N + base;
+    float* row = dst + (k * Rg::RY + wy + 1) * Rg::PW;
+    if (R.valid) cp_async8(row + 2 * lane, src + R.row + R.x);
+    if (R.edge) cp_async4(row + 64 + lane, src + R.rowe);
+    if (wy == (k0 + k) % TY && xin) {
+      cp_async8(dst + (k * Rg::RY) * Rg::PW + 2 * lane, src + R.rowm + R.x);
+      cp_async8(dst + (k * Rg::RY + R.vy + 1) * Rg::PW + 2 * lane, src + R.rowp + R.x);
+    }
+  }
+}
+
+__device__ __forceinline__ f2 sh2(const float* p) { return f2(*reinterpret_cast<const float2*>(p)); }
+
+// Values of component k at the pair's own column and its six neighbours
+// (the order of face_neighbours) in ring plane slot, from slots sm (z - 1)
+// and sp (z + 1).
+template <int NC, int TY>
+__device__ __forceinline__ void ring_gather(const float* ring, const RingLane& R, int k, int s0, int sm, int sp,
+                                            f2& own, f2 n[6]) {
+  using Rg = Ring<NC, TY>;
+  const int off = (k * Rg::RY + (int)threadIdx.y + 1) * Rg::PW, c = 2 * (int)threadIdx.x;
+  const float* p = ring + s0 * Rg::PLANE + off;
+  own = sh2(p + c);
+  n[0] = f2(own.v.y, p[R.ri]);
+  n[1] = f2(p[R.li], own.v.x);
+  n[2] = sh2(p + Rg::PW + c);
+  n[3] = sh2(p - Rg::PW + c);
+  n[4] = sh2(ring + sp * Rg::PLANE + off + c);
+  n[5] = sh2(ring + sm * Rg::PLANE + off + c);
+}
+
+__device__ __forceinline__ bool plain_node(unsigned m) { return (m & (IDMASK | NEAR)) == 0; }
+
+// Store v for the nodes of a pair that the tile path evaluates (a: the first,
+// b: the second).
+__device__ __forceinline__ void st2_keep_if(float* p, f2 v, bool a, bool b, uint64_t pol) {
+  if (a && b) st2_keep(p, v, pol);
+  else if (a) st_hint(p, v.v.x, pol);
+  else if (b) st_hint(p + 1, v.v.y, pol);
+}
+
+// Stress of a tile of plain nodes, two nodes per lane, Q from the ring.
+template <int TY>
+__device__ __forceinline__ void stress_ring(const DevBox& B, const LcK<f2>& K2, const int4 td, int zc, float* ring) {
+  if (!B.p.lc_on) return;
+  const float* __restrict__ Q = static_cast<const float*>(B.Q[B.st->qpar]);
+  float* __restrict__ Hb = static_cast<float*>(B.H);
+  float* __restrict__ Pb = static_cast<float*>(B.P);
+  const RingLane R = ring_lane<TY>(B, td);
+  const int nz = B.nz, zend = min(td.w + zc, nz);
+  const size_t N = (size_t)B.N;
+  const uint64_t keep = l2_keep();
+  const bool chiral = B.p.q0 != 0.0, flow = B.p.flow_on != 0;
+  const uint8_t* mp = B.mask + R.x + R.row;
+  const int plane = B.nx * B.ny;
+  __syncthreads();  // the ring's last reads (previous tile) are done
+#pragma unroll 1
+  for (int k = -1; k <= 1; ++k) ring_load<5, TY, 5>(ring, B, R, Q, 0, td.w + k, (k + 1) & 3);
+  cp_async_commit();
+  unsigned m2 = R.valid ? (unsigned)*reinterpret_cast<const uint16_t*>(mp + (size_t)plane * td.w) : 0x0101u;
+  for (int z = td.w; z < zend; ++z) {
+    const int s0 = (z - td.w + 1) & 3;
+    cp_async_wait0();
+    __syncthreads();
+    const bool pa = plain_node(m2 & 0xffu), pb = plain_node(m2 >> 8);
+    if (z + 1 < zend) {
+      ring_load<5, TY, 5>(ring, B, R, Q, 0, z + 2, (s0 + 2) & 3);
+      if (R.valid) m2 = (unsigned)*reinterpret_cast<const uint16_t*>(mp + (size_t)plane * (z + 1));
+    }
+    cp_async_commit();
+    if (!pa && !pb) continue;
+    f2 qi[5], dq[3][5], lap[5], h[5], p[9], fp;
+#pragma unroll
+    for (int k = 0; k < 5; ++k) {
+      f2 n[6];
+      ring_gather<5, TY>(ring, R, k, s0, (s0 + 3) & 3, (s0 + 1) & 3, qi[k], n);
+      dq[0][k] = n[0] - n[1];
+      dq[1][k] = n[2] - n[3];
+      dq[2][k] = n[4] - n[5];
+      lap[k] = ((n[0] + n[1]) + (n[2] + n[3]) + (n[4] + n[5])) + K2.nsix * qi[k];
+    }
+    lc_node_d<f2>(K2, chiral, qi, dq, lap, h, p, &fp);
+    const size_t i = (size_t)R.x + R.row + (size_t)plane * z;
+#pragma unroll
+    for (int c = 0; c < 5; ++c) st2_keep_if(Hb + c * N + i, h[c], pa, pb, keep);
+    if (flow) {  // with the flow frozen nothing reads the stress
+#pragma unroll
+      for (int c = 0; c < 9; ++c) st2_keep_if(Pb + c * N + i, p[c], pa, pb, keep);
+    }
+  }
+}
+
+// Stress of a tile of plain nodes, one node per lane (odd widths, FP64).
+template <typename T>
+__device__ __forceinline__ void stress_plain(const DevBox& B, const int4 td, int zc) {
+  if (!B.p.lc_on) return;
+  const int lane = threadIdx.x;
+  const T* __restrict__ Q = static_cast<const T*>(B.Q[B.st->qpar]);
+  const int nx = B.nx, ny = B.ny, x = td.y + lane, y = td.z + (int)threadIdx.y;
+  const int zend = min(td.w + zc, B.nz);
+  const bool valid = x < nx && y < ny;
+  T qz[2][5];
+  column_start<T, 5>(B, Q, x, y, td.w, valid, qz);
+  for (int z = td.w; z < zend; ++z) {
+    const int i = x + nx * (y + ny * z);
+    const uint8_t m = valid ? B.mask[i] : (uint8_t)1;
+    T pq[5][5];
+    column_next<T, 5>(B, Q, x, y, z, valid, qz, pq);
+    x_neighbours<T, 5>(Q, (size_t)B.N, pq[0], lane, x, nx, nx * (y + ny * z), valid, &pq[1]);
+    if (plain_node(m))
+      stress_node<T>(B, phys<T>(B), Q, static_cast<T*>(B.H), static_cast<T*>(B.P), x, y, z, i, pq);
+    column_roll<T, 5>(qz, pq);
+  }
+}
+
+// H and P stored once per fluid node, and the colloid LC force from the near
+// nodes.
 template <typename T, int TY>
-__global__ void __launch_bounds__(TX * TY, (sizeof(T) == 4 ? 384 : 256) / (TX * TY)) k_stress(
-    const DevBox* __restrict__ boxes, const int4* __restrict__ tiles, int ntiles, int zc, int mode,
-    double* __restrict__ part) {
+__global__ void __launch_bounds__(TX * TY, (sizeof(T) == 4 ? 512 : 256) / (TX * TY)) k_stress(Launch L, int mode) {
   __shared__ DevBox B;
-  __shared__ int sq[TY][2 * TX];  // per-warp queue of near fluid nodes
+  __shared__ LcK<f2> K2;
+  extern __shared__ __align__(16) float ring[];
   int cur_box = -1;
-  for (int t = blockIdx.x; t < ntiles; t += gridDim.x) {
-    const int4 td = tiles[t];
-    load_box(B, boxes, td.x, cur_box);
+  const int nn = L.ngroups / TY, units = nn + L.ntiles;
+  for (int t = blockIdx.x; t < units; t += gridDim.x) {
+    if (t < nn) {
+      load_box(B, K2, L.boxes, L.groups[t * TY].x, cur_box);
+      if (!B.p.lc_on) continue;
+      near_group<TY>(B, L.groups, t, [&](int j) {
+        near_stress<T>(B, j, mode, reinterpret_cast<NearScratch<T>*>(ring)[threadIdx.y]);
+      });
+      __syncthreads();
+      continue;
+    }
+    const int4 td = L.tiles[t - nn];
+    load_box(B, K2, L.boxes, td.x, cur_box);
     if constexpr (sizeof(T) == 4) {
       if (pair_box(B)) {
-        stress_tile_pair<TY>(B, td, zc, mode, sq);
+        stress_ring<TY>(B, K2, td, L.zc, ring);
         continue;
       }
     }
-    stress_tile<T, TY>(B, td, zc, mode, sq);
+    stress_plain<T>(B, td, L.zc);
   }
 }
 
@@ -956,17 +1286,47 @@ __device__ __forceinline__ void lbp_tile(const DevBox& B, const int4 td, int zc,
   __syncwarp();
 }
 
+// Tile of k_lbp: the plain nodes collided, solid nodes given the colloid's
+// velocity.
+template <typename T>
+__device__ __forceinline__ void lbp_plain(const DevBox& B, const int4 td, int zc) {
+  const int nx = B.nx, ny = B.ny, x = td.y + (int)threadIdx.x, y = td.z + (int)threadIdx.y;
+  if (x >= nx || y >= ny) return;
+  const int fpar = B.st->fpar, zend = min(td.w + zc, B.nz);
+  const bool pre = B.st->pre_valid != 0, lc = B.p.lc_on != 0;
+  const T* __restrict__ fin = static_cast<const T*>(B.f[fpar]);
+  T* __restrict__ fout = static_cast<T*>(B.f[fpar ^ 1]);
+  for (int z = td.w; z < zend; ++z) {
+    const int i = x + nx * (y + ny * z);
+    const uint8_t m = B.mask[i];
+    if (plain_node(m))
+      lbp_node<T, false>(B, phys<T>(B), fin, fout, static_cast<const T*>(B.P), static_cast<T*>(B.u), x, y, z, i, m,
+                         pre, lc);
+    else if (m & IDMASK)
+      solid_velocity(B, static_cast<T*>(B.u), x, y, z, i, m);
+  }
+}
+
 template <typename T, int TY>
-__global__ void __launch_bounds__(TX * TY, (sizeof(T) == 4 ? 768 : 384) / (TX * TY)) k_lbp(
-    const DevBox* __restrict__ boxes, const int4* __restrict__ tiles, int ntiles, int zc, int mode,
-    double* __restrict__ part) {
+__global__ void __launch_bounds__(TX * TY, (sizeof(T) == 4 ? 1024 : 384) / (TX * TY)) k_lbp(Launch L) {
   __shared__ DevBox B;
-  __shared__ int sq[TY][2 * TX];
   int cur_box = -1;
-  for (int t = blockIdx.x; t < ntiles; t += gridDim.x) {
-    const int4 td = tiles[t];
-    load_box(B, boxes, td.x, cur_box);
-    lbp_tile<T, TY, false>(B, td, zc, sq);
+  const int nn = L.ngroups / TY, units = nn + L.ntiles;
+  for (int t = blockIdx.x; t < units; t += gridDim.x) {
+    const int4 td = t < nn ? make_int4(L.groups[t * TY].x, 0, 0, 0) : L.tiles[t - nn];
+    load_box(B, L.boxes, td.x, cur_box);
+    if (!B.p.flow_on) continue;
+    if (t < nn) {
+      near_group<TY>(B, L.groups, t, [&](int j) {
+        if (j < 0) return;
+        const int fpar = B.st->fpar;
+        lbp_node<T, true>(B, phys<T>(B), static_cast<const T*>(B.f[fpar]), static_cast<T*>(B.f[fpar ^ 1]),
+                          static_cast<const T*>(B.P), static_cast<T*>(B.u), j % B.nx, (j / B.nx) % B.ny,
+                          j / (B.nx * B.ny), j, B.mask[j], B.st->pre_valid != 0, B.p.lc_on != 0);
+      });
+      continue;
+    }
+    lbp_plain<T>(B, td, L.zc);
   }
 }
 
@@ -1083,17 +1443,16 @@ __device__ __forceinline__ void lc_update_node(const DevBox& B, const PhysT<T>& 
                                                const T (*pq)[5] = nullptr, const T (*pu)[3] = nullptr,
                                                const float* plo = nullptr) {
   const int N = B.N;
-  // BF16 remainder of the node's own Q (FP32 storage), loaded with the other
-  // inputs so that its latency overlaps theirs
+  // H of this node was stored by the stress kernel of this step; Q of the
+  // fluid face neighbours is needed only for the advective fluxes (zero
+  // across solid faces), so no surface values are formed here.  Near nodes
+  // read the six mask bytes first and then everything else in one round of
+  // independent loads (a closed face loads the node's own Q, unused).
   float lo[5];
   if constexpr (sizeof(T) == 4) {
 #pragma unroll
     for (int c = 0; c < 5; ++c) lo[c] = NEAR_NODE ? __bfloat162float(Lin[(size_t)c * N + i]) : plo[c];
   }
-  const T Gam = PP.Gamma, xi = PP.xi;
-  // H of this node was stored by the stress kernel of this step; Q of the
-  // fluid face neighbours is needed only for the advective fluxes (zero
-  // across solid faces), so no surface values are formed here
   const T* __restrict__ Hb = static_cast<const T*>(B.H);
   T qi[5], qn[6][5], h[5];
 #pragma unroll
@@ -1108,9 +1467,10 @@ __device__ __forceinline__ void lc_update_node(const DevBox& B, const PhysT<T>& 
 #pragma unroll
   for (int a = 0; a < 3; ++a) ui[a] = NEAR_NODE ? ldx<CG>(U + (size_t)a * N + i) : pu[0][a];
 #pragma unroll
+  for (int d = 0; d < 6; ++d) fl[d] = !NEAR_NODE || (nb[d] >= 0 && (B.mask[nb[d] < 0 ? i : nb[d]] & IDMASK) == 0);
+#pragma unroll
   for (int d = 0; d < 6; ++d) {
     const int j = nb[d];
-    fl[d] = !NEAR_NODE || (j >= 0 && (B.mask[j] & IDMASK) == 0);
     if (!NEAR_NODE && d < 2) {
 #pragma unroll
       for (int a = 0; a < 3; ++a) un[d][a] = pu[1 + d][a];
@@ -1118,113 +1478,34 @@ __device__ __forceinline__ void lc_update_node(const DevBox& B, const PhysT<T>& 
       for (int c = 0; c < 5; ++c) qn[d][c] = pq[1 + d][c];
       continue;
     }
+    const size_t ju = NEAR_NODE && j < 0 ? i : j, jq = fl[d] ? j : i;
 #pragma unroll
-    for (int a = 0; a < 3; ++a) un[d][a] = (!NEAR_NODE || j >= 0) ? ldx<CG>(U + (size_t)a * N + j) : T(0);
+    for (int a = 0; a < 3; ++a) {
+      un[d][a] = ldx<CG>(U + (size_t)a * N + ju);
+      if (NEAR_NODE && j < 0) un[d][a] = T(0);
+    }
 #pragma unroll
-    for (int c = 0; c < 5; ++c) qn[d][c] = fl[d] ? ldg(Q + (size_t)c * N + j) : T(0);
+    for (int c = 0; c < 5; ++c) qn[d][c] = ldg(Q + (size_t)c * N + jq);
   }
-  // velocity gradient W_ab = d_b u_a
-  T W[3][3];
-#pragma unroll
-  for (int a = 0; a < 3; ++a)
-#pragma unroll
-    for (int b = 0; b < 3; ++b) W[a][b] = T(0.5) * (un[2 * b][a] - un[2 * b + 1][a]);
-  // advective fluxes through the six faces (zero across solid faces)
-  T adv[5] = {T(0), T(0), T(0), T(0), T(0)};
-#pragma unroll
-  for (int d = 0; d < 6; ++d) {
-    if (!fl[d]) continue;
-    const int ax = d >> 1;
-    const T uf = T(0.5) * (ui[ax] + un[d][ax]);
-    const bool plus = (d & 1) == 0;
-    // + face: upwind is i when uf > 0; - face: upwind is the neighbour when uf > 0
-    const bool take_i = plus ? (uf > T(0)) : !(uf > T(0));
-#pragma unroll
-    for (int k = 0; k < 5; ++k) {
-      const T fl_ = uf * (take_i ? qi[k] : qn[d][k]);
-      adv[k] += plus ? fl_ : -fl_;
-    }
-  }
-  // co-rotation S = xi (D Qt + Qt D) + (Om Q - Q Om) - 2 xi Qt Tr(Q W), Qt = Q + I/3
-  T D[3][3], Om[3][3];
-#pragma unroll
-  for (int a = 0; a < 3; ++a)
-#pragma unroll
-    for (int b = 0; b < 3; ++b) {
-      D[a][b] = T(0.5) * (W[a][b] + W[b][a]);
-      Om[a][b] = T(0.5) * (W[a][b] - W[b][a]);
-    }
-  T trQW = T(0);
-#pragma unroll
-  for (int a = 0; a < 3; ++a)
-#pragma unroll
-    for (int b = 0; b < 3; ++b) trQW += qab(qi, a, b) * D[a][b];
-  T dQ[3][3];
-#pragma unroll
-  for (int a = 0; a < 3; ++a)
-#pragma unroll
-    for (int b = 0; b < 3; ++b) {
-      T s = T(0);
-#pragma unroll
-      for (int c = 0; c < 3; ++c)
-        s += xi * (D[a][c] * qab(qi, c, b) + qab(qi, a, c) * D[c][b]) + Om[a][c] * qab(qi, c, b) -
-             qab(qi, a, c) * Om[c][b];
-      s += xi * T(2) / T(3) * D[a][b];
-      s -= T(2) * xi * (qab(qi, a, b) + (a == b ? T(1) / T(3) : T(0))) * trQW;
-      dQ[a][b] = s;
-    }
-  const T tr = dQ[0][0] + dQ[1][1] + dQ[2][2];
-  const int ia[5] = {0, 0, 0, 1, 1}, ib[5] = {0, 1, 2, 1, 2};
-  if constexpr (sizeof(T) == 4) {
-    // H was evaluated at hi; the stored Q is hi + lo.  Add the local part of
-    // H(hi + lo) - H(hi) to first order: the bulk terms' derivative at hi
-    // applied to lo, and lo's own term -6 K lo of the Laplacian (the
-    // neighbours' lo enter K lap and the gradient terms at the ~1e-9 level).
-    // Without it the relaxation stalls where A0 lo ~ the residual.
-    const T A0 = PP.A0, g = PP.gamma, K = PP.K, q0 = PP.q0;
-    T Qm[3][3], Lm[3][3];
-#pragma unroll
-    for (int a = 0; a < 3; ++a)
-#pragma unroll
-      for (int b = 0; b < 3; ++b) {
-        Qm[a][b] = qab(qi, a, b);
-        Lm[a][b] = qab(lo, a, b);
-      }
-    T trq2 = T(0), trql = T(0);
-#pragma unroll
-    for (int a = 0; a < 3; ++a)
-#pragma unroll
-      for (int b = 0; b < 3; ++b) {
-        trq2 += Qm[a][b] * Qm[a][b];
-        trql += Qm[a][b] * Lm[a][b];
-      }
-    const T cb = -A0 * (T(1) - g / T(3)) - A0 * g * trq2 - T(4) * K * q0 * q0 - T(6) * K;
-    const T A0g = A0 * g;
-#pragma unroll
-    for (int k = 0; k < 5; ++k) {
-      const int a = ia[k], b = ib[k];
-      T ql = T(0);
-#pragma unroll
-      for (int c = 0; c < 3; ++c) ql += Qm[a][c] * Lm[c][b] + Lm[a][c] * Qm[c][b];
-      if (a == b) ql -= T(2) / T(3) * trql;
-      h[k] += cb * lo[k] + A0g * ql - T(2) * A0g * trql * qi[k];
-    }
-  }
-  T d5[5];
+  T G[9], cd[6], self, adv[5], d5[5];
+  flow_terms<T>(lck<T>(B), ui, un, fl, G, cd, self);
 #pragma unroll
   for (int k = 0; k < 5; ++k) {
-    T v = Gam * h[k] + dQ[ia[k]][ib[k]] - adv[k];
-    if (ia[k] == ib[k]) v -= tr / T(3);
-    d5[k] = v;
+    const T n[6] = {qn[0][k], qn[1][k], qn[2][k], qn[3][k], qn[4][k], qn[5][k]};
+    adv[k] = advect(cd, self, qi[k], n);
+  }
+  q_increment<sizeof(T) == 4, true, T>(lck<T>(B), qi, adv, G, h, reinterpret_cast<const T*>(lo), d5);
+#pragma unroll
+  for (int k = 0; k < 5; ++k) {
     if constexpr (sizeof(T) == 4) {
       // compensated FP32 storage: hi + lo + increment carried exactly into hi, to BF16 in lo
       float hi;
       __nv_bfloat16 lo_out;
-      add_compensated(qi[k], lo[k], v, hi, lo_out);
+      add_compensated(qi[k], lo[k], d5[k], hi, lo_out);
       Qo[(size_t)k * N + i] = hi;
       Lout[(size_t)k * N + i] = lo_out;
     } else {
-      Qo[(size_t)k * N + i] = qi[k] + v;
+      Qo[(size_t)k * N + i] = qi[k] + d5[k];
     }
   }
   const T dzz = -d5[0] - d5[3];
@@ -1304,114 +1585,24 @@ __device__ __forceinline__ void lc_tile(const DevBox& B, const int4 td, int zc, 
 // Q update, two nodes per lane (FP32 boxes of even width; tiles 64 wide): the
 // Beris-Edwards update of lc_update_node for the nodes x, x + 1 at once, in
 // packed FP32x2 arithmetic, with Q, u, H and the BF16 remainder of Q moved as
-// pairs.  The upwind choice of each face flux is taken per node.
-__device__ __forceinline__ f2 sel2(bool ca, bool cb, f2 a, f2 b) {
-  return f2(ca ? a.v.x : b.v.x, cb ? a.v.y : b.v.y);
-}
-
-__device__ __forceinline__ void lc_update_pair(const DevBox& B, float* __restrict__ Qo,
+// pairs.
+__device__ __forceinline__ void lc_update_pair(const DevBox& B, const LcK<f2>& K2, float* __restrict__ Qo,
                                                __nv_bfloat16* __restrict__ Lout, int i, const f2 qi[5],
-                                               const f2 qn[6][5], const f2 ui[3], const f2 un[6][3], const f2 h_[5],
+                                               const f2 qn[6][5], const f2 ui[3], const f2 un[6][3], const f2 h[5],
                                                const f2 lo[5], float& rsum, float& rmax) {
-  const PhysT<float>& PP = B.pf;
   const size_t N = (size_t)B.N;
-  const float Gam = PP.Gamma, xi = PP.xi;
-  f2 h[5];
-#pragma unroll
-  for (int k = 0; k < 5; ++k) h[k] = h_[k];
-  // velocity gradient W_ab = d_b u_a
-  f2 W[3][3];
-#pragma unroll
-  for (int a = 0; a < 3; ++a)
-#pragma unroll
-    for (int b = 0; b < 3; ++b) W[a][b] = f2(0.5f * (un[2 * b][a] - un[2 * b + 1][a]));
-  // upwind advective fluxes through the six faces (no solid faces here)
-  f2 adv[5] = {f2(0.f), f2(0.f), f2(0.f), f2(0.f), f2(0.f)};
-#pragma unroll
-  for (int d = 0; d < 6; ++d) {
-    const int ax = d >> 1;
-    const f2 uf = f2(0.5f * (ui[ax] + un[d][ax]));
-    const bool plus = (d & 1) == 0;
-    const bool pa = uf.v.x > 0.f, pb = uf.v.y > 0.f;
-    const bool ta = plus ? pa : !pa, tb = plus ? pb : !pb;
-#pragma unroll
-    for (int k = 0; k < 5; ++k) {
-      const f2 up = sel2(ta, tb, qi[k], qn[d][k]);
-      adv[k] = plus ? adv[k] + uf * up : adv[k] - uf * up;
-    }
-  }
-  // co-rotation S = xi (D Qt + Qt D) + (Om Q - Q Om) - 2 xi Qt Tr(Q W), Qt = Q + I/3
-  f2 D[3][3], Om[3][3], Qm[3][3];
-#pragma unroll
-  for (int a = 0; a < 3; ++a)
-#pragma unroll
-    for (int b = 0; b < 3; ++b) {
-      D[a][b] = f2(0.5f * (W[a][b] + W[b][a]));
-      Om[a][b] = f2(0.5f * (W[a][b] - W[b][a]));
-      Qm[a][b] = qab(qi, a, b);
-    }
-  f2 trQW = f2(0.f);
-#pragma unroll
-  for (int a = 0; a < 3; ++a)
-#pragma unroll
-    for (int b = 0; b < 3; ++b) trQW = trQW + Qm[a][b] * D[a][b];
-  const int ia[5] = {0, 0, 0, 1, 1}, ib[5] = {0, 1, 2, 1, 2};
-  const float twoxi = 2.f * xi, xi23 = 2.f * xi / 3.f, third = 1.f / 3.f;
-  f2 dQ[3][3];
-#pragma unroll
-  for (int a = 0; a < 3; ++a)
-#pragma unroll
-    for (int b = 0; b < 3; ++b) {
-      f2 sacc = f2(0.f);
-#pragma unroll
-      for (int c = 0; c < 3; ++c) {
-        const f2 dq = D[a][c] * Qm[c][b] + Qm[a][c] * D[c][b];
-        sacc = sacc + xi * dq;
-        sacc = sacc + Om[a][c] * Qm[c][b];
-        sacc = sacc - Qm[a][c] * Om[c][b];
-      }
-      sacc = sacc + xi23 * D[a][b];
-      const f2 qt = a == b ? Qm[a][b] + third : Qm[a][b];
-      sacc = sacc - twoxi * (qt * trQW);
-      dQ[a][b] = sacc;
-    }
-  const f2 tr = dQ[0][0] + dQ[1][1] + dQ[2][2];
-  {
-    // local part of H(hi + lo) - H(hi) to first order (as lc_update_node)
-    const float A0 = PP.A0, g = PP.gamma, K = PP.K, q0 = PP.q0;
-    f2 Lm[3][3];
-#pragma unroll
-    for (int a = 0; a < 3; ++a)
-#pragma unroll
-      for (int b = 0; b < 3; ++b) Lm[a][b] = qab(lo, a, b);
-    f2 trq2 = f2(0.f), trql = f2(0.f);
-#pragma unroll
-    for (int a = 0; a < 3; ++a)
-#pragma unroll
-      for (int b = 0; b < 3; ++b) {
-        trq2 = trq2 + Qm[a][b] * Qm[a][b];
-        trql = trql + Qm[a][b] * Lm[a][b];
-      }
-    const float A0g = A0 * g;
-    const f2 cb = (-A0 * (1.f - g / 3.f) - 4.f * K * q0 * q0 - 6.f * K) - A0g * trq2;
-    const f2 trql2 = f2(2.f * A0g * trql);
-#pragma unroll
-    for (int k = 0; k < 5; ++k) {
-      const int a = ia[k], b = ib[k];
-      f2 ql = f2(0.f);
-#pragma unroll
-      for (int c = 0; c < 3; ++c) ql = ql + Qm[a][c] * Lm[c][b] + Lm[a][c] * Qm[c][b];
-      if (a == b) ql = ql - (2.f / 3.f) * trql;
-      h[k] = h[k] + cb * lo[k] + A0g * ql - trql2 * qi[k];
-    }
-  }
-  f2 d5[5];
-  const f2 tr3 = f2(third * tr);
+  const bool open[6] = {true, true, true, true, true, true};
+  f2 G[9], cd[6], self, adv[5], d5[5];
+  flow_terms<f2>(K2, ui, un, open, G, cd, self);
 #pragma unroll
   for (int k = 0; k < 5; ++k) {
-    f2 v = Gam * h[k] + dQ[ia[k]][ib[k]] - adv[k];
-    if (ia[k] == ib[k]) v = v - tr3;
-    d5[k] = v;
+    const f2 n[6] = {qn[0][k], qn[1][k], qn[2][k], qn[3][k], qn[4][k], qn[5][k]};
+    adv[k] = advect(cd, self, qi[k], n);
+  }
+  q_increment<true, true, f2>(K2, qi, adv, G, h, lo, d5);
+#pragma unroll
+  for (int k = 0; k < 5; ++k) {
+    const f2 v = d5[k];
     // compensated storage: hi + lo + v carried exactly into (hi, lo) (two-sum)
     const f2 sv = lo[k] + v;
     const f2 hn = qi[k] + sv;
@@ -1430,7 +1621,7 @@ __device__ __forceinline__ void lc_update_pair(const DevBox& B, float* __restric
 }
 
 template <int TY, bool CG>
-__device__ __forceinline__ void lc_tile_pair(const DevBox& B, const int4 td, int zc, double* part,
+__device__ __forceinline__ void lc_tile_pair(const DevBox& B, const LcK<f2>& K2, const int4 td, int zc, double* part,
                                              int (*sq)[2 * TX]) {
   if (!B.p.lc_on) return;
   const int lane = threadIdx.x, wy = threadIdx.y;
@@ -1489,7 +1680,7 @@ __device__ __forceinline__ void lc_tile_pair(const DevBox& B, const int4 td, int
       for (int a = 0; a < 3; ++a)
 #pragma unroll
         for (int d = 0; d < 4; ++d) un[2 + d][a] = ldx2<CG>(U + a * N + jr[d]);
-      lc_update_pair(B, Qo, Lout, i, qi, qn, ui, un, h, lo, rsum, rmax);
+      lc_update_pair(B, K2, Qo, Lout, i, qi, qn, ui, un, h, lo, rsum, rmax);
     }
     queue_push(sq, wy, lane, nq, valid && fA && !plain, i, near_fn);
     queue_push(sq, wy, lane, nq, valid && fB && !plain, i + 1, near_fn);
@@ -1497,27 +1688,6 @@ __device__ __forceinline__ void lc_tile_pair(const DevBox& B, const int4 td, int
   if (lane < nq) near_fn(sq[wy][lane]);
   __syncwarp();
   if (part) warp_residual<float>(part, wy, lane, rsum, rmax);
-}
-
-template <typename T, int TY>
-__global__ void __launch_bounds__(TX * TY, (sizeof(T) == 4 ? 512 : 256) / (TX * TY)) k_lc(
-    const DevBox* __restrict__ boxes, const int4* __restrict__ tiles, int ntiles, int zc, int mode,
-    double* __restrict__ part) {
-  __shared__ DevBox B;
-  __shared__ int sq[TY][2 * TX];
-  int cur_box = -1;
-  for (int t = blockIdx.x; t < ntiles; t += gridDim.x) {
-    const int4 td = tiles[t];
-    load_box(B, boxes, td.x, cur_box);
-    double* pt = (mode & LC_RESID) ? part + 2 * (size_t)t * TY : nullptr;
-    if constexpr (sizeof(T) == 4) {
-      if (pair_box(B)) {
-        lc_tile_pair<TY, false>(B, td, zc, pt, sq);
-        continue;
-      }
-    }
-    lc_tile<T, TY, false>(B, td, zc, pt, sq);
-  }
 }
 
 // ---------------------------------------------------------------------------
@@ -1564,31 +1734,29 @@ __device__ __forceinline__ void links_chunk(const DevBox& B, int l0, int n, doub
 #undef LCLB_CASE
         default: break;
       }
-      const double w = (q <= 6) ? 1.0 / 18.0 : 1.0 / 36.0;
       const DevColloid& C = B.col[c];
-      double d[3], ubv[3];
+      double d[3];
       disp(B, x + 0.5 * qx, y + 0.5 * qy, z + 0.5 * qz, C.X, d);
-      rigid_velocity(C.V, C.W, d, ubv);
-      const double corr = 6.0 * w * B.p.rho0 * (qx * ubv[0] + qy * ubv[1] + qz * ubv[2]);
-      const double mag = 2.0 * dfq - corr;
-      const double dp[3] = {qx * mag, qy * mag, qz * mag};
-      const double tq[3] = {d[1] * dp[2] - d[2] * dp[1], d[2] * dp[0] - d[0] * dp[2], d[0] * dp[1] - d[1] * dp[0]};
+      // with rc = d x c_b, c_b.(V + W x d) = c_b.V + W.rc and the torque of
+      // dp = mag c_b is mag rc
+      const double cc[3] = {(double)qx, (double)qy, (double)qz};
+      const double rc[3] = {d[1] * cc[2] - d[2] * cc[1], d[2] * cc[0] - d[0] * cc[2], d[0] * cc[1] - d[1] * cc[0]};
+      const double zk = (q <= 6 ? 6.0 / 18.0 : 6.0 / 36.0) * B.p.rho0;
+      const double cub = cc[0] * C.V[0] + cc[1] * C.V[1] + cc[2] * C.V[2] + rc[0] * C.W[0] + rc[1] * C.W[1] + rc[2] * C.W[2];
+      const double mag = 2.0 * dfq - zk * cub;
       my_c = c;
       for (int a = 0; a < 3; ++a) {
-        v[a] = dp[a];
-        v[3 + a] = tq[a];
+        v[a] = cc[a] * mag;
+        v[3 + a] = rc[a] * mag;
       }
       mob = C.mobile != 0;
       if (mob) {
         // the part of dp linear in the rigid velocity, -6 w rho0 c (c.(V + W x d)):
         // coefficients 6 w rho0 c c (V-V) and 6 w rho0 (d x c)(d x c) (W-W)
-        const double zk = 6.0 * w * B.p.rho0;
-        const double cc[3] = {(double)qx, (double)qy, (double)qz};
-        const double rc[3] = {d[1] * cc[2] - d[2] * cc[1], d[2] * cc[0] - d[0] * cc[2], d[0] * cc[1] - d[1] * cc[0]};
         const int ia[6] = {0, 0, 0, 1, 1, 2}, ib[6] = {0, 1, 2, 1, 2, 2};
 #pragma unroll
         for (int k = 0; k < 6; ++k) {
-          v[6 + k] = zk * cc[ia[k]] * cc[ib[k]];
+          v[6 + k] = zk * (cc[ia[k]] * cc[ib[k]]);
           v[12 + k] = zk * rc[ia[k]] * rc[ib[k]];
         }
       }
@@ -1673,7 +1841,7 @@ __device__ int contact_partner(const DevBox& B, int c) {
 // colloid index of that pass) is kept in the box state and flagged in the
 // group's error words; the host reports it as LC_ERR_OVERLAP.  All threads of
 // the block call this (it holds block barriers).
-__device__ void resolve_contacts(DevBox& B, int tid, int nthr) {
+__device__ void resolve_contacts(const DevBox& B, int tid, int nthr) {
   __shared__ signed char s_hit[MAXCOL];  // -2 no contact, else the partner
   __shared__ unsigned char s_back[MAXCOL];
   __shared__ int s_any;
@@ -1711,7 +1879,7 @@ __device__ void resolve_contacts(DevBox& B, int tid, int nthr) {
 }
 
 template <bool CG>
-__device__ __forceinline__ void colloid_box(DevBox& B, bool commit = true) {
+__device__ __forceinline__ void colloid_box(const DevBox& B, bool commit = true) {
   const int tid = threadIdx.x + blockDim.x * threadIdx.y;
   const int nthr = blockDim.x * blockDim.y;
   if (!commit) {
@@ -1772,7 +1940,236 @@ __device__ __forceinline__ void colloid_box(DevBox& B, bool commit = true) {
   }
 }
 
-__global__ void k_colloid(DevBox* __restrict__ boxes, int nboxes) {
+// ---------------------------------------------------------------------------
+// k_lc: Q update, link exchange and colloid update in one launch
+// ---------------------------------------------------------------------------
+// Q update of a tile of plain nodes, two nodes per lane: Q and u from the
+// ring, H and the remainder of Q from global memory, issued before the ring
+// reads of the plane.
+template <int TY>
+__device__ __forceinline__ void lc_ring(const DevBox& B, const LcK<f2>& K2, const int4 td, int zc, float* ring,
+                                        float& rsum, float& rmax) {
+  if (!B.p.lc_on) return;
+  const int qpar = B.st->qpar;
+  const float* __restrict__ Q = static_cast<const float*>(B.Q[qpar]);
+  float* __restrict__ Qo = static_cast<float*>(B.Q[qpar ^ 1]);
+  const __nv_bfloat16* __restrict__ Lin = B.Qlo[qpar];
+  __nv_bfloat16* __restrict__ Lout = B.Qlo[qpar ^ 1];
+  const float* __restrict__ U = static_cast<const float*>(B.u);
+  const float* __restrict__ Hb = static_cast<const float*>(B.H);
+  const RingLane R = ring_lane<TY>(B, td);
+  const int nz = B.nz, zend = min(td.w + zc, nz), plane = B.nx * B.ny;
+  const size_t N = (size_t)B.N;
+  const uint8_t* mp = B.mask + R.x + R.row;
+  __syncthreads();
+#pragma unroll 1
+  for (int k = -1; k <= 1; ++k) {
+    ring_load<8, TY, 5>(ring, B, R, Q, 0, td.w + k, (k + 1) & 3);
+    ring_load<8, TY, 3>(ring, B, R, U, 5, td.w + k, (k + 1) & 3);
+  }
+  cp_async_commit();
+  unsigned m2 = R.valid ? (unsigned)*reinterpret_cast<const uint16_t*>(mp + (size_t)plane * td.w) : 0x0101u;
+  for (int z = td.w; z < zend; ++z) {
+    const int s0 = (z - td.w + 1) & 3, sm = (s0 + 3) & 3, sp = (s0 + 1) & 3;
+    const size_t i = (size_t)R.x + R.row + (size_t)plane * z;
+    const bool pa = plain_node(m2 & 0xffu), pb = plain_node(m2 >> 8);
+    float2 hr[5];
+    __nv_bfloat162 lr[5];
+    if (pa || pb) {
+#pragma unroll
+      for (int k = 0; k < 5; ++k) {
+        hr[k] = __ldg(reinterpret_cast<const float2*>(Hb + k * N + i));
+        lr[k] = *reinterpret_cast<const __nv_bfloat162*>(Lin + k * N + i);
+      }
+    }
+    cp_async_wait0();
+    __syncthreads();
+    if (z + 1 < zend) {
+      ring_load<8, TY, 5>(ring, B, R, Q, 0, z + 2, (s0 + 2) & 3);
+      ring_load<8, TY, 3>(ring, B, R, U, 5, z + 2, (s0 + 2) & 3);
+      if (R.valid) m2 = (unsigned)*reinterpret_cast<const uint16_t*>(mp + (size_t)plane * (z + 1));
+    }
+    cp_async_commit();
+    if (!pa && !pb) continue;
+    f2 qi[5], G[9], cd[6], self, adv[5], d5[5];
+    {
+      f2 ui[3], un[6][3];
+#pragma unroll
+      for (int a = 0; a < 3; ++a) {
+        f2 n[6];
+        ring_gather<8, TY>(ring, R, 5 + a, s0, sm, sp, ui[a], n);
+#pragma unroll
+        for (int d = 0; d < 6; ++d) un[d][a] = n[d];
+      }
+      const bool open[6] = {true, true, true, true, true, true};
+      flow_terms<f2>(K2, ui, un, open, G, cd, self);
+    }
+    // one component's neighbours at a time: read all together, the 35 values
+    // of Q would push the kernel past its registers
+#pragma unroll
+    for (int k = 0; k < 5; ++k) {
+      f2 n[6];
+      asm volatile("" ::: "memory");
+      ring_gather<8, TY>(ring, R, k, s0, sm, sp, qi[k], n);
+      adv[k] = advect(cd, self, qi[k], n);
+    }
+    asm volatile("" ::: "memory");
+    f2 h[5], lo[5];
+#pragma unroll
+    for (int k = 0; k < 5; ++k) {
+      h[k] = f2(hr[k]);
+      lo[k] = f2(__bfloat1622float2(lr[k]));
+    }
+    q_increment<true, true, f2>(K2, qi, adv, G, h, lo, d5);
+#pragma unroll
+    for (int k = 0; k < 5; ++k) {
+      // compensated storage: hi + lo + increment carried exactly into (hi, lo) (two-sum)
+      const f2 sv = lo[k] + d5[k];
+      const f2 hn = qi[k] + sv;
+      const f2 bb = hn - qi[k];
+      const f2 err = (qi[k] - (hn - bb)) + (sv - bb);
+      const __nv_bfloat162 l2 = __float22bfloat162_rn(err.v);
+      float* q = Qo + (size_t)k * N + i;
+      __nv_bfloat16* l = Lout + (size_t)k * N + i;
+      if (pa && pb) {
+        st2(q, hn);
+        *reinterpret_cast<__nv_bfloat162*>(l) = l2;
+      } else if (pa) {
+        q[0] = hn.v.x;
+        l[0] = l2.x;
+      } else {
+        q[1] = hn.v.y;
+        l[1] = l2.y;
+      }
+    }
+    const f2 dzz = -(d5[0] + d5[3]);
+    const f2 r2 = d5[0] * d5[0] + d5[3] * d5[3] + dzz * dzz + 2.f * (d5[1] * d5[1] + d5[2] * d5[2] + d5[4] * d5[4]);
+    float mx = fabsf(dzz.v.x), my = fabsf(dzz.v.y);
+#pragma unroll
+    for (int k = 0; k < 5; ++k) {
+      mx = fmaxf(mx, fabsf(d5[k].v.x));
+      my = fmaxf(my, fabsf(d5[k].v.y));
+    }
+    if (pa) {
+      rsum += r2.v.x;
+      rmax = fmaxf(rmax, mx);
+    }
+    if (pb) {
+      rsum += r2.v.y;
+      rmax = fmaxf(rmax, my);
+    }
+  }
+}
+
+// Q update of a tile of plain nodes, one node per lane.
+template <typename T>
+__device__ __forceinline__ void lc_plain(const DevBox& B, const int4 td, int zc, T& rsum, T& rmax) {
+  if (!B.p.lc_on) return;
+  const int lane = threadIdx.x, qpar = B.st->qpar;
+  const T* __restrict__ Q = static_cast<const T*>(B.Q[qpar]);
+  const __nv_bfloat16* __restrict__ Lin = B.Qlo[qpar];
+  const T* __restrict__ U = static_cast<const T*>(B.u);
+  const int nx = B.nx, ny = B.ny, x = td.y + lane, y = td.z + (int)threadIdx.y;
+  const int zend = min(td.w + zc, B.nz);
+  const bool valid = x < nx && y < ny;
+  for (int z = td.w; z < zend; ++z) {
+    const int row = nx * (y + ny * z), i = x + row;
+    const uint8_t m = valid ? B.mask[i] : (uint8_t)1;
+    const bool plain = plain_node(m);
+    T pq[3][5], pu[3][3];
+    float plo[5];
+#pragma unroll
+    for (int k = 0; k < 5; ++k) pq[0][k] = valid ? ldg(Q + (size_t)k * B.N + i) : T(0);
+#pragma unroll
+    for (int a = 0; a < 3; ++a) pu[0][a] = valid ? ldg(U + (size_t)a * B.N + i) : T(0);
+    if constexpr (sizeof(T) == 4) {
+#pragma unroll
+      for (int k = 0; k < 5; ++k) plo[k] = plain ? __bfloat162float(Lin[(size_t)k * B.N + i]) : 0.f;
+    }
+    x_neighbours<T, 5>(Q, (size_t)B.N, pq[0], lane, x, nx, row, valid, &pq[1]);
+    x_neighbours<T, 3>(U, (size_t)B.N, pu[0], lane, x, nx, row, valid, &pu[1]);
+    if (plain)
+      lc_update_node<T, false>(B, phys<T>(B), Q, static_cast<T*>(B.Q[qpar ^ 1]), Lin, B.Qlo[qpar ^ 1], U, x, y, z, i, m,
+                               rsum, rmax, pq, pu, plo);
+  }
+}
+
+// The work units of a box are counted as they finish; the block that finishes
+// the last one of a box (near groups, link chunks and tiles) runs its colloid
+// update and parity flip, so a step takes no separate launches for the link
+// exchange and the colloid update (16 and 6 us beside or after a 62 us update
+// at 128^3, and most of the step of a small box).  The counter is zero again
+// when the launch ends.  All threads of the block call this.
+__device__ __forceinline__ void lc_commit(const Launch& L, int b, unsigned n) {
+  __shared__ int s_last;
+  __threadfence();
+  __syncthreads();
+  if (threadIdx.x + threadIdx.y == 0) s_last = atomicAdd(L.done + b, n) + n == L.total[b];
+  __syncthreads();
+  if (s_last) {
+    __threadfence();
+    colloid_box<true>(L.boxes[b]);
+    if (threadIdx.x + threadIdx.y == 0) L.done[b] = 0;
+  }
+  __syncthreads();
+}
+
+template <typename T, int TY>
+__global__ void __launch_bounds__(TX * TY, (sizeof(T) == 4 ? 512 : 256) / (TX * TY)) k_lc(Launch L, int mode,
+                                                                                         double* __restrict__ part) {
+  __shared__ DevBox B;
+  __shared__ LcK<f2> K2;
+  __shared__ double sblk[18];
+  __shared__ int sc0;
+  extern __shared__ __align__(16) float ring[];
+  const bool commit = (mode & LC_COMMIT) != 0;
+  const int lane = threadIdx.x, wy = threadIdx.y;
+  const int nn = L.ngroups / TY, nl = commit ? L.nchunks : 0, units = nn + nl + L.ntiles;
+  int cur_box = -1, run_box = -1;
+  unsigned run_n = 0;
+  for (int t = blockIdx.x; t < units; t += gridDim.x) {
+    const int4 td = t < nn ? make_int4(L.groups[t * TY].x, 0, 0, 0)
+                           : (t < nn + nl ? make_int4(L.chunks[t - nn].x, L.chunks[t - nn].y, 0, 0) : L.tiles[t - nn - nl]);
+    if (commit && td.x != run_box) {
+      if (run_n) lc_commit(L, run_box, run_n);
+      run_box = td.x;
+      run_n = 0;
+    }
+    ++run_n;
+    load_box(B, K2, L.boxes, td.x, cur_box);
+    T rsum = T(0), rmax = T(0);  // per-thread residual (sum of squares, max), in T
+    if (t < nn) {
+      if (B.p.lc_on)
+        near_group<TY>(B, L.groups, t, [&](int j) {
+          if (j < 0) return;
+          const int qpar = B.st->qpar;
+          lc_update_node<T, true>(B, phys<T>(B), static_cast<const T*>(B.Q[qpar]), static_cast<T*>(B.Q[qpar ^ 1]),
+                                  B.Qlo[qpar], B.Qlo[qpar ^ 1], static_cast<const T*>(B.u), j % B.nx,
+                                  (j / B.nx) % B.ny, j / (B.nx * B.ny), j, B.mask[j], rsum, rmax);
+        });
+      __syncwarp();
+      if (mode & LC_RESID) warp_residual<T>(L.npart + 2 * (size_t)t * TY, wy, lane, rsum, rmax);
+      continue;
+    }
+    if (t < nn + nl) {
+      links_chunk<T, false>(B, td.y, TX * TY, sblk, &sc0);
+      continue;
+    }
+    bool done = false;
+    if constexpr (sizeof(T) == 4) {
+      if (pair_box(B)) {
+        lc_ring<TY>(B, K2, td, L.zc, ring, rsum, rmax);
+        done = true;
+      }
+    }
+    if (!done) lc_plain<T>(B, td, L.zc, rsum, rmax);
+    __syncwarp();
+    if (mode & LC_RESID) warp_residual<T>(part + 2 * (size_t)(t - nn - nl) * TY, wy, lane, rsum, rmax);
+  }
+  if (commit && run_n) lc_commit(L, run_box, run_n);
+}
+
+__global__ void k_colloid(const DevBox* __restrict__ boxes, int nboxes) {
   const int b = blockIdx.x;
   if (b >= nboxes) return;
   colloid_box<false>(boxes[b]);
@@ -1805,9 +2202,12 @@ __global__ void __launch_bounds__(TX * TY, (sizeof(T) == 4 ? 512 : 256) / (TX * 
     DevBox* __restrict__ boxes, const StepItem* __restrict__ items, int nitems, int zc, unsigned* __restrict__ sync,
     double* __restrict__ part, int spin_limit, int commit, int* __restrict__ err) {
   __shared__ DevBox B;
+  __shared__ LcK<f2> K2;
   __shared__ double sblk[18];
   __shared__ int sq[TY][2 * TX];
   __shared__ int s_item, s_ok, s_sc0;
+  extern __shared__ __align__(16) float step_smem[];
+  NearScratch<T>& sc = reinterpret_cast<NearScratch<T>*>(step_smem)[threadIdx.y];
   const int tid = threadIdx.x + TX * threadIdx.y;
   int cur_box = -1;
   for (;;) {
@@ -1836,23 +2236,23 @@ __global__ void __launch_bounds__(TX * TY, (sizeof(T) == 4 ? 512 : 256) / (TX * 
     }
     __syncthreads();
     if (s_ok) {
-      load_box(B, boxes, I.box, cur_box);
+      load_box(B, K2, boxes, I.box, cur_box);
       const int4 td = make_int4(I.box, I.x0, I.y0, I.z0);
       switch (I.kind) {
         case ITEM_STRESS:
           if constexpr (sizeof(T) == 4) {
             if (pair_box(B)) {
-              stress_tile_pair<TY>(B, td, zc, FORCE_ACC, sq);
+              stress_tile_pair<TY>(B, K2, td, zc, FORCE_ACC, sq, sc);
               break;
             }
           }
-          stress_tile<T, TY>(B, td, zc, FORCE_ACC, sq);
+          stress_tile<T, TY>(B, td, zc, FORCE_ACC, sq, sc);
           break;
         case ITEM_LB: lbp_tile<T, TY, true>(B, td, zc, sq); break;
         case ITEM_LC:
           if constexpr (sizeof(T) == 4) {
             if (pair_box(B)) {
-              lc_tile_pair<TY, true>(B, td, zc, part + 2 * (size_t)I.part * TY, sq);
+              lc_tile_pair<TY, true>(B, K2, td, zc, part + 2 * (size_t)I.part * TY, sq);
               break;
             }
           }
@@ -1907,6 +2307,24 @@ __global__ void k_near(DevBox* __restrict__ boxes, int b) {
     if (B.mask[j] & IDMASK) near = true;
   }
   B.mask[i] = near ? (uint8_t)(m | NEAR) : (uint8_t)(m & ~NEAR);
+}
+
+// Appends the near nodes of a warp's 32 nodes to the box's list (all lanes call it).
+__device__ __forceinline__ void near_append(const DevBox& B, int i, bool near) {
+  const unsigned m = __ballot_sync(0xffffffffu, near);
+  if (!m) return;
+  const int lane = threadIdx.x & 31, leader = __ffs(m) - 1;
+  int at = 0;
+  if (lane == leader) at = atomicAdd(B.nnear, __popc(m));
+  at = __shfl_sync(0xffffffffu, at, leader) + __popc(m & ((1u << lane) - 1u));
+  if (!near) return;
+  if (at < B.near_cap) B.near_node[at] = i;
+}
+
+__global__ void __launch_bounds__(256) k_near_list(const DevBox* __restrict__ boxes, int b) {
+  const DevBox& B = boxes[b];
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  near_append(B, i, i < B.N && (B.mask[i] & NEAR) && (B.mask[i] & IDMASK) == 0);
 }
 
 // Number of links from fluid node i into colloid c (bit q set in *bits).
@@ -2444,18 +2862,26 @@ __global__ void __launch_bounds__(256) k_rd_near(DevBox* __restrict__ boxes, con
   }
 }
 
-// Rebuild the boundary links of boxes whose solid set changed (unordered;
-// lc_lb_get_links sorts them).  Block 0 of the grid first clears the count
+// Rebuild the boundary links (unordered; lc_lb_get_links sorts them) and the
+// near-node lists of boxes whose solid set changed.  Block 0 of the grid first clears the count
 // in a separate launch (k_rd_links_reset).
 __global__ void k_rd_links_reset(DevBox* __restrict__ boxes, int nboxes) {
   const int b = blockIdx.x * blockDim.x + threadIdx.x;
-  if (b < nboxes && boxes[b].st->nchg > 0) *boxes[b].nlinks = 0;
+  if (b < nboxes && boxes[b].st->nchg > 0) {
+    *boxes[b].nlinks = 0;
+    *boxes[b].nnear = 0;
+  }
 }
 
 __global__ void __launch_bounds__(256) k_rd_links(DevBox* __restrict__ boxes, int nboxes) {
   for (int b = 0; b < nboxes; ++b) {
     const DevBox& B = boxes[b];
     if (B.st->nchg == 0) continue;
+    const int nthr = gridDim.x * gridDim.y * blockDim.x;
+    for (int base = (blockIdx.y * gridDim.x + blockIdx.x) * blockDim.x; base < B.N; base += nthr) {
+      const int i = base + threadIdx.x;
+      near_append(B, i, i < B.N && (B.mask[i] & NEAR) && (B.mask[i] & IDMASK) == 0);
+    }
     for (int c = blockIdx.y; c < B.ncol; c += gridDim.y) {
       const DevColloid& C = B.col[c];
       const int n = region_size(B, C);
@@ -2501,7 +2927,7 @@ __global__ void k_rd_finish(DevBox* __restrict__ boxes, int nboxes) {
       for (int a = 0; a < 3; ++a) C.V[a] += C.rdp[a] / C.M;
     for (int a = 0; a < 3; ++a) C.rdp[a] = 0.0;
   }
-  if (*B.nlinks > B.nlinks_cap) atomicOr(&st->err, 1);
+  if (*B.nlinks > B.nlinks_cap || *B.nnear > B.near_cap) atomicOr(&st->err, 1);
 }
 
 // ---------------------------------------------------------------------------
@@ -2539,21 +2965,35 @@ static cudaError_t launch_flb_t(const Launch& L, int mode, double* part) {
   return cudaGetLastError();
 }
 
+// Dynamic shared memory of the kernels that march with a Ring (0: FP64).
+template <typename T, int NC, int TY>
+constexpr size_t ring_bytes() { return sizeof(T) == 4 ? Ring<NC, TY>::BYTES : 0; }
+
 template <typename T, int TY>
-static cudaError_t launch_stress_t(const Launch& L, int mode, double* part) {
-  k_stress<T, TY><<<L.grid, dim3(TX, TY), 0, L.stream>>>(L.boxes, L.tiles, L.ntiles, L.zc, mode, part);
+static cudaError_t launch_stress_t(const Launch& L, int mode, double*) {
+  constexpr size_t ring = ring_bytes<T, 5, TY>(), near = sizeof(NearScratch<T>) * TY, smem = ring > near ? ring : near;
+  if (smem > 0) {
+    cudaError_t e = cudaFuncSetAttribute(k_stress<T, TY>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+  }
+  k_stress<T, TY><<<L.grid, dim3(TX, TY), smem, L.stream>>>(L, mode);
   return cudaGetLastError();
 }
 
 template <typename T, int TY>
-static cudaError_t launch_lbp_t(const Launch& L, int mode, double* part) {
-  k_lbp<T, TY><<<L.grid, dim3(TX, TY), 0, L.stream>>>(L.boxes, L.tiles, L.ntiles, L.zc, mode, part);
+static cudaError_t launch_lbp_t(const Launch& L, int, double*) {
+  k_lbp<T, TY><<<L.grid, dim3(TX, TY), 0, L.stream>>>(L);
   return cudaGetLastError();
 }
 
 template <typename T, int TY>
 static cudaError_t launch_lc_t(const Launch& L, int mode, double* part) {
-  k_lc<T, TY><<<L.grid, dim3(TX, TY), 0, L.stream>>>(L.boxes, L.tiles, L.ntiles, L.zc, mode, part);
+  constexpr size_t smem = ring_bytes<T, 8, TY>();
+  if (smem > 0) {
+    cudaError_t e = cudaFuncSetAttribute(k_lc<T, TY>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+  }
+  k_lc<T, TY><<<L.grid, dim3(TX, TY), smem, L.stream>>>(L, mode, part);
   return cudaGetLastError();
 }
 
@@ -2604,8 +3044,8 @@ cudaError_t launch_lbp(int prec, const Launch& L, int mode, double* part) {
 
 cudaError_t launch_links(int prec, const DevBox* boxes, const int2* chunks, int nchunks, int grid, cudaStream_t s) {
   if (nchunks <= 0) return cudaSuccess;
-  if (prec == 0) k_links<float><<<grid, 256, 0, s>>>(boxes, chunks, nchunks);
-  else k_links<double><<<grid, 256, 0, s>>>(boxes, chunks, nchunks);
+  if (prec == 0) k_links<float><<<grid, LINK_CHUNK, 0, s>>>(boxes, chunks, nchunks);
+  else k_links<double><<<grid, LINK_CHUNK, 0, s>>>(boxes, chunks, nchunks);
   return cudaGetLastError();
 }
 
@@ -2617,7 +3057,10 @@ cudaError_t launch_colloid(DevBox* boxes, int nboxes, cudaStream_t s) {
 template <typename T, int TY>
 static cudaError_t launch_step_t(DevBox* boxes, const StepItem* items, int nitems, int zc, unsigned* sync,
                                  double* part, int spin_limit, int commit, int* err, int grid, cudaStream_t s) {
-  k_step<T, TY><<<grid, dim3(TX, TY), 0, s>>>(boxes, items, nitems, zc, sync, part, spin_limit, commit, err);
+  constexpr size_t smem = sizeof(NearScratch<T>) * TY;
+  cudaError_t e = cudaFuncSetAttribute(k_step<T, TY>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e != cudaSuccess) return e;
+  k_step<T, TY><<<grid, dim3(TX, TY), smem, s>>>(boxes, items, nitems, zc, sync, part, spin_limit, commit, err);
   return cudaGetLastError();
 }
 
@@ -2638,7 +3081,11 @@ int step_blocks_per_sm(int prec, int ty) {
   int n = 0;
   cudaError_t e = cudaErrorInvalidValue;
 #define LCLB_OCC(T, Y) \
-  case Y: e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_step<T, Y>, TX * Y, 0); break;
+  case Y: \
+    e = cudaFuncSetAttribute(k_step<T, Y>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(NearScratch<T>) * Y); \
+    if (e == cudaSuccess) \
+      e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_step<T, Y>, TX * Y, sizeof(NearScratch<T>) * Y); \
+    break;
   if (prec == 0) {
     switch (ty) { LCLB_OCC(float, 2) LCLB_OCC(float, 4) LCLB_OCC(float, 8) default: break; }
   } else {
@@ -2653,6 +3100,11 @@ static inline int nblk(int N, int bs) { return (N + bs - 1) / bs; }
 cudaError_t launch_geometry(DevBox* boxes, int b, int N, cudaStream_t s) {
   k_mask<<<nblk(N, 256), 256, 0, s>>>(boxes, b);
   k_near<<<nblk(N, 256), 256, 0, s>>>(boxes, b);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_near_list(DevBox* boxes, int b, int N, cudaStream_t s) {
+  k_near_list<<<nblk(N, 256), 256, 0, s>>>(boxes, b);
   return cudaGetLastError();
 }
 

@@ -1,0 +1,46 @@
+"""Step kernels at the edges of their tiles against the FP64 oracle: widths around the 64-column tiles of the
+two-node path, a two-node-wide box, odd widths (one node per lane), ragged heights, boxes one to three planes deep,
+walls, near-node lists that fill less than a group of 32 and several groups, and boxes without any near node.
+Tolerances as the other parity tests (FP32 storage 1e-5 in Q, 1e-6 in u; FP64 1e-10, 1e-12)."""
+import numpy as np
+import pytest
+
+import oracle
+import synth
+
+pytestmark = pytest.mark.gpu
+
+CASES = [((64, 9, 3), False, None), ((66, 7, 5), False, (20.3, 3.1, 2.2, 1.6)), ((62, 5, 33), False, (30.2, 2.4, 15.7, 2.3)),
+         ((130, 6, 10), True, (64.4, 2.9, 4.6, 2.6)), ((2, 3, 4), False, None), ((4, 1, 1), False, None),
+         ((12, 10, 2), False, None), ((68, 12, 1), False, None), ((33, 17, 9), True, (15.1, 8.3, 4.4, 3.2)),
+         ((1, 2, 3), False, None), ((20, 33, 18), False, (10.2, 16.4, 8.9, 7.1))]
+
+
+@pytest.mark.parametrize("L,wall,col", CASES)
+@pytest.mark.parametrize("prec", ["f32", "f64"])
+@pytest.mark.parametrize("pitch,flow", [(0.0, True), (12.0, True), (12.0, False)])
+def test_step_edges(L, wall, col, prec, pitch, flow):
+    import paper_1102_2193_gb300 as P
+    prm = dict(synth.NEMATIC, q0=2 * np.pi / pitch if pitch else 0.0)
+    q = synth.random_q((L[2], L[1], L[0]), 5, amp=0.02, base=(-0.1, 0.05, 0.02, -0.12, 0.03))
+    s = P.Solver(*L, wall_z=wall, precision=P.LC_FP32 if prec == "f32" else P.LC_FP64, flow=flow, **prm)
+    o = oracle.Oracle(*L, wall_z=wall, flow=flow, **prm)
+    for k in (s, o):
+        k.set_Q(q)
+        if col:
+            k.add_colloid(col[:3], col[3], 1, 0.02)
+        k.step(5)
+    fl = o.get_solid() < 0
+    assert np.abs(s.get_Q() - o.get_Q())[:, fl].max() < (1e-5 if prec == "f32" else 1e-10)
+    if flow:
+        _, u = s.get_rho_u()
+        _, ur = o.get_rho_u()
+        assert np.abs(u - ur)[:, fl].max() < (1e-6 if prec == "f32" else 1e-12)
+    r, ro = s.diag(), o.diag()
+    assert abs(r["resid_rms"] - ro["resid_rms"]) <= (1e-4 if prec == "f32" else 1e-9) * ro["resid_rms"]
+    assert abs(r["resid_max"] - ro["resid_max"]) <= (1e-3 if prec == "f32" else 1e-9) * ro["resid_max"]
+    if col:
+        a, b = s.colloid(0), o.colloid(0)
+        F = np.abs(b["F_lc"]).max() + np.abs(b["F_hyd"]).max()
+        tol = 1e-4 if prec == "f32" else 1e-9
+        assert np.abs(a["F_lc"] - b["F_lc"]).max() <= tol * F and np.abs(a["F_hyd"] - b["F_hyd"]).max() <= tol * F
