@@ -249,9 +249,9 @@ Launch phase_launch(Group* g, int k, int mode, int box = -1) {
   } else {
     L.tiles = P.d_tiles + P.start[box];
     L.ntiles = P.count[box];
-    L.ngroups = 0;
+    L.ngroups = has_groups(k) ? g->gcount[box] : 0;
   }
-  L.groups = g->d_groups;
+  L.groups = g->d_groups + (box < 0 || !has_groups(k) ? 0 : g->gstart[box]);
   L.npart = g->d_npart;
   L.chunks = g->d_lchunks;
   L.nchunks = g->nlchunks;
@@ -1697,17 +1697,27 @@ int lc_lb_get_fields(lc_lb* h, int which, void* dst, size_t bytes, int dst_is_de
     default: return fail(&h->err, LC_ERR_ARG, "unknown field %d", which);
   }
   if (!dst || bytes < nc * N * sizeof(double)) return fail(&h->err, LC_ERR_ARG, "destination too small");
-  int rc = ensure_scratch(g, nc * N);
-  if (rc) return rc;
+  // a device destination is written by the export itself, a host one through scratch
+  const bool direct = dst_is_device && (reinterpret_cast<uintptr_t>(dst) & 7) == 0;
+  if (!direct)
+    if (int rc = ensure_scratch(g, nc * N)) return rc;
+  double* out = direct ? static_cast<double*>(dst) : g->d_scratch;
   if ((which == LC_U || which == LC_FORCE) && h->hb.p.lc_on) {
-    // body force of the current Q (no colloid accumulation)
-    CK(launch_phase(g, 0, 0, h->index), &h->err);
+    // stress of the current Q (no colloid accumulation); H and the stress are
+    // what the next step writes again
+    CK(launch_phase(g, 4, FORCE_P, h->index), &h->err);
   }
-  CK(launch_export(g->prec, g->d_boxes, h->index, h->hb.N, which, g->d_scratch, g->stream), &h->err);
-  CK(cudaMemcpyAsync(dst, g->d_scratch, nc * N * sizeof(double),
-                     dst_is_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost, g->stream),
-     &h->err);
-  CK(cudaStreamSynchronize(g->stream), &h->err);
+  if (which == LC_Q) {
+    auto al16 = [](const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15) == 0; };
+    const bool vec = al16(out) && al16(h->hb.Q[0]) && al16(h->hb.Q[1]) && al16(h->hb.Qlo[0]) && al16(h->hb.Qlo[1]);
+    CK(launch_export_q(g->prec, g->d_boxes, h->index, h->hb.N, vec, out, g->stream), &h->err);
+  } else {
+    CK(launch_export(g->prec, g->d_boxes, h->index, h->hb.N, which, out, g->stream), &h->err);
+  }
+  if (!direct)
+    CK(cudaMemcpyAsync(dst, g->d_scratch, nc * N * sizeof(double),
+                       dst_is_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost, g->stream),
+       &h->err);
   return check_step_err(g, &h->err);
 }
 

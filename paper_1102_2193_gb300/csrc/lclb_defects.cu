@@ -87,12 +87,16 @@ __global__ void __launch_bounds__(256) k_def_init(const DevBox* __restrict__ box
   if (i >= B.N) return;
   int v = -1;
   if ((B.mask[i] & IDMASK) == 0) {
-    double q[5];
+    float qf[5];
+    load_q_f32<T>(B, B.st->qpar, i, qf);
+    int low = below_f32(qf, (float)(thr / 1.5));
+    if (low < 0) {
+      double q[5];
 #pragma unroll
-    for (int k = 0; k < 5; ++k) q[k] = load_q<T>(B, i, k);
-    const float qf[5] = {(float)q[0], (float)q[1], (float)q[2], (float)q[3], (float)q[4]};
-    const int fast = below_f32(qf, (float)(thr / 1.5));
-    if (fast < 0 ? def_is_defect(q, thr / 1.5) : fast) v = i;
+      for (int k = 0; k < 5; ++k) q[k] = load_q<T>(B, i, k);
+      low = def_is_defect(q, thr / 1.5);
+    }
+    if (low) v = i;
   }
   parent[i] = v;
 }

@@ -255,20 +255,55 @@ __device__ __forceinline__ int below_f32(const float q[5], float t) {
 // Sum and first moments of the 19 deviations in FP64, through the sums and
 // differences of opposite directions (39 additions instead of the 76 of the
 // 19 x 4 products; FP64 issue bounds the kernels that call it).
-template <typename T>
-__device__ __forceinline__ void moments_f64(const T df[NQ], double& drho, double m[3], bool want_m = true) {
-  drho = (double)df[0];
-  m[0] = m[1] = m[2] = 0.0;
+template <typename S, typename V>
+__device__ __forceinline__ void pair_moments(const V v[NQ], S& sum, S m[3]) {
+  sum = v[0];
+  m[0] = m[1] = m[2] = S(0);
 #pragma unroll
   for (int q = 1; q < NQ; q += 2) {
-    const double a = (double)df[q], b = (double)df[q + 1];
-    drho += a + b;
-    if (want_m) {
-      const double d = a - b;
-      if (cx(q)) m[0] += cx(q) > 0 ? d : -d;
-      if (cy(q)) m[1] += cy(q) > 0 ? d : -d;
-      if (cz(q)) m[2] += cz(q) > 0 ? d : -d;
-    }
+    const S a = v[q], b = v[q + 1], d = a - b;
+    sum += a + b;
+    if (cx(q)) m[0] += cx(q) > 0 ? d : -d;
+    if (cy(q)) m[1] += cy(q) > 0 ? d : -d;
+    if (cz(q)) m[2] += cz(q) > 0 ? d : -d;
+  }
+}
+__device__ __forceinline__ void moments_f64(const double df[NQ], double& drho, double m[3]) {
+  pair_moments<double>(df, drho, m);
+}
+// FP32 deviations: added as 64-bit integers at 2^-57 of the largest, which
+// loses less than FP64 additions (2^-53 of the partial sums) and takes 8 FP64
+// operations instead of 58; infinities and NaN take the FP64 sums.
+__device__ __forceinline__ void moments_f64(const float df[NQ], double& drho, double m[3]) {
+  unsigned top = 0;
+#pragma unroll
+  for (int q = 0; q < NQ; ++q) top = max(top, __float_as_uint(df[q]) & 0x7fffffffu);
+  if (top >= 0x7f800000u) {
+    pair_moments<double>(df, drho, m);
+    return;
+  }
+  const int k = min(126, 183 - (int)(top >> 23));  // |df| 2^k < 2^57, so 19 of them fit 63 bits
+  const float scale = __int_as_float((k + 127) << 23);
+  long long v[NQ], s, ms[3];
+#pragma unroll
+  for (int q = 0; q < NQ; ++q) v[q] = __float2ll_rn(df[q] * scale);
+  pair_moments<long long>(v, s, ms);
+  const double inv = __hiloint2double((1023 - k) << 20, 0);
+  drho = (double)s * inv;
+#pragma unroll
+  for (int a = 0; a < 3; ++a) m[a] = (double)ms[a] * inv;
+}
+
+// The stored Q of node i rounded to FP32 (for decisions taken in FP32).
+template <typename T>
+__device__ __forceinline__ void load_q_f32(const DevBox& B, int qpar, int i, float q[5]) {
+#pragma unroll
+  for (int k = 0; k < 5; ++k) {
+    const size_t o = (size_t)k * B.N + i;
+    if constexpr (sizeof(T) == 4)
+      q[k] = static_cast<const float*>(B.Q[qpar])[o] + __bfloat162float(B.Qlo[qpar][o]);
+    else
+      q[k] = (float)static_cast<const double*>(B.Q[qpar])[o];
   }
 }
 

@@ -10,6 +10,7 @@ namespace lclb {
 // mode bits
 constexpr int FORCE_ACC = 1;  // accumulate colloid LC force/torque
 constexpr int FORCE_FE = 2;   // write free-energy partials (one double per tile)
+constexpr int FORCE_P = 4;    // k_stress: store the stress also with the flow frozen (exports read it)
 constexpr int LB_MOM = 1;     // write mass/momentum partials (4 doubles per tile)
 constexpr int LC_RESID = 1;   // write residual partials (sum of squares, max; 2 doubles per tile)
 constexpr int LC_COMMIT = 2;  // k_lc also runs the link exchange and, when a box is done, its colloid update and parity flip
@@ -83,6 +84,10 @@ cudaError_t launch_link_build(DevBox* boxes, int b, int N, int c, int* blocksum,
 cudaError_t launch_init_q(int prec, DevBox* boxes, int b, int N, int kind, const double* n, double amp,
                           unsigned long long seed, cudaStream_t s);
 cudaError_t launch_set_field(int prec, DevBox* boxes, int b, int N, int which, const double* src, cudaStream_t s);
+// Q as FP64 into out (device); vec: out and the Q buffers are 16-byte aligned.
+cudaError_t launch_export_q(int prec, const DevBox* boxes, int b, int N, bool vec, double* out, cudaStream_t s);
+// Other fields; U and FORCE take the force from the stored stress (k_stress
+// with FORCE_P has run on the current Q).
 cudaError_t launch_export(int prec, const DevBox* boxes, int b, int N, int which, double* out, cudaStream_t s);
 int diag_state_blocks(int N);
 cudaError_t launch_diag_state(int prec, const DevBox* boxes, int b, int N, double* part, cudaStream_t s);

@@ -701,7 +701,7 @@ __device__ __noinline__ void near_stress(const DevBox& B, int i, int mode, NearS
     T* Pb = static_cast<T*>(B.P);
 #pragma unroll
     for (int c = 0; c < 5; ++c) Hb[(size_t)c * N + i] = h[c];
-    if (B.p.flow_on) {  // with the flow frozen nothing reads the stress
+    if (B.p.flow_on || (mode & FORCE_P)) {  // with the flow frozen only exports read the stress
 #pragma unroll
       for (int c = 0; c < 9; ++c) Pb[(size_t)c * N + i] = p[c];
     }
@@ -735,7 +735,7 @@ __device__ __noinline__ void near_stress(const DevBox& B, int i, int mode, NearS
 template <typename T>
 __device__ __forceinline__ void stress_node(const DevBox& B, const PhysT<T>& PP, const T* __restrict__ Q,
                                             T* __restrict__ Hb, T* __restrict__ Pb, int x, int y, int z, int i,
-                                            const T (*pq)[5]) {
+                                            const T (*pq)[5], int mode) {
   const int N = B.N;
   T qi[5], qn[6][5], h[5], p[9], fp;
   int nb[6], zz[2];
@@ -755,7 +755,7 @@ __device__ __forceinline__ void stress_node(const DevBox& B, const PhysT<T>& PP,
   lc_node<T>(B, qi, qn, h, p, &fp);
 #pragma unroll
   for (int c = 0; c < 5; ++c) Hb[(size_t)c * N + i] = h[c];
-  if (B.p.flow_on) {  // with the flow frozen nothing reads the stress
+  if (B.p.flow_on || (mode & FORCE_P)) {  // with the flow frozen only exports read the stress
 #pragma unroll
     for (int c = 0; c < 9; ++c) Pb[(size_t)c * N + i] = p[c];
   }
@@ -790,7 +790,7 @@ __device__ __forceinline__ void stress_tile(const DevBox& B, const int4 td, int 
     T pq[5][5];
     column_next<T, 5>(B, Q, x, y, z, valid, qz, pq);
     x_neighbours<T, 5>(Q, (size_t)B.N, pq[0], lane, x, nx, nx * (y + ny * z), valid, &pq[1]);
-    if (fluid && !near) stress_node<T>(B, PP, Q, Hb, Pb, x, y, z, i, pq);
+    if (fluid && !near) stress_node<T>(B, PP, Q, Hb, Pb, x, y, z, i, pq, mode);
     const unsigned nb = __ballot_sync(0xffffffffu, near);
     if (nb) {
       if (near) sq[wy][nq + __popc(nb & ((1u << lane) - 1u))] = i;
@@ -1077,7 +1077,8 @@ __device__ __forceinline__ void st2_keep_if(float* p, f2 v, bool a, bool b, uint
 
 // Stress of a tile of plain nodes, two nodes per lane, Q from the ring.
 template <int TY>
-__device__ __forceinline__ void stress_ring(const DevBox& B, const LcK<f2>& K2, const int4 td, int zc, float* ring) {
+__device__ __forceinline__ void stress_ring(const DevBox& B, const LcK<f2>& K2, const int4 td, int zc, int mode,
+                                            float* ring) {
   if (!B.p.lc_on) return;
   const float* __restrict__ Q = static_cast<const float*>(B.Q[B.st->qpar]);
   float* __restrict__ Hb = static_cast<float*>(B.H);
@@ -1086,7 +1087,7 @@ __device__ __forceinline__ void stress_ring(const DevBox& B, const LcK<f2>& K2, 
   const int nz = B.nz, zend = min(td.w + zc, nz);
   const size_t N = (size_t)B.N;
   const uint64_t keep = l2_keep();
-  const bool chiral = B.p.q0 != 0.0, flow = B.p.flow_on != 0;
+  const bool chiral = B.p.q0 != 0.0, store_p = B.p.flow_on || (mode & FORCE_P);
   const uint8_t* mp = B.mask + R.x + R.row;
   const int plane = B.nx * B.ny;
   __syncthreads();  // the ring's last reads (previous tile) are done
@@ -1119,7 +1120,7 @@ __device__ __forceinline__ void stress_ring(const DevBox& B, const LcK<f2>& K2, 
     const size_t i = (size_t)R.x + R.row + (size_t)plane * z;
 #pragma unroll
     for (int c = 0; c < 5; ++c) st2_keep_if(Hb + c * N + i, h[c], pa, pb, keep);
-    if (flow) {  // with the flow frozen nothing reads the stress
+    if (store_p) {  // with the flow frozen only exports read the stress
 #pragma unroll
       for (int c = 0; c < 9; ++c) st2_keep_if(Pb + c * N + i, p[c], pa, pb, keep);
     }
@@ -1128,7 +1129,7 @@ __device__ __forceinline__ void stress_ring(const DevBox& B, const LcK<f2>& K2, 
 
 // Stress of a tile of plain nodes, one node per lane (odd widths, FP64).
 template <typename T>
-__device__ __forceinline__ void stress_plain(const DevBox& B, const int4 td, int zc) {
+__device__ __forceinline__ void stress_plain(const DevBox& B, const int4 td, int zc, int mode) {
   if (!B.p.lc_on) return;
   const int lane = threadIdx.x;
   const T* __restrict__ Q = static_cast<const T*>(B.Q[B.st->qpar]);
@@ -1144,7 +1145,7 @@ __device__ __forceinline__ void stress_plain(const DevBox& B, const int4 td, int
     column_next<T, 5>(B, Q, x, y, z, valid, qz, pq);
     x_neighbours<T, 5>(Q, (size_t)B.N, pq[0], lane, x, nx, nx * (y + ny * z), valid, &pq[1]);
     if (plain_node(m))
-      stress_node<T>(B, phys<T>(B), Q, static_cast<T*>(B.H), static_cast<T*>(B.P), x, y, z, i, pq);
+      stress_node<T>(B, phys<T>(B), Q, static_cast<T*>(B.H), static_cast<T*>(B.P), x, y, z, i, pq, mode);
     column_roll<T, 5>(qz, pq);
   }
 }
@@ -1172,11 +1173,11 @@ __global__ void __launch_bounds__(TX * TY, (sizeof(T) == 4 ? 512 : 256) / (TX * 
     load_box(B, K2, L.boxes, td.x, cur_box);
     if constexpr (sizeof(T) == 4) {
       if (pair_box(B)) {
-        stress_ring<TY>(B, K2, td, L.zc, ring);
+        stress_ring<TY>(B, K2, td, L.zc, mode, ring);
         continue;
       }
     }
-    stress_plain<T>(B, td, L.zc);
+    stress_plain<T>(B, td, L.zc, mode);
   }
 }
 
@@ -2509,26 +2510,52 @@ __global__ void k_set_field(DevBox* __restrict__ boxes, int b, int which, const 
   }
 }
 
-// Exports.  which: LC_Q, LC_F_PRE, LC_RHO, LC_U, LC_FORCE, LC_SOLID.
+// Exports.  Q: the 5 N stored values in order, VEC per thread (hi + lo, or the
+// FP64 values).
+template <typename T, int VEC>
+__global__ void __launch_bounds__(256) k_export_q(const DevBox* __restrict__ boxes, int b, double* __restrict__ out) {
+  const DevBox& B = boxes[b];
+  const int qpar = B.st->qpar;
+  const size_t n = 5 * (size_t)B.N, e0 = (blockIdx.x * (size_t)256 + threadIdx.x) * VEC;
+  const T* __restrict__ Q = static_cast<const T*>(B.Q[qpar]);
+  const __nv_bfloat16* __restrict__ lo = B.Qlo[qpar];
+  if constexpr (sizeof(T) == 4 && VEC == 4) {
+    if (e0 + 4 <= n) {
+      const float4 h = *reinterpret_cast<const float4*>(Q + e0);
+      const __nv_bfloat162 l0 = *reinterpret_cast<const __nv_bfloat162*>(lo + e0);
+      const __nv_bfloat162 l1 = *reinterpret_cast<const __nv_bfloat162*>(lo + e0 + 2);
+      double2* o = reinterpret_cast<double2*>(out + e0);
+      o[0] = make_double2((double)h.x + (double)__low2float(l0), (double)h.y + (double)__high2float(l0));
+      o[1] = make_double2((double)h.z + (double)__low2float(l1), (double)h.w + (double)__high2float(l1));
+      return;
+    }
+  }
+  for (size_t e = e0; e < e0 + VEC && e < n; ++e) {
+    if constexpr (sizeof(T) == 4) out[e] = (double)Q[e] + (double)__bfloat162float(lo[e]);
+    else out[e] = Q[e];
+  }
+}
+
+// Other fields.  which: LC_F_PRE, LC_RHO, LC_U, LC_FORCE, LC_SOLID.  The force
+// is the face divergence of the stored stress, as the LB kernel takes it.
 template <typename T>
-__global__ void k_export(const DevBox* __restrict__ boxes, int b, int which, double* __restrict__ out) {
+__global__ void __launch_bounds__(256) k_export(const DevBox* __restrict__ boxes, int b, int which,
+                                                double* __restrict__ out) {
   const DevBox& B = boxes[b];
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= B.N) return;
   const int N = B.N;
   const uint8_t m = B.mask[i];
   const int x = i % B.nx, y = (i / B.nx) % B.ny, z = i / (B.nx * B.ny);
-  if (which == EXP_Q) {
-    for (int k = 0; k < 5; ++k) out[(size_t)k * N + i] = load_q<T>(B, i, k);
-    return;
-  }
   if (which == EXP_SOLID) {
     out[i] = (m & IDMASK) ? (double)((m & IDMASK) - 1) : -1.0;
     return;
   }
+  T F[3] = {T(0), T(0), T(0)};
+  if ((which == EXP_FORCE || which == EXP_U) && !(m & IDMASK) && B.p.lc_on)
+    stored_force<T>(B, static_cast<const T*>(B.P), x, y, z, i, m, F);
   if (which == EXP_FORCE) {
-    const T* F = static_cast<const T*>(B.F);
-    for (int a = 0; a < 3; ++a) out[(size_t)a * N + i] = (m & IDMASK) || !B.p.lc_on ? 0.0 : (double)F[(size_t)a * N + i];
+    for (int a = 0; a < 3; ++a) out[(size_t)a * N + i] = (double)F[a];
     return;
   }
   if (m & IDMASK) {
@@ -2552,24 +2579,20 @@ __global__ void k_export(const DevBox* __restrict__ boxes, int b, int which, dou
     return;
   }
   double drho, mm[3];
-  moments_f64(df, drho, mm, which != EXP_RHO);
+  moments_f64(df, drho, mm);
   const double rho = B.p.rho0 + drho;
   if (which == EXP_RHO) {
     out[i] = rho;
     return;
   }
-  const T* F = static_cast<const T*>(B.F);
   const double inv = 1.0 / rho;
-  for (int a = 0; a < 3; ++a) {
-    const double Fa = (B.p.lc_on ? (double)F[(size_t)a * N + i] : 0.0) + B.p.g[a];
-    out[(size_t)a * N + i] = (mm[a] + 0.5 * Fa) * inv;
-  }
+  for (int a = 0; a < 3; ++a) out[(size_t)a * N + i] = (mm[a] + 0.5 * ((double)F[a] + B.p.g[a])) * inv;
 }
 
 // Diagnostics per block: [0] sum(df), [1..3] sum(df c), [4] fluid nodes,
 // [5] defect nodes (3/2 lambda_max(Q) < 0.435).  Bound by FP64 issue: the
-// moments take 39 FP64 additions per node, a thread sums DIAG_PER nodes before
-// the block reduction, and the defect test runs in FP32 except at nodes too
+// moments of FP32 populations are summed as integers, a thread sums DIAG_PER
+// nodes before the block reduction, and the defect test runs in FP32 except at nodes too
 // close to the threshold (with the closed-form eigenvalue in FP64 at every
 // node and 19 x 4 products: 1102 us at 128^3).
 constexpr int DIAG_PER = 4;
@@ -2579,7 +2602,7 @@ __global__ void __launch_bounds__(256) k_diag_state(const DevBox* __restrict__ b
   double v[6] = {0, 0, 0, 0, 0, 0};
   __shared__ double sred[32 * 6];
   int nfl = 0, ndef = 0;
-  const int nx = B.nx, ny = B.ny, N = B.N;
+  const int nx = B.nx, ny = B.ny, N = B.N, qpar = B.st->qpar;
   for (int r = 0; r < DIAG_PER; ++r) {
     const long long il = ((long long)blockIdx.x * DIAG_PER + r) * 256 + threadIdx.x;
     if (il >= N) break;
@@ -2596,11 +2619,12 @@ __global__ void __launch_bounds__(256) k_diag_state(const DevBox* __restrict__ b
     v[2] += mom[1];
     v[3] += mom[2];
     ++nfl;
-    double q[5];
-    for (int k = 0; k < 5; ++k) q[k] = load_q<T>(B, i, k);
-    const float qf[5] = {(float)q[0], (float)q[1], (float)q[2], (float)q[3], (float)q[4]};
+    float qf[5];
+    load_q_f32<T>(B, qpar, i, qf);
     int low = below_f32(qf, 0.29f);
     if (low < 0) {
+      double q[5];
+      for (int k = 0; k < 5; ++k) q[k] = load_q<T>(B, i, k);
       // largest eigenvalue of the traceless symmetric Q (closed form, as in principal_dir)
       double a00 = q[0], a01 = q[1], a02 = q[2], a11 = q[3], a12 = q[4], a22 = -q[0] - q[3];
       double p1 = a01 * a01 + a02 * a02 + a12 * a12;
@@ -3127,6 +3151,15 @@ cudaError_t launch_init_q(int prec, DevBox* boxes, int b, int N, int kind, const
 cudaError_t launch_set_field(int prec, DevBox* boxes, int b, int N, int which, const double* src, cudaStream_t s) {
   if (prec == 0) k_set_field<float><<<nblk(N, 256), 256, 0, s>>>(boxes, b, which, src);
   else k_set_field<double><<<nblk(N, 256), 256, 0, s>>>(boxes, b, which, src);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_export_q(int prec, const DevBox* boxes, int b, int N, bool vec, double* out, cudaStream_t s) {
+  const size_t n = 5 * (size_t)N;
+  const unsigned g1 = (unsigned)((n + 255) / 256), g4 = (unsigned)((n + 1023) / 1024);
+  if (prec != 0) k_export_q<double, 1><<<g1, 256, 0, s>>>(boxes, b, out);
+  else if (vec) k_export_q<float, 4><<<g4, 256, 0, s>>>(boxes, b, out);
+  else k_export_q<float, 1><<<g1, 256, 0, s>>>(boxes, b, out);
   return cudaGetLastError();
 }
 
