@@ -152,6 +152,7 @@ struct Group {
   cudaGraph_t graph = nullptr;
   cudaGraphExec_t gexec = nullptr;
   bool dirty = true, tuned = false;
+  bool frozen = false;    // every box has its flow frozen: a step is k_relax alone (except the dataflow variant)
   int graph_kernels = 0;  // kernel nodes of the captured step
   int nsm = 0;
   int dev = 0;            // the device current when the group was created
@@ -320,12 +321,12 @@ int build_groups(Group* g) {
 int build_totals(Group* g) {
   const Phase& P = g->ph[2];
   std::vector<unsigned> tot(g->boxes.size());
-  std::vector<int2> ch;
+  std::vector<int2> ch;  // (none with the flow frozen)
   for (size_t b = 0; b < g->boxes.size(); ++b) {
     const lc_lb* h = g->boxes[b];
     const int step = 32 * P.cfg.ty, n = h->hb.nmobile > 0 ? h->hb.nlinks_cap : h->nlinks;
     const size_t at = ch.size();
-    for (int s = 0; s < n; s += step) ch.push_back(make_int2((int)b, s));
+    for (int s = 0; s < n && !g->frozen; s += step) ch.push_back(make_int2((int)b, s));
     tot[b] = (unsigned)(P.count[b] + g->gcount[b] / P.cfg.ty) + (unsigned)(ch.size() - at);
   }
   if ((int)ch.size() > g->lchunk_cap) {
@@ -443,6 +444,7 @@ void fill_lck(LcK<T>& o, const DevParams& p) {
 
 // Allocate and initialise one box inside group g.
 int make_box(Group* g, const lc_grid* G, const lc_params* p, lc_lb* h) {
+  g->frozen = !p->flow_enabled && (h->index == 0 || g->frozen);
   h->grid = *G;
   h->params = *p;
   DevBox& B = h->hb;
@@ -630,7 +632,7 @@ cudaError_t launch_phase(Group* g, int k, int mode, int box = -1) {
                  (box < 0 ? 0 : (size_t)g->ph[k].start[box] * PART_WIDTH[k] * part_records(g->ph[k], k));
   if (k == 0) return launch_force(g->prec, L, mode, part);
   if (k == 1) return launch_lb(g->prec, L, mode, part);
-  if (k == 2) return launch_lc(g->prec, L, mode, part);
+  if (k == 2) return g->frozen ? launch_relax(g->prec, L, mode, part) : launch_lc(g->prec, L, mode, part);
   if (k == 4) return launch_stress(g->prec, L, mode, part);
   if (k == 5) return launch_lbp(g->prec, L, mode, part);
   return launch_flb(g->prec, L, mode, part);
@@ -1163,6 +1165,7 @@ int check_step_err(Group* g, std::string* err) {
 // One coupled step: stress, body force and collide/stream, then one launch
 // for the Q update, the link momentum exchange and the colloid update.
 int enqueue_force_lb(Group* g) {
+  if (g->frozen) return LC_OK;
   if (g->variant == 1) return enqueue_split(g, FORCE_ACC);
   if (g->variant == 2) {
     CK(launch_phase(g, 4, FORCE_ACC), &g->err);
@@ -1275,9 +1278,9 @@ int group_profile(Group* g, int n, double* ms) {
   const int k2 = g->variant == 0 ? -1 : (g->variant == 1 ? 1 : 5);
   for (int s = 0; s < n; ++s) {
     CK(cudaEventRecord(ev[0], g->stream), &g->err);
-    CK(launch_phase(g, k1, FORCE_ACC), &g->err);
+    if (!g->frozen) CK(launch_phase(g, k1, FORCE_ACC), &g->err);
     CK(cudaEventRecord(ev[5], g->stream), &g->err);
-    if (k2 >= 0) CK(launch_phase(g, k2, 0), &g->err);
+    if (k2 >= 0 && !g->frozen) CK(launch_phase(g, k2, 0), &g->err);
     CK(cudaEventRecord(ev[1], g->stream), &g->err);
     CK(launch_phase(g, 2, LC_RESID), &g->err);
     CK(cudaEventRecord(ev[2], g->stream), &g->err);

@@ -657,8 +657,8 @@ __device__ __forceinline__ void derivatives(const T qi[5], const T qn[6][5], T d
 // q0 = 0 (uniform over a box).  Products are added, never subtracted, with the
 // sign on a factor that is reused: the packed f2 form has no negated multiply.
 // T is the arithmetic type (float, double, or f2: two nodes at once); chiral:
-// q0 != 0.
-template <typename T>
+// q0 != 0; NEED_P false: the molecular field alone.
+template <typename T, bool NEED_P = true>
 __device__ __forceinline__ void lc_node_d(const LcK<T>& P, bool chiral, const T qi[5], const T dq[3][5],
                                           const T lap[5], T h[5], T p[9], T* fprime) {
   const T a = qi[0], b = qi[1], c = qi[2], d = qi[3], e = qi[4];
@@ -687,6 +687,7 @@ __device__ __forceinline__ void lc_node_d(const LcK<T>& P, bool chiral, const T 
   h[2] = T(cb * c + P.A0g * s2) + T(P.K * lap[2] + P.nKq0 * c2);
   h[3] = T(P.nA3 * trq2 + T(cb * d + P.A0g * s3)) + T(P.K * lap[3] + P.n2Kq0 * c3);
   h[4] = T(cb * e + P.A0g * s4) + T(P.K * lap[4] + P.nKq0 * c4);
+  if constexpr (!NEED_P) return;
   const T hz = -h[0] - h[3];
   // <2 d_a Q, 2 d_b Q> for the six pairs (double contraction over the five
   // stored components of two traceless symmetric tensors)
@@ -733,12 +734,12 @@ __device__ __forceinline__ void lc_node_d(const LcK<T>& P, bool chiral, const T 
   *fprime = fp;
 }
 
-template <typename T>
+template <typename T, bool NEED_P = true>
 __device__ __forceinline__ void lc_node(const DevBox& B, const T qi[5], const T qn[6][5], T h[5], T p[9],
                                         T* fprime) {
   T dq[3][5], lap[5];
   derivatives(qi, qn, dq, lap);
-  lc_node_d<T>(lck<T>(B), B.p.q0 != 0.0, qi, dq, lap, h, p, fprime);
+  lc_node_d<T, NEED_P>(lck<T>(B), B.p.q0 != 0.0, qi, dq, lap, h, p, fprime);
 }
 
 // Per-node choice ca ? a : b (f2: per lane value).

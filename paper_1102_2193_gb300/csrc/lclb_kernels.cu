@@ -590,8 +590,34 @@ struct NearScratch {
   T dn[192][5];        // Qs - Q of each solid face
 };
 
+// FROZEN (flow frozen): the node's Q is updated at once, dQ = Gamma H, and its
+// residual added to rs (sum of squares, max), instead of storing H and P.
 template <typename T>
-__device__ __noinline__ void near_stress(const DevBox& B, int i, int mode, NearScratch<T>& sc) {
+__device__ __forceinline__ void store_q_next(const DevBox& B, int qpar, size_t i, int k, T q, float lo, T d) {
+  const size_t o = (size_t)k * B.N + i;
+  if constexpr (sizeof(T) == 4) {
+    // compensated FP32 storage: hi + lo + increment carried exactly into hi, to BF16 in lo
+    float hi;
+    __nv_bfloat16 lo_out;
+    add_compensated(q, lo, d, hi, lo_out);
+    static_cast<float*>(B.Q[qpar ^ 1])[o] = hi;
+    B.Qlo[qpar ^ 1][o] = lo_out;
+  } else {
+    static_cast<T*>(B.Q[qpar ^ 1])[o] = q + d;
+  }
+}
+template <typename T>
+__device__ __forceinline__ void add_residual(const T d5[5], T& rsum, T& rmax) {
+  const T dzz = -d5[0] - d5[3];
+  rsum += d5[0] * d5[0] + d5[3] * d5[3] + dzz * dzz + T(2) * (d5[1] * d5[1] + d5[2] * d5[2] + d5[4] * d5[4]);
+  T mx = fabs(dzz);
+#pragma unroll
+  for (int k = 0; k < 5; ++k) mx = fmax(mx, fabs(d5[k]));
+  rmax = fmax(rmax, mx);
+}
+
+template <typename T, bool FROZEN = false>
+__device__ __noinline__ void near_stress(const DevBox& B, int i, int mode, NearScratch<T>& sc, T* rs = nullptr) {
   const unsigned full = 0xffffffffu;
   const int lane = threadIdx.x & 31;
   const bool valid = i >= 0;
@@ -696,7 +722,15 @@ __device__ __noinline__ void near_stress(const DevBox& B, int i, int mode, NearS
     lap[k] = (dn[0][k] + dn[1][k]) + (dn[2][k] + dn[3][k]) + (dn[4][k] + dn[5][k]);
   }
   lc_node_d<T>(lck<T>(B), B.p.q0 != 0.0, qi, dq, lap, h, p, &fp);
-  if (valid) {
+  if constexpr (FROZEN) {
+    if (valid) {
+      T d5[5];
+      q_increment<comp, false, T>(lck<T>(B), qh, nullptr, nullptr, h, reinterpret_cast<const T*>(ql), d5);
+#pragma unroll
+      for (int k = 0; k < 5; ++k) store_q_next<T>(B, qpar, i, k, qh[k], ql[k], d5[k]);
+      add_residual(d5, rs[0], rs[1]);
+    }
+  } else if (valid) {
     T* Hb = static_cast<T*>(B.H);
     T* Pb = static_cast<T*>(B.P);
 #pragma unroll
@@ -1308,6 +1342,16 @@ __device__ __forceinline__ void lbp_plain(const DevBox& B, const int4 td, int zc
   }
 }
 
+// Near node of k_lbp.
+template <typename T>
+__device__ __forceinline__ void near_lbp(const DevBox& B, int j) {
+  if (j < 0) return;
+  const int fpar = B.st->fpar;
+  lbp_node<T, true>(B, phys<T>(B), static_cast<const T*>(B.f[fpar]), static_cast<T*>(B.f[fpar ^ 1]),
+                    static_cast<const T*>(B.P), static_cast<T*>(B.u), j % B.nx, (j / B.nx) % B.ny,
+                    j / (B.nx * B.ny), j, B.mask[j], B.st->pre_valid != 0, B.p.lc_on != 0);
+}
+
 template <typename T, int TY>
 __global__ void __launch_bounds__(TX * TY, (sizeof(T) == 4 ? 1024 : 384) / (TX * TY)) k_lbp(Launch L) {
   __shared__ DevBox B;
@@ -1318,13 +1362,7 @@ __global__ void __launch_bounds__(TX * TY, (sizeof(T) == 4 ? 1024 : 384) / (TX *
     load_box(B, L.boxes, td.x, cur_box);
     if (!B.p.flow_on) continue;
     if (t < nn) {
-      near_group<TY>(B, L.groups, t, [&](int j) {
-        if (j < 0) return;
-        const int fpar = B.st->fpar;
-        lbp_node<T, true>(B, phys<T>(B), static_cast<const T*>(B.f[fpar]), static_cast<T*>(B.f[fpar ^ 1]),
-                          static_cast<const T*>(B.P), static_cast<T*>(B.u), j % B.nx, (j / B.nx) % B.ny,
-                          j / (B.nx * B.ny), j, B.mask[j], B.st->pre_valid != 0, B.p.lc_on != 0);
-      });
+      near_group<TY>(B, L.groups, t, [&](int j) { near_lbp<T>(B, j); });
       continue;
     }
     lbp_plain<T>(B, td, L.zc);
@@ -1438,9 +1476,8 @@ __global__ void __launch_bounds__(32 * (BY + 3), (sizeof(T) == 4 && BY <= 4) ? 2
 // against 71 us).
 template <typename T, bool NEAR_NODE, bool CG = false>
 __device__ __forceinline__ void lc_update_node(const DevBox& B, const PhysT<T>& PP, const T* __restrict__ Q,
-                                               T* __restrict__ Qo, const __nv_bfloat16* __restrict__ Lin,
-                                               __nv_bfloat16* __restrict__ Lout, const T* __restrict__ U, int x,
-                                               int y, int z, int i, uint8_t m, T& rsum, T& rmax,
+                                               const __nv_bfloat16* __restrict__ Lin, const T* __restrict__ U, int qpar,
+                                               int x, int y, int z, int i, T& rsum, T& rmax,
                                                const T (*pq)[5] = nullptr, const T (*pu)[3] = nullptr,
                                                const float* plo = nullptr) {
   const int N = B.N;
@@ -1497,24 +1534,8 @@ __device__ __forceinline__ void lc_update_node(const DevBox& B, const PhysT<T>& 
   }
   q_increment<sizeof(T) == 4, true, T>(lck<T>(B), qi, adv, G, h, reinterpret_cast<const T*>(lo), d5);
 #pragma unroll
-  for (int k = 0; k < 5; ++k) {
-    if constexpr (sizeof(T) == 4) {
-      // compensated FP32 storage: hi + lo + increment carried exactly into hi, to BF16 in lo
-      float hi;
-      __nv_bfloat16 lo_out;
-      add_compensated(qi[k], lo[k], d5[k], hi, lo_out);
-      Qo[(size_t)k * N + i] = hi;
-      Lout[(size_t)k * N + i] = lo_out;
-    } else {
-      Qo[(size_t)k * N + i] = qi[k] + d5[k];
-    }
-  }
-  const T dzz = -d5[0] - d5[3];
-  rsum += d5[0] * d5[0] + d5[3] * d5[3] + dzz * dzz + T(2) * (d5[1] * d5[1] + d5[2] * d5[2] + d5[4] * d5[4]);
-  T mx = fabs(dzz);
-#pragma unroll
-  for (int k = 0; k < 5; ++k) mx = fmax(mx, fabs(d5[k]));
-  rmax = fmax(rmax, mx);
+  for (int k = 0; k < 5; ++k) store_q_next<T>(B, qpar, i, k, qi[k], sizeof(T) == 4 ? lo[k] : 0.f, d5[k]);
+  add_residual(d5, rsum, rmax);
 }
 
 // k_lc: Beris-Edwards update; plain nodes of a warp's row together, nodes
@@ -1527,9 +1548,7 @@ __device__ __forceinline__ void lc_tile(const DevBox& B, const int4 td, int zc, 
   const int lane = threadIdx.x, wy = threadIdx.y;
   const int qpar = B.st->qpar;
   const T* __restrict__ Q = static_cast<const T*>(B.Q[qpar]);
-  T* __restrict__ Qo = static_cast<T*>(B.Q[qpar ^ 1]);
   const __nv_bfloat16* __restrict__ Lin = B.Qlo[qpar];
-  __nv_bfloat16* __restrict__ Lout = B.Qlo[qpar ^ 1];
   const T* __restrict__ U = static_cast<const T*>(B.u);
   const int nx = B.nx, ny = B.ny;
   const int x = td.y + lane, y = td.z + wy;
@@ -1557,7 +1576,7 @@ __device__ __forceinline__ void lc_tile(const DevBox& B, const int4 td, int zc, 
     x_neighbours<T, 5>(Q, (size_t)B.N, pq[0], lane, x, nx, row, valid, &pq[1]);
     x_neighbours<T, 3, CG>(U, (size_t)B.N, pu[0], lane, x, nx, row, valid, &pu[1]);
     if (fluid && !near)
-      lc_update_node<T, false, CG>(B, PP, Q, Qo, Lin, Lout, U, x, y, z, i, m, rsum, rmax, pq, pu, plo);
+      lc_update_node<T, false, CG>(B, PP, Q, Lin, U, qpar, x, y, z, i, rsum, rmax, pq, pu, plo);
     const unsigned nb = __ballot_sync(0xffffffffu, near);
     if (nb) {
       if (near) sq[wy][nq + __popc(nb & ((1u << lane) - 1u))] = i;
@@ -1565,8 +1584,7 @@ __device__ __forceinline__ void lc_tile(const DevBox& B, const int4 td, int zc, 
       __syncwarp();
       if (nq >= TX) {
         const int j = sq[wy][lane];
-        lc_update_node<T, true, CG>(B, PP, Q, Qo, Lin, Lout, U, j % nx, (j / nx) % ny, j / (nx * ny), j, B.mask[j],
-                                    rsum, rmax);
+        lc_update_node<T, true, CG>(B, PP, Q, Lin, U, qpar, j % nx, (j / nx) % ny, j / (nx * ny), j, rsum, rmax);
         __syncwarp();
         nq -= TX;
         if (lane < nq) sq[wy][lane] = sq[wy][TX + lane];
@@ -1576,8 +1594,7 @@ __device__ __forceinline__ void lc_tile(const DevBox& B, const int4 td, int zc, 
   }
   if (lane < nq) {
     const int j = sq[wy][lane];
-    lc_update_node<T, true, CG>(B, PP, Q, Qo, Lin, Lout, U, j % nx, (j / nx) % ny, j / (nx * ny), j, B.mask[j], rsum,
-                                rmax);
+    lc_update_node<T, true, CG>(B, PP, Q, Lin, U, qpar, j % nx, (j / nx) % ny, j / (nx * ny), j, rsum, rmax);
   }
   __syncwarp();
   if (part) warp_residual<T>(part, wy, lane, rsum, rmax);
@@ -1642,8 +1659,7 @@ __device__ __forceinline__ void lc_tile_pair(const DevBox& B, const LcK<f2>& K2,
   float rsum = 0.f, rmax = 0.f;
   int nq = 0;
   auto near_fn = [&](int j) {
-    lc_update_node<float, true, CG>(B, B.pf, Q, Qo, Lin, Lout, U, j % nx, (j / nx) % ny, j / (nx * ny), j, B.mask[j],
-                                    rsum, rmax);
+    lc_update_node<float, true, CG>(B, B.pf, Q, Lin, U, qpar, j % nx, (j / nx) % ny, j / (nx * ny), j, rsum, rmax);
   };
   for (int z = td.w; z < zend; ++z) {
     const int row = nx * (y + ny * z);
@@ -1941,6 +1957,47 @@ __device__ __forceinline__ void colloid_box(const DevBox& B, bool commit = true)
   }
 }
 
+// Stores Q + d5 of a pair (compensated: hi + lo + increment carried exactly into
+// (hi, lo) by two-sum) for the nodes that the tile path evaluates, and adds
+// their residual.
+__device__ __forceinline__ void store_pair(float* q, __nv_bfloat16* l, size_t N, const f2 qi[5], const f2 lo[5],
+                                           const f2 d5[5], bool pa, bool pb, float& rsum, float& rmax) {
+#pragma unroll
+  for (int k = 0; k < 5; ++k) {
+    const f2 sv = lo[k] + d5[k];
+    const f2 hn = qi[k] + sv;
+    const f2 bb = hn - qi[k];
+    const f2 err = (qi[k] - (hn - bb)) + (sv - bb);
+    const __nv_bfloat162 l2 = __float22bfloat162_rn(err.v);
+    if (pa && pb) {
+      st2(q + k * N, hn);
+      *reinterpret_cast<__nv_bfloat162*>(l + k * N) = l2;
+    } else if (pa) {
+      q[k * N] = hn.v.x;
+      l[k * N] = l2.x;
+    } else {
+      q[k * N + 1] = hn.v.y;
+      l[k * N + 1] = l2.y;
+    }
+  }
+  const f2 dzz = -(d5[0] + d5[3]);
+  const f2 r2 = d5[0] * d5[0] + d5[3] * d5[3] + dzz * dzz + 2.f * (d5[1] * d5[1] + d5[2] * d5[2] + d5[4] * d5[4]);
+  float mx = fabsf(dzz.v.x), my = fabsf(dzz.v.y);
+#pragma unroll
+  for (int k = 0; k < 5; ++k) {
+    mx = fmaxf(mx, fabsf(d5[k].v.x));
+    my = fmaxf(my, fabsf(d5[k].v.y));
+  }
+  if (pa) {
+    rsum += r2.v.x;
+    rmax = fmaxf(rmax, mx);
+  }
+  if (pb) {
+    rsum += r2.v.y;
+    rmax = fmaxf(rmax, my);
+  }
+}
+
 // ---------------------------------------------------------------------------
 // k_lc: Q update, link exchange and colloid update in one launch
 // ---------------------------------------------------------------------------
@@ -2022,43 +2079,7 @@ __device__ __forceinline__ void lc_ring(const DevBox& B, const LcK<f2>& K2, cons
       lo[k] = f2(__bfloat1622float2(lr[k]));
     }
     q_increment<true, true, f2>(K2, qi, adv, G, h, lo, d5);
-#pragma unroll
-    for (int k = 0; k < 5; ++k) {
-      // compensated storage: hi + lo + increment carried exactly into (hi, lo) (two-sum)
-      const f2 sv = lo[k] + d5[k];
-      const f2 hn = qi[k] + sv;
-      const f2 bb = hn - qi[k];
-      const f2 err = (qi[k] - (hn - bb)) + (sv - bb);
-      const __nv_bfloat162 l2 = __float22bfloat162_rn(err.v);
-      float* q = Qo + (size_t)k * N + i;
-      __nv_bfloat16* l = Lout + (size_t)k * N + i;
-      if (pa && pb) {
-        st2(q, hn);
-        *reinterpret_cast<__nv_bfloat162*>(l) = l2;
-      } else if (pa) {
-        q[0] = hn.v.x;
-        l[0] = l2.x;
-      } else {
-        q[1] = hn.v.y;
-        l[1] = l2.y;
-      }
-    }
-    const f2 dzz = -(d5[0] + d5[3]);
-    const f2 r2 = d5[0] * d5[0] + d5[3] * d5[3] + dzz * dzz + 2.f * (d5[1] * d5[1] + d5[2] * d5[2] + d5[4] * d5[4]);
-    float mx = fabsf(dzz.v.x), my = fabsf(dzz.v.y);
-#pragma unroll
-    for (int k = 0; k < 5; ++k) {
-      mx = fmaxf(mx, fabsf(d5[k].v.x));
-      my = fmaxf(my, fabsf(d5[k].v.y));
-    }
-    if (pa) {
-      rsum += r2.v.x;
-      rmax = fmaxf(rmax, mx);
-    }
-    if (pb) {
-      rsum += r2.v.y;
-      rmax = fmaxf(rmax, my);
-    }
+    store_pair(Qo + i, Lout + i, N, qi, lo, d5, pa, pb, rsum, rmax);
   }
 }
 
@@ -2090,9 +2111,20 @@ __device__ __forceinline__ void lc_plain(const DevBox& B, const int4 td, int zc,
     x_neighbours<T, 5>(Q, (size_t)B.N, pq[0], lane, x, nx, row, valid, &pq[1]);
     x_neighbours<T, 3>(U, (size_t)B.N, pu[0], lane, x, nx, row, valid, &pu[1]);
     if (plain)
-      lc_update_node<T, false>(B, phys<T>(B), Q, static_cast<T*>(B.Q[qpar ^ 1]), Lin, B.Qlo[qpar ^ 1], U, x, y, z, i, m,
-                               rsum, rmax, pq, pu, plo);
+      lc_update_node<T, false>(B, phys<T>(B), Q, Lin, U, qpar, x, y, z, i, rsum, rmax, pq, pu, plo);
   }
+}
+
+// Near node of k_lc.
+template <typename T>
+__device__ __forceinline__ void near_lc(const DevBox& B, int j, T& rsum, T& rmax) {
+  if (j < 0) return;
+  const int qpar = B.st->qpar;
+  T rs = T(0), rm = T(0);
+  lc_update_node<T, true>(B, phys<T>(B), static_cast<const T*>(B.Q[qpar]), B.Qlo[qpar], static_cast<const T*>(B.u),
+                          qpar, j % B.nx, (j / B.nx) % B.ny, j / (B.nx * B.ny), j, rs, rm);
+  rsum += rs;
+  rmax = fmax(rmax, rm);
 }
 
 // The work units of a box are counted as they finish; the block that finishes
@@ -2141,13 +2173,7 @@ __global__ void __launch_bounds__(TX * TY, (sizeof(T) == 4 ? 512 : 256) / (TX * 
     T rsum = T(0), rmax = T(0);  // per-thread residual (sum of squares, max), in T
     if (t < nn) {
       if (B.p.lc_on)
-        near_group<TY>(B, L.groups, t, [&](int j) {
-          if (j < 0) return;
-          const int qpar = B.st->qpar;
-          lc_update_node<T, true>(B, phys<T>(B), static_cast<const T*>(B.Q[qpar]), static_cast<T*>(B.Q[qpar ^ 1]),
-                                  B.Qlo[qpar], B.Qlo[qpar ^ 1], static_cast<const T*>(B.u), j % B.nx,
-                                  (j / B.nx) % B.ny, j / (B.nx * B.ny), j, B.mask[j], rsum, rmax);
-        });
+        near_group<TY>(B, L.groups, t, [&](int j) { near_lc<T>(B, j, rsum, rmax); });
       __syncwarp();
       if (mode & LC_RESID) warp_residual<T>(L.npart + 2 * (size_t)t * TY, wy, lane, rsum, rmax);
       continue;
@@ -2166,6 +2192,151 @@ __global__ void __launch_bounds__(TX * TY, (sizeof(T) == 4 ? 512 : 256) / (TX * 
     if (!done) lc_plain<T>(B, td, L.zc, rsum, rmax);
     __syncwarp();
     if (mode & LC_RESID) warp_residual<T>(part + 2 * (size_t)(t - nn - nl) * TY, wy, lane, rsum, rmax);
+  }
+  if (commit && run_n) lc_commit(L, run_box, run_n);
+}
+
+// ---------------------------------------------------------------------------
+// k_relax: the whole step of boxes whose flow is frozen
+// ---------------------------------------------------------------------------
+// With u = 0 the step is dQ = Gamma H (Eq. 2): no stress, no populations, no
+// flux, so H is used where it is formed and each node moves its Q twice (60
+// bytes with the remainder) instead of the 190 of the separate stress and Q
+// update.  Near nodes still take their stress for the colloid's LC force.
+// Bound by issue of the molecular field (about 130 packed operations a pair).
+template <int TY>
+__device__ __forceinline__ void relax_ring(const DevBox& B, const LcK<f2>& K2, const int4 td, int zc, float* ring,
+                                           float& rsum, float& rmax) {
+  const int qpar = B.st->qpar;
+  const float* __restrict__ Q = static_cast<const float*>(B.Q[qpar]);
+  float* __restrict__ Qo = static_cast<float*>(B.Q[qpar ^ 1]);
+  const __nv_bfloat16* __restrict__ Lin = B.Qlo[qpar];
+  __nv_bfloat16* __restrict__ Lout = B.Qlo[qpar ^ 1];
+  const RingLane R = ring_lane<TY>(B, td);
+  const int zend = min(td.w + zc, B.nz), plane = B.nx * B.ny;
+  const size_t N = (size_t)B.N;
+  const bool chiral = B.p.q0 != 0.0;
+  const uint8_t* mp = B.mask + R.x + R.row;
+  __syncthreads();
+#pragma unroll 1
+  for (int k = -1; k <= 1; ++k) ring_load<5, TY, 5>(ring, B, R, Q, 0, td.w + k, (k + 1) & 3);
+  cp_async_commit();
+  unsigned m2 = R.valid ? (unsigned)*reinterpret_cast<const uint16_t*>(mp + (size_t)plane * td.w) : 0x0101u;
+  for (int z = td.w; z < zend; ++z) {
+    const int s0 = (z - td.w + 1) & 3;
+    const size_t i = (size_t)R.x + R.row + (size_t)plane * z;
+    const bool pa = plain_node(m2 & 0xffu), pb = plain_node(m2 >> 8);
+    __nv_bfloat162 lr[5];
+    if (pa || pb) {
+#pragma unroll
+      for (int k = 0; k < 5; ++k) lr[k] = *reinterpret_cast<const __nv_bfloat162*>(Lin + k * N + i);
+    }
+    cp_async_wait0();
+    __syncthreads();
+    if (z + 1 < zend) {
+      ring_load<5, TY, 5>(ring, B, R, Q, 0, z + 2, (s0 + 2) & 3);
+      if (R.valid) m2 = (unsigned)*reinterpret_cast<const uint16_t*>(mp + (size_t)plane * (z + 1));
+    }
+    cp_async_commit();
+    if (!pa && !pb) continue;
+    f2 qi[5], dq[3][5], lap[5], h[5], p[9], fp, lo[5], d5[5];
+#pragma unroll
+    for (int k = 0; k < 5; ++k) {
+      f2 n[6];
+      ring_gather<5, TY>(ring, R, k, s0, (s0 + 3) & 3, (s0 + 1) & 3, qi[k], n);
+      dq[0][k] = n[0] - n[1];
+      dq[1][k] = n[2] - n[3];
+      dq[2][k] = n[4] - n[5];
+      lap[k] = ((n[0] + n[1]) + (n[2] + n[3]) + (n[4] + n[5])) + K2.nsix * qi[k];
+      lo[k] = f2(__bfloat1622float2(lr[k]));
+    }
+    lc_node_d<f2, false>(K2, chiral, qi, dq, lap, h, p, &fp);
+    q_increment<true, false, f2>(K2, qi, nullptr, nullptr, h, lo, d5);
+    store_pair(Qo + i, Lout + i, N, qi, lo, d5, pa, pb, rsum, rmax);
+  }
+}
+
+template <typename T>
+__device__ __forceinline__ void relax_plain(const DevBox& B, const int4 td, int zc, T& rsum, T& rmax) {
+  const int lane = threadIdx.x, qpar = B.st->qpar;
+  const T* __restrict__ Q = static_cast<const T*>(B.Q[qpar]);
+  const size_t N = (size_t)B.N;
+  const int nx = B.nx, ny = B.ny, x = td.y + lane, y = td.z + (int)threadIdx.y;
+  const int zend = min(td.w + zc, B.nz);
+  const bool valid = x < nx && y < ny;
+  T qz[2][5];
+  column_start<T, 5>(B, Q, x, y, td.w, valid, qz);
+  for (int z = td.w; z < zend; ++z) {
+    const int row = nx * (y + ny * z), i = x + row;
+    const bool plain = valid && plain_node(B.mask[i]);
+    T pq[5][5];
+    column_next<T, 5>(B, Q, x, y, z, valid, qz, pq);
+    x_neighbours<T, 5>(Q, N, pq[0], lane, x, nx, row, valid, &pq[1]);
+    if (plain) {
+      float lo[5] = {0.f, 0.f, 0.f, 0.f, 0.f};
+      T qn[6][5], h[5], p[9], fp, d5[5];
+      const int yp = nx * ((y + 1 == ny ? 0 : y + 1) + ny * z) + x, ym = nx * ((y == 0 ? ny - 1 : y - 1) + ny * z) + x;
+#pragma unroll
+      for (int k = 0; k < 5; ++k) {
+        if constexpr (sizeof(T) == 4) lo[k] = __bfloat162float(B.Qlo[qpar][k * N + i]);
+        qn[0][k] = pq[1][k];
+        qn[1][k] = pq[2][k];
+        qn[2][k] = ldg(Q + k * N + yp);
+        qn[3][k] = ldg(Q + k * N + ym);
+        qn[4][k] = pq[3][k];
+        qn[5][k] = pq[4][k];
+      }
+      lc_node<T, false>(B, pq[0], qn, h, p, &fp);
+      q_increment<sizeof(T) == 4, false, T>(lck<T>(B), pq[0], nullptr, nullptr, h, reinterpret_cast<const T*>(lo), d5);
+#pragma unroll
+      for (int k = 0; k < 5; ++k) store_q_next<T>(B, qpar, i, k, pq[0][k], lo[k], d5[k]);
+      add_residual(d5, rsum, rmax);
+    }
+    column_roll<T, 5>(qz, pq);
+  }
+}
+
+template <typename T, int TY>
+__global__ void __launch_bounds__(TX * TY, (sizeof(T) == 4 ? 640 : 256) / (TX * TY)) k_relax(Launch L, int mode,
+                                                                                            double* __restrict__ part) {
+  __shared__ DevBox B;
+  __shared__ LcK<f2> K2;
+  extern __shared__ __align__(16) float ring[];
+  const bool commit = (mode & LC_COMMIT) != 0;
+  const int lane = threadIdx.x, wy = threadIdx.y;
+  const int nn = L.ngroups / TY, units = nn + L.ntiles;
+  int cur_box = -1, run_box = -1;
+  unsigned run_n = 0;
+  for (int t = blockIdx.x; t < units; t += gridDim.x) {
+    const int4 td = t < nn ? make_int4(L.groups[t * TY].x, 0, 0, 0) : L.tiles[t - nn];
+    if (commit && td.x != run_box) {
+      if (run_n) lc_commit(L, run_box, run_n);
+      run_box = td.x;
+      run_n = 0;
+    }
+    ++run_n;
+    load_box(B, K2, L.boxes, td.x, cur_box);
+    T rs[2] = {T(0), T(0)};
+    if (B.p.lc_on) {
+      if (t < nn) {
+        near_group<TY>(B, L.groups, t, [&](int j) {
+          near_stress<T, true>(B, j, commit ? FORCE_ACC : 0, reinterpret_cast<NearScratch<T>*>(ring)[wy], rs);
+        });
+        __syncthreads();
+      } else {
+        bool done = false;
+        if constexpr (sizeof(T) == 4) {
+          if (pair_box(B)) {
+            relax_ring<TY>(B, K2, td, L.zc, ring, rs[0], rs[1]);
+            done = true;
+          }
+        }
+        if (!done) relax_plain<T>(B, td, L.zc, rs[0], rs[1]);
+      }
+    }
+    __syncwarp();
+    if (mode & LC_RESID)
+      warp_residual<T>(t < nn ? L.npart + 2 * (size_t)t * TY : part + 2 * (size_t)(t - nn) * TY, wy, lane, rs[0], rs[1]);
   }
   if (commit && run_n) lc_commit(L, run_box, run_n);
 }
@@ -3021,6 +3192,15 @@ static cudaError_t launch_lc_t(const Launch& L, int mode, double* part) {
   return cudaGetLastError();
 }
 
+template <typename T, int TY>
+static cudaError_t launch_relax_t(const Launch& L, int mode, double* part) {
+  constexpr size_t ring = ring_bytes<T, 5, TY>(), near = sizeof(NearScratch<T>) * TY, smem = ring > near ? ring : near;
+  cudaError_t e = cudaFuncSetAttribute(k_relax<T, TY>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e != cudaSuccess) return e;
+  k_relax<T, TY><<<L.grid, dim3(TX, TY), smem, L.stream>>>(L, mode, part);
+  return cudaGetLastError();
+}
+
 #define LCLB_DISPATCH_TY(FN, T)                      \
   switch (L.ty) {                                    \
     case 2: return FN<T, 2>(L, mode, part);          \
@@ -3056,6 +3236,10 @@ cudaError_t launch_flb(int prec, const Launch& L, int mode, double* part) {
 cudaError_t launch_lc(int prec, const Launch& L, int mode, double* part) {
   if (prec == 0) { LCLB_DISPATCH_TY(launch_lc_t, float) }
   LCLB_DISPATCH_TY(launch_lc_t, double)
+}
+cudaError_t launch_relax(int prec, const Launch& L, int mode, double* part) {
+  if (prec == 0) { LCLB_DISPATCH_TY(launch_relax_t, float) }
+  LCLB_DISPATCH_TY(launch_relax_t, double)
 }
 cudaError_t launch_stress(int prec, const Launch& L, int mode, double* part) {
   if (prec == 0) { LCLB_DISPATCH_TY(launch_stress_t, float) }
