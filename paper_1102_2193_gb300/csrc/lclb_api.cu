@@ -1134,7 +1134,7 @@ int check_step_err(Group* g, std::string* err) {
   CK(cudaStreamSynchronize(g->stream), err);
   if (hv[0] == 0 && hv[1] == 0) return LC_OK;
   const bool timeout = hv[0] != 0;
-  CK(cudaMemsetAsync(g->d_err, 0, 2 * sizeof(int), g->stream), err);
+  CK(cudaMemsetAsync(g->d_err, 0, (timeout ? 4 : 2) * sizeof(int), g->stream), err);  // [2]: grid barrier of k_rediscretise
   long long cstep = -1;
   int cbox = -1, ccol = -1, cpartner = -2;
   for (size_t b = 0; b < g->boxes.size(); ++b) {
@@ -1153,7 +1153,7 @@ int check_step_err(Group* g, std::string* err) {
     CK(cudaMemcpyAsync(g->boxes[b]->hb.st, &st, sizeof(st), cudaMemcpyHostToDevice, g->stream), err);
   }
   CK(cudaStreamSynchronize(g->stream), err);
-  if (timeout) return fail(err, LC_ERR_TIMEOUT, "a dependency wait of the persistent step kernel gave up; the state is invalid");
+  if (timeout) return fail(err, LC_ERR_TIMEOUT, "a bounded wait of a step kernel gave up; the state is invalid");
   if (cbox < 0) return fail(err, LC_ERR_STATE, "contact flagged with no box recording it");
   char with[32];
   if (cpartner == -1) snprintf(with, sizeof(with), "a wall");
@@ -1180,14 +1180,16 @@ int enqueue_step(Group* g) {
   if (g->variant == 3) {
     CK(launch_dataflow(g, 1), &g->err);
     if (g->nmob > 0)
-      CK(launch_rediscretise(g->prec, g->d_boxes, (int)g->boxes.size(), g->d_mob, g->nmob, g->nsm, g->stream),
+      CK(launch_rediscretise(g->prec, g->d_boxes, (int)g->boxes.size(), g->d_mob, g->nmob, g->nsm,
+                           reinterpret_cast<unsigned*>(g->d_err) + 2, g->d_err, spin_limit(), g->stream),
          &g->err);
     return LC_OK;
   }
   if (int rc = enqueue_force_lb(g)) return rc;
   CK(launch_phase(g, 2, LC_RESID | LC_COMMIT), &g->err);
   if (g->nmob > 0)
-    CK(launch_rediscretise(g->prec, g->d_boxes, (int)g->boxes.size(), g->d_mob, g->nmob, g->nsm, g->stream), &g->err);
+    CK(launch_rediscretise(g->prec, g->d_boxes, (int)g->boxes.size(), g->d_mob, g->nmob, g->nsm,
+                           reinterpret_cast<unsigned*>(g->d_err) + 2, g->d_err, spin_limit(), g->stream), &g->err);
   return LC_OK;
 }
 
@@ -1288,7 +1290,8 @@ int group_profile(Group* g, int n, double* ms) {
     CK(cudaEventRecord(ev[3], g->stream), &g->err);
     CK(launch_colloid(g->d_boxes, (int)g->boxes.size(), g->stream), &g->err);
     if (g->nmob > 0)
-      CK(launch_rediscretise(g->prec, g->d_boxes, (int)g->boxes.size(), g->d_mob, g->nmob, g->nsm, g->stream),
+      CK(launch_rediscretise(g->prec, g->d_boxes, (int)g->boxes.size(), g->d_mob, g->nmob, g->nsm,
+                           reinterpret_cast<unsigned*>(g->d_err) + 2, g->d_err, spin_limit(), g->stream),
          &g->err);
     CK(cudaEventRecord(ev[4], g->stream), &g->err);
     CK(cudaEventSynchronize(ev[4]), &g->err);
@@ -1311,7 +1314,8 @@ int group_profile(Group* g, int n, double* ms) {
     for (int s = 0; s < n; ++s) {
       CK(launch_dataflow(g, 1), &g->err);
       if (g->nmob > 0)
-        CK(launch_rediscretise(g->prec, g->d_boxes, (int)g->boxes.size(), g->d_mob, g->nmob, g->nsm, g->stream),
+        CK(launch_rediscretise(g->prec, g->d_boxes, (int)g->boxes.size(), g->d_mob, g->nmob, g->nsm,
+                           reinterpret_cast<unsigned*>(g->d_err) + 2, g->d_err, spin_limit(), g->stream),
            &g->err);
     }
     CK(cudaEventRecord(ev[4], g->stream), &g->err);

@@ -78,6 +78,10 @@ struct DevColloid {
   double Fh[3], Th[3], Flc[3], Tlc[3];
   double imp[3], aimp[3];
   double rdp[3];  // momentum exchanged by the running re-discretisation
+  // mobile colloids: the position of the last search for changed nodes and the
+  // least distance of a node from the surface then; until the colloid has moved
+  // that far no node can change (0: not searched yet)
+  double Xref[3], margin;
 };
 
 // Per-box state flags kept on the device (the step kernels flip the buffer
@@ -88,7 +92,7 @@ struct DevState {
   int pre_valid;  // f[fpar] holds pre-collision values: next collide reads them in place
   int err;        // sticky error bits (1: link list overflow, 2: change list overflow, 4: overlap, 8: contact)
   int nchg;       // nodes whose solid/fluid status changes after the colloid update of this step
-  int pad;
+  int scan;       // 1: a mobile colloid has moved past its margin; search for changed nodes
   long long step;
   // first contact since the host last read it (see resolve_contacts): the
   // step, the colloid and its partner (-1: a z wall); cstep < 0: none

@@ -75,9 +75,11 @@ cudaError_t launch_colloid(DevBox* boxes, int nboxes, cudaStream_t s);
 cudaError_t launch_step(int prec, int ty, DevBox* boxes, const StepItem* items, int nitems, int zc, unsigned* sync,
                         double* part, int spin_limit, int commit, int* err, int grid, cudaStream_t s);
 int step_blocks_per_sm(int prec, int ty);
-// Re-discretisation after the colloid update; mob lists (box, colloid) of mobile colloids.
+// Re-discretisation after the colloid update; mob lists (box, colloid) of
+// mobile colloids, bar the grid barrier's counter (never reset but after an
+// error), err the group's error words.
 cudaError_t launch_rediscretise(int prec, DevBox* boxes, int nboxes, const int2* mob, int nmob, int nsm,
-                                cudaStream_t s);
+                                unsigned* bar, int* err, int spin_limit, cudaStream_t s);
 // Fills box b's list of near nodes (up to its capacity) and its count, which
 // the caller has zeroed.
 cudaError_t launch_near_list(DevBox* boxes, int b, int N, cudaStream_t s);

@@ -1944,7 +1944,30 @@ __device__ __forceinline__ void colloid_box(const DevBox& B, bool commit = true)
     }
     for (int k = 0; k < 24; ++k) C.acc[k] = 0.0;
   }
-  if (B.nmobile) resolve_contacts(B, tid, nthr);
+  if (B.nmobile) {
+    resolve_contacts(B, tid, nthr);
+    // has a colloid moved as far as the node nearest to its surface?  (1e-9:
+    // far above the rounding of the solid test, far below any margin that
+    // saves a search)
+    __shared__ int s_scan;
+    if (tid == 0) s_scan = 0;
+    __syncthreads();
+    for (int c = tid; c < B.ncol; c += nthr) {
+      const DevColloid& C = B.col[c];
+      if (!C.mobile) continue;
+      double r[3];
+      disp(B, C.X[0], C.X[1], C.X[2], C.Xref, r);
+      if (!(sqrt(r[0] * r[0] + r[1] * r[1] + r[2] * r[2]) + 1e-9 < C.margin)) s_scan = 1;
+    }
+    __syncthreads();
+    if (s_scan)
+      for (int c = tid; c < B.ncol; c += nthr) {
+        DevColloid& C = B.col[c];
+        for (int a = 0; a < 3; ++a) C.Xref[a] = C.X[a];
+        C.margin = 1.0;
+      }
+    if (tid == 0) B.st->scan = s_scan;
+  }
   if (tid == 0) {
     DevState* st = B.st;
     if (B.p.flow_on) {
@@ -2843,18 +2866,24 @@ __global__ void __launch_bounds__(256) k_reduce(const double* __restrict__ part,
 // ---------------------------------------------------------------------------
 // re-discretisation of moving colloids (Sec. 2.2, last paragraph)
 // ---------------------------------------------------------------------------
-// Run after the colloid update of every step for the (box, colloid) pairs of
-// mobile colloids; every kernel returns at once when nothing changed.
-//   k_rd_find     nodes of the colloid's bounding region whose solid test at
-//                 the new X differs from the mask -> change list
-//   k_rd_pull     pre-collision populations of the step just streamed, pulled
-//                 with the old mask and the old colloid state, into the other
-//                 buffer (the next collide reads them in place)
-//   k_rd_apply    covered nodes hand their momentum sum_q df_q c_q to the
-//                 colloid; uncovered nodes take f_eq(rho_bar, u_b) and the
-//                 mean Q of their fluid face neighbours (fluid before and after)
-//   k_rd_mask     mask bits of the changed nodes; k_rd_near the near flags of
-//                 the region; k_rd_links the boundary links of the box.
+// One launch (k_rediscretise) after the colloid update, which has flagged the
+// boxes where a mobile colloid moved past its margin (DevState::scan); without
+// one every block returns at once.  Phases, with a grid barrier between them
+// (the launch is cooperative, so all its blocks are resident):
+//   rd_find   nodes of the colloid's bounding region whose solid test at the
+//             new X differs from the mask -> change list; the least distance
+//             of a node from the surface -> margin
+//   rd_pull   pre-collision populations of the step just streamed, pulled
+//             with the old mask and the old colloid state, into the other
+//             buffer (the next collide reads them in place)
+//   rd_apply  covered nodes hand their momentum sum_q df_q c_q to the
+//             colloid; uncovered nodes take f_eq(rho_bar, u_b) and the
+//             mean Q of their fluid face neighbours (fluid before and after)
+//   rd_mask   mask bits of the changed nodes; rd_near the near flags of the
+//             region; rd_links the boundary links and near list of the box;
+//             rd_finish the box state.
+// As eight launches that returned at once they took 52 us of the 113 us step
+// of a 64^3 box with one mobile colloid.
 __device__ __forceinline__ int region_lo(double c, double r) { return (int)floor(c - r - 2.0); }
 
 // Node (x,y,z) of the bounding region of colloid C: index k of n = nx*ny*nz region
@@ -2887,18 +2916,25 @@ __device__ __forceinline__ int new_owner(const DevBox& B, int x, int y, int z) {
   return 0;
 }
 
-__global__ void __launch_bounds__(256) k_rd_find(DevBox* __restrict__ boxes, const int2* __restrict__ mob, int nmob) {
-  for (int p = blockIdx.y; p < nmob; p += gridDim.y) {
+// Words that other blocks of the same launch write: read through L2.
+__device__ __forceinline__ int ld_state(const int* p) { return __ldcg(p); }
+
+__device__ void rd_find(DevBox* __restrict__ boxes, const int2* __restrict__ mob, int nmob) {
+  for (int p = 0; p < nmob; ++p) {
     const DevBox& B = boxes[mob[p].x];
-    const DevColloid& C = B.col[mob[p].y];
-    const int n = region_size(B, C);
+    if (!B.st->scan) continue;
+    DevColloid& C = B.col[mob[p].y];
+    const int c = mob[p].y, n = region_size(B, C);
+    double gap = 1.0;
     for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < n; k += gridDim.x * blockDim.x) {
       int x, y, z;
       if (!region_node(B, C, k, x, y, z)) continue;
       const int i = x + B.nx * (y + B.ny * z);
       const int old = B.mask[i] & IDMASK;
       const bool in_new = inside_colloid(B, x, y, z, C);
-      const int c = mob[p].y;
+      double r[3];
+      disp(B, (double)x, (double)y, (double)z, C.X, r);
+      gap = fmin(gap, fabs(sqrt(r[0] * r[0] + r[1] * r[1] + r[2] * r[2]) - C.a0));
       int code = -1;
       if (in_new && old == 0) code = c << 1;                 // covered
       else if (!in_new && old == c + 1) code = (c << 1) | 1;  // uncovered
@@ -2913,14 +2949,16 @@ __global__ void __launch_bounds__(256) k_rd_find(DevBox* __restrict__ boxes, con
         }
       }
     }
+    // positive doubles order as their bits
+    if (gap < 1.0) atomicMin(reinterpret_cast<unsigned long long*>(&C.margin), (unsigned long long)__double_as_longlong(gap));
   }
 }
 
 template <typename T>
-__global__ void __launch_bounds__(256) k_rd_pull(DevBox* __restrict__ boxes, int nboxes) {
+__device__ void rd_pull(DevBox* __restrict__ boxes, int nboxes) {
   for (int b = 0; b < nboxes; ++b) {
     const DevBox& B = boxes[b];
-    if (B.st->nchg == 0 || !B.p.flow_on) continue;
+    if (ld_state(&B.st->nchg) == 0 || !B.p.flow_on) continue;
     const int fpar = B.st->fpar;
     const bool pre = B.st->pre_valid != 0;
     const T* fin = static_cast<const T*>(B.f[fpar]);
@@ -2938,10 +2976,10 @@ __global__ void __launch_bounds__(256) k_rd_pull(DevBox* __restrict__ boxes, int
 }
 
 template <typename T>
-__global__ void __launch_bounds__(256) k_rd_apply(DevBox* __restrict__ boxes, int nboxes) {
+__device__ void rd_apply(DevBox* __restrict__ boxes, int nboxes) {
   for (int b = 0; b < nboxes; ++b) {
     DevBox& B = boxes[b];
-    const int nchg = min(B.st->nchg, B.chg_cap);
+    const int nchg = min(ld_state(&B.st->nchg), B.chg_cap);
     if (nchg == 0) continue;
     const int fpar = B.st->fpar;
     T* fpre = static_cast<T*>(B.f[fpar ^ 1]);
@@ -3015,10 +3053,10 @@ __global__ void __launch_bounds__(256) k_rd_apply(DevBox* __restrict__ boxes, in
   }
 }
 
-__global__ void __launch_bounds__(256) k_rd_mask(DevBox* __restrict__ boxes, int nboxes) {
+__device__ void rd_mask(DevBox* __restrict__ boxes, int nboxes) {
   for (int b = 0; b < nboxes; ++b) {
     const DevBox& B = boxes[b];
-    const int nchg = min(B.st->nchg, B.chg_cap);
+    const int nchg = min(ld_state(&B.st->nchg), B.chg_cap);
     if (nchg == 0) continue;
     for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < nchg; k += gridDim.x * blockDim.x) {
       const int i = B.chg[2 * k], code = B.chg[2 * k + 1];
@@ -3027,10 +3065,10 @@ __global__ void __launch_bounds__(256) k_rd_mask(DevBox* __restrict__ boxes, int
   }
 }
 
-__global__ void __launch_bounds__(256) k_rd_near(DevBox* __restrict__ boxes, const int2* __restrict__ mob, int nmob) {
-  for (int p = blockIdx.y; p < nmob; p += gridDim.y) {
+__device__ void rd_near(DevBox* __restrict__ boxes, const int2* __restrict__ mob, int nmob) {
+  for (int p = 0; p < nmob; ++p) {
     const DevBox& B = boxes[mob[p].x];
-    if (B.st->nchg == 0) continue;
+    if (ld_state(&B.st->nchg) == 0) continue;
     const DevColloid& C = B.col[mob[p].y];
     const int n = region_size(B, C);
     for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < n; k += gridDim.x * blockDim.x) {
@@ -3058,26 +3096,18 @@ __global__ void __launch_bounds__(256) k_rd_near(DevBox* __restrict__ boxes, con
 }
 
 // Rebuild the boundary links (unordered; lc_lb_get_links sorts them) and the
-// near-node lists of boxes whose solid set changed.  Block 0 of the grid first clears the count
-// in a separate launch (k_rd_links_reset).
-__global__ void k_rd_links_reset(DevBox* __restrict__ boxes, int nboxes) {
-  const int b = blockIdx.x * blockDim.x + threadIdx.x;
-  if (b < nboxes && boxes[b].st->nchg > 0) {
-    *boxes[b].nlinks = 0;
-    *boxes[b].nnear = 0;
-  }
-}
-
-__global__ void __launch_bounds__(256) k_rd_links(DevBox* __restrict__ boxes, int nboxes) {
+// near-node lists of boxes whose solid set changed (their counts are zeroed
+// with the near flags).
+__device__ void rd_links(DevBox* __restrict__ boxes, int nboxes) {
   for (int b = 0; b < nboxes; ++b) {
     const DevBox& B = boxes[b];
-    if (B.st->nchg == 0) continue;
-    const int nthr = gridDim.x * gridDim.y * blockDim.x;
-    for (int base = (blockIdx.y * gridDim.x + blockIdx.x) * blockDim.x; base < B.N; base += nthr) {
+    if (ld_state(&B.st->nchg) == 0) continue;
+    const int nthr = gridDim.x * blockDim.x;
+    for (int base = blockIdx.x * blockDim.x; base < B.N; base += nthr) {
       const int i = base + threadIdx.x;
       near_append(B, i, i < B.N && (B.mask[i] & NEAR) && (B.mask[i] & IDMASK) == 0);
     }
-    for (int c = blockIdx.y; c < B.ncol; c += gridDim.y) {
+    for (int c = 0; c < B.ncol; ++c) {
       const DevColloid& C = B.col[c];
       const int n = region_size(B, C);
       for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < n; k += gridDim.x * blockDim.x) {
@@ -3106,12 +3136,10 @@ __global__ void __launch_bounds__(256) k_rd_links(DevBox* __restrict__ boxes, in
 
 // The next collide reads the pulled populations in place; the momentum
 // exchanged by the re-discretisation changes each mobile colloid's velocity.
-__global__ void k_rd_finish(DevBox* __restrict__ boxes, int nboxes) {
-  const int b = blockIdx.x * blockDim.x + threadIdx.x;
-  if (b >= nboxes) return;
+__device__ void rd_finish(DevBox* __restrict__ boxes, int b) {
   DevBox& B = boxes[b];
   DevState* st = B.st;
-  if (st->nchg == 0) return;
+  if (ld_state(&st->nchg) == 0) return;
   if (B.p.flow_on) {
     st->fpar ^= 1;
     st->pre_valid = 1;
@@ -3122,7 +3150,64 @@ __global__ void k_rd_finish(DevBox* __restrict__ boxes, int nboxes) {
       for (int a = 0; a < 3; ++a) C.V[a] += C.rdp[a] / C.M;
     for (int a = 0; a < 3; ++a) C.rdp[a] = 0.0;
   }
-  if (*B.nlinks > B.nlinks_cap || *B.nnear > B.near_cap) atomicOr(&st->err, 1);
+  if (ld_state(B.nlinks) > B.nlinks_cap || ld_state(B.nnear) > B.near_cap) atomicOr(&st->err, 1);
+}
+
+// Grid barrier: every block arrives on a counter that only grows and waits for
+// the multiple of the grid size that its arrival belongs to.  Bounded: after
+// spin_limit polls the error word is set and the block gives up.
+__device__ bool grid_barrier(unsigned* bar, int* err, int spin_limit) {
+  __shared__ int s_ok;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    __threadfence();
+    const unsigned n = gridDim.x, target = (atomicAdd(bar, 1u) / n + 1u) * n;
+    int ok = 0;
+    for (int spin = 0; spin <= spin_limit; ++spin) {
+      if ((int)(ld_acquire_u32(bar) - target) >= 0) {
+        ok = 1;
+        break;
+      }
+      __nanosleep(40);
+    }
+    if (!ok) atomicOr(err, 1);
+    s_ok = ok;
+    __threadfence();
+  }
+  __syncthreads();
+  return s_ok != 0;
+}
+
+template <typename T>
+__global__ void __launch_bounds__(256) k_rediscretise(DevBox* __restrict__ boxes, int nboxes,
+                                                      const int2* __restrict__ mob, int nmob, unsigned* bar, int* err,
+                                                      int spin_limit) {
+  bool any = false;
+  for (int b = threadIdx.x; b < nboxes; b += blockDim.x) any = any || (boxes[b].nmobile && boxes[b].st->scan);
+  if (!__syncthreads_or(any)) return;
+  rd_find(boxes, mob, nmob);
+  if (!grid_barrier(bar, err, spin_limit)) return;
+  any = false;
+  for (int b = threadIdx.x; b < nboxes; b += blockDim.x) any = any || ld_state(&boxes[b].st->nchg) != 0;
+  if (!__syncthreads_or(any)) return;
+  rd_pull<T>(boxes, nboxes);
+  if (!grid_barrier(bar, err, spin_limit)) return;
+  rd_apply<T>(boxes, nboxes);
+  if (!grid_barrier(bar, err, spin_limit)) return;
+  rd_mask(boxes, nboxes);
+  if (!grid_barrier(bar, err, spin_limit)) return;
+  rd_near(boxes, mob, nmob);
+  if (blockIdx.x == 0)
+    for (int b = threadIdx.x; b < nboxes; b += blockDim.x)
+      if (ld_state(&boxes[b].st->nchg) > 0) {
+        *boxes[b].nlinks = 0;
+        *boxes[b].nnear = 0;
+      }
+  if (!grid_barrier(bar, err, spin_limit)) return;
+  rd_links(boxes, nboxes);
+  if (!grid_barrier(bar, err, spin_limit)) return;
+  if (blockIdx.x == 0)
+    for (int b = threadIdx.x; b < nboxes; b += blockDim.x) rd_finish(boxes, b);
 }
 
 // ---------------------------------------------------------------------------
@@ -3355,18 +3440,13 @@ cudaError_t launch_export(int prec, const DevBox* boxes, int b, int N, int which
 
 
 cudaError_t launch_rediscretise(int prec, DevBox* boxes, int nboxes, const int2* mob, int nmob, int nsm,
-                                cudaStream_t s) {
+                                unsigned* bar, int* err, int spin_limit, cudaStream_t s) {
   if (nmob <= 0) return cudaSuccess;
-  k_rd_find<<<dim3(8, nmob), 256, 0, s>>>(boxes, mob, nmob);
-  if (prec == 0) k_rd_pull<float><<<nsm * 2, 256, 0, s>>>(boxes, nboxes);
-  else k_rd_pull<double><<<nsm * 2, 256, 0, s>>>(boxes, nboxes);
-  if (prec == 0) k_rd_apply<float><<<4, 256, 0, s>>>(boxes, nboxes);
-  else k_rd_apply<double><<<4, 256, 0, s>>>(boxes, nboxes);
-  k_rd_mask<<<4, 256, 0, s>>>(boxes, nboxes);
-  k_rd_near<<<dim3(8, nmob), 256, 0, s>>>(boxes, mob, nmob);
-  k_rd_links_reset<<<(nboxes + 127) / 128, 128, 0, s>>>(boxes, nboxes);
-  k_rd_links<<<dim3(8, 4), 256, 0, s>>>(boxes, nboxes);
-  k_rd_finish<<<(nboxes + 127) / 128, 128, 0, s>>>(boxes, nboxes);
+  // one block per SM: all resident, which the cooperative launch guarantees
+  void* args[] = {&boxes, &nboxes, &mob, &nmob, &bar, &err, &spin_limit};
+  const void* fn = prec == 0 ? (const void*)k_rediscretise<float> : (const void*)k_rediscretise<double>;
+  cudaError_t e = cudaLaunchCooperativeKernel(fn, dim3(nsm), dim3(256), args, 0, s);
+  if (e != cudaSuccess) return e;
   return cudaGetLastError();
 }
 
