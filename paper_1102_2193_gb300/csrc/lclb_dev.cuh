@@ -350,21 +350,24 @@ __device__ __forceinline__ void rigid_velocity(const double* V, const double* W,
 // matrix (Smith, CACM 1961) and a cross product of two rows of (A - l I).
 // FP64: the eigenvalue of the FP32 evaluation refined by two Newton steps on
 // the characteristic polynomial det(A - l I) = -l^3 + (Tr A^2 / 2) l + det A
-// (no FP64 transcendental functions), then the FP64 cross products.
+// (no FP64 transcendental functions; the slope in FP32, whose 1e-7 leaves the
+// steps 1e-7 -> 1e-14 -> rounding), then the FP64 cross products.  One warp
+// runs this chain per 32 nodes next to a planar colloid, and in a small box
+// the step waits for it, so FP64 divisions and square roots are kept out.
 template <typename T>
 __device__ void principal_dir(const T* q, T n[3]);
 
 __device__ __forceinline__ double principal_lambda_f64(const double* q) {
   const double a00 = q[0], a01 = q[1], a02 = q[2], a11 = q[3], a12 = q[4], a22 = -q[0] - q[3];
-  const float qf[5] = {(float)q[0], (float)q[1], (float)q[2], (float)q[3], (float)q[4]};
   // FP32 seed: the largest eigenvalue by the trigonometric formula
-  const float f00 = qf[0], f01 = qf[1], f02 = qf[2], f11 = qf[3], f12 = qf[4], f22 = -qf[0] - qf[3];
+  const float f00 = (float)q[0], f01 = (float)q[1], f02 = (float)q[2], f11 = (float)q[3], f12 = (float)q[4];
+  const float f22 = -f00 - f11;
   const float p1 = f01 * f01 + f02 * f02 + f12 * f12;
   const float p2 = f00 * f00 + f11 * f11 + f22 * f22 + 2.f * p1;
   float lam32 = 0.f;
   if (p2 > 0.f) {
-    const float pp = sqrtf(p2 / 6.f);
-    const float b00 = f00 / pp, b01 = f01 / pp, b02 = f02 / pp, b11 = f11 / pp, b12 = f12 / pp, b22 = f22 / pp;
+    const float pp = sqrtf(p2 / 6.f), ip = 1.f / pp;
+    const float b00 = f00 * ip, b01 = f01 * ip, b02 = f02 * ip, b11 = f11 * ip, b12 = f12 * ip, b22 = f22 * ip;
     float r = (b00 * (b11 * b22 - b12 * b12) - b01 * (b01 * b22 - b12 * b02) + b02 * (b01 * b12 - b11 * b02)) / 2.f;
     r = fminf(1.f, fmaxf(-1.f, r));
     lam32 = 2.f * pp * cosf(acosf(r) / 3.f);
@@ -374,11 +377,21 @@ __device__ __forceinline__ double principal_lambda_f64(const double* q) {
   double lam = (double)lam32;
 #pragma unroll
   for (int it = 0; it < 2; ++it) {
-    const double f = -lam * lam * lam + t2 * lam + det;
-    const double df = -3.0 * lam * lam + t2;
-    if (df != 0.0) lam -= f / df;
+    const double f = (t2 - lam * lam) * lam + det;
+    const float df = (float)(t2 - 3.0 * lam * lam);
+    if (df != 0.f) lam -= f * (double)(1.f / df);
   }
   return lam;
+}
+
+// 1/sqrt(v) in FP64 from the FP32 estimate and Newton steps (FP32 storage:
+// one, relative error ~1e-14; FP64 storage: two, to rounding).
+template <int STEPS>
+__device__ __forceinline__ double rsqrt_f64(double v) {
+  double r = (double)rsqrtf((float)v);
+#pragma unroll
+  for (int k = 0; k < STEPS; ++k) r = r * (1.5 - 0.5 * v * r * r);
+  return r;
 }
 
 template <typename T>
@@ -409,16 +422,28 @@ __device__ void principal_dir(const T* q, T n[3]) {
   T n0 = c0[0] * c0[0] + c0[1] * c0[1] + c0[2] * c0[2];
   T n1 = c1[0] * c1[0] + c1[1] * c1[1] + c1[2] * c1[2];
   T n2 = c2[0] * c2[0] + c2[1] * c2[1] + c2[2] * c2[2];
-  const T* c = c0;
   T nn = n0;
-  if (n1 > nn) { c = c1; nn = n1; }
-  if (n2 > nn) { c = c2; nn = n2; }
+#pragma unroll
+  for (int a = 0; a < 3; ++a) n[a] = c0[a];
+  if (n1 > nn) {
+    nn = n1;
+#pragma unroll
+    for (int a = 0; a < 3; ++a) n[a] = c1[a];
+  }
+  if (n2 > nn) {
+    nn = n2;
+#pragma unroll
+    for (int a = 0; a < 3; ++a) n[a] = c2[a];
+  }
   if (!(nn > T(0))) {
     n[0] = T(1); n[1] = T(0); n[2] = T(0);
     return;
   }
-  T s = T(1) / sqrt(nn);
-  n[0] = c[0] * s; n[1] = c[1] * s; n[2] = c[2] * s;
+  T s;
+  // the FP32 estimate needs a normal FP32 argument (nn is a fourth power of Q's anisotropy)
+  if constexpr (sizeof(T) == 8) s = nn > 1e-30 && nn < 1e30 ? rsqrt_f64<2>(nn) : T(1) / sqrt(nn);
+  else s = T(1) / sqrt(nn);
+  n[0] *= s; n[1] *= s; n[2] *= s;
 }
 
 // Surface order Q0 = S0 (n0 n0 - delta/3) (Eq. 7) at solid node (sx,sy,sz) of
@@ -570,16 +595,6 @@ __device__ __forceinline__ void gather_q(const DevBox& B, const T* __restrict__ 
       ghost_q(B, c, sx, sy, sz, qi, qn[d], surf);
     }
   }
-}
-
-// 1/sqrt(v) in FP64 from the FP32 estimate and Newton steps (FP32 storage:
-// one, relative error ~1e-14; FP64 storage: two, to rounding).
-template <int STEPS>
-__device__ __forceinline__ double rsqrt_f64(double v) {
-  double r = (double)rsqrtf((float)v);
-#pragma unroll
-  for (int k = 0; k < STEPS; ++k) r = r * (1.5 - 0.5 * v * r * r);
-  return r;
 }
 
 // Surface order Q0 (Eq. 7) in FP64: the unit normal s at solid node

@@ -324,6 +324,52 @@ __global__ void __launch_bounds__(TX * TY) k_force(const DevBox* __restrict__ bo
   }
 }
 
+// Moving-surface term of the bounced populations: ms[q] is the mask byte of
+// node r - c_q (colloid id + 1, 0 fluid, WALLFLAG).  The colloid's state is
+// read and converted once per node (a node rarely touches two), and a colloid
+// at rest adds nothing.
+template <typename T>
+__device__ __forceinline__ void bounce_correction(const DevBox& B, int x, int y, int z, const uint8_t ms[NQ],
+                                                  T df[NQ]) {
+  const T rho0 = phys<T>(B).rho0;
+  unsigned todo = 0;
+#pragma unroll
+  for (int q = 1; q < NQ; ++q)
+    if (ms[q] != 0 && ms[q] != WALLFLAG) todo |= 1u << q;
+  while (todo) {
+    int id = 0;
+    const int first = __ffs(todo) - 1;
+#pragma unroll
+    for (int q = 1; q < NQ; ++q)
+      if (q == first) id = ms[q];
+    const DevColloid& C = B.col[id - 1];
+    T X[3], V[3], W[3];
+    bool moving = false;
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+      X[a] = T(C.Xb[a]);
+      V[a] = T(C.Vb[a]);
+      W[a] = T(C.Wb[a]);
+      moving = moving || V[a] != T(0) || W[a] != T(0);
+    }
+#pragma unroll
+    for (int q = 1; q < NQ; ++q) {
+      if (ms[q] != id) continue;
+      todo &= ~(1u << q);
+      if (!moving) continue;
+      // u_b = V + W x d at the link midpoint r - c_q / 2
+      const T d0 = minimg_t(T(x) - T(0.5 * cx(q)) - X[0], B.nx, true);
+      const T d1 = minimg_t(T(y) - T(0.5 * cy(q)) - X[1], B.ny, true);
+      const T d2 = minimg_t(T(z) - T(0.5 * cz(q)) - X[2], B.nz, !B.wall_z);
+      T cub = T(0);
+      if (cx(q)) cub += T(cx(q)) * (V[0] + W[1] * d2 - W[2] * d1);
+      if (cy(q)) cub += T(cy(q)) * (V[1] + W[2] * d0 - W[0] * d2);
+      if (cz(q)) cub += T(cz(q)) * (V[2] + W[0] * d1 - W[1] * d0);
+      df[q] += T(6.0 * wq(q)) * rho0 * cub;
+    }
+  }
+}
+
 // ---------------------------------------------------------------------------
 // pull with bounce-back (shared by the LB kernels and the export/diagnostic kernels)
 // ---------------------------------------------------------------------------
@@ -361,7 +407,6 @@ __device__ __forceinline__ void pull(const DevBox& B, const T* __restrict__ fin,
   // near node: the 18 mask bytes, then the 19 populations, each in one round of
   // independent loads (taken direction by direction, the dependent pairs of
   // loads were most of the time of a small box's LB kernel)
-  const T rho0 = phys<T>(B).rho0;
   int s[NQ];
   uint8_t ms[NQ];
   s[0] = i;
@@ -376,15 +421,7 @@ __device__ __forceinline__ void pull(const DevBox& B, const T* __restrict__ fin,
   }
 #pragma unroll
   for (int q = 0; q < NQ; ++q) df[q] = ldg(fin + (ms[q] == 0 ? (size_t)q * N + s[q] : (size_t)opp(q) * N + i));
-#pragma unroll
-  for (int q = 1; q < NQ; ++q) {
-    if (ms[q] == 0 || ms[q] == WALLFLAG) continue;
-    const DevColloid& C = B.col[ms[q] - 1];
-    T ub[3];
-    rigid_velocity_t<T>(B, T(x) - T(0.5 * cx(q)), T(y) - T(0.5 * cy(q)), T(z) - T(0.5 * cz(q)), C.Xb, C.Vb, C.Wb, ub);
-    const T cub = T(cx(q)) * ub[0] + T(cy(q)) * ub[1] + T(cz(q)) * ub[2];
-    df[q] += T(6.0 * wq(q)) * rho0 * cub;
-  }
+  bounce_correction<T>(B, x, y, z, ms, df);
 }
 
 // Collide at fluid node i with force (Fx,Fy,Fz) (BGK + Guo, deviation form):
@@ -641,13 +678,25 @@ __device__ __noinline__ void near_stress(const DevBox& B, int i, int mode, NearS
 #pragma unroll
   for (int d = 0; d < 6; ++d) cf[d] = (int)(B.mask[nb[d] < 0 ? j0 : nb[d]] & IDMASK);
   unsigned solid = 0;  // solid faces of the node
-  bool planar = false;
+#pragma unroll
+  for (int d = 0; d < 6; ++d)
+    if (valid && (nb[d] < 0 || cf[d] != 0)) solid |= 1u << d;
+  // differences to the fluid neighbours (their loads are in flight under the
+  // arithmetic of the surface values)
+  T dn[6][5];
 #pragma unroll
   for (int d = 0; d < 6; ++d) {
-    const int c = nb[d] < 0 ? -1 : cf[d] - 1;
-    if (valid && (nb[d] < 0 || c >= 0)) solid |= 1u << d;
-    if (valid && c >= 0 && B.col[c].anchoring != 0) planar = true;
+    const size_t j = ((solid >> d) & 1u) || nb[d] < 0 ? j0 : nb[d];
+#pragma unroll
+    for (int k = 0; k < 5; ++k) {
+      dn[d][k] = ldg(Q + (size_t)k * N + j) - qh[k];
+      if constexpr (comp) dn[d][k] += __bfloat162float(Lo[(size_t)k * N + j]) - ql[k];
+    }
   }
+  bool planar = false;
+#pragma unroll
+  for (int d = 0; d < 6; ++d)
+    if (((solid >> d) & 1u) && nb[d] >= 0 && B.col[cf[d] - 1].anchoring != 0) planar = true;
   double nf[3] = {1.0, 0.0, 0.0};
   if (planar) {
     double qid[5];
@@ -670,12 +719,15 @@ __device__ __noinline__ void near_stress(const DevBox& B, int i, int mode, NearS
     const int e = t < nface ? sc.face[t] : lane;
     own = e & 31;
     d = e >> 8;
-    const int o = __shfl_sync(full, j0, own);
-    s[0] = o % nx; s[1] = (o / nx) % ny; s[2] = o / (nx * ny);
-    const int ax = d >> 1, v = s[ax] + ((d & 1) ? -1 : 1);
-    const int L = ax == 0 ? nx : (ax == 1 ? ny : B.nz);
-    const bool out = ax == 2 && B.wall_z && (v < 0 || v >= L);
-    s[ax] = out ? v : wrap1(v, L);
+    s[0] = __shfl_sync(full, x, own);
+    s[1] = __shfl_sync(full, y, own);
+    s[2] = __shfl_sync(full, z, own);
+    const int ax = d >> 1, up = (d & 1) ? -1 : 1;
+    s[0] = ax == 0 ? wrap1(s[0] + up, nx) : s[0];
+    s[1] = ax == 1 ? wrap1(s[1] + up, ny) : s[1];
+    const int zs = ax == 2 ? s[2] + up : s[2];
+    const bool out = B.wall_z && (zs < 0 || zs >= B.nz);
+    s[2] = out ? zs : wrap1(zs, B.nz);
     c = t < nface && !out ? (int)(B.mask[s[0] + nx * (s[1] + ny * s[2])] & IDMASK) - 1 : -1;
   };
   for (int t0 = 0; t0 < nface; t0 += 32) {
@@ -700,18 +752,11 @@ __device__ __noinline__ void near_stress(const DevBox& B, int i, int mode, NearS
     }
   }
   __syncwarp();
-  T dn[6][5];
 #pragma unroll
-  for (int d = 0; d < 6; ++d) {
-    const bool so = (solid >> d) & 1u;
-    const size_t j = so || nb[d] < 0 ? j0 : nb[d];
+  for (int d = 0; d < 6; ++d)
+    if ((solid >> d) & 1u)
 #pragma unroll
-    for (int k = 0; k < 5; ++k) {
-      T v = ldg(Q + (size_t)k * N + j) - qh[k];
-      if constexpr (comp) v += __bfloat162float(Lo[(size_t)k * N + j]) - ql[k];
-      dn[d][k] = so ? sc.dn[slot[d]][k] : v;
-    }
-  }
+      for (int k = 0; k < 5; ++k) dn[d][k] = sc.dn[slot[d]][k];
   T qi[5], dq[3][5], lap[5], h[5], p[9], fp;
 #pragma unroll
   for (int k = 0; k < 5; ++k) {
@@ -756,8 +801,10 @@ __device__ __noinline__ void near_stress(const DevBox& B, int i, int mode, NearS
       const T pcv[3] = {ax == 0 ? po[0] : (ax == 1 ? po[1] : po[2]), ax == 0 ? po[3] : (ax == 1 ? po[4] : po[5]),
                         ax == 0 ? po[6] : (ax == 1 ? po[7] : po[8])};
       // the fluid node: one step back from the solid node
-      const int L = ax == 0 ? nx : (ax == 1 ? ny : B.nz);
-      s[ax] = wrap1(s[ax] + ((d & 1) ? 1 : -1), L);
+      const int back = (d & 1) ? 1 : -1;
+      s[0] = ax == 0 ? wrap1(s[0] + back, nx) : s[0];
+      s[1] = ax == 1 ? wrap1(s[1] + back, ny) : s[1];
+      s[2] = ax == 2 ? wrap1(s[2] + back, B.nz) : s[2];
       colloid_face(B, c, ax, sgn, pcv, s[0], s[1], s[2], my_c, my_acc);
     }
   }
@@ -1234,21 +1281,26 @@ __device__ __forceinline__ void stored_force(const DevBox& B, const T* __restric
     }
     return;
   }
+  // near node: the six mask bytes, then all stress values, in one round of
+  // loads each (a closed face reads P(i), which is its face value)
+  size_t j[6];
+#pragma unroll
+  for (int d = 0; d < 6; ++d) j[d] = nb[d] >= 0 && (B.mask[nb[d] < 0 ? i : nb[d]] & IDMASK) == 0 ? nb[d] : i;
+  T v[6][3], pc[9];
+#pragma unroll
+  for (int c = 0; c < 9; ++c) pc[c] = ldx<CG>(Pb + (size_t)c * N + i);
+#pragma unroll
+  for (int d = 0; d < 6; ++d)
+#pragma unroll
+    for (int a = 0; a < 3; ++a) v[d][a] = ldx<CG>(Pb + (size_t)(3 * a + (d >> 1)) * N + j[d]);
   F[0] = F[1] = F[2] = T(0);
 #pragma unroll
-  for (int d = 0; d < 6; ++d) {
-    const int j = nb[d];
-    const bool fluid = j >= 0 && (B.mask[j] & IDMASK) == 0;
-    const int ax = d >> 1;
-    const T sgn = (d & 1) ? T(-1) : T(1);
+  for (int d = 0; d < 6; ++d)
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
-      const T* Pc = Pb + (size_t)(3 * a + ax) * N;
-      const T pc = ldx<CG>(Pc + i);
-      const T face = fluid ? T(0.5) * (pc + ldx<CG>(Pc + j)) : pc;
-      F[a] += sgn * face;
+      const T face = T(0.5) * (pc[3 * a + (d >> 1)] + v[d][a]);
+      F[a] += (d & 1) ? -face : face;
     }
-  }
 }
 
 // One fluid node of k_lbp: pull (bounce-back only for near nodes), body force
