@@ -425,6 +425,7 @@ void fill_phys(PhysT<T>& o, const DevParams& p) {
   o.ptau = (T)(p.tau - 0.5);
   o.K = (T)p.K;
   o.S0 = (T)p.S0;
+  o.S0l = (T)(p.S0 - (double)o.S0);
   for (int a = 0; a < 3; ++a) o.g[a] = (T)p.g[a];
 }
 
@@ -1586,6 +1587,9 @@ int lc_lb_add_colloid(lc_lb* h, const double X[3], double a0, int anchoring, dou
   C.w = w;
   C.strong = (!(w > 0.0) || std::isinf(w)) ? 1 : 0;
   C.wfac = C.strong ? 1.0 : w / (h->hb.p.K + w);
+  C.ws[0] = (float)C.wfac;
+  C.ws[1] = (float)(C.wfac - (double)C.ws[0]);
+  split_position(C);
   C.anchoring = anchoring;
   C.mobile = mobile ? 1 : 0;
   C.M = h->params.rho0 * 4.0 / 3.0 * M_PI * a0 * a0 * a0;

@@ -43,7 +43,7 @@ struct DevParams {
 template <typename T>
 struct PhysT {
   T rho0, omega, ptau;  // rho0, 1/tau, (1 - 1/(2 tau)) tau = tau - 1/2
-  T K, S0;
+  T K, S0, S0l;  // S0l: the part of S0 that FP32 drops
   T g[3];
 };
 
@@ -74,6 +74,8 @@ struct DevColloid {
   double Fext[3], Text[3];  // external force and torque
   int anchoring, mobile, strong, pad;
   double wfac;     // weight of Q0 in the surface value: w / (K + w), 1 for strong anchoring
+  float ws[2];     // wfac and X as sums of two floats (48 bits), for the FP32 surface values
+  float Xs[3][2];
   double acc[24];  // step sums: F_hyd, T_hyd, F_lc, T_lc, then the link drag tensors zv, zw (6 each, xx xy xz yy yz zz)
   double Fh[3], Th[3], Flc[3], Tlc[3];
   double imp[3], aimp[3];
@@ -83,6 +85,13 @@ struct DevColloid {
   // that far no node can change (0: not searched yet)
   double Xref[3], margin;
 };
+
+__host__ __device__ inline void split_position(DevColloid& C) {
+  for (int a = 0; a < 3; ++a) {
+    C.Xs[a][0] = (float)C.X[a];
+    C.Xs[a][1] = (float)(C.X[a] - (double)C.Xs[a][0]);
+  }
+}
 
 // Per-box state flags kept on the device (the step kernels flip the buffer
 // parities without a host round trip).
@@ -168,13 +177,20 @@ __device__ __forceinline__ int wrapn(int v, int n) {
   return r < 0 ? r + n : r;
 }
 
+// Orders doubles (no NaN) as integers: an FP64 comparison takes a slot of the
+// FP64 pipe (one instruction per 64 cycles for a warp), these do not.
+__device__ __forceinline__ bool f64_ge(double a, double b) {
+  const long long x = __double_as_longlong(a), y = __double_as_longlong(b);
+  return (x ^ ((x >> 63) & 0x7fffffffffffffffll)) >= (y ^ ((y >> 63) & 0x7fffffffffffffffll));
+}
+
 // Minimum-image displacement r - X along one axis (FP64, round-to-nearest
 // operations only, matching a plain C evaluation).
 __device__ __forceinline__ double minimg(double d, int L, bool periodic) {
   if (!periodic) return d;
-  double h = 0.5 * (double)L;
-  if (d >= h) d = __dsub_rn(d, (double)L);
-  else if (d < -h) d = __dadd_rn(d, (double)L);
+  const double h = 0.5 * (double)L;
+  if (f64_ge(d, h)) d = __dsub_rn(d, (double)L);
+  else if (!f64_ge(d, -h)) d = __dadd_rn(d, (double)L);
   return d;
 }
 
@@ -416,6 +432,28 @@ __device__ void principal_dir(const T* q, T n[3]) {
     lam = T(2) * p * cos(phi);
   }
   T r0[3] = {a00 - lam, a01, a02}, r1[3] = {a01, a11 - lam, a12}, r2[3] = {a02, a12, a22 - lam};
+  if constexpr (sizeof(T) == 8) {
+    // the longest of the three row products, found in FP32, then that one in
+    // FP64 (the others would be 24 of the chain's 110 FP64 instructions)
+    const float f0[3] = {(float)r0[0], (float)r0[1], (float)r0[2]}, f1[3] = {f0[1], (float)r1[1], (float)r1[2]};
+    const float f2[3] = {f0[2], f1[2], (float)r2[2]};
+    auto len = [](const float* u, const float* v) {
+      const float x = u[1] * v[2] - u[2] * v[1], y = u[2] * v[0] - u[0] * v[2], z = u[0] * v[1] - u[1] * v[0];
+      return x * x + y * y + z * z;
+    };
+    const float l0 = len(f0, f1), l1 = len(f0, f2), l2 = len(f1, f2);
+    if (fmaxf(l0, fmaxf(l1, l2)) > 1e-24f) {
+      const bool u1 = l2 > l0 && l2 > l1, v2 = u1 || l1 > l0;  // rows (0,1), (0,2) or (1,2)
+      const T u[3] = {u1 ? r1[0] : r0[0], u1 ? r1[1] : r0[1], u1 ? r1[2] : r0[2]};
+      const T v[3] = {v2 ? r2[0] : r1[0], v2 ? r2[1] : r1[1], v2 ? r2[2] : r1[2]};
+      n[0] = u[1] * v[2] - u[2] * v[1];
+      n[1] = u[2] * v[0] - u[0] * v[2];
+      n[2] = u[0] * v[1] - u[1] * v[0];
+      const T sc = rsqrt_f64<2>(n[0] * n[0] + n[1] * n[1] + n[2] * n[2]);
+      n[0] *= sc; n[1] *= sc; n[2] *= sc;
+      return;
+    }
+  }
   T c0[3] = {r0[1] * r1[2] - r0[2] * r1[1], r0[2] * r1[0] - r0[0] * r1[2], r0[0] * r1[1] - r0[1] * r1[0]};
   T c1[3] = {r0[1] * r2[2] - r0[2] * r2[1], r0[2] * r2[0] - r0[0] * r2[2], r0[0] * r2[1] - r0[1] * r2[0]};
   T c2[3] = {r1[1] * r2[2] - r1[2] * r2[1], r1[2] * r2[0] - r1[0] * r2[2], r1[0] * r2[1] - r1[1] * r2[0]};
@@ -439,10 +477,7 @@ __device__ void principal_dir(const T* q, T n[3]) {
     n[0] = T(1); n[1] = T(0); n[2] = T(0);
     return;
   }
-  T s;
-  // the FP32 estimate needs a normal FP32 argument (nn is a fourth power of Q's anisotropy)
-  if constexpr (sizeof(T) == 8) s = nn > 1e-30 && nn < 1e30 ? rsqrt_f64<2>(nn) : T(1) / sqrt(nn);
-  else s = T(1) / sqrt(nn);
+  const T s = T(1) / sqrt(nn);
   n[0] *= s; n[1] *= s; n[2] *= s;
 }
 
@@ -641,6 +676,72 @@ __device__ __forceinline__ void surface_q0_near(const DevBox& B, int c, int sx, 
   q0[2] = S0 * n[0] * n[2];
   q0[3] = S0 * (n[1] * n[1] - third);
   q0[4] = S0 * n[1] * n[2];
+}
+
+// w (Q0 - Q) for a homeotropic solid face in FP32 storage, in sums of two
+// floats (48 bits; every step below keeps the error of the FP32 operation
+// before it): n0 = d / |d| from the split position of the colloid, 1/|d| by one
+// corrected estimate, and the difference to Q = qh + ql rounded once at the
+// end, as the FP64 evaluation of surface_q0_near rounds it.  The FP64 one is
+// some 100 instructions of 64 cycles each for a lone warp, this one as many
+// FP32 instructions.
+__device__ __forceinline__ void surface_dn_normal(const DevBox& B, const DevColloid& C, const int s[3],
+                                                  const float qh[5], const float ql[5], float dn[5]) {
+  float dh[3], dl[3];
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
+    const int L = a == 0 ? B.nx : (a == 1 ? B.ny : B.nz);
+    // integer minus X: exact in the high part; the minimum image decided on both parts
+    float t = (float)s[a] - C.Xs[a][0];
+    const float xl = C.Xs[a][1];
+    if (a < 2 || !B.wall_z) {
+      const float h = 0.5f * (float)L;
+      if (t - h >= xl) t -= (float)L;
+      else if (t + h < xl) t += (float)L;
+    }
+    dh[a] = t - xl;
+    dl[a] = (t - dh[a]) - xl;
+  }
+  // |d|^2 = rh + rl
+  float ph[3], rl = 0.f;
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
+    ph[a] = dh[a] * dh[a];
+    rl += fmaf(dh[a], dh[a], -ph[a]) + 2.f * dh[a] * dl[a];
+  }
+  const float s01 = ph[0] + ph[1], b01 = s01 - ph[0];
+  rl += (ph[0] - (s01 - b01)) + (ph[1] - b01);
+  const float rh = s01 + ph[2], b2 = rh - s01;
+  rl += (s01 - (rh - b2)) + (ph[2] - b2);
+  // 1/|d| = r + rc
+  const float r = rsqrtf(rh), rr = r * r, re = fmaf(r, r, -rr);
+  const float eps = -(fmaf(rr, rh, -1.f) + fmaf(rr, rl, re * rh));
+  const float rc = 0.5f * r * eps;
+  float nh[3], nl[3];
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
+    const float p = dh[a] * r, e = fmaf(dh[a], r, -p) + fmaf(dh[a], rc, dl[a] * r);
+    nh[a] = p + e;
+    nl[a] = e - (nh[a] - p);
+  }
+  const float th = 1.f / 3.f, tl = -9.934107e-9f;  // 1/3 - th
+  const float S0h = B.pf.S0, S0l = B.pf.S0l, wh = C.ws[0], wl = C.ws[1];
+  const int ia[5] = {0, 0, 0, 1, 1}, ib[5] = {0, 1, 2, 1, 2};
+#pragma unroll
+  for (int k = 0; k < 5; ++k) {
+    const int a = ia[k], b = ib[k];
+    float ph2 = nh[a] * nh[b], pl = fmaf(nh[a], nh[b], -ph2) + fmaf(nh[a], nl[b], nl[a] * nh[b]);
+    if (a == b) {
+      const float t = ph2 - th, bb = t - ph2;
+      pl += ((ph2 - (t - bb)) + (-th - bb)) - tl;
+      ph2 = t;
+    }
+    // S0 (n n - delta/3) - qh - ql
+    const float q = S0h * ph2, qe = fmaf(S0h, ph2, -q) + fmaf(S0h, pl, S0l * ph2);
+    const float t = q - qh[k], bb = t - q;
+    const float D = t, E = ((q - (t - bb)) + (-qh[k] - bb)) + (qe - ql[k]);
+    dn[k] = fmaf(D, wh, fmaf(E, wh, D * wl));
+  }
 }
 
 // Derivatives from the face-neighbour values: twice the central first

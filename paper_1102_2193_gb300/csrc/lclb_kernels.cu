@@ -110,22 +110,50 @@ __device__ __forceinline__ void warp_residual(double* part, int wy, int lane, T 
   }
 }
 
-// Add per-lane contributions v[0..5] (for colloid id c, -1: none) into
+// Sums of NV values over the 32 lanes, eight at a time: each exchange halves
+// the values a lane carries, so a sum takes 9 FP64 additions per eight values
+// instead of 40 (an FP64 instruction occupies a warp for 64 cycles).  fn(k, sum)
+// is called once per value by one lane.  All lanes call it.
+template <int NV, typename Fn>
+__device__ __forceinline__ void warp_sums(const double* v, Fn fn) {
+  const int lane = threadIdx.x & 31;
+#pragma unroll
+  for (int k0 = 0; k0 < NV; k0 += 8) {
+    double t[8];
+#pragma unroll
+    for (int k = 0; k < 8; ++k) t[k] = k0 + k < NV ? v[k0 + k] : 0.0;
+#pragma unroll
+    for (int w = 4, o = 16; w >= 1; w >>= 1, o >>= 1) {
+      const bool up = (lane & o) != 0;
+#pragma unroll
+      for (int k = 0; k < w; ++k) {
+        const double give = up ? t[k] : t[k + w], keep = up ? t[k + w] : t[k];
+        t[k] = keep + __shfl_xor_sync(0xffffffffu, give, o);
+      }
+    }
+    t[0] += __shfl_xor_sync(0xffffffffu, t[0], 2);
+    t[0] += __shfl_xor_sync(0xffffffffu, t[0], 1);
+    const int k = k0 + (lane >> 2);
+    if ((lane & 3) == 0 && k < NV) fn(k, t[0]);
+  }
+}
+
+// Add per-lane contributions v[0..NV-1] (for colloid id c, -1: none) into
 // acc[off..off+NV-1] of each colloid with one FP64 atomic per (warp, colloid,
 // component).  Must be called by all 32 lanes of a converged warp.
 template <int NV = 6>
 __device__ __forceinline__ void warp_flush_colloid(DevColloid* col, int c, const double* v, int off) {
   unsigned pend = __ballot_sync(0xffffffffu, c >= 0);
-  const int lane = threadIdx.x & 31;
   while (pend) {
     const int leader = __ffs(pend) - 1;
     const int cc = __shfl_sync(0xffffffffu, c, leader);
     const bool mine = (c == cc);
+    double w[NV];
 #pragma unroll
-    for (int k = 0; k < NV; ++k) {
-      const double t = warp_sum(mine ? v[k] : 0.0);  // total lands in lane 0
-      if (lane == 0 && t != 0.0) atomicAdd(&col[cc].acc[off + k], t);
-    }
+    for (int k = 0; k < NV; ++k) w[k] = mine ? v[k] : 0.0;
+    warp_sums<NV>(w, [&](int k, double t) {
+      if (t != 0.0) atomicAdd(&col[cc].acc[off + k], t);
+    });
     if (mine) c = -1;
     pend = __ballot_sync(0xffffffffu, c >= 0);
   }
@@ -697,13 +725,18 @@ __device__ __noinline__ void near_stress(const DevBox& B, int i, int mode, NearS
 #pragma unroll
   for (int d = 0; d < 6; ++d)
     if (((solid >> d) & 1u) && nb[d] >= 0 && B.col[cf[d] - 1].anchoring != 0) planar = true;
-  double nf[3] = {1.0, 0.0, 0.0};
-  if (planar) {
-    double qid[5];
+  // Q in FP64 where a face evaluates its surface value in FP64: planar
+  // anchoring, walls, FP64 storage
+  const bool wall_face = B.wall_z && (((solid >> 4) & 1u && nb[4] < 0) || ((solid >> 5) & 1u && nb[5] < 0));
+  double nf[3] = {1.0, 0.0, 0.0}, qid[5];
+  if (!comp || planar || wall_face || max(nx, max(ny, B.nz)) >= (1 << 22)) {
 #pragma unroll
-    for (int k = 0; k < 5; ++k) qid[k] = (double)qh[k] + (double)ql[k];
-    principal_dir<double>(qid, nf);
+    for (int k = 0; k < 5; ++k) qid[k] = comp ? (double)qh[k] + (double)ql[k] : (double)qh[k];
+  } else {
+#pragma unroll
+    for (int k = 0; k < 5; ++k) qid[k] = 0.0;
   }
+  if (planar) principal_dir<double>(qid, nf);
   // queue of solid faces; slot[d]: position of this node's face d
   int slot[6], nface = 0;
 #pragma unroll
@@ -734,21 +767,32 @@ __device__ __noinline__ void near_stress(const DevBox& B, int i, int mode, NearS
     const int t = t0 + lane;
     int own, d, c, s[3];
     face_of(t, own, d, c, s);
-    double nfo[3], qo[5];
-    float lo[5];
+    // (node coordinates are exact in FP32 up to 2^24)
+    const bool normal = comp && c >= 0 && B.col[c].anchoring == 0 && max(nx, max(ny, B.nz)) < (1 << 22);
+    if constexpr (comp) {
+      if (__ballot_sync(full, t < nface && normal)) {
+        float ho[5], lo[5];
 #pragma unroll
-    for (int a = 0; a < 3; ++a) nfo[a] = __shfl_sync(full, nf[a], own);
-#pragma unroll
-    for (int k = 0; k < 5; ++k) {
-      qo[k] = (double)__shfl_sync(full, qh[k], own);
-      lo[k] = __shfl_sync(full, ql[k], own);
+        for (int k = 0; k < 5; ++k) {
+          ho[k] = __shfl_sync(full, qh[k], own);
+          lo[k] = __shfl_sync(full, ql[k], own);
+        }
+        if (t < nface && normal) surface_dn_normal(B, B.col[c], s, ho, lo, sc.dn[t]);
+      }
     }
-    if (t < nface) {
-      double q0[5];
-      surface_q0_near<T>(B, c, s[0], s[1], s[2], nfo, q0);
-      const double w = c < 0 ? 1.0 : B.col[c].wfac;
+    if (__ballot_sync(full, t < nface && !normal)) {
+      double nfo[3], qo[5];
 #pragma unroll
-      for (int k = 0; k < 5; ++k) sc.dn[t][k] = (T)(w * ((q0[k] - qo[k]) - (double)lo[k]));
+      for (int a = 0; a < 3; ++a) nfo[a] = __shfl_sync(full, nf[a], own);
+#pragma unroll
+      for (int k = 0; k < 5; ++k) qo[k] = __shfl_sync(full, qid[k], own);
+      if (t < nface && !normal) {
+        double q0[5];
+        surface_q0_near<T>(B, c, s[0], s[1], s[2], nfo, q0);
+        const double w = c < 0 ? 1.0 : B.col[c].wfac;
+#pragma unroll
+        for (int k = 0; k < 5; ++k) sc.dn[t][k] = (T)(w * (q0[k] - qo[k]));
+      }
     }
   }
   __syncwarp();
@@ -786,8 +830,6 @@ __device__ __noinline__ void near_stress(const DevBox& B, int i, int mode, NearS
     }
   }
   if (!(mode & FORCE_ACC)) return;
-  int my_c = -1;
-  double my_acc[6] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
   for (int t0 = 0; t0 < nface; t0 += 32) {
     const int t = t0 + lane;
     int own, d, c, s[3];
@@ -795,21 +837,35 @@ __device__ __noinline__ void near_stress(const DevBox& B, int i, int mode, NearS
     T po[9];
 #pragma unroll
     for (int k = 0; k < 9; ++k) po[k] = __shfl_sync(full, p[k], own);
+    double v[6] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
     if (t < nface && c >= 0) {
+      // the colloid takes -sgn P_{.,ax} of the fluid node (Eq. 8) at the face
+      // centre, half a step back from the solid node, with the moment about
+      // its centre (arm from the FP64 offset, taken in T)
       const int ax = d >> 1;
       const T sgn = (d & 1) ? T(-1) : T(1);
-      const T pcv[3] = {ax == 0 ? po[0] : (ax == 1 ? po[1] : po[2]), ax == 0 ? po[3] : (ax == 1 ? po[4] : po[5]),
-                        ax == 0 ? po[6] : (ax == 1 ? po[7] : po[8])};
-      // the fluid node: one step back from the solid node
+      const T ff[3] = {-sgn * (ax == 0 ? po[0] : (ax == 1 ? po[1] : po[2])),
+                       -sgn * (ax == 0 ? po[3] : (ax == 1 ? po[4] : po[5])),
+                       -sgn * (ax == 0 ? po[6] : (ax == 1 ? po[7] : po[8]))};
       const int back = (d & 1) ? 1 : -1;
-      s[0] = ax == 0 ? wrap1(s[0] + back, nx) : s[0];
-      s[1] = ax == 1 ? wrap1(s[1] + back, ny) : s[1];
-      s[2] = ax == 2 ? wrap1(s[2] + back, B.nz) : s[2];
-      colloid_face(B, c, ax, sgn, pcv, s[0], s[1], s[2], my_c, my_acc);
+      double fc[3], rd[3];
+#pragma unroll
+      for (int a = 0; a < 3; ++a) {
+        const int L = a == 0 ? nx : (a == 1 ? ny : B.nz);
+        fc[a] = (double)(ax == a ? wrap1(s[a] + back, L) : s[a]);
+        if (ax == a) fc[a] -= 0.5 * back;
+      }
+      disp(B, fc[0], fc[1], fc[2], B.col[c].X, rd);
+      const T r[3] = {T(rd[0]), T(rd[1]), T(rd[2])};
+#pragma unroll
+      for (int a = 0; a < 3; ++a) v[a] = (double)ff[a];
+      v[3] = (double)(r[1] * ff[2] - r[2] * ff[1]);
+      v[4] = (double)(r[2] * ff[0] - r[0] * ff[2]);
+      v[5] = (double)(r[0] * ff[1] - r[1] * ff[0]);
     }
+    __syncwarp();
+    warp_flush_colloid(B.col, t < nface ? c : -1, v, 6);
   }
-  __syncwarp();
-  warp_flush_colloid(B.col, my_c, my_acc, 6);
 }
 
 // Plain node, one per lane: own Q and that of the x- and z-neighbours from pq.
@@ -1835,12 +1891,11 @@ __device__ __forceinline__ void links_chunk(const DevBox& B, int l0, int n, doub
     const bool warp_main = __all_sync(0xffffffffu, main || my_c < 0);
     const bool warp_mob = __any_sync(0xffffffffu, mob);
     if (warp_main) {
-#pragma unroll
-      for (int k = 0; k < 18; ++k) {
-        if (k >= 6 && !warp_mob) break;
-        const double t = warp_sum(v[k]);
-        if ((tid & 31) == 0 && t != 0.0) atomicAdd(&sblk[k], t);
-      }
+      auto add = [&](int k, double t) {
+        if (t != 0.0) atomicAdd(&sblk[k], t);
+      };
+      if (warp_mob) warp_sums<18>(v, add);
+      else warp_sums<6>(v, add);
     } else {
       warp_flush_colloid<6>(B.col, my_c, v, 0);
       if (warp_mob) warp_flush_colloid<12>(B.col, mob ? my_c : -1, v + 6, 12);
@@ -2012,6 +2067,8 @@ __device__ __forceinline__ void colloid_box(const DevBox& B, bool commit = true)
       if (!(sqrt(r[0] * r[0] + r[1] * r[1] + r[2] * r[2]) + 1e-9 < C.margin)) s_scan = 1;
     }
     __syncthreads();
+    for (int c = tid; c < B.ncol; c += nthr)
+      if (B.col[c].mobile) split_position(B.col[c]);
     if (s_scan)
       for (int c = tid; c < B.ncol; c += nthr) {
         DevColloid& C = B.col[c];

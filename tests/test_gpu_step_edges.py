@@ -44,3 +44,21 @@ def test_step_edges(L, wall, col, prec, pitch, flow):
         F = np.abs(b["F_lc"]).max() + np.abs(b["F_hyd"]).max()
         tol = 1e-4 if prec == "f32" else 1e-9
         assert np.abs(a["F_lc"] - b["F_lc"]).max() <= tol * F and np.abs(a["F_hyd"] - b["F_hyd"]).max() <= tol * F
+
+
+@pytest.mark.parametrize("anchoring,w", [(0, 0.02), (0, float("inf")), (1, 0.03)])
+def test_surface_values_far_from_origin(anchoring, w):
+    """FP32 surface values of colloids at positions that FP32 does not hold (the normal ones are summed in pairs of
+    FP32 numbers) and across the periodic boundary: the colloid's LC force and torque after one step."""
+    import paper_1102_2193_gb300 as P
+    L, X, a0 = (130, 40, 34), (128.7, 39.2, 0.4), 9.3
+    prm = dict(synth.NEMATIC, q0=2 * np.pi / 17)
+    s, o = P.Solver(*L, precision=P.LC_FP32, **prm), oracle.Oracle(*L, **prm)
+    q = synth.random_q((L[2], L[1], L[0]), 9, amp=0.05, base=(0.2, 0.05, 0.02, -0.1, 0.03))
+    for k in (s, o):
+        k.set_Q(q)
+        k.add_colloid(X, a0, anchoring, w)
+        k.step(1)
+    a, b = s.colloid(0), o.colloid(0)
+    assert np.abs(a["F_lc"] - b["F_lc"]).max() <= 2e-5 * np.abs(b["F_lc"]).max()
+    assert np.abs(a["T_lc"] - b["T_lc"]).max() <= 1e-4 * a0 * np.abs(b["F_lc"]).max()
