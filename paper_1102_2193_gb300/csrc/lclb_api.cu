@@ -149,8 +149,11 @@ struct Group {
   double* h_red = nullptr;      // pinned
   int* d_iwork = nullptr;       // link-build block sums
   size_t iwork_cap = 0;
+  // the captured step, and GRAPH_STEPS steps in one graph (built once a handle
+  // has stepped GRAPH_AFTER times)
   cudaGraph_t graph = nullptr;
-  cudaGraphExec_t gexec = nullptr;
+  cudaGraphExec_t gexec = nullptr, gexec_many = nullptr;
+  long long stepped = 0;
   bool dirty = true, tuned = false;
   bool frozen = false;    // every box has its flow frozen: a step is k_relax alone (except the dataflow variant)
   int graph_kernels = 0;  // kernel nodes of the captured step
@@ -346,15 +349,11 @@ int build_totals(Group* g) {
 // exact capacity, boxes with a mobile colloid a bound over its motion (near
 // nodes lie within sqrt 2 of the surface; a shell's nodes are at most the
 // volume of the shell widened by half a cell diagonal).
-int build_near(lc_lb* h) {
+// n: the near nodes that launch_near_list has counted.
+int build_near(lc_lb* h, int n) {
   Group* g = h->g;
   DevBox& B = h->hb;
   cudaStream_t s = g->stream;
-  int n = 0;
-  CK(cudaMemsetAsync(B.nnear, 0, sizeof(int), s), &h->err);
-  CK(launch_near_list(g->d_boxes, h->index, B.N, s), &h->err);
-  CK(cudaMemcpyAsync(&n, B.nnear, sizeof(int), cudaMemcpyDeviceToHost, s), &h->err);
-  CK(cudaStreamSynchronize(s), &h->err);
   double bound = n;
   if (B.nmobile > 0) {
     double m = B.wall_z ? 2.0 * B.nx * B.ny : 0.0;
@@ -552,11 +551,18 @@ Group* new_group(int prec, void* stream, int nboxes, std::string* err) {
   return g;
 }
 
+void drop_graphs(Group* g) {
+  if (g->gexec) cudaGraphExecDestroy(g->gexec);
+  if (g->gexec_many) cudaGraphExecDestroy(g->gexec_many);
+  if (g->graph) cudaGraphDestroy(g->graph);
+  g->gexec = g->gexec_many = nullptr;
+  g->graph = nullptr;
+}
+
 void free_group(Group* g) {
   if (!g) return;
   cudaStreamSynchronize(g->stream);
-  if (g->gexec) cudaGraphExecDestroy(g->gexec);
-  if (g->graph) cudaGraphDestroy(g->graph);
+  drop_graphs(g);
   g->mem.release(g->al);
   if (g->h_red) cudaFreeHost(g->h_red);
   if (g->side2) {
@@ -1228,19 +1234,16 @@ int build_mobile(Group* g) {
   return LC_OK;
 }
 
-int capture(Group* g) {
-  if (!g->dirty && g->gexec) return LC_OK;
-  if (g->gexec) {
-    cudaGraphExecDestroy(g->gexec);
-    g->gexec = nullptr;
-  }
-  if (g->graph) {
-    cudaGraphDestroy(g->graph);
-    g->graph = nullptr;
-  }
-  if (int rc = g->variant == 3 ? build_items(g) : build_totals(g)) return rc;
+// Steps per launch of the second graph: one graph launch, and the gap before
+// its first kernel, per eight steps (two colloids in 37 x 29 x 23: 43 -> 39 us a
+// step, 96^3 relaxation 28.7 -> 26.3).  Capturing it takes 0.1 ms, so a handle
+// that is stepped only a few times does without.
+constexpr int GRAPH_STEPS = 8, GRAPH_AFTER = 64;
+
+int capture_steps(Group* g, int steps, cudaGraph_t* out) {
   CK(cudaStreamBeginCapture(g->stream, cudaStreamCaptureModeThreadLocal), &g->err);
-  int rc = enqueue_step(g);
+  int rc = LC_OK;
+  for (int s = 0; s < steps && !rc; ++s) rc = enqueue_step(g);
   cudaGraph_t gr = nullptr;
   cudaError_t e = cudaStreamEndCapture(g->stream, &gr);
   if (rc) {
@@ -1248,6 +1251,26 @@ int capture(Group* g) {
     return rc;
   }
   CK(e, &g->err);
+  *out = gr;
+  return LC_OK;
+}
+
+int capture_many(Group* g) {
+  if (g->gexec_many) return LC_OK;
+  cudaGraph_t gr = nullptr;
+  if (int rc = capture_steps(g, GRAPH_STEPS, &gr)) return rc;
+  const cudaError_t e = cudaGraphInstantiate(&g->gexec_many, gr, 0);
+  cudaGraphDestroy(gr);
+  CK(e, &g->err);
+  return LC_OK;
+}
+
+int capture(Group* g) {
+  if (!g->dirty && g->gexec) return LC_OK;
+  drop_graphs(g);
+  if (int rc = g->variant == 3 ? build_items(g) : build_totals(g)) return rc;
+  cudaGraph_t gr = nullptr;
+  if (int rc = capture_steps(g, 1, &gr)) return rc;
   g->graph = gr;
   CK(cudaGraphInstantiate(&g->gexec, gr, 0), &g->err);
   size_t nn = 0;
@@ -1342,10 +1365,7 @@ int group_step(Group* g, int n) {
   if (env && env[0] == '1') {
     if (g->dirty) {
       if ((rc = g->variant == 3 ? build_items(g) : build_totals(g))) return rc;
-      if (g->gexec) {  // the graph of the old work lists
-        cudaGraphExecDestroy(g->gexec);
-        g->gexec = nullptr;
-      }
+      drop_graphs(g);  // of the old work lists
       g->dirty = false;
     }
     for (int s = 0; s < n; ++s)
@@ -1353,7 +1373,13 @@ int group_step(Group* g, int n) {
     return LC_OK;
   }
   if ((rc = capture(g))) return rc;
-  for (int s = 0; s < n; ++s) CK(cudaGraphLaunch(g->gexec, g->stream), &g->err);
+  int s = 0;
+  if (n >= GRAPH_STEPS && g->stepped + n >= GRAPH_AFTER) {
+    if ((rc = capture_many(g))) return rc;
+    for (; s + GRAPH_STEPS <= n; s += GRAPH_STEPS) CK(cudaGraphLaunch(g->gexec_many, g->stream), &g->err);
+  }
+  for (; s < n; ++s) CK(cudaGraphLaunch(g->gexec, g->stream), &g->err);
+  g->stepped += n;
   return LC_OK;
 }
 
@@ -1397,11 +1423,16 @@ int rebuild_geometry(lc_lb* h) {
   int rc = upload_box(g, h);
   if (rc) return rc;
   CK(launch_geometry(g->d_boxes, h->index, h->hb.N, s), &h->err);
-  if ((rc = build_near(h))) return rc;
-  // boundary links, colloid by colloid, in node order
+  // near nodes; boundary links, colloid by colloid, in node order
   const int nb = (h->hb.N + 255) / 256;
   if ((rc = ensure_iwork(g, (size_t)nb + 8))) return rc;
-  int total = 0;
+  int total = 0, nnear = 0;
+  CK(cudaMemsetAsync(h->hb.nnear, 0, sizeof(int), s), &h->err);
+  if (!h->col.empty() || h->hb.wall_z) {
+    CK(launch_near_list(g->d_boxes, h->index, h->hb.N, s), &h->err);
+    CK(cudaMemcpyAsync(&nnear, h->hb.nnear, sizeof(int), cudaMemcpyDeviceToHost, s), &h->err);
+    if (h->col.empty()) CK(cudaStreamSynchronize(s), &h->err);  // else the link counts below wait
+  }
   std::vector<int> counts(h->col.size());
   for (size_t c = 0; c < h->col.size(); ++c) {
     CK(launch_link_build(g->d_boxes, h->index, h->hb.N, (int)c, g->d_iwork, total, g->d_iwork + nb, s), &h->err);
@@ -1410,6 +1441,7 @@ int rebuild_geometry(lc_lb* h) {
     CK(cudaStreamSynchronize(s), &h->err);
     total = t;
   }
+  if ((rc = build_near(h, nnear))) return rc;
   if (total > h->hb.nlinks_cap) {
     if (h->hb.link_node) {
       g->mem.put(h->hb.link_node, g->al);

@@ -334,6 +334,61 @@ __global__ void __launch_bounds__(288) k_wgrad_tile(const __nv_bfloat16* __restr
       }
 }
 
+// Partial dW of the 1x1x1 kernel: block (chunk, 16 output x 16 input channels)
+// takes its chunk 512 positions at a time through shared memory, as
+// k_wgrad_tile without taps: eight warps take every eighth group of 16
+// positions, and their sums are added in warp order (k_conv_wgrad, with its
+// 2-byte loads, 105 us for 16 x 16 channels at 64^3).
+__global__ void __launch_bounds__(256) k_wgrad_1(const __nv_bfloat16* __restrict__ dout,
+                                                 const __nv_bfloat16* __restrict__ in, float* __restrict__ part,
+                                                 int npos, int cin, int cout, int chunk) {
+  constexpr int NP = 512;
+  __shared__ __align__(128) unsigned char buf[2 * NP * 32];
+  const uint32_t sI = smem_addr(buf), sD = sI + NP * 32;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int nci = cin / 16, co0 = (blockIdx.y / nci) * 16, ci0 = (blockIdx.y % nci) * 16;
+  const int pend = min(npos, (int)(blockIdx.x + 1) * chunk);
+  const int ar = ((lane >> 4) & 1) * 8 + (lane & 7), ah = (lane >> 3) & 1;
+  const int br = ((lane >> 3) & 1) * 8 + (lane & 7), bh = lane >> 4;
+  float acc[2][4] = {{0.f, 0.f, 0.f, 0.f}, {0.f, 0.f, 0.f, 0.f}};
+  for (int p0 = blockIdx.x * chunk; p0 < pend; p0 += NP) {
+    __syncthreads();
+    for (int m = tid; m < NP; m += 256) {
+      const int p = p0 + m;
+      if (p < pend) {
+        cp16(sI + row32(m, 0), in + (size_t)p * cin + ci0);
+        cp16(sI + row32(m, 1), in + (size_t)p * cin + ci0 + 8);
+        cp16(sD + row32(m, 0), dout + (size_t)p * cout + co0);
+        cp16(sD + row32(m, 1), dout + (size_t)p * cout + co0 + 8);
+      } else {
+        uint4* a = reinterpret_cast<uint4*>(buf + m * 32);
+        uint4* b = reinterpret_cast<uint4*>(buf + NP * 32 + m * 32);
+        a[0] = a[1] = b[0] = b[1] = make_uint4(0u, 0u, 0u, 0u);
+      }
+    }
+    cp_wait_all();
+    __syncthreads();
+    for (int g = warp; g < NP / 16; g += 8) {
+      uint32_t a[4], b[4];
+      ldm4t(a, sD + row32(g * 16 + ar, ah));
+      ldm4t(b, sI + row32(g * 16 + br, bh));
+      mma_bf16(acc[0], a, b);
+      mma_bf16(acc[1], a, b + 2);
+    }
+  }
+  __syncthreads();
+  float* red = reinterpret_cast<float*>(buf);  // [warp][16 co][16 ci]
+  const int g = lane >> 2, tg = lane & 3;
+#pragma unroll
+  for (int j = 0; j < 2; ++j)
+#pragma unroll
+    for (int k = 0; k < 4; ++k) red[warp * 256 + (g + (k >> 1) * 8) * 16 + j * 8 + tg * 2 + (k & 1)] = acc[j][k];
+  __syncthreads();
+  float v = 0.f;
+  for (int w = 0; w < 8; ++w) v += red[w * 256 + tid];
+  part[(size_t)blockIdx.x * cout * cin + (size_t)(co0 + tid / 16) * cin + ci0 + tid % 16] = v;
+}
+
 // Partial dW[co][t][ci] = sum_p dout[p][co] in[tap(p, t)][ci] over one chunk
 // of positions, stored for the chunk (part[chunk][co][t][ci]); one warp per
 // (chunk, tap, 16 output channels).  A = dout^T (16 C_out x 16 positions),
@@ -413,42 +468,59 @@ __global__ void k_flip_weights(const __nv_bfloat16* __restrict__ w, __nv_bfloat1
   wt[((size_t)ci * taps + (taps - 1 - t)) * cout + co] = w[i];
 }
 
-// db[ch] += sum_p dout[p][ch]: a cluster of eight blocks takes up to 16
-// channels; a thread adds every position of its residue class for its channel
-// (coalesced rows), the block sums go through distributed shared memory and
-// are added in block order, so the result is the same on every run.  One
-// block per channel, striding over whole rows, read each line c times from
-// too few SMs (16 channels at 64^3: 223 us).
-constexpr int BIAS_CLUSTER = 8, BIAS_THREADS = 512;
-__global__ void __cluster_dims__(BIAS_CLUSTER, 1, 1) __launch_bounds__(BIAS_THREADS)
-    k_bias_grad(const float* __restrict__ dout, float* __restrict__ db, int npos, int c) {
-  __shared__ float s[BIAS_THREADS];
+// db[ch] += sum_p dout[p][ch]: a cluster of 16 blocks takes up to 16 channels;
+// a thread adds the positions of its residue class for its V channels (rows of
+// 16 bytes, eight in flight per thread: 64 KB per SM cover the latency of the
+// memory), the block sums go through distributed shared memory and are added
+// in block order, so the result is the same on every run.  16 channels at 64^3:
+// one block per channel 223 us, clusters of 8 with 4-byte loads 80 us.
+constexpr int BIAS_CLUSTER = 16, BIAS_THREADS = 512;
+template <int V>
+__global__ void __launch_bounds__(BIAS_THREADS) k_bias_grad(const float* __restrict__ dout, float* __restrict__ db,
+                                                            int npos, int c) {
+  constexpr int COLS = 16 / V, ROWS = BIAS_THREADS / COLS, UNROLL = 8;
+  __shared__ float s[ROWS][17];
   __shared__ float tot[16];
   const int tid = threadIdx.x, rank = blockIdx.x % BIAS_CLUSTER, c0 = (blockIdx.x / BIAS_CLUSTER) * 16;
-  const int ch = tid & 15, row = tid >> 4;
-  constexpr int ROWS = BIAS_THREADS / 16;
-  float v[4] = {0.f, 0.f, 0.f, 0.f};
-  if (c0 + ch < c) {
+  const int col = (tid % COLS) * V, row = tid / COLS;
+  float v[V];
+#pragma unroll
+  for (int j = 0; j < V; ++j) v[j] = 0.f;
+  if (c0 + col < c) {
     const size_t step = (size_t)ROWS * BIAS_CLUSTER;
     size_t p = (size_t)rank * ROWS + row;
-    for (; p + 3 * step < (size_t)npos; p += 4 * step)
+    const float* src = dout + c0 + col;
+    for (; p + (UNROLL - 1) * step < (size_t)npos; p += UNROLL * step) {
+      float t[UNROLL][V];
 #pragma unroll
-      for (int k = 0; k < 4; ++k) v[k] += dout[(p + k * step) * c + c0 + ch];
-    for (; p < (size_t)npos; p += step) v[0] += dout[p * c + c0 + ch];
+      for (int k = 0; k < UNROLL; ++k) {
+        if constexpr (V == 4) *reinterpret_cast<float4*>(t[k]) = *reinterpret_cast<const float4*>(src + (p + k * step) * c);
+        else t[k][0] = src[(p + k * step) * c];
+      }
+#pragma unroll
+      for (int k = 0; k < UNROLL; ++k)
+#pragma unroll
+        for (int j = 0; j < V; ++j) v[j] += t[k][j];
+    }
+    for (; p < (size_t)npos; p += step)
+#pragma unroll
+      for (int j = 0; j < V; ++j) v[j] += src[p * c + j];
   }
-  s[tid] = (v[0] + v[1]) + (v[2] + v[3]);
+#pragma unroll
+  for (int j = 0; j < V; ++j) s[row][col + j] = v[j];
   __syncthreads();
-  for (int d = ROWS / 2; d > 0; d >>= 1) {
-    if (row < d) s[tid] += s[tid + d * 16];
-    __syncthreads();
-  }
-  if (tid < 16) tot[tid] = s[tid];
+  // 32 threads per channel add the rows in a fixed tree
+  const int ch = tid >> 5, lane = tid & 31;
+  float t = 0.f;
+  for (int r = lane; r < ROWS; r += 32) t += s[r][ch];
+  for (int o = 16; o > 0; o >>= 1) t += __shfl_down_sync(0xffffffffu, t, o);
+  if (lane == 0) tot[ch] = t;
   cooperative_groups::cluster_group cl = cooperative_groups::this_cluster();
   cl.sync();
   if (rank == 0 && tid < 16 && c0 + tid < c) {
-    float t = 0.f;
-    for (int r = 0; r < BIAS_CLUSTER; ++r) t += cl.map_shared_rank(tot, r)[tid];
-    db[c0 + tid] += t;
+    float u = 0.f;
+    for (int r = 0; r < BIAS_CLUSTER; ++r) u += cl.map_shared_rank(tot, r)[tid];
+    db[c0 + tid] += u;
   }
   cl.sync();
 }
@@ -469,19 +541,43 @@ __global__ void k_cast_bf16(const float* __restrict__ a, __nv_bfloat16* __restri
 }
 
 // 2x2x2 mean pooling (channels last) and its adjoint.
+template <int VEC>
 __global__ void k_pool2(const __nv_bfloat16* __restrict__ in, __nv_bfloat16* __restrict__ out, int S, int c) {
-  const int So = S / 2;
-  const size_t n = (size_t)So * So * So * c;
+  const int So = S / 2, cv = c / VEC;
+  const size_t n = (size_t)So * So * So * cv;
   for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
-    const int ch = (int)(i % c);
-    const size_t p = i / c;
-    const int x = (int)(p % So), y = (int)((p / So) % So), z = (int)(p / ((size_t)So * So));
-    float s = 0.f;
+    const unsigned p = n >> 32 ? (unsigned)(i / (unsigned)cv) : (unsigned)i / (unsigned)cv;
+    const int ch = (int)(i - (size_t)p * cv) * VEC;
+    const int x = p % So, y = (p / So) % So, z = p / ((unsigned)So * So);
+    float s[VEC];
+#pragma unroll
+    for (int j = 0; j < VEC; ++j) s[j] = 0.f;
+#pragma unroll
     for (int k = 0; k < 8; ++k) {
       const int xx = 2 * x + (k & 1), yy = 2 * y + ((k >> 1) & 1), zz = 2 * z + (k >> 2);
-      s += __bfloat162float(in[((size_t)xx + (size_t)S * (yy + (size_t)S * zz)) * c + ch]);
+      const __nv_bfloat16* src = in + ((size_t)xx + (size_t)S * (yy + (size_t)S * zz)) * c + ch;
+      if constexpr (VEC == 8) {
+        const uint4 q = *reinterpret_cast<const uint4*>(src);
+        const __nv_bfloat162* h = reinterpret_cast<const __nv_bfloat162*>(&q);
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          const float2 f = __bfloat1622float2(h[j]);
+          s[2 * j] += f.x;
+          s[2 * j + 1] += f.y;
+        }
+      } else {
+        s[0] += __bfloat162float(src[0]);
+      }
     }
-    out[i] = __float2bfloat16_rn(0.125f * s);
+    if constexpr (VEC == 8) {
+      uint4 q;
+      __nv_bfloat162* h = reinterpret_cast<__nv_bfloat162*>(&q);
+#pragma unroll
+      for (int j = 0; j < 4; ++j) h[j] = __floats2bfloat162_rn(0.125f * s[2 * j], 0.125f * s[2 * j + 1]);
+      reinterpret_cast<uint4*>(out)[i] = q;
+    } else {
+      out[i] = __float2bfloat16_rn(0.125f * s[0]);
+    }
   }
 }
 
@@ -644,8 +740,12 @@ __global__ void k_pack_input(const double* __restrict__ solid, const double* __r
                              double* __restrict__ nfluid, int npos, int cpad, bool vec) {
   int cnt = 0;
   for (int p = blockIdx.x * blockDim.x + threadIdx.x; p < npos; p += gridDim.x * blockDim.x) {
-    cnt += solid[p] < 0.0;
-    const bool sol = solid[p] >= 0.0;
+    // solid < 0, >= 0 by the bits (an FP64 comparison is a slot of the FP64 pipe;
+    // NaN is neither)
+    const long long sb = __double_as_longlong(solid[p]);
+    const bool nan = (sb & 0x7fffffffffffffffll) > 0x7ff0000000000000ll, zero = (sb << 1) == 0;
+    cnt += !nan && !zero && sb < 0;
+    const bool sol = !nan && (zero || sb > 0);
     float v[9] = {sol ? 1.f : 0.f, 0, 0, 0, 0, 0, r / 32.f, pitch / 64.f, 20.f * w};
     for (int c = 0; c < 5; ++c) {
       v[1 + c] = (float)q[(size_t)c * npos + p];
@@ -755,6 +855,22 @@ static int conv_tiled(const __nv_bfloat16* in, const __nv_bfloat16* w, const flo
   return launch_conv_tile<2, 2, 4, 8, 4, 4>(in, w, bias, out32, out16, W, H, D, cin, cout, relu, s);
 }
 
+static int launch_bias_grad(const float* dout, float* db, int npos, int c, cudaStream_t s) {
+  auto* fn = c % 4 == 0 && aligned16(dout) ? k_bias_grad<4> : k_bias_grad<1>;
+  if (cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) return LC_NN_ERR_CUDA;
+  cudaLaunchConfig_t cfg{};
+  cudaLaunchAttribute at{};
+  cfg.gridDim = dim3((c + 15) / 16 * BIAS_CLUSTER);
+  cfg.blockDim = dim3(BIAS_THREADS);
+  cfg.stream = s;
+  at.id = cudaLaunchAttributeClusterDimension;
+  at.val.clusterDim.x = BIAS_CLUSTER;
+  at.val.clusterDim.y = at.val.clusterDim.z = 1;
+  cfg.attrs = &at;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, fn, dout, db, npos, c) == cudaSuccess ? LC_NN_OK : LC_NN_ERR_CUDA;
+}
+
 template <int TPW, int TY, int TZ>
 static int launch_wgrad_tile(const __nv_bfloat16* dout, const __nv_bfloat16* in, float* part, int W, int H, int D,
                              int cin, int cout, int nchunk, cudaStream_t s) {
@@ -847,6 +963,11 @@ int lc_nn_conv3d_wgrad(const void* dout, const void* in, float* dw, float* parti
     k_wgrad_sum<<<sgrid, sblk, 0, s>>>(partial, dw, nchunk, nw);
     return cudaGetLastError() == cudaSuccess ? LC_NN_OK : LC_NN_ERR_CUDA;
   }
+  if (taps == 1 && cin % 16 == 0 && aligned16(dout) && aligned16(in)) {
+    k_wgrad_1<<<dim3(nchunk, (cout / 16) * (cin / 16)), 256, 0, s>>>(a, b, partial, npos, cin, cout, chunk);
+    k_wgrad_sum<<<sgrid, sblk, 0, s>>>(partial, dw, nchunk, nw);
+    return cudaGetLastError() == cudaSuccess ? LC_NN_OK : LC_NN_ERR_CUDA;
+  }
   switch (cin / 8) {
     case 1: k_conv_wgrad<1><<<grid, 32, 0, s>>>(a, b, partial, npos, W, H, D, cin, cout, taps, chunk); break;
     case 2: k_conv_wgrad<2><<<grid, 32, 0, s>>>(a, b, partial, npos, W, H, D, cin, cout, taps, chunk); break;
@@ -860,8 +981,7 @@ int lc_nn_conv3d_wgrad(const void* dout, const void* in, float* dw, float* parti
 }
 
 int lc_nn_bias_grad(const float* dout, float* db, int npos, int c, void* stream) {
-  k_bias_grad<<<(c + 15) / 16 * BIAS_CLUSTER, BIAS_THREADS, 0, (cudaStream_t)stream>>>(dout, db, npos, c);
-  return cudaGetLastError() == cudaSuccess ? LC_NN_OK : LC_NN_ERR_CUDA;
+  return launch_bias_grad(dout, db, npos, c, (cudaStream_t)stream);
 }
 
 int lc_nn_relu_bwd(const float* dy, const void* y, float* dz32, void* dz16, size_t n, void* stream) {
@@ -876,8 +996,11 @@ int lc_nn_cast_bf16(const float* a, void* b, size_t n, void* stream) {
 
 int lc_nn_pool2(const void* in, void* out, int S, int c, void* stream) {
   if (S % 2) return LC_NN_ERR_ARG;
-  k_pool2<<<grid_for((size_t)S * S * S * c / 8), 256, 0, (cudaStream_t)stream>>>((const __nv_bfloat16*)in,
-                                                                                   (__nv_bfloat16*)out, S, c);
+  const size_t n = (size_t)(S / 2) * (S / 2) * (S / 2) * c;
+  if (c % 8 == 0 && aligned16(in) && aligned16(out))
+    k_pool2<8><<<grid_for(n / 8), 256, 0, (cudaStream_t)stream>>>((const __nv_bfloat16*)in, (__nv_bfloat16*)out, S, c);
+  else
+    k_pool2<1><<<grid_for(n), 256, 0, (cudaStream_t)stream>>>((const __nv_bfloat16*)in, (__nv_bfloat16*)out, S, c);
   return cudaGetLastError() == cudaSuccess ? LC_NN_OK : LC_NN_ERR_CUDA;
 }
 
