@@ -205,7 +205,8 @@ int lc_lb_get_links(lc_lb* h, int32_t* node, int8_t* dir, int16_t* colloid, size
  * *n_defect and *n_comp receive the totals (either may be NULL).  Labels
  * and counts are exact; the FP64 sums are accumulated in an unspecified
  * order.  Device memory: 3 N + N/256 + 2 ints kept by the handle, plus
- * 64 bytes per component during the call.  Synchronises the stream.
+ * 136 bytes per component and 16 per lattice line (nx + ny + nz) during the
+ * call.  Synchronises the stream.
  * LC_ERR_ARG for a threshold that is not positive and finite;
  * LC_ERR_TIMEOUT if a bounded device loop gave up (not expected). */
 int lc_lb_defects(lc_lb* h, double thr, size_t cap, long long* n_defect, long long* n_comp, long long* root,

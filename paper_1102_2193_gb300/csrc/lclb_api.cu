@@ -115,7 +115,7 @@ struct Group {
   int2* d_groups = nullptr;      // near-node groups (box, first entry), a multiple of NEAR_PAD per box
   int ngroups = 0, group_cap = 0;
   std::vector<int> gstart, gcount;  // groups of each box
-  double* d_npart = nullptr;     // residual record of each group
+  double* d_npart = nullptr;     // residual record of each group (2), then free energies (1)
   unsigned* d_done = nullptr;    // finished work units per box of k_lc, then the totals
   unsigned* d_total = nullptr;
   // Step variant: 0 = fused stress/force/LB kernel; 1 = split: the stress/
@@ -257,6 +257,7 @@ Launch phase_launch(Group* g, int k, int mode, int box = -1) {
   }
   L.groups = g->d_groups + (box < 0 || !has_groups(k) ? 0 : g->gstart[box]);
   L.npart = g->d_npart;
+  L.fepart = g->d_npart + 2 * (size_t)g->group_cap;
   L.chunks = g->d_lchunks;
   L.nchunks = g->nlchunks;
   L.done = g->d_done;
@@ -307,7 +308,7 @@ int build_groups(Group* g) {
     if (g->d_npart) g->mem.put(g->d_npart, g->al);
     g->group_cap = (int)gr.size() + 64;
     g->d_groups = (int2*)galloc(g, sizeof(int2) * g->group_cap);
-    g->d_npart = (double*)galloc(g, sizeof(double) * 2 * g->group_cap);
+    g->d_npart = (double*)galloc(g, sizeof(double) * 3 * g->group_cap);
     if (!g->d_groups || !g->d_npart) return fail(&g->err, LC_ERR_OOM, "near group allocation failed");
     CK(cudaMemsetAsync(g->d_npart, 0, sizeof(double) * 2 * g->group_cap, g->stream), &g->err);
   }
@@ -1866,15 +1867,17 @@ int lc_lb_defects(lc_lb* h, double thr, size_t cap, long long* n_defect, long lo
   std::vector<double> hc((size_t)3 * nc), hg((size_t)6 * nc);
   if (nc > 0) {
     const size_t ib = ((sizeof(int) * (size_t)nc + 15) / 16) * 16;
-    char* tmp = (char*)galloc(g, ib + sizeof(double) * 15 * (size_t)nc);
+    const int sides = h->hb.nx + h->hb.ny + h->hb.nz;
+    char* tmp = (char*)galloc(g, ib + sizeof(double) * (15 * (size_t)nc + 2 * (size_t)sides));
     if (!tmp) return fail(&h->err, LC_ERR_OOM, "defect statistics allocation failed");
     int* dsz = (int*)tmp;
     double* circ = (double*)(tmp + ib);
     double* cen = circ + 6 * (size_t)nc;
     double* gyr = cen + 3 * (size_t)nc;
+    double* trig = gyr + 6 * (size_t)nc;
     int rc = LC_OK;
     if (cudaMemsetAsync(tmp, 0, ib + sizeof(double) * 15 * (size_t)nc, g->stream) != cudaSuccess ||
-        launch_defects_stats(g->d_boxes, h->index, N, h->hb.nx + h->hb.ny + h->hb.nz, nc, h->def, h->def + N, dsz, circ, cen, gyr, g->stream) !=
+        launch_defects_stats(g->d_boxes, h->index, N, sides, nc, h->def, h->def + N, dsz, circ, cen, gyr, trig, g->stream) !=
             cudaSuccess ||
         cudaMemcpyAsync(hl.data(), h->def + 2 * (size_t)N, sizeof(int) * nc, cudaMemcpyDeviceToHost, g->stream) !=
             cudaSuccess ||
@@ -1928,12 +1931,14 @@ int lc_lb_diagnostics(lc_lb* h, lc_diag* out) {
   out->mass = (double)nf * h->hb.p.rho0 + sums[0];
   for (int a = 0; a < 3; ++a) out->momentum[a] = sums[1 + a];
   if (h->hb.p.lc_on) {
-    CK(launch_phase(g, 0, FORCE_FE, h->index), &h->err);
-    Phase& P = g->ph[0];
+    CK(launch_phase(g, 4, FORCE_FE, h->index), &h->err);
+    Phase& P = g->ph[4];
+    const int nblk = g->gcount[h->index] / P.cfg.ty;
     CK(launch_reduce(P.d_part, P.start[h->index], P.count[h->index], 1, 0u, g->d_red, g->stream), &h->err);
-    CK(cudaMemcpyAsync(g->h_red, g->d_red, sizeof(double), cudaMemcpyDeviceToHost, g->stream), &h->err);
+    CK(launch_reduce(g->d_npart + 2 * (size_t)g->group_cap, 0, nblk, 1, 0u, g->d_red + 1, g->stream), &h->err);
+    CK(cudaMemcpyAsync(g->h_red, g->d_red, 2 * sizeof(double), cudaMemcpyDeviceToHost, g->stream), &h->err);
     CK(cudaStreamSynchronize(g->stream), &h->err);
-    out->free_energy = g->h_red[0];
+    out->free_energy = g->h_red[0] + (nblk > 0 ? g->h_red[1] : 0.0);
     double rms = 0, mx = 0;
     if ((rc = box_residual(g, h->index, &rms, &mx, nf))) return rc;
     out->resid_rms = rms;

@@ -185,19 +185,33 @@ __global__ void __launch_bounds__(256) k_def_rank(int N, const int* __restrict__
 // threads meet first is summed in registers and added with one atomic per
 // value at the end; nodes of other components add directly.  The values
 // depend on one coordinate each (PASS 2: for one component), so the block
-// tabulates them per axis in shared memory (table; boxes whose tables do not
-// fit evaluate them per node).  With one FP64 atomic per node and value, a
+// keeps them per axis in shared memory (table; boxes whose tables do not fit
+// read them from global memory, or evaluate them per node).  With one FP64 atomic per node and value, a
 // loop of 10^5 nodes serialised on six addresses (1.69 and 1.45 ms at 128^3).
 __device__ __forceinline__ double def_disp(double x, double cen, double L, bool periodic) {
   const double d = x - cen;
   return periodic ? d - L * floor(d / L + 0.5) : d;
 }
 
+// cos, sin of 2 pi x / L for every coordinate of the three axes (in FP64, some
+// 200 instructions each: once per call, not once per block).
+__global__ void k_def_trig(const DevBox* __restrict__ boxes, int b, double* __restrict__ trig) {
+  const DevBox& B = boxes[b];
+  const int k = blockIdx.x * blockDim.x + threadIdx.x;
+  if (k >= B.nx + B.ny + B.nz) return;
+  const int a = k < B.nx ? 0 : (k < B.nx + B.ny ? 1 : 2);
+  const int L[3] = {B.nx, B.ny, B.nz}, at[3] = {0, B.nx, B.nx + B.ny};
+  const double th = DEF_TWO_PI * (double)(k - at[a]) / (double)L[a];
+  trig[2 * k] = cos(th);
+  trig[2 * k + 1] = sin(th);
+}
+
 template <int PASS>
 __global__ void __launch_bounds__(256) k_def_sum(const DevBox* __restrict__ boxes, int b,
                                                  const int* __restrict__ parent, const int* __restrict__ comp,
                                                  const double* __restrict__ cen, int* __restrict__ size,
-                                                 double* __restrict__ out, int per, int table) {
+                                                 double* __restrict__ out, const double* __restrict__ trig, int per,
+                                                 int table) {
   extern __shared__ double tab[];  // PASS 1: cos, sin per coordinate; PASS 2: displacement per coordinate
   __shared__ long long s_key[8];
   __shared__ double s_sum[8][7];
@@ -223,9 +237,8 @@ __global__ void __launch_bounds__(256) k_def_sum(const DevBox* __restrict__ boxe
       const int a = k < nx ? 0 : (k < nx + ny ? 1 : 2);
       const double x = (double)(k - at[a]);
       if (PASS == 1) {
-        const double th = DEF_TWO_PI * x / (double)L[a];
-        tab[2 * k] = cos(th);
-        tab[2 * k + 1] = sin(th);
+        tab[2 * k] = trig[2 * k];
+        tab[2 * k + 1] = trig[2 * k + 1];
       } else {
         tab[k] = def_disp(x, cen[3 * main_c + a], (double)L[a], !(a == 2 && wall));
       }
@@ -246,13 +259,10 @@ __global__ void __launch_bounds__(256) k_def_sum(const DevBox* __restrict__ boxe
         if (a == 2 && wall) {
           v[4] = (double)co[2];
           v[5] = 0.0;
-        } else if (table) {
-          v[2 * a] = tab[2 * (at[a] + co[a])];
-          v[2 * a + 1] = tab[2 * (at[a] + co[a]) + 1];
         } else {
-          const double th = DEF_TWO_PI * (double)co[a] / (double)L[a];
-          v[2 * a] = cos(th);
-          v[2 * a + 1] = sin(th);
+          const double* t = table ? tab : trig;
+          v[2 * a] = t[2 * (at[a] + co[a])];
+          v[2 * a + 1] = t[2 * (at[a] + co[a]) + 1];
         }
       }
     } else {
@@ -339,16 +349,18 @@ cudaError_t launch_defects_label(int prec, const DevBox* boxes, int b, int N, do
 }
 
 cudaError_t launch_defects_stats(const DevBox* boxes, int b, int N, int sides, int ncomp, const int* parent, const int* comp,
-                                 int* size, double* circ, double* cen, double* gyr, cudaStream_t s) {
+                                 int* size, double* circ, double* cen, double* gyr, double* trig,
+                                 cudaStream_t s) {
   if (ncomp <= 0) return cudaSuccess;
   // up to eight blocks per SM, whole rows of 256 nodes each
   const int per = 256 * std::max(1, def_blocks(def_blocks(N, 256), 8 * 152));
   const int nb = (N - 1) / per + 1;
   const size_t rows = sides * sizeof(double);
   const bool t1 = 2 * rows <= 40960, t2 = rows <= 40960;
-  k_def_sum<1><<<nb, 256, t1 ? 2 * rows : 0, s>>>(boxes, b, parent, comp, cen, size, circ, per, t1);
+  k_def_trig<<<def_blocks(sides, 64), 64, 0, s>>>(boxes, b, trig);
+  k_def_sum<1><<<nb, 256, t1 ? 2 * rows : 0, s>>>(boxes, b, parent, comp, cen, size, circ, trig, per, t1);
   k_def_centroid<<<def_blocks(ncomp, 128), 128, 0, s>>>(boxes, b, ncomp, size, circ, cen);
-  k_def_sum<2><<<nb, 256, t2 ? rows : 0, s>>>(boxes, b, parent, comp, cen, size, gyr, per, t2);
+  k_def_sum<2><<<nb, 256, t2 ? rows : 0, s>>>(boxes, b, parent, comp, cen, size, gyr, trig, per, t2);
   k_def_final<<<def_blocks(6 * ncomp, 256), 256, 0, s>>>(ncomp, size, gyr);
   return cudaGetLastError();
 }

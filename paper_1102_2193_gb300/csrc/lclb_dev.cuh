@@ -10,6 +10,8 @@
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
+#include "f64_bits.cuh"
+
 namespace lclb {
 
 constexpr int NQ = 19;
@@ -292,7 +294,7 @@ __device__ __forceinline__ void moments_f64(const double df[NQ], double& drho, d
   pair_moments<double>(df, drho, m);
 }
 // FP32 deviations: added as 64-bit integers at 2^-57 of the largest, which
-// loses less than FP64 additions (2^-53 of the partial sums) and takes 8 FP64
+// loses less than FP64 additions (2^-53 of the partial sums) and takes 4 FP64
 // operations instead of 58; infinities and NaN take the FP64 sums.
 __device__ __forceinline__ void moments_f64(const float df[NQ], double& drho, double m[3]) {
   unsigned top = 0;
@@ -302,11 +304,10 @@ __device__ __forceinline__ void moments_f64(const float df[NQ], double& drho, do
     pair_moments<double>(df, drho, m);
     return;
   }
-  const int k = min(126, 183 - (int)(top >> 23));  // |df| 2^k < 2^57, so 19 of them fit 63 bits
-  const float scale = __int_as_float((k + 127) << 23);
+  const int k = 183 - (int)(top >> 23);  // |df| 2^k < 2^57, so 19 of them fit 63 bits
   long long v[NQ], s, ms[3];
 #pragma unroll
-  for (int q = 0; q < NQ; ++q) v[q] = __float2ll_rn(df[q] * scale);
+  for (int q = 0; q < NQ; ++q) v[q] = f32_to_fixed(df[q], k);
   pair_moments<long long>(v, s, ms);
   const double inv = __hiloint2double((1023 - k) << 20, 0);
   drho = (double)s * inv;
@@ -326,6 +327,9 @@ __device__ __forceinline__ void load_q_f32(const DevBox& B, int qpar, int i, flo
       q[k] = (float)static_cast<const double*>(B.Q[qpar])[o];
   }
 }
+
+__device__ __forceinline__ double to_f64(float v) { return f32_to_f64(v); }
+__device__ __forceinline__ double to_f64(double v) { return v; }
 
 template <typename T>
 __device__ __forceinline__ T ldg(const T* p) { return __ldg(p); }
@@ -390,12 +394,12 @@ __device__ __forceinline__ double principal_lambda_f64(const double* q) {
   }
   const double t2 = 0.5 * (a00 * a00 + a11 * a11 + a22 * a22 + 2.0 * (a01 * a01 + a02 * a02 + a12 * a12));
   const double det = a00 * (a11 * a22 - a12 * a12) - a01 * (a01 * a22 - a12 * a02) + a02 * (a01 * a12 - a11 * a02);
-  double lam = (double)lam32;
+  double lam = f32_to_f64(lam32);
 #pragma unroll
   for (int it = 0; it < 2; ++it) {
     const double f = (t2 - lam * lam) * lam + det;
     const float df = (float)(t2 - 3.0 * lam * lam);
-    if (df != 0.f) lam -= f * (double)(1.f / df);
+    if (df != 0.f) lam -= f * f32_to_f64(1.f / df);
   }
   return lam;
 }
@@ -404,7 +408,7 @@ __device__ __forceinline__ double principal_lambda_f64(const double* q) {
 // one, relative error ~1e-14; FP64 storage: two, to rounding).
 template <int STEPS>
 __device__ __forceinline__ double rsqrt_f64(double v) {
-  double r = (double)rsqrtf((float)v);
+  double r = f32_to_f64(rsqrtf((float)v));
 #pragma unroll
   for (int k = 0; k < STEPS; ++k) r = r * (1.5 - 0.5 * v * r * r);
   return r;

@@ -48,6 +48,7 @@ struct Launch {
   const int2* groups;
   int ngroups;
   double* npart;      // k_lc: residual record (sum of squares, max) of each group
+  double* fepart;     // k_stress with FORCE_FE: free energy of each block of groups
   const int2* chunks; // k_lc with LC_COMMIT: link chunks (box, first link)
   int nchunks;
   unsigned* done;       // k_lc with LC_COMMIT: finished work units per box (zero between launches)
@@ -104,11 +105,12 @@ cudaError_t launch_reduce(const double* part, int rec0, int n, int w, unsigned m
 // defect_blocks(N) ints; *total = number of components; *err set when a
 // bounded loop gave up.  Statistics: size (ncomp ints), circ (6 ncomp),
 // cen (3 ncomp), gyr (6 ncomp) doubles, size/circ/gyr zeroed by the caller;
-// sides = nx + ny + nz.
+// trig 2 sides doubles, sides = nx + ny + nz.
 int defect_blocks(int N);
 cudaError_t launch_defects_label(int prec, const DevBox* boxes, int b, int N, double thr, int* parent, int* comp,
                                  int* list, int* blockcnt, int* total, int* err, cudaStream_t s);
 cudaError_t launch_defects_stats(const DevBox* boxes, int b, int N, int sides, int ncomp, const int* parent, const int* comp,
-                                 int* size, double* circ, double* cen, double* gyr, cudaStream_t s);
+                                 int* size, double* circ, double* cen, double* gyr, double* trig,
+                                 cudaStream_t s);
 
 }  // namespace lclb

@@ -682,7 +682,8 @@ __device__ __forceinline__ void add_residual(const T d5[5], T& rsum, T& rmax) {
 }
 
 template <typename T, bool FROZEN = false>
-__device__ __noinline__ void near_stress(const DevBox& B, int i, int mode, NearScratch<T>& sc, T* rs = nullptr) {
+__device__ __noinline__ void near_stress(const DevBox& B, int i, int mode, NearScratch<T>& sc, T* rs = nullptr,
+                                         double* fe = nullptr) {
   const unsigned full = 0xffffffffu;
   const int lane = threadIdx.x & 31;
   const bool valid = i >= 0;
@@ -731,7 +732,7 @@ __device__ __noinline__ void near_stress(const DevBox& B, int i, int mode, NearS
   double nf[3] = {1.0, 0.0, 0.0}, qid[5];
   if (!comp || planar || wall_face || max(nx, max(ny, B.nz)) >= (1 << 22)) {
 #pragma unroll
-    for (int k = 0; k < 5; ++k) qid[k] = comp ? (double)qh[k] + (double)ql[k] : (double)qh[k];
+    for (int k = 0; k < 5; ++k) qid[k] = comp ? to_f64(qh[k]) + f32_to_f64(ql[k]) : to_f64(qh[k]);
   } else {
 #pragma unroll
     for (int k = 0; k < 5; ++k) qid[k] = 0.0;
@@ -829,6 +830,22 @@ __device__ __noinline__ void near_stress(const DevBox& B, int i, int mode, NearS
       for (int c = 0; c < 9; ++c) Pb[(size_t)c * N + i] = p[c];
     }
   }
+  if (fe && valid) {
+    // free energy of the node, and of its weakly anchored faces (w/2)|Qs - Q0|^2
+    // with Qs - Q0 = -(1/wfac - 1)(Qs - Q)
+    *fe += to_f64(fp);
+#pragma unroll
+    for (int d = 0; d < 6; ++d) {
+      if (!((solid >> d) & 1u) || nb[d] < 0) continue;
+      const DevColloid& C = B.col[cf[d] - 1];
+      if (C.strong) continue;
+      const T dz = dn[d][0] + dn[d][3];
+      const T s2 = dn[d][0] * dn[d][0] + dn[d][3] * dn[d][3] + dz * dz +
+                   T(2) * (dn[d][1] * dn[d][1] + dn[d][2] * dn[d][2] + dn[d][4] * dn[d][4]);
+      const double r = 1.0 / C.wfac - 1.0;
+      *fe += 0.5 * C.w * r * r * to_f64(s2);
+    }
+  }
   if (!(mode & FORCE_ACC)) return;
   for (int t0 = 0; t0 < nface; t0 += 32) {
     const int t = t0 + lane;
@@ -858,10 +875,10 @@ __device__ __noinline__ void near_stress(const DevBox& B, int i, int mode, NearS
       disp(B, fc[0], fc[1], fc[2], B.col[c].X, rd);
       const T r[3] = {T(rd[0]), T(rd[1]), T(rd[2])};
 #pragma unroll
-      for (int a = 0; a < 3; ++a) v[a] = (double)ff[a];
-      v[3] = (double)(r[1] * ff[2] - r[2] * ff[1]);
-      v[4] = (double)(r[2] * ff[0] - r[0] * ff[2]);
-      v[5] = (double)(r[0] * ff[1] - r[1] * ff[0]);
+      for (int a = 0; a < 3; ++a) v[a] = to_f64(ff[a]);
+      v[3] = to_f64(r[1] * ff[2] - r[2] * ff[1]);
+      v[4] = to_f64(r[2] * ff[0] - r[0] * ff[2]);
+      v[5] = to_f64(r[0] * ff[1] - r[1] * ff[0]);
     }
     __syncwarp();
     warp_flush_colloid(B.col, t < nface ? c : -1, v, 6);
@@ -872,9 +889,9 @@ __device__ __noinline__ void near_stress(const DevBox& B, int i, int mode, NearS
 template <typename T>
 __device__ __forceinline__ void stress_node(const DevBox& B, const PhysT<T>& PP, const T* __restrict__ Q,
                                             T* __restrict__ Hb, T* __restrict__ Pb, int x, int y, int z, int i,
-                                            const T (*pq)[5], int mode) {
+                                            const T (*pq)[5], int mode, T& fp) {
   const int N = B.N;
-  T qi[5], qn[6][5], h[5], p[9], fp;
+  T qi[5], qn[6][5], h[5], p[9];
   int nb[6], zz[2];
   face_neighbours(B, x, y, z, nb, zz);
 #pragma unroll
@@ -927,7 +944,8 @@ __device__ __forceinline__ void stress_tile(const DevBox& B, const int4 td, int 
     T pq[5][5];
     column_next<T, 5>(B, Q, x, y, z, valid, qz, pq);
     x_neighbours<T, 5>(Q, (size_t)B.N, pq[0], lane, x, nx, nx * (y + ny * z), valid, &pq[1]);
-    if (fluid && !near) stress_node<T>(B, PP, Q, Hb, Pb, x, y, z, i, pq, mode);
+    T fp;
+    if (fluid && !near) stress_node<T>(B, PP, Q, Hb, Pb, x, y, z, i, pq, mode, fp);
     const unsigned nb = __ballot_sync(0xffffffffu, near);
     if (nb) {
       if (near) sq[wy][nq + __popc(nb & ((1u << lane) - 1u))] = i;
@@ -1213,9 +1231,9 @@ __device__ __forceinline__ void st2_keep_if(float* p, f2 v, bool a, bool b, uint
 }
 
 // Stress of a tile of plain nodes, two nodes per lane, Q from the ring.
-template <int TY>
+template <int TY, bool FE>
 __device__ __forceinline__ void stress_ring(const DevBox& B, const LcK<f2>& K2, const int4 td, int zc, int mode,
-                                            float* ring) {
+                                            float* ring, double& fe) {
   if (!B.p.lc_on) return;
   const float* __restrict__ Q = static_cast<const float*>(B.Q[B.st->qpar]);
   float* __restrict__ Hb = static_cast<float*>(B.H);
@@ -1254,6 +1272,10 @@ __device__ __forceinline__ void stress_ring(const DevBox& B, const LcK<f2>& K2, 
       lap[k] = ((n[0] + n[1]) + (n[2] + n[3]) + (n[4] + n[5])) + K2.nsix * qi[k];
     }
     lc_node_d<f2>(K2, chiral, qi, dq, lap, h, p, &fp);
+    if constexpr (FE) {
+      if (pa) fe += f32_to_f64(fp.v.x);
+      if (pb) fe += f32_to_f64(fp.v.y);
+    }
     const size_t i = (size_t)R.x + R.row + (size_t)plane * z;
 #pragma unroll
     for (int c = 0; c < 5; ++c) st2_keep_if(Hb + c * N + i, h[c], pa, pb, keep);
@@ -1265,8 +1287,8 @@ __device__ __forceinline__ void stress_ring(const DevBox& B, const LcK<f2>& K2, 
 }
 
 // Stress of a tile of plain nodes, one node per lane (odd widths, FP64).
-template <typename T>
-__device__ __forceinline__ void stress_plain(const DevBox& B, const int4 td, int zc, int mode) {
+template <typename T, bool FE>
+__device__ __forceinline__ void stress_plain(const DevBox& B, const int4 td, int zc, int mode, double& fe) {
   if (!B.p.lc_on) return;
   const int lane = threadIdx.x;
   const T* __restrict__ Q = static_cast<const T*>(B.Q[B.st->qpar]);
@@ -1281,40 +1303,61 @@ __device__ __forceinline__ void stress_plain(const DevBox& B, const int4 td, int
     T pq[5][5];
     column_next<T, 5>(B, Q, x, y, z, valid, qz, pq);
     x_neighbours<T, 5>(Q, (size_t)B.N, pq[0], lane, x, nx, nx * (y + ny * z), valid, &pq[1]);
-    if (plain_node(m))
-      stress_node<T>(B, phys<T>(B), Q, static_cast<T*>(B.H), static_cast<T*>(B.P), x, y, z, i, pq, mode);
+    if (plain_node(m)) {
+      T fp;
+      stress_node<T>(B, phys<T>(B), Q, static_cast<T*>(B.H), static_cast<T*>(B.P), x, y, z, i, pq, mode, fp);
+      if constexpr (FE) fe += to_f64(fp);
+    }
     column_roll<T, 5>(qz, pq);
   }
 }
 
+// Sum of fe over the block's TY warps in warp order, by thread (0, 0) into *out.
+template <int TY>
+__device__ __forceinline__ void block_fe(double fe, double* out) {
+  __shared__ double s_fe[TY];
+  warp_sums<1>(&fe, [&](int, double t) { s_fe[threadIdx.y] = t; });
+  __syncthreads();
+  if (threadIdx.x + threadIdx.y == 0) {
+    double t = 0.0;
+    for (int k = 0; k < TY; ++k) t += s_fe[k];
+    *out = t;
+  }
+  __syncthreads();
+}
+
 // H and P stored once per fluid node, and the colloid LC force from the near
-// nodes.
-template <typename T, int TY>
-__global__ void __launch_bounds__(TX * TY, (sizeof(T) == 4 ? 512 : 256) / (TX * TY)) k_stress(Launch L, int mode) {
+// nodes.  FE (diagnostics): the free energy of each tile into part and of each
+// block of near groups into L.fepart.
+template <typename T, int TY, bool FE>
+__global__ void __launch_bounds__(TX * TY, (sizeof(T) == 4 ? 512 : 256) / (TX * TY)) k_stress(Launch L, int mode,
+                                                                                             double* __restrict__ part) {
   __shared__ DevBox B;
   __shared__ LcK<f2> K2;
   extern __shared__ __align__(16) float ring[];
   int cur_box = -1;
   const int nn = L.ngroups / TY, units = nn + L.ntiles;
   for (int t = blockIdx.x; t < units; t += gridDim.x) {
-    if (t < nn) {
-      load_box(B, K2, L.boxes, L.groups[t * TY].x, cur_box);
-      if (!B.p.lc_on) continue;
-      near_group<TY>(B, L.groups, t, [&](int j) {
-        near_stress<T>(B, j, mode, reinterpret_cast<NearScratch<T>*>(ring)[threadIdx.y]);
-      });
-      __syncthreads();
-      continue;
-    }
-    const int4 td = L.tiles[t - nn];
+    const int4 td = t < nn ? make_int4(L.groups[t * TY].x, 0, 0, 0) : L.tiles[t - nn];
     load_box(B, K2, L.boxes, td.x, cur_box);
-    if constexpr (sizeof(T) == 4) {
-      if (pair_box(B)) {
-        stress_ring<TY>(B, K2, td, L.zc, mode, ring);
-        continue;
+    double fe = 0.0;
+    if (t < nn) {
+      if (B.p.lc_on)
+        near_group<TY>(B, L.groups, t, [&](int j) {
+          near_stress<T>(B, j, mode, reinterpret_cast<NearScratch<T>*>(ring)[threadIdx.y], nullptr, FE ? &fe : nullptr);
+        });
+      __syncthreads();
+    } else {
+      bool done = false;
+      if constexpr (sizeof(T) == 4) {
+        if (pair_box(B)) {
+          stress_ring<TY, FE>(B, K2, td, L.zc, mode, ring, fe);
+          done = true;
+        }
       }
+      if (!done) stress_plain<T, FE>(B, td, L.zc, mode, fe);
     }
-    stress_plain<T>(B, td, L.zc, mode);
+    if constexpr (FE) block_fe<TY>(fe, t < nn ? L.fepart + t : part + (t - nn));
   }
 }
 
@@ -1848,7 +1891,7 @@ __device__ __forceinline__ void links_chunk(const DevBox& B, int l0, int n, doub
       const int q = B.link_dir[l];
       const int c = B.link_col[l];
       const T* fout = static_cast<const T*>(B.f[B.st->fpar ^ 1]);
-      const double dfq = (double)ldx<CG>(fout + (size_t)q * B.N + i);
+      const double dfq = to_f64(ldx<CG>(fout + (size_t)q * B.N + i));
       const int x = i % B.nx, y = (i / B.nx) % B.ny, z = i / (B.nx * B.ny);
       int qx = 0, qy = 0, qz = 0;
       switch (q) {
@@ -2828,8 +2871,8 @@ __global__ void __launch_bounds__(256) k_export_q(const DevBox* __restrict__ box
       const __nv_bfloat162 l0 = *reinterpret_cast<const __nv_bfloat162*>(lo + e0);
       const __nv_bfloat162 l1 = *reinterpret_cast<const __nv_bfloat162*>(lo + e0 + 2);
       double2* o = reinterpret_cast<double2*>(out + e0);
-      o[0] = make_double2((double)h.x + (double)__low2float(l0), (double)h.y + (double)__high2float(l0));
-      o[1] = make_double2((double)h.z + (double)__low2float(l1), (double)h.w + (double)__high2float(l1));
+      o[0] = make_double2(f32_to_f64(h.x) + f32_to_f64(__low2float(l0)), f32_to_f64(h.y) + f32_to_f64(__high2float(l0)));
+      o[1] = make_double2(f32_to_f64(h.z) + f32_to_f64(__low2float(l1)), f32_to_f64(h.w) + f32_to_f64(__high2float(l1)));
       return;
     }
   }
@@ -2838,6 +2881,9 @@ __global__ void __launch_bounds__(256) k_export_q(const DevBox* __restrict__ box
     else out[e] = Q[e];
   }
 }
+
+__device__ __forceinline__ double half_f64(float v) { return f32_to_f64(0.5f * v); }
+__device__ __forceinline__ double half_f64(double v) { return 0.5 * v; }
 
 // Other fields.  which: LC_F_PRE, LC_RHO, LC_U, LC_FORCE, LC_SOLID.  The force
 // is the face divergence of the stored stress, as the LB kernel takes it.
@@ -2888,8 +2934,22 @@ __global__ void __launch_bounds__(256) k_export(const DevBox* __restrict__ boxes
     out[i] = rho;
     return;
   }
-  const double inv = 1.0 / rho;
-  for (int a = 0; a < 3; ++a) out[(size_t)a * N + i] = (mm[a] + 0.5 * ((double)F[a] + B.p.g[a])) * inv;
+  // 1/rho by Newton from the FP32 reciprocal (to rounding in two steps)
+  const float rf = (float)rho;
+  double inv;
+  if (rf > 1e-30f && rf < 1e30f) {
+    inv = f32_to_f64(1.f / rf);
+    inv = inv * (2.0 - rho * inv);
+    inv = inv * (2.0 - rho * inv);
+  } else {
+    inv = 1.0 / rho;
+  }
+  const bool forced = B.p.g[0] != 0.0 || B.p.g[1] != 0.0 || B.p.g[2] != 0.0;
+  for (int a = 0; a < 3; ++a) {
+    double m = mm[a] + half_f64(F[a]);
+    if (forced) m += 0.5 * B.p.g[a];
+    out[(size_t)a * N + i] = m * inv;
+  }
 }
 
 // Diagnostics per block: [0] sum(df), [1..3] sum(df c), [4] fluid nodes,
@@ -3359,13 +3419,12 @@ template <typename T, int NC, int TY>
 constexpr size_t ring_bytes() { return sizeof(T) == 4 ? Ring<NC, TY>::BYTES : 0; }
 
 template <typename T, int TY>
-static cudaError_t launch_stress_t(const Launch& L, int mode, double*) {
+static cudaError_t launch_stress_t(const Launch& L, int mode, double* part) {
   constexpr size_t ring = ring_bytes<T, 5, TY>(), near = sizeof(NearScratch<T>) * TY, smem = ring > near ? ring : near;
-  if (smem > 0) {
-    cudaError_t e = cudaFuncSetAttribute(k_stress<T, TY>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-  }
-  k_stress<T, TY><<<L.grid, dim3(TX, TY), smem, L.stream>>>(L, mode);
+  auto* fn = (mode & FORCE_FE) ? k_stress<T, TY, true> : k_stress<T, TY, false>;
+  cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e != cudaSuccess) return e;
+  fn<<<L.grid, dim3(TX, TY), smem, L.stream>>>(L, mode, part);
   return cudaGetLastError();
 }
 

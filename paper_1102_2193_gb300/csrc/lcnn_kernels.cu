@@ -12,6 +12,7 @@
 #include <cstdint>
 
 #include "../../include/lc_nn.h"
+#include "f64_bits.cuh"
 
 namespace lcnn {
 
@@ -780,7 +781,10 @@ __global__ void k_from_soa(const double* __restrict__ q, float* __restrict__ a, 
 __global__ void k_to_soa(const float* __restrict__ a, const float* __restrict__ base, double* __restrict__ q, int npos,
                          int cout) {
   for (int p = blockIdx.x * blockDim.x + threadIdx.x; p < npos; p += gridDim.x * blockDim.x)
-    for (int c = 0; c < 5; ++c) q[(size_t)c * npos + p] = (double)a[(size_t)p * cout + c] + (base ? base[(size_t)p * 5 + c] : 0.0);
+    for (int c = 0; c < 5; ++c) {
+      const double v = f32_to_f64(a[(size_t)p * cout + c]);
+      q[(size_t)c * npos + p] = base ? v + f32_to_f64(base[(size_t)p * 5 + c]) : v + 0.0;
+    }
 }
 
 // Trilinear x2 upsampling of a periodic SoA field [c][S^3] (cell-centred: the
