@@ -9,6 +9,7 @@
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cstdint>
 
 #include "../../include/lc_nn.h"
@@ -136,16 +137,20 @@ __device__ __forceinline__ int modn(int v, int n) {
 // k_conv_fwd, which this replaces for 3x3x3 kernels, read every position 27
 // times through L1 with 4-byte loads (16 -> 16 channels at 128^3: 740 us).
 // A warp holds MT 16-position tiles x NT 8-channel tiles, so one B fragment
-// serves MT products; MT and NT are bounded by the accumulator registers, the
-// tile by 2 blocks per SM.  FP32 accumulation in the order (16-channel group,
+// serves MT products; in boxes 16 wide its tiles are MT consecutive rows of y,
+// so the MT + 2 rows of A that one (dx, dz) needs serve all three dy (shared
+// memory reads bound the kernel: 61 % of its wavefronts with 12 loads of A per
+// (dx, dz) instead of 6).  MT and NT are bounded by the accumulator registers,
+// the tile by 2 or 3 blocks per SM.  FP32 accumulation in the order (16-channel group,
 // tap).  blockIdx.y picks the group of NT * 8 output channels.
 template <int NT, int MT, int NW, int TX, int TY, int TZ>
-__global__ void __launch_bounds__(32 * NW) k_conv_tile(const __nv_bfloat16* __restrict__ in,
+__global__ void __launch_bounds__(32 * NW, NW == 8 ? (NT <= 2 ? 3 : (NT <= 4 ? 2 : 1)) : 6) k_conv_tile(const __nv_bfloat16* __restrict__ in,
                                                        const __nv_bfloat16* __restrict__ w,
                                                        const float* __restrict__ bias, float* __restrict__ out32,
                                                        __nv_bfloat16* __restrict__ out16, int W, int H, int D, int cin,
                                                        int cout, int relu, int ntx, int nty) {
   static_assert(TX * TY * TZ == 16 * MT * NW, "one 16-position tile per (warp, MT)");
+  static_assert(TX != 16 || TY % MT == 0, "a warp's rows share z");
   constexpr int HX = TX + 2, HY = TY + 2, HZ = TZ + 2, HP = HX * HY * HZ, NTHR = 32 * NW;
   constexpr int NPT = (HP + NTHR - 1) / NTHR, NWR = 27 * NT * 8;
   extern __shared__ __align__(128) unsigned char smem[];
@@ -192,29 +197,40 @@ __global__ void __launch_bounds__(32 * NW) k_conv_tile(const __nv_bfloat16* __re
     }
     cp_wait_all();
     __syncthreads();
+    // B fragments of tap t
+    auto load_b = [&](int t, uint32_t b[NT][2]) {
+#pragma unroll
+      for (int j = 0; j + 1 < NT; j += 2) {
+        uint32_t q[4];
+        ldm4(q, sW + row32(t * NT * 8 + j * 8 + brow, bhalf));
+        b[j][0] = q[0];
+        b[j][1] = q[1];
+        b[j + 1][0] = q[2];
+        b[j + 1][1] = q[3];
+      }
+      if constexpr (NT & 1) ldm2(b[NT - 1], sW + row32(t * NT * 8 + (NT - 1) * 8 + (lane & 7), bhalf));
+    };
 #pragma unroll 1
     for (int dz = 0; dz < 3; ++dz)
 #pragma unroll
-      for (int dyx = 0; dyx < 9; ++dyx) {
-        const int t = dz * 9 + dyx;
-        const int off = dyx % 3 + HX * (dyx / 3 + HY * dz);
-        uint32_t a[MT][4], b[NT][2];
+      for (int dx = 0; dx < 3; ++dx) {
+        uint32_t a[MT + 2][4], b[NT][2];
+        if constexpr (TX == 16) {
 #pragma unroll
-        for (int i = 0; i < MT; ++i) ldm4(a[i], sA + row32(rowp[i] + off, ahalf));
-#pragma unroll
-        for (int j = 0; j + 1 < NT; j += 2) {
-          uint32_t q[4];
-          ldm4(q, sW + row32(t * NT * 8 + j * 8 + brow, bhalf));
-          b[j][0] = q[0];
-          b[j][1] = q[1];
-          b[j + 1][0] = q[2];
-          b[j + 1][1] = q[3];
+          for (int i = 0; i < MT + 2; ++i) ldm4(a[i], sA + row32(rowp[0] + dx + HX * (i + HY * dz), ahalf));
         }
-        if constexpr (NT & 1) ldm2(b[NT - 1], sW + row32(t * NT * 8 + (NT - 1) * 8 + (lane & 7), bhalf));
 #pragma unroll
-        for (int i = 0; i < MT; ++i)
+        for (int dy = 0; dy < 3; ++dy) {
+          if constexpr (TX != 16) {
 #pragma unroll
-          for (int j = 0; j < NT; ++j) mma_bf16(acc[i][j], a[i], b[j]);
+            for (int i = 0; i < MT; ++i) ldm4(a[i + dy], sA + row32(rowp[i] + dx + HX * (dy + HY * dz), ahalf));
+          }
+          load_b(dz * 9 + dy * 3 + dx, b);
+#pragma unroll
+          for (int i = 0; i < MT; ++i)
+#pragma unroll
+            for (int j = 0; j < NT; ++j) mma_bf16(acc[i][j], a[i + dy], b[j]);
+        }
       }
   }
   const int g = lane >> 2, tg = lane & 3;
@@ -474,8 +490,9 @@ __global__ void k_flip_weights(const __nv_bfloat16* __restrict__ w, __nv_bfloat1
 // 16 bytes, eight in flight per thread: 64 KB per SM cover the latency of the
 // memory), the block sums go through distributed shared memory and are added
 // in block order, so the result is the same on every run.  16 channels at 64^3:
-// one block per channel 223 us, clusters of 8 with 4-byte loads 80 us.
-constexpr int BIAS_CLUSTER = 16, BIAS_THREADS = 512;
+// one block per channel 223 us, clusters of 8 with 4-byte loads 80 us, with
+// 512 threads 17 us.
+constexpr int BIAS_CLUSTER = 16, BIAS_THREADS = 1024;
 template <int V>
 __global__ void __launch_bounds__(BIAS_THREADS) k_bias_grad(const float* __restrict__ dout, float* __restrict__ db,
                                                             int npos, int c) {
@@ -510,12 +527,14 @@ __global__ void __launch_bounds__(BIAS_THREADS) k_bias_grad(const float* __restr
 #pragma unroll
   for (int j = 0; j < V; ++j) s[row][col + j] = v[j];
   __syncthreads();
-  // 32 threads per channel add the rows in a fixed tree
+  // a warp per channel adds the rows in a fixed tree
   const int ch = tid >> 5, lane = tid & 31;
-  float t = 0.f;
-  for (int r = lane; r < ROWS; r += 32) t += s[r][ch];
-  for (int o = 16; o > 0; o >>= 1) t += __shfl_down_sync(0xffffffffu, t, o);
-  if (lane == 0) tot[ch] = t;
+  if (ch < 16) {
+    float t = 0.f;
+    for (int r = lane; r < ROWS; r += 32) t += s[r][ch];
+    for (int o = 16; o > 0; o >>= 1) t += __shfl_down_sync(0xffffffffu, t, o);
+    if (lane == 0) tot[ch] = t;
+  }
   cooperative_groups::cluster_group cl = cooperative_groups::this_cluster();
   cl.sync();
   if (rank == 0 && tid < 16 && c0 + tid < c) {
@@ -648,11 +667,28 @@ __global__ void k_up2_concat_bwd(const float* __restrict__ dout, float* __restri
 // pred = base + out[:, 0:5] (out has cout channels); grad w.r.t. out.
 __global__ void k_mse(const float* __restrict__ out, const float* __restrict__ base, const float* __restrict__ target,
                       const float* __restrict__ fluid, float* __restrict__ grad, double* __restrict__ loss, int npos,
-                      int cout, double inv_count) {
+                      int cout, double inv_count, bool vec) {
   __shared__ double s[256];
   double acc = 0.0;
   for (int p = blockIdx.x * blockDim.x + threadIdx.x; p < npos; p += gridDim.x * blockDim.x) {
     const float m = fluid[p];
+    if (cout == 16 && vec) {  // the position's gradient row in four 16-byte stores
+      float g[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+      if (m > 0.f)
+        for (int c = 0; c < 5; ++c) {
+          const float d = out[(size_t)p * 16 + c] + base[(size_t)p * 5 + c] - target[(size_t)p * 5 + c];
+          const double dd = f32_to_f64(d);
+          acc += dd * dd;
+          g[c] = (float)(2.0 * inv_count) * d;
+        }
+      if (grad) {
+        float4* o = reinterpret_cast<float4*>(grad + (size_t)p * 16);
+        o[0] = make_float4(g[0], g[1], g[2], g[3]);
+        o[1] = make_float4(g[4], 0.f, 0.f, 0.f);
+        o[2] = o[3] = make_float4(0.f, 0.f, 0.f, 0.f);
+      }
+      continue;
+    }
     for (int c = 0; c < cout; ++c) {
       float gv = 0.f;
       if (c < 5 && m > 0.f) {
@@ -736,38 +772,68 @@ __global__ void k_adam(float* __restrict__ p, const float* __restrict__ g, float
 
 // Network input (channels last, cpad >= 9 channels, the rest zero):
 // [solid indicator, Q xx,xy,xz,yy,yz, R/32, p/64, 20 w] from FP64 SoA fields.
-__global__ void k_pack_input(const double* __restrict__ solid, const double* __restrict__ q, float r, float pitch,
-                             float w, __nv_bfloat16* __restrict__ x16, float* __restrict__ base, float* __restrict__ fluid,
-                             double* __restrict__ nfluid, int npos, int cpad, bool vec) {
+// vec (cpad == 16, x16 and base 16-byte aligned): the position's 32 bytes in two
+// stores, and the base of the block's 256 positions through shared memory in
+// whole lines.
+__global__ void __launch_bounds__(256) k_pack_input(const double* __restrict__ solid, const double* __restrict__ q,
+                                                    float r, float pitch, float w, __nv_bfloat16* __restrict__ x16,
+                                                    float* __restrict__ base, float* __restrict__ fluid,
+                                                    double* __restrict__ nfluid, int npos, int cpad, bool vec) {
+  __shared__ __align__(16) float sb[256 * 5];
   int cnt = 0;
-  for (int p = blockIdx.x * blockDim.x + threadIdx.x; p < npos; p += gridDim.x * blockDim.x) {
-    // solid < 0, >= 0 by the bits (an FP64 comparison is a slot of the FP64 pipe;
-    // NaN is neither)
-    const long long sb = __double_as_longlong(solid[p]);
-    const bool nan = (sb & 0x7fffffffffffffffll) > 0x7ff0000000000000ll, zero = (sb << 1) == 0;
-    cnt += !nan && !zero && sb < 0;
-    const bool sol = !nan && (zero || sb > 0);
-    float v[9] = {sol ? 1.f : 0.f, 0, 0, 0, 0, 0, r / 32.f, pitch / 64.f, 20.f * w};
-    for (int c = 0; c < 5; ++c) {
-      v[1 + c] = (float)q[(size_t)c * npos + p];
-      if (base) base[(size_t)p * 5 + c] = v[1 + c];
-    }
-    if (vec) {  // cpad == 16: the position's 32 bytes in two stores
-      __nv_bfloat162 h[8];
+  for (int p0 = blockIdx.x * 256; p0 < npos; p0 += gridDim.x * 256) {
+    const int p = p0 + threadIdx.x;
+    const bool in = p < npos;
+    float v[9] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, r / 32.f, pitch / 64.f, 20.f * w};
+    if (in) {
+      // solid < 0, >= 0 by the bits (an FP64 comparison is a slot of the FP64 pipe;
+      // NaN is neither)
+      const long long sbits = __double_as_longlong(solid[p]);
+      const bool nan = (sbits & 0x7fffffffffffffffll) > 0x7ff0000000000000ll, zero = (sbits << 1) == 0;
+      cnt += !nan && !zero && sbits < 0;
+      const bool sol = !nan && (zero || sbits > 0);
+      v[0] = sol ? 1.f : 0.f;
+      for (int c = 0; c < 5; ++c) v[1 + c] = (float)q[(size_t)c * npos + p];
+      if (vec) {
+        __nv_bfloat162 h[8];
 #pragma unroll
-      for (int k = 0; k < 8; ++k)
-        h[k] = __floats2bfloat162_rn(2 * k < 9 ? v[2 * k] : 0.f, 2 * k + 1 < 9 ? v[2 * k + 1] : 0.f);
-      uint4* d = reinterpret_cast<uint4*>(x16 + (size_t)p * 16);
-      d[0] = *reinterpret_cast<uint4*>(h);
-      d[1] = *reinterpret_cast<uint4*>(h + 4);
-    } else {
-      for (int c = 0; c < cpad; ++c) x16[(size_t)p * cpad + c] = __float2bfloat16_rn(c < 9 ? v[c] : 0.f);
+        for (int k = 0; k < 8; ++k)
+          h[k] = __floats2bfloat162_rn(2 * k < 9 ? v[2 * k] : 0.f, 2 * k + 1 < 9 ? v[2 * k + 1] : 0.f);
+        uint4* d = reinterpret_cast<uint4*>(x16 + (size_t)p * 16);
+        d[0] = *reinterpret_cast<uint4*>(h);
+        d[1] = *reinterpret_cast<uint4*>(h + 4);
+      } else {
+        for (int c = 0; c < cpad; ++c) x16[(size_t)p * cpad + c] = __float2bfloat16_rn(c < 9 ? v[c] : 0.f);
+        if (base)
+          for (int c = 0; c < 5; ++c) base[(size_t)p * 5 + c] = v[1 + c];
+      }
+      if (fluid) fluid[p] = sol ? 0.f : 1.f;
     }
-    if (fluid) fluid[p] = sol ? 0.f : 1.f;
+    if (vec && base) {
+      __syncthreads();
+      for (int c = 0; c < 5; ++c) sb[threadIdx.x * 5 + c] = v[1 + c];
+      __syncthreads();
+      const int n = min(256, npos - p0) * 5;
+      float* dst = base + (size_t)p0 * 5;
+      for (int k = threadIdx.x * 4; k < n; k += 1024) {
+        if (k + 4 <= n) *reinterpret_cast<float4*>(dst + k) = *reinterpret_cast<const float4*>(sb + k);
+        else
+          for (int j = k; j < n; ++j) dst[j] = sb[j];
+      }
+    }
   }
   if (nfluid) {
-    for (int o = 16; o > 0; o >>= 1) cnt += __shfl_down_sync(0xffffffffu, cnt, o);
-    if ((threadIdx.x & 31) == 0 && cnt) atomicAdd(nfluid, (double)cnt);
+    // one FP64 atomic per block of a grid that fits the GPU (one per warp, all
+    // to one address, was the kernel's time: 131 us at 128^3 for 32 us of bytes)
+    __shared__ int sc[8];
+    cnt = __reduce_add_sync(0xffffffffu, cnt);
+    if ((threadIdx.x & 31) == 0) sc[threadIdx.x >> 5] = cnt;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      int t = 0;
+      for (int k = 0; k < 8; ++k) t += sc[k];
+      if (t) atomicAdd(nfluid, (double)t);
+    }
   }
 }
 
@@ -837,8 +903,9 @@ static int launch_conv_tile(const __nv_bfloat16* in, const __nv_bfloat16* w, con
 }
 
 // Boxes of 16 x 8 x 4 positions and all output channels per block while they
-// fill the GPU (152 SMs x 2 blocks), else boxes of 8 x 4 x 4 positions with
-// the output channels split in groups of 16 over the blocks.
+// fill the GPU (152 SMs x 2 blocks), else boxes of 128 positions (16 x 4 x 2, or
+// 8 x 4 x 4 where the tensor is no wider than 8) with the output channels split
+// in groups of 16 over the blocks.
 static int conv_tiled(const __nv_bfloat16* in, const __nv_bfloat16* w, const float* bias, float* out32,
                       __nv_bfloat16* out16, int W, int H, int D, int cin, int cout, int relu, cudaStream_t s) {
   if (cout != 8 && cout % 16) return LC_NN_ERR_ARG;
@@ -855,6 +922,10 @@ static int conv_tiled(const __nv_bfloat16* in, const __nv_bfloat16* w, const flo
     }
   }
 #undef LCNN_BIG
+  if (W > 8) {
+    if (cout == 8) return launch_conv_tile<1, 2, 4, 16, 4, 2>(in, w, bias, out32, out16, W, H, D, cin, cout, relu, s);
+    return launch_conv_tile<2, 2, 4, 16, 4, 2>(in, w, bias, out32, out16, W, H, D, cin, cout, relu, s);
+  }
   if (cout == 8) return launch_conv_tile<1, 2, 4, 8, 4, 4>(in, w, bias, out32, out16, W, H, D, cin, cout, relu, s);
   return launch_conv_tile<2, 2, 4, 8, 4, 4>(in, w, bias, out32, out16, W, H, D, cin, cout, relu, s);
 }
@@ -1032,7 +1103,8 @@ int lc_nn_up2_concat_bwd(const float* dout, float* dlo, float* dskip, int S, int
 
 int lc_nn_mse(const float* out, const float* base, const float* target, const float* fluid, float* grad,
               double* loss, int npos, int cout, double inv_count, void* stream) {
-  k_mse<<<grid_for(npos), 256, 0, (cudaStream_t)stream>>>(out, base, target, fluid, grad, loss, npos, cout, inv_count);
+  k_mse<<<grid_for(npos), 256, 0, (cudaStream_t)stream>>>(out, base, target, fluid, grad, loss, npos, cout, inv_count,
+                                                            aligned16(grad));
   return cudaGetLastError() == cudaSuccess ? LC_NN_OK : LC_NN_ERR_CUDA;
 }
 
@@ -1057,9 +1129,9 @@ int lc_nn_adam(float* p, const float* g, float* m, float* v, void* p16, size_t n
 int lc_nn_pack_input(const double* solid, const double* q, double R, double pitch, double w, void* x16, float* base,
                      float* fluid, double* nfluid, int npos, int cpad, void* stream) {
   if (cpad < 9) return LC_NN_ERR_ARG;
-  k_pack_input<<<grid_for(npos), 256, 0, (cudaStream_t)stream>>>(solid, q, (float)R, (float)pitch, (float)w,
+  k_pack_input<<<std::min(grid_for(npos), 8 * 152), 256, 0, (cudaStream_t)stream>>>(solid, q, (float)R, (float)pitch, (float)w,
                                                                    (__nv_bfloat16*)x16, base, fluid, nfluid, npos, cpad,
-                                                                   cpad == 16 && aligned16(x16));
+                                                                   cpad == 16 && aligned16(x16) && aligned16(base));
   return cudaGetLastError() == cudaSuccess ? LC_NN_OK : LC_NN_ERR_CUDA;
 }
 

@@ -54,18 +54,29 @@ class UNet:
         self.sp = C.c_void_p(self.stream.cuda_stream)
         g = np.random.default_rng(seed)
         self.params = {}
+        # parameters, gradients and moments of all layers lie in one buffer each
+        # (segments of whole 64-element blocks), so that clearing the gradients
+        # and the Adam step are one launch, not one per layer and tensor
+        size = lambda n: (n + 63) // 64 * 64  # noqa: E731
+        total = sum(size(cout * taps * cin) + size(cout) for _, cin, cout, taps, _, _ in LAYERS)
+        self.flat = {k: torch.zeros(total, device=self.dev) for k in ("", "g", "m", "v")}
+        self.flat16 = torch.zeros(total, dtype=torch.bfloat16, device=self.dev)
+        at = 0
         for name, cin, cout, taps, relu, lvl in LAYERS:
             fan_in = cin * taps
             scale = math.sqrt(2.0 / fan_in) if relu else 0.0  # the head starts at zero: pred = Q_init
             w = (g.standard_normal((cout, taps, cin)) * scale).astype(np.float32)
             if name == "c0a":
                 w[:, :, 9:] = 0.0
-            P = {"w": torch.tensor(w, device=self.dev), "b": torch.zeros(cout, device=self.dev)}
-            for k in ("w", "b"):
-                P["g" + k] = torch.zeros_like(P[k])
-                P["m" + k] = torch.zeros_like(P[k])
-                P["v" + k] = torch.zeros_like(P[k])
-            P["w16"] = torch.empty(P["w"].shape, dtype=torch.bfloat16, device=self.dev)
+            P = {}
+            for k, shape in (("w", w.shape), ("b", (cout,))):
+                n = math.prod(shape)
+                for pre, buf in self.flat.items():
+                    P[pre + k] = buf[at:at + n].view(shape)
+                if k == "w":
+                    P["w16"] = self.flat16[at:at + n].view(shape)
+                at += size(n)
+            P["w"].copy_(torch.tensor(w))
             P["wt"] = torch.empty(P["w"].numel(), dtype=torch.bfloat16, device=self.dev)
             self.params[name] = P
             self._cast(P["w"], P["w16"])
@@ -184,9 +195,7 @@ class UNet:
 
     def backward(self):
         t, S, a, L, sp = self.torch, self.S, self.a, self.L, self.sp
-        for P in self.params.values():
-            P["gw"].zero_()
-            P["gb"].zero_()
+        self.flat["g"].zero_()
         n0, n1, n2 = S**3, (S // 2)**3, (S // 4)**3
         new = lambda n, c: t.empty((n, c), dtype=t.float32, device=self.dev)  # noqa: E731
         d_c4 = new(n0, 16)
@@ -219,11 +228,9 @@ class UNet:
 
     def adam(self, lr=1e-3, b1=0.9, b2=0.999, eps=1e-8):
         self.step_count += 1
-        for P in self.params.values():
-            for k in ("w", "b"):
-                _ok(self.L.lc_nn_adam(_p(P[k]), _p(P["g" + k]), _p(P["m" + k]), _p(P["v" + k]),
-                                      _p(P["w16"]) if k == "w" else None, P[k].numel(), lr, b1, b2, eps,
-                                      self.step_count, self.sp), "adam")
+        f = self.flat
+        _ok(self.L.lc_nn_adam(_p(f[""]), _p(f["g"]), _p(f["m"]), _p(f["v"]), _p(self.flat16), f[""].numel(), lr, b1,
+                              b2, eps, self.step_count, self.sp), "adam")
 
     def predict_soa(self):
         """Q = Q_init + y[:, :5] as a [5][S^3] FP64 device tensor."""
