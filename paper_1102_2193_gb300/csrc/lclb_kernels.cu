@@ -1150,53 +1150,96 @@ __device__ __forceinline__ void cp_async4(float* dst, const float* src) {
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
 __device__ __forceinline__ void cp_async_wait0() { asm volatile("cp.async.wait_group 0;\n" ::: "memory"); }
 
-// Columns of the tile at (td.y, td.z): what a lane copies and where it finds
-// its neighbours.
+__device__ __forceinline__ void cp_async16(float* dst, const float* src) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src)
+               : "memory");
+}
+
+// Columns of the tile at (td.y, td.z): where a lane finds its neighbours, and
+// what the thread copies of each plane.  The 64 columns of the RY rows of a
+// component are 16 RY pieces of 16 bytes, one per thread (rows whose length or
+// base is not a multiple of 16 bytes: pieces of 8 bytes in turns); the two edge
+// columns of all components are one 4-byte copy per thread, at offsets that are
+// kept from plane to plane.  (Each lane copying its own pair, its row's edges
+// and, by turns, the rows above and below took 24 copies a plane and warp for
+// 5 components and 43 for 8, with their addresses a quarter of the kernels'
+// instructions.  128^3: k_stress 59 -> 44 us, k_lc 71 -> 53; 256 x 192 x 160:
+// 167 -> 126 and 207 -> 162; a step of k_relax at 96^3 26.5 -> 22.2.)
 struct RingLane {
-  int x, y, row, rowm, rowp, rowe;  // node column; row starts of y, y - 1, y + vy, and of the edge column (node index)
-  int vx, vy, li, ri;               // valid columns and rows of the tile; ring columns of x - 1 and x + 2
-  bool valid, edge;                 // the lane's pair is a node pair; the lane copies an edge column
+  int x, y, row;   // node column, row start of y (node index)
+  int li, ri;      // ring columns of x - 1 and x + 2
+  int src, dst;    // first piece: offset in a plane of a component (-1: none), ring index
+  int esrc, edst;  // edge value: offset in a plane (-1: none), ring index
+  bool wide;       // pieces of 16 bytes
+  bool valid;      // the lane's pair is a node pair
 };
-template <int TY>
-__device__ __forceinline__ RingLane ring_lane(const DevBox& B, const int4 td) {
+
+// Start of ring row r (0 .. RY - 1) of the tile in a plane, or -1: not read.
+__device__ __forceinline__ int ring_row(const DevBox& B, const int4 td, int vy, int r) {
+  if (r > vy + 1) return -1;
+  int y = td.z + r - 1;
+  y = y < 0 ? B.ny - 1 : (y >= B.ny ? 0 : y);
+  return B.nx * y;
+}
+
+// Components 0 .. NF - 1 of the ring are F's, the next NC - NF are G's.
+template <int NC, int TY, int NF>
+__device__ __forceinline__ RingLane ring_lane(const DevBox& B, const int4 td, const float* F, const float* G) {
+  using Rg = Ring<NC, TY>;
+  static_assert(16 * Rg::RY <= 32 * TY && 2 * NC <= 32, "one piece and one edge value per thread");
   RingLane R;
-  const int lane = threadIdx.x, nx = B.nx, ny = B.ny;
-  R.vx = min(64, nx - td.y);
-  R.vy = min(TY, ny - td.z);
+  const int lane = threadIdx.x, nx = B.nx, ny = B.ny, t = lane + 32 * (int)threadIdx.y;
+  const int vx = min(64, nx - td.y), vy = min(TY, ny - td.z);
   R.x = td.y + 2 * lane;
   R.y = td.z + (int)threadIdx.y;
   R.valid = R.x < nx && R.y < ny;
   R.row = nx * R.y;
-  R.rowm = nx * (td.z == 0 ? ny - 1 : td.z - 1);
-  R.rowp = nx * (td.z + R.vy >= ny ? 0 : td.z + R.vy);
-  R.edge = lane < 2 && R.y < ny;
-  R.rowe = R.row + (lane == 0 ? (td.y == 0 ? nx - 1 : td.y - 1) : (td.y + R.vx >= nx ? 0 : td.y + R.vx));
   R.li = lane == 0 ? 64 : 2 * lane - 1;
-  R.ri = 2 * lane + 2 >= R.vx ? 65 : 2 * lane + 2;
+  R.ri = 2 * lane + 2 >= vx ? 65 : 2 * lane + 2;
+  R.wide = (nx & 3) == 0 && ((reinterpret_cast<uintptr_t>(F) | reinterpret_cast<uintptr_t>(G)) & 15) == 0;
+  const int r = R.wide ? t >> 4 : t >> 5, c = R.wide ? 4 * (t & 15) : 2 * lane;
+  const int row = r < Rg::RY && c < vx ? ring_row(B, td, vy, r) : -1;
+  R.src = row < 0 ? -1 : row + td.y + c;
+  R.dst = r * Rg::PW + c;
+  const int k = t / (2 * TY), ry = (t >> 1) % TY, side = t & 1;
+  const int xe = side ? (td.y + vx >= nx ? 0 : td.y + vx) : (td.y == 0 ? nx - 1 : td.y - 1);
+  R.esrc = k < NC && ry < vy ? xe + nx * (td.z + ry) : -1;
+  R.edst = (k * Rg::RY + ry + 1) * Rg::PW + 64 + side;
   return R;
 }
 
-// Copies plane z (-1 .. nz; wrapped, or nothing beyond a wall) of components
-// k0 .. k0 + NF - 1 (field F, component stride N) into the ring.
+// Copies plane z (-1 .. nz; wrapped, or nothing beyond a wall) of all
+// components (strides N) into the ring.
 template <int NC, int TY, int NF>
-__device__ __forceinline__ void ring_load(float* ring, const DevBox& B, const RingLane& R, const float* __restrict__ F,
-                                          int k0, int z, int slot) {
+__device__ __forceinline__ void ring_load(float* ring, const DevBox& B, const RingLane& R, const int4 td,
+                                          const float* __restrict__ F, const float* __restrict__ G, int z, int slot) {
   using Rg = Ring<NC, TY>;
-  const int nz = B.nz, lane = threadIdx.x, wy = threadIdx.y;
+  const int nz = B.nz;
   if (B.wall_z && (z < 0 || z >= nz)) return;
   const size_t base = (size_t)B.nx * B.ny * (z < 0 ? z + nz : (z >= nz ? z - nz : z));
-  float* dst = ring + slot * Rg::PLANE + k0 * Rg::RY * Rg::PW;
-  const bool xin = R.x < B.nx;
+  const size_t N = (size_t)B.N;
+  float* dst = ring + slot * Rg::PLANE;
+  if (R.esrc >= 0) {
+    const int k = ((int)threadIdx.x + 32 * (int)threadIdx.y) / (2 * TY);
+    cp_async4(dst + R.edst, (k < NF ? F + k * N : G + (k - NF) * N) + base + R.esrc);
+  }
+  if (R.wide) {
+    if (R.src >= 0) {
+      const float* p = F + base + R.src;
+      const float* q = G + base + R.src;
 #pragma unroll
-  for (int k = 0; k < NF; ++k) {
-    const float* src = F + (size_t)k * B.N + base;
-    float* row = dst + (k * Rg::RY + wy + 1) * Rg::PW;
-    if (R.valid) cp_async8(row + 2 * lane, src + R.row + R.x);
-    if (R.edge) cp_async4(row + 64 + lane, src + R.rowe);
-    if (wy == (k0 + k) % TY && xin) {
-      cp_async8(dst + (k * Rg::RY) * Rg::PW + 2 * lane, src + R.rowm + R.x);
-      cp_async8(dst + (k * Rg::RY + R.vy + 1) * Rg::PW + 2 * lane, src + R.rowp + R.x);
+      for (int k = 0; k < NC; ++k)
+        cp_async16(dst + k * (Rg::RY * Rg::PW) + R.dst, k < NF ? p + k * N : q + (k - NF) * N);
     }
+  } else {
+    const int vx = min(64, B.nx - td.y), vy = min(TY, B.ny - td.z), c = 2 * (int)threadIdx.x;
+    if (c < vx)
+#pragma unroll 1
+      for (int e = threadIdx.y; e < NC * (vy + 2); e += TY) {
+        const int k = e / (vy + 2), r = e % (vy + 2);
+        cp_async8(dst + (k * Rg::RY + r) * Rg::PW + c,
+                  (k < NF ? F + k * N : G + (k - NF) * N) + base + ring_row(B, td, vy, r) + td.y + c);
+      }
   }
 }
 
@@ -1222,14 +1265,6 @@ __device__ __forceinline__ void ring_gather(const float* ring, const RingLane& R
 
 __device__ __forceinline__ bool plain_node(unsigned m) { return (m & (IDMASK | NEAR)) == 0; }
 
-// Store v for the nodes of a pair that the tile path evaluates (a: the first,
-// b: the second).
-__device__ __forceinline__ void st2_keep_if(float* p, f2 v, bool a, bool b, uint64_t pol) {
-  if (a && b) st2_keep(p, v, pol);
-  else if (a) st_hint(p, v.v.x, pol);
-  else if (b) st_hint(p + 1, v.v.y, pol);
-}
-
 // Stress of a tile of plain nodes, two nodes per lane, Q from the ring.
 template <int TY, bool FE>
 __device__ __forceinline__ void stress_ring(const DevBox& B, const LcK<f2>& K2, const int4 td, int zc, int mode,
@@ -1238,7 +1273,7 @@ __device__ __forceinline__ void stress_ring(const DevBox& B, const LcK<f2>& K2, 
   const float* __restrict__ Q = static_cast<const float*>(B.Q[B.st->qpar]);
   float* __restrict__ Hb = static_cast<float*>(B.H);
   float* __restrict__ Pb = static_cast<float*>(B.P);
-  const RingLane R = ring_lane<TY>(B, td);
+  const RingLane R = ring_lane<5, TY, 5>(B, td, Q, Q);
   const int nz = B.nz, zend = min(td.w + zc, nz);
   const size_t N = (size_t)B.N;
   const uint64_t keep = l2_keep();
@@ -1247,7 +1282,7 @@ __device__ __forceinline__ void stress_ring(const DevBox& B, const LcK<f2>& K2, 
   const int plane = B.nx * B.ny;
   __syncthreads();  // the ring's last reads (previous tile) are done
 #pragma unroll 1
-  for (int k = -1; k <= 1; ++k) ring_load<5, TY, 5>(ring, B, R, Q, 0, td.w + k, (k + 1) & 3);
+  for (int k = -1; k <= 1; ++k) ring_load<5, TY, 5>(ring, B, R, td, Q, Q, td.w + k, (k + 1) & 3);
   cp_async_commit();
   unsigned m2 = R.valid ? (unsigned)*reinterpret_cast<const uint16_t*>(mp + (size_t)plane * td.w) : 0x0101u;
   for (int z = td.w; z < zend; ++z) {
@@ -1256,7 +1291,7 @@ __device__ __forceinline__ void stress_ring(const DevBox& B, const LcK<f2>& K2, 
     __syncthreads();
     const bool pa = plain_node(m2 & 0xffu), pb = plain_node(m2 >> 8);
     if (z + 1 < zend) {
-      ring_load<5, TY, 5>(ring, B, R, Q, 0, z + 2, (s0 + 2) & 3);
+      ring_load<5, TY, 5>(ring, B, R, td, Q, Q, z + 2, (s0 + 2) & 3);
       if (R.valid) m2 = (unsigned)*reinterpret_cast<const uint16_t*>(mp + (size_t)plane * (z + 1));
     }
     cp_async_commit();
@@ -1277,11 +1312,21 @@ __device__ __forceinline__ void stress_ring(const DevBox& B, const LcK<f2>& K2, 
       if (pb) fe += f32_to_f64(fp.v.y);
     }
     const size_t i = (size_t)R.x + R.row + (size_t)plane * z;
+    if (pa && pb) {
 #pragma unroll
-    for (int c = 0; c < 5; ++c) st2_keep_if(Hb + c * N + i, h[c], pa, pb, keep);
-    if (store_p) {  // with the flow frozen only exports read the stress
+      for (int c = 0; c < 5; ++c) st2_keep(Hb + c * N + i, h[c], keep);
+      if (store_p) {  // with the flow frozen only exports read the stress
 #pragma unroll
-      for (int c = 0; c < 9; ++c) st2_keep_if(Pb + c * N + i, p[c], pa, pb, keep);
+        for (int c = 0; c < 9; ++c) st2_keep(Pb + c * N + i, p[c], keep);
+      }
+    } else {  // one node of the pair is a near or solid node
+      const size_t j = i + (pa ? 0 : 1);
+#pragma unroll
+      for (int c = 0; c < 5; ++c) st_hint(Hb + c * N + j, pa ? h[c].v.x : h[c].v.y, keep);
+      if (store_p) {
+#pragma unroll
+        for (int c = 0; c < 9; ++c) st_hint(Pb + c * N + j, pa ? p[c].v.x : p[c].v.y, keep);
+      }
     }
   }
 }
@@ -2137,22 +2182,28 @@ __device__ __forceinline__ void colloid_box(const DevBox& B, bool commit = true)
 // their residual.
 __device__ __forceinline__ void store_pair(float* q, __nv_bfloat16* l, size_t N, const f2 qi[5], const f2 lo[5],
                                            const f2 d5[5], bool pa, bool pb, float& rsum, float& rmax) {
+  f2 hn[5];
+  __nv_bfloat162 l2[5];
 #pragma unroll
   for (int k = 0; k < 5; ++k) {
     const f2 sv = lo[k] + d5[k];
-    const f2 hn = qi[k] + sv;
-    const f2 bb = hn - qi[k];
-    const f2 err = (qi[k] - (hn - bb)) + (sv - bb);
-    const __nv_bfloat162 l2 = __float22bfloat162_rn(err.v);
-    if (pa && pb) {
-      st2(q + k * N, hn);
-      *reinterpret_cast<__nv_bfloat162*>(l + k * N) = l2;
-    } else if (pa) {
-      q[k * N] = hn.v.x;
-      l[k * N] = l2.x;
-    } else {
-      q[k * N + 1] = hn.v.y;
-      l[k * N + 1] = l2.y;
+    hn[k] = qi[k] + sv;
+    const f2 bb = hn[k] - qi[k];
+    const f2 err = (qi[k] - (hn[k] - bb)) + (sv - bb);
+    l2[k] = __float22bfloat162_rn(err.v);
+  }
+  if (pa && pb) {
+#pragma unroll
+    for (int k = 0; k < 5; ++k) {
+      st2(q + k * N, hn[k]);
+      *reinterpret_cast<__nv_bfloat162*>(l + k * N) = l2[k];
+    }
+  } else {
+    const int o = pa ? 0 : 1;
+#pragma unroll
+    for (int k = 0; k < 5; ++k) {
+      q[k * N + o] = pa ? hn[k].v.x : hn[k].v.y;
+      l[k * N + o] = pa ? l2[k].x : l2[k].y;
     }
   }
   const f2 dzz = -(d5[0] + d5[3]);
@@ -2190,16 +2241,13 @@ __device__ __forceinline__ void lc_ring(const DevBox& B, const LcK<f2>& K2, cons
   __nv_bfloat16* __restrict__ Lout = B.Qlo[qpar ^ 1];
   const float* __restrict__ U = static_cast<const float*>(B.u);
   const float* __restrict__ Hb = static_cast<const float*>(B.H);
-  const RingLane R = ring_lane<TY>(B, td);
+  const RingLane R = ring_lane<8, TY, 5>(B, td, Q, U);
   const int nz = B.nz, zend = min(td.w + zc, nz), plane = B.nx * B.ny;
   const size_t N = (size_t)B.N;
   const uint8_t* mp = B.mask + R.x + R.row;
   __syncthreads();
 #pragma unroll 1
-  for (int k = -1; k <= 1; ++k) {
-    ring_load<8, TY, 5>(ring, B, R, Q, 0, td.w + k, (k + 1) & 3);
-    ring_load<8, TY, 3>(ring, B, R, U, 5, td.w + k, (k + 1) & 3);
-  }
+  for (int k = -1; k <= 1; ++k) ring_load<8, TY, 5>(ring, B, R, td, Q, U, td.w + k, (k + 1) & 3);
   cp_async_commit();
   unsigned m2 = R.valid ? (unsigned)*reinterpret_cast<const uint16_t*>(mp + (size_t)plane * td.w) : 0x0101u;
   for (int z = td.w; z < zend; ++z) {
@@ -2218,8 +2266,7 @@ __device__ __forceinline__ void lc_ring(const DevBox& B, const LcK<f2>& K2, cons
     cp_async_wait0();
     __syncthreads();
     if (z + 1 < zend) {
-      ring_load<8, TY, 5>(ring, B, R, Q, 0, z + 2, (s0 + 2) & 3);
-      ring_load<8, TY, 3>(ring, B, R, U, 5, z + 2, (s0 + 2) & 3);
+      ring_load<8, TY, 5>(ring, B, R, td, Q, U, z + 2, (s0 + 2) & 3);
       if (R.valid) m2 = (unsigned)*reinterpret_cast<const uint16_t*>(mp + (size_t)plane * (z + 1));
     }
     cp_async_commit();
@@ -2387,14 +2434,14 @@ __device__ __forceinline__ void relax_ring(const DevBox& B, const LcK<f2>& K2, c
   float* __restrict__ Qo = static_cast<float*>(B.Q[qpar ^ 1]);
   const __nv_bfloat16* __restrict__ Lin = B.Qlo[qpar];
   __nv_bfloat16* __restrict__ Lout = B.Qlo[qpar ^ 1];
-  const RingLane R = ring_lane<TY>(B, td);
+  const RingLane R = ring_lane<5, TY, 5>(B, td, Q, Q);
   const int zend = min(td.w + zc, B.nz), plane = B.nx * B.ny;
   const size_t N = (size_t)B.N;
   const bool chiral = B.p.q0 != 0.0;
   const uint8_t* mp = B.mask + R.x + R.row;
   __syncthreads();
 #pragma unroll 1
-  for (int k = -1; k <= 1; ++k) ring_load<5, TY, 5>(ring, B, R, Q, 0, td.w + k, (k + 1) & 3);
+  for (int k = -1; k <= 1; ++k) ring_load<5, TY, 5>(ring, B, R, td, Q, Q, td.w + k, (k + 1) & 3);
   cp_async_commit();
   unsigned m2 = R.valid ? (unsigned)*reinterpret_cast<const uint16_t*>(mp + (size_t)plane * td.w) : 0x0101u;
   for (int z = td.w; z < zend; ++z) {
@@ -2409,7 +2456,7 @@ __device__ __forceinline__ void relax_ring(const DevBox& B, const LcK<f2>& K2, c
     cp_async_wait0();
     __syncthreads();
     if (z + 1 < zend) {
-      ring_load<5, TY, 5>(ring, B, R, Q, 0, z + 2, (s0 + 2) & 3);
+      ring_load<5, TY, 5>(ring, B, R, td, Q, Q, z + 2, (s0 + 2) & 3);
       if (R.valid) m2 = (unsigned)*reinterpret_cast<const uint16_t*>(mp + (size_t)plane * (z + 1));
     }
     cp_async_commit();

@@ -1,6 +1,6 @@
 """Step kernels at the edges of their tiles against the FP64 oracle: widths around the 64-column tiles of the
-two-node path, a two-node-wide box, odd widths (one node per lane), ragged heights, boxes one to three planes deep,
-walls, near-node lists that fill less than a group of 32 and several groups, and boxes without any near node.
+two-node path, rows of whole 16-byte pieces and others, a two-node-wide box, odd widths (one node per lane), ragged
+heights, boxes one to three planes deep, walls, near-node lists that fill less than a group of 32 and several groups, and boxes without any near node.
 Tolerances as the other parity tests (FP32 storage 1e-5 in Q, 1e-6 in u; FP64 1e-10, 1e-12)."""
 import numpy as np
 import pytest
@@ -13,7 +13,8 @@ pytestmark = pytest.mark.gpu
 CASES = [((64, 9, 3), False, None), ((66, 7, 5), False, (20.3, 3.1, 2.2, 1.6)), ((62, 5, 33), False, (30.2, 2.4, 15.7, 2.3)),
          ((130, 6, 10), True, (64.4, 2.9, 4.6, 2.6)), ((2, 3, 4), False, None), ((4, 1, 1), False, None),
          ((12, 10, 2), False, None), ((68, 12, 1), False, None), ((33, 17, 9), True, (15.1, 8.3, 4.4, 3.2)),
-         ((1, 2, 3), False, None), ((20, 33, 18), False, (10.2, 16.4, 8.9, 7.1))]
+         ((1, 2, 3), False, None), ((20, 33, 18), False, (10.2, 16.4, 8.9, 7.1)),
+         ((132, 7, 6), True, (66.1, 3.2, 2.7, 1.9)), ((36, 2, 5), False, None), ((128, 10, 4), False, (1.2, 9.1, 2.1, 1.7))]
 
 
 @pytest.mark.parametrize("L,wall,col", CASES)
