@@ -1,13 +1,17 @@
 // lclb_kernels.cu -- sm_103a kernels of one coupled step (Lintuvuori et al., Sec. 2.2):
-//   k_force   LC stress at fluid nodes, its face divergence (body force) and the
-//             colloid LC force/torque (Eqs. 4, 8); z-marching tiles with the
-//             stress of three planes in shared memory.
-//   k_lb      pull-scheme stream + BGK collide with Guo forcing, bounce-back on
-//             links inline (moving-surface term), writes df* and u.
+//   k_stress  molecular field H and stress P of every fluid node, stored, and
+//             the colloid LC force/torque (Eqs. 4, 8).
+//   k_lbp     pull-scheme stream + BGK collide with Guo forcing, bounce-back on
+//             links inline (moving-surface term), body force from the stored P;
+//             writes df* and u.
 //   k_lc      Beris-Edwards update of Q (Eq. 2 with co-rotation and upwind
-//             advective face fluxes), residual partials.
-//   k_links   momentum exchange over the boundary-link list -> F_hyd, T_hyd.
-//   k_colloid colloid update and buffer-parity flip.
+//             advective face fluxes), residual partials, momentum exchange over
+//             the boundary links -> F_hyd, T_hyd, colloid update and
+//             buffer-parity flip.
+//   k_relax   the whole step when the flow is frozen.
+// Other variants of the step: k_flb (stress and LB fused), k_force + k_lb (body
+// force stored), k_step (all phases in one launch), and k_links and k_colloid,
+// the last two parts of k_lc as launches of their own.
 // All step kernels walk a work list of (box, x0, y0, z0) tiles, so that one
 // launch serves one box or a batch of boxes of different sizes.
 #include <cstdio>
@@ -204,14 +208,13 @@ __device__ __forceinline__ void load_box(DevBox& sb, LcK<f2>& k2, const DevBox* 
 // Q update of the same step.
 template <typename T>
 __device__ __forceinline__ uint8_t stress_at(const DevBox& B, const PhysT<T>& PP, const T* __restrict__ Q, int gx,
-                                             int gy, int kk, T* sP, int HP, bool fe, double* fe_acc, T* hout) {
+                                             int gy, int kk, T* sP, int HP, T* hout) {
   const int i = gx + B.nx * (gy + B.ny * kk);
   const uint8_t m = B.mask[i];
   const uint8_t flag = m & IDMASK;
   if (flag != 0) return flag;
   T qi[5], qn[6][5], h[5], p[9], fp;
-  double surf = 0.0;
-  gather_q(B, Q, gx, gy, kk, i, m, qi, qn, fe ? &surf : nullptr);
+  gather_q(B, Q, gx, gy, kk, i, m, qi, qn, nullptr);
   lc_node<T>(B, qi, qn, h, p, &fp);
 #pragma unroll
   for (int c = 0; c < 9; ++c) sP[c * HP] = p[c];
@@ -219,7 +222,6 @@ __device__ __forceinline__ uint8_t stress_at(const DevBox& B, const PhysT<T>& PP
 #pragma unroll
     for (int c = 0; c < 5; ++c) hout[(size_t)c * B.N + i] = h[c];
   }
-  if (fe) *fe_acc += (double)fp + surf;
   return 0;
 }
 
@@ -281,7 +283,7 @@ __device__ __forceinline__ void face_force(const DevBox& B, const T* sP, const u
 }
 
 // ---------------------------------------------------------------------------
-// k_force: body force (and, in diagnostic mode, free-energy partials) alone
+// k_force: body force alone
 // ---------------------------------------------------------------------------
 // Shared memory: P of three z planes over the tile plus a one-node halo,
 // [3][9][(TX+2)(TY+2)] in T, then one flag byte per position.
@@ -293,7 +295,6 @@ __global__ void __launch_bounds__(TX * TY) k_force(const DevBox* __restrict__ bo
   T* sP = reinterpret_cast<T*>(smem_raw);
   uint8_t* sFl = smem_raw + sizeof(T) * 27 * HP;
   __shared__ DevBox B;
-  __shared__ double sred[32 * 1];
   const int tid = threadIdx.x + TX * threadIdx.y;
 
   int cur_box = -1;
@@ -310,7 +311,6 @@ __global__ void __launch_bounds__(TX * TY) k_force(const DevBox* __restrict__ bo
     const int nx = B.nx, ny = B.ny, nz = B.nz, N = B.N;
     const int vx = min(TX, nx - x0), vy = min(TY, ny - y0);
     const int zend = min(z0 + zc, nz);
-    double fe_acc = 0.0;
     __syncthreads();
     for (int k = z0 - 1; k <= zend; ++k) {
       const int slot = (k - z0 + 1) % 3;
@@ -323,7 +323,7 @@ __global__ void __launch_bounds__(TX * TY) k_force(const DevBox* __restrict__ bo
         if (!wallplane) {
           const bool inner = hx >= 1 && hx <= vx && hy >= 1 && hy <= vy && k >= z0 && k < zend;
           flag = stress_at(B, PP, Q, wrapn(x0 - 1 + hx, nx), wrapn(y0 - 1 + hy, ny), kk, sP + slot * 9 * HP + pidx,
-                           HP, inner && (mode & FORCE_FE), &fe_acc, inner ? static_cast<T*>(B.H) : (T*)nullptr);
+                           HP, inner ? static_cast<T*>(B.H) : (T*)nullptr);
         }
         sFl[slot * HP + pidx] = flag;
       }
@@ -344,11 +344,6 @@ __global__ void __launch_bounds__(TX * TY) k_force(const DevBox* __restrict__ bo
       __syncthreads();
     }
     if (mode & FORCE_ACC) warp_flush_colloid(B.col, my_c, my_acc, 6);
-    if (mode & FORCE_FE) {
-      double v[1] = {fe_acc};
-      block_sum<1>(v, sred);
-      if (tid == 0) part[t] = v[0];
-    }
   }
 }
 
@@ -1374,6 +1369,15 @@ __device__ __forceinline__ void block_fe(double fe, double* out) {
 // H and P stored once per fluid node, and the colloid LC force from the near
 // nodes.  FE (diagnostics): the free energy of each tile into part and of each
 // block of near groups into L.fepart.
+// FP32 tiles of even width: two nodes per lane from the ring, packed arithmetic
+// (about 450 of them, 2 cycles each, and as many other instructions a pair), 16
+// warps per SM at 128 registers; bound by issue and by the FP32 pipe, for 48
+// bytes a node of traffic.  One or two rows of a tile per thread, and 168
+// registers with fewer warps, measured the same or slower.  FP64: bound by the
+// FP64 pipe (84 % busy).  Near groups: a chain of FP64 surface values, 64 cycles
+// an instruction and warp, spread over all SMs.  128^3 with one
+// colloid: near nodes queued by tiles and Q by shuffles and loads 75 us, near
+// groups and the ring 58, its copies in 16-byte pieces 44.
 template <typename T, int TY, bool FE>
 __global__ void __launch_bounds__(TX * TY, (sizeof(T) == 4 ? 512 : 256) / (TX * TY)) k_stress(Launch L, int mode,
                                                                                              double* __restrict__ part) {
@@ -1548,6 +1552,12 @@ __device__ __forceinline__ void near_lbp(const DevBox& B, int j) {
                     j / (B.nx * B.ny), j, B.mask[j], B.st->pre_valid != 0, B.p.lc_on != 0);
 }
 
+// Bound by the memory system: 38 population streams of 4 bytes a node, 18
+// stress values and 3 velocities: 159 MB of populations read and written and 75
+// MB of stress at 128^3 (70 us under the profiler, 5.0 TB/s; 79 in the step).  What hides the
+// latency is warps: 64 registers for 32 warps per SM 77 us, 80 registers 87, 48
+// registers 88.  The rows of the next plane staged in shared memory by 16-byte
+// asynchronous copies, which leaves 20 warps per SM: 94.
 template <typename T, int TY>
 __global__ void __launch_bounds__(TX * TY, (sizeof(T) == 4 ? 1024 : 384) / (TX * TY)) k_lbp(Launch L) {
   __shared__ DevBox B;
@@ -1625,11 +1635,10 @@ __global__ void __launch_bounds__(32 * (BY + 3), (sizeof(T) == 4 && BY <= 4) ? 2
       if (lc && mypos) {
         const bool wallplane = B.wall_z && (k < 0 || k >= nz);
         const int kk = B.wall_z ? k : wrapn(k, nz);
-        double dummy = 0.0;
         const bool inner = hx >= 1 && hx <= vx && hy >= 1 && hy <= vy && k >= z0 && k < zend;
         sFl[slot * HP + pidx] =
             wallplane ? WALLFLAG
-                      : stress_at(B, PP, Q, gx, gy, kk, sP + slot * 9 * HP + pidx, HP, false, &dummy,
+                      : stress_at(B, PP, Q, gx, gy, kk, sP + slot * 9 * HP + pidx, HP,
                                   inner ? static_cast<T*>(B.H) : (T*)nullptr);
       }
       __syncthreads();
@@ -2369,6 +2378,12 @@ __device__ __forceinline__ void lc_commit(const Launch& L, int b, unsigned n) {
   __syncthreads();
 }
 
+// Q update of all nodes, link exchange and colloid update.  FP32 tiles of even
+// width: as k_stress, Q and u from the ring (8 components), H and the remainder
+// of Q loaded per pair ahead of the plane's barrier; 128 registers, one
+// component's neighbours read at a time (all at once spill).  Bound by issue:
+// 128^3 67 + 16 us (links) + 6 (colloid) at the start, 53 us for all of it now;
+// 256 x 192 x 160 162 us.
 template <typename T, int TY>
 __global__ void __launch_bounds__(TX * TY, (sizeof(T) == 4 ? 512 : 256) / (TX * TY)) k_lc(Launch L, int mode,
                                                                                          double* __restrict__ part) {
@@ -2425,7 +2440,9 @@ __global__ void __launch_bounds__(TX * TY, (sizeof(T) == 4 ? 512 : 256) / (TX * 
 // flux, so H is used where it is formed and each node moves its Q twice (60
 // bytes with the remainder) instead of the 190 of the separate stress and Q
 // update.  Near nodes still take their stress for the colloid's LC force.
-// Bound by issue of the molecular field (about 130 packed operations a pair).
+// Bound by issue of the molecular field (about 130 packed operations a pair);
+// 96^3: 105 us for the launches of the general step, 69 without its stores and
+// loads, 30 as one launch, 22 with the ring copied in 16-byte pieces.
 template <int TY>
 __device__ __forceinline__ void relax_ring(const DevBox& B, const LcK<f2>& K2, const int4 td, int zc, float* ring,
                                            float& rsum, float& rmax) {
