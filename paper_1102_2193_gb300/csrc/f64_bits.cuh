@@ -16,6 +16,19 @@ __device__ __forceinline__ double f32_to_f64(float x) {
   return __hiloint2double((int)hi, (int)(u << 29));
 }
 
+// s 2^-k rounded to nearest even (|k| < 900: the result is normal).
+__device__ __forceinline__ double fixed_to_f64(long long s, int k) {
+  if (s == 0) return 0.0;
+  unsigned long long u = s < 0 ? 0ull - (unsigned long long)s : (unsigned long long)s;
+  const int lz = __clzll((long long)u);
+  u <<= lz;
+  const unsigned rem = (unsigned)u & 0x7ffu;
+  unsigned long long m = u >> 11;
+  m += rem > 0x400u || (rem == 0x400u && (m & 1ull)) ? 1ull : 0ull;
+  m += (unsigned long long)(1085 - lz - k) << 52;  // the mantissa's leading one adds 1 to the exponent
+  return __longlong_as_double((long long)(m | ((unsigned long long)s & 0x8000000000000000ull)));
+}
+
 // x 2^k as a 64-bit integer, |x| 2^k < 2^57, bits below 1 dropped.
 __device__ __forceinline__ long long f32_to_fixed(float x, int k) {
   const unsigned u = __float_as_uint(x), e = (u >> 23) & 0xffu;

@@ -293,26 +293,38 @@ __device__ __forceinline__ void pair_moments(const V v[NQ], S& sum, S m[3]) {
 __device__ __forceinline__ void moments_f64(const double df[NQ], double& drho, double m[3]) {
   pair_moments<double>(df, drho, m);
 }
-// FP32 deviations: added as 64-bit integers at 2^-57 of the largest, which
-// loses less than FP64 additions (2^-53 of the partial sums) and takes 4 FP64
-// operations instead of 58; infinities and NaN take the FP64 sums.
-__device__ __forceinline__ void moments_f64(const float df[NQ], double& drho, double m[3]) {
+// FP32 deviations: added as 64-bit integers at 2^-56 of the largest, which
+// loses less than FP64 additions (2^-53 of the partial sums), and rounded to
+// FP64 by integer instructions: no FP64 operation where there were 58, then 4
+// and 4 conversions; infinities and NaN take the FP64 sums.
+// F: a force whose half is added to the momentum.
+__device__ __forceinline__ void moments_f64(const double df[NQ], const double F[3], double& drho, double m[3]) {
+  pair_moments<double>(df, drho, m);
+  for (int a = 0; a < 3; ++a) m[a] += 0.5 * F[a];
+}
+__device__ __forceinline__ void moments_f64(const float df[NQ], const float F[3], double& drho, double m[3]) {
   unsigned top = 0;
 #pragma unroll
   for (int q = 0; q < NQ; ++q) top = max(top, __float_as_uint(df[q]) & 0x7fffffffu);
+#pragma unroll
+  for (int a = 0; a < 3; ++a) top = max(top, __float_as_uint(F[a]) & 0x7fffffffu);
   if (top >= 0x7f800000u) {
     pair_moments<double>(df, drho, m);
+    for (int a = 0; a < 3; ++a) m[a] += 0.5 * (double)F[a];
     return;
   }
-  const int k = 183 - (int)(top >> 23);  // |df| 2^k < 2^57, so 19 of them fit 63 bits
+  const int k = 182 - (int)(top >> 23);  // |df| 2^k < 2^56: 20 of them and the force fit 63 bits
   long long v[NQ], s, ms[3];
 #pragma unroll
   for (int q = 0; q < NQ; ++q) v[q] = f32_to_fixed(df[q], k);
   pair_moments<long long>(v, s, ms);
-  const double inv = __hiloint2double((1023 - k) << 20, 0);
-  drho = (double)s * inv;
+  drho = fixed_to_f64(s, k);
 #pragma unroll
-  for (int a = 0; a < 3; ++a) m[a] = (double)ms[a] * inv;
+  for (int a = 0; a < 3; ++a) m[a] = fixed_to_f64(ms[a] + f32_to_fixed(F[a], k - 1), k);
+}
+__device__ __forceinline__ void moments_f64(const float df[NQ], double& drho, double m[3]) {
+  const float none[3] = {0.f, 0.f, 0.f};
+  moments_f64(df, none, drho, m);
 }
 
 // The stored Q of node i rounded to FP32 (for decisions taken in FP32).

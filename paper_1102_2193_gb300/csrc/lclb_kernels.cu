@@ -2946,13 +2946,15 @@ __global__ void __launch_bounds__(256) k_export_q(const DevBox* __restrict__ box
   }
 }
 
-__device__ __forceinline__ double half_f64(float v) { return f32_to_f64(0.5f * v); }
-__device__ __forceinline__ double half_f64(double v) { return 0.5 * v; }
-
 // Other fields.  which: LC_F_PRE, LC_RHO, LC_U, LC_FORCE, LC_SOLID.  The force
 // is the face divergence of the stored stress, as the LB kernel takes it.
+// Velocity from FP32 storage: 37 loads a node, so 64 registers for 32 warps per
+// SM (98 registers: 16 warps), and 8 FP64 operations a node with the half force
+// added among the integers (23 with conversions before): 256 x 192 x 160 694 ->
+// 364 us (a quarter more than the LB kernel, which loads the same), 128^3 189 ->
+// 98.
 template <typename T>
-__global__ void __launch_bounds__(256) k_export(const DevBox* __restrict__ boxes, int b, int which,
+__global__ void __launch_bounds__(256, sizeof(T) == 4 ? 4 : 2) k_export(const DevBox* __restrict__ boxes, int b, int which,
                                                 double* __restrict__ out) {
   const DevBox& B = boxes[b];
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
@@ -2992,7 +2994,7 @@ __global__ void __launch_bounds__(256) k_export(const DevBox* __restrict__ boxes
     return;
   }
   double drho, mm[3];
-  moments_f64(df, drho, mm);
+  moments_f64(df, F, drho, mm);
   const double rho = B.p.rho0 + drho;
   if (which == EXP_RHO) {
     out[i] = rho;
@@ -3010,7 +3012,7 @@ __global__ void __launch_bounds__(256) k_export(const DevBox* __restrict__ boxes
   }
   const bool forced = B.p.g[0] != 0.0 || B.p.g[1] != 0.0 || B.p.g[2] != 0.0;
   for (int a = 0; a < 3; ++a) {
-    double m = mm[a] + half_f64(F[a]);
+    double m = mm[a];
     if (forced) m += 0.5 * B.p.g[a];
     out[(size_t)a * N + i] = m * inv;
   }
@@ -3022,9 +3024,10 @@ __global__ void __launch_bounds__(256) k_export(const DevBox* __restrict__ boxes
 // nodes before the block reduction, and the defect test runs in FP32 except at nodes too
 // close to the threshold (with the closed-form eigenvalue in FP64 at every
 // node and 19 x 4 products: 1102 us at 128^3).
+// (FP32: 64 registers, 32 warps per SM, 158 -> 115 us at 128^3.)
 constexpr int DIAG_PER = 4;
 template <typename T>
-__global__ void __launch_bounds__(256) k_diag_state(const DevBox* __restrict__ boxes, int b, double* __restrict__ part) {
+__global__ void __launch_bounds__(256, sizeof(T) == 4 ? 4 : 2) k_diag_state(const DevBox* __restrict__ boxes, int b, double* __restrict__ part) {
   const DevBox& B = boxes[b];
   double v[6] = {0, 0, 0, 0, 0, 0};
   __shared__ double sred[32 * 6];

@@ -63,3 +63,28 @@ def test_surface_values_far_from_origin(anchoring, w):
     a, b = s.colloid(0), o.colloid(0)
     assert np.abs(a["F_lc"] - b["F_lc"]).max() <= 2e-5 * np.abs(b["F_lc"]).max()
     assert np.abs(a["T_lc"] - b["T_lc"]).max() <= 1e-4 * a0 * np.abs(b["F_lc"]).max()
+
+
+@pytest.mark.parametrize("scale", [0.0, 1e-12, 1e-3, 1.0, 1e6])
+@pytest.mark.parametrize("prec", ["f32", "f64"])
+def test_exported_moments(scale, prec):
+    """Density and velocity of populations of mixed magnitudes (the FP32 kernel adds them as integers at a common
+    exponent) against FP64 sums of the exported populations.  Tolerance: 19 roundings of f, 18 of the sum and 3 of the
+    quotient, 2^-53 of the sum of |f| each."""
+    import paper_1102_2193_gb300 as P
+    rng = np.random.default_rng(3)
+    L = (33, 9, 5)
+    d = rng.random((19, L[2], L[1], L[0])) * 10.0 ** rng.integers(-6, 1, (19, 1, L[1], L[0]))
+    s = P.Solver(*L, precision=P.LC_FP32 if prec == "f32" else P.LC_FP64, **synth.NEMATIC)
+    s.set_Q(np.zeros((5, L[2], L[1], L[0])))
+    w = oracle.feq(1.0, (0, 0, 0)).reshape(19, 1, 1, 1)
+    c = np.array([[0, 0, 0], [1, 0, 0], [-1, 0, 0], [0, 1, 0], [0, -1, 0], [0, 0, 1], [0, 0, -1], [1, 1, 0], [-1, -1, 0],
+                  [1, -1, 0], [-1, 1, 0], [1, 0, 1], [-1, 0, -1], [1, 0, -1], [-1, 0, 1], [0, 1, 1], [0, -1, -1],
+                  [0, 1, -1], [0, -1, 1]], dtype=float)
+    s.set_f(w * (1.0 + scale * d))
+    f, (rho, u) = s.get_f(), s.get_rho_u()
+    total = np.abs(f).sum(0)
+    eps = 40 * 2.0**-53
+    assert (np.abs(rho - f.sum(0)) <= eps * total).all()
+    m = np.einsum("qa,qzyx->azyx", c, f)
+    assert (np.abs(u - m / f.sum(0)) <= 2 * eps * total / f.sum(0)).all()
