@@ -252,7 +252,10 @@ int lc_lb_diagnostics_noalloc(lc_lb* h, lc_diag* out);
  * stress kernel stores H and P, the LB kernel takes the face divergence of
  * the stored P) and [6], [7] the milliseconds of its two kernels (fused:
  * [7] = 0).  LCLB_VARIANT=fused|split|stored in the environment overrides the
- * tuned variant.  The state advances by nsteps.  Synchronises. */
+ * tuned variant.  The link exchange and the colloid update, which the stored
+ * variant's step runs inside the Q update's launch, are launches of their own
+ * here; with the flow frozen [1] is the one launch of the whole step.  The
+ * state advances by nsteps.  Synchronises. */
 int lc_lb_profile(lc_lb* h, int nsteps, double ms_out[5]);
 int lc_lb_batch_profile(lc_lb_batch* b, int nsteps, double ms_out[5]);
 int lc_lb_profile_detail(lc_lb* h, int nsteps, double ms_out[8]);

@@ -1369,10 +1369,10 @@ __device__ __forceinline__ void block_fe(double fe, double* out) {
 // H and P stored once per fluid node, and the colloid LC force from the near
 // nodes.  FE (diagnostics): the free energy of each tile into part and of each
 // block of near groups into L.fepart.
-// FP32 tiles of even width: two nodes per lane from the ring, packed arithmetic
-// (about 450 of them, 2 cycles each, and as many other instructions a pair), 16
-// warps per SM at 128 registers; bound by issue and by the FP32 pipe, for 48
-// bytes a node of traffic.  One or two rows of a tile per thread, and 168
+// FP32 tiles of even width: two nodes per lane from the ring, packed arithmetic,
+// 597 instructions a pair and warp, 16 warps per SM at 128 registers; bound by
+// issue and by the FP32 pipe, which a packed instruction holds for two cycles
+// (76 bytes a node: 23 us at 128^3).  One or two rows of a tile per thread, and 168
 // registers with fewer warps, measured the same or slower.  FP64: bound by the
 // FP64 pipe (84 % busy).  Near groups: a chain of FP64 surface values, 64 cycles
 // an instruction and warp, spread over all SMs.  128^3 with one
@@ -3021,13 +3021,14 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 4 : 2) k_export(const De
 // Diagnostics per block: [0] sum(df), [1..3] sum(df c), [4] fluid nodes,
 // [5] defect nodes (3/2 lambda_max(Q) < 0.435).  Bound by FP64 issue: the
 // moments of FP32 populations are summed as integers, a thread sums DIAG_PER
-// nodes before the block reduction, and the defect test runs in FP32 except at nodes too
-// close to the threshold (with the closed-form eigenvalue in FP64 at every
-// node and 19 x 4 products: 1102 us at 128^3).
-// (FP32: 64 registers, 32 warps per SM, 158 -> 115 us at 128^3.)
+// nodes before the block reduction, and the defect test runs in FP32 except at
+// nodes too close to the threshold (with the closed-form eigenvalue in FP64 at
+// every node and 19 x 4 products: 1102 us at 128^3).  At 64 registers 32 warps
+// fit an SM: 158 -> 115 us at 128^3.
 constexpr int DIAG_PER = 4;
 template <typename T>
-__global__ void __launch_bounds__(256, sizeof(T) == 4 ? 4 : 2) k_diag_state(const DevBox* __restrict__ boxes, int b, double* __restrict__ part) {
+__global__ void __launch_bounds__(256, sizeof(T) == 4 ? 4 : 2) k_diag_state(const DevBox* __restrict__ boxes, int b,
+                                                                              double* __restrict__ part) {
   const DevBox& B = boxes[b];
   double v[6] = {0, 0, 0, 0, 0, 0};
   __shared__ double sred[32 * 6];
