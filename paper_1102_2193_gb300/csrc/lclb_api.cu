@@ -348,8 +348,9 @@ int build_totals(Group* g) {
 
 // Near-node list of box h after its geometry is built: static boxes get the
 // exact capacity, boxes with a mobile colloid a bound over its motion (near
-// nodes lie within sqrt 2 of the surface; a shell's nodes are at most the
-// volume of the shell widened by half a cell diagonal).
+// nodes lie within sqrt 2 of the surface, the other nodes of their pairs one
+// node further; a shell's nodes are at most the volume of the shell widened by
+// half a cell diagonal).
 // n: the near nodes that launch_near_list has counted.
 int build_near(lc_lb* h, int n) {
   Group* g = h->g;
@@ -359,7 +360,7 @@ int build_near(lc_lb* h, int n) {
   if (B.nmobile > 0) {
     double m = B.wall_z ? 2.0 * B.nx * B.ny : 0.0;
     for (const DevColloid& C : h->col) {
-      const double o = C.a0 + 2.4, i = std::max(0.0, C.a0 - 0.9);
+      const double o = C.a0 + (B.pair ? 3.4 : 2.4), i = std::max(0.0, C.a0 - 0.9);
       m += 4.0 / 3.0 * M_PI * (o * o * o - i * i * i) + 64.0;
     }
     bound = std::min((double)B.N, std::max(bound, m));
@@ -422,8 +423,9 @@ template <typename T>
 void fill_phys(PhysT<T>& o, const DevParams& p) {
   o.rho0 = (T)p.rho0;
   o.omega = (T)(1.0 / p.tau);
+  o.pref = (T)(1.0 - 0.5 / p.tau);
   o.ptau = (T)(p.tau - 0.5);
-  o.K = (T)p.K;
+  o.A0 = (T)p.A0; o.gamma = (T)p.gamma; o.K = (T)p.K; o.q0 = (T)p.q0; o.xi = (T)p.xi; o.Gamma = (T)p.Gamma;
   o.S0 = (T)p.S0;
   o.S0l = (T)(p.S0 - (double)o.S0);
   for (int a = 0; a < 3; ++a) o.g[a] = (T)p.g[a];
@@ -432,15 +434,14 @@ void fill_phys(PhysT<T>& o, const DevParams& p) {
 template <typename T>
 void fill_lck(LcK<T>& o, const DevParams& p) {
   const double A0g = p.A0 * p.gamma, lin = -p.A0 * (1.0 - p.gamma / 3.0) - 4.0 * p.K * p.q0 * p.q0;
-  o.A0g = (T)A0g; o.nA0g = (T)-A0g; o.nA3 = (T)(-A0g / 3.0); o.c_lin = (T)lin; o.c_lo = (T)(lin - 6.0 * p.K);
+  o.A0g = (T)A0g; o.nA0g = (T)-A0g; o.nA3 = (T)(-A0g / 3.0); o.c_lin = (T)lin;
   o.K = (T)p.K; o.nKq0 = (T)(-p.K * p.q0); o.n2Kq0 = (T)(-2.0 * p.K * p.q0); o.Kq0 = (T)(p.K * p.q0);
   o.f2c = (T)(0.5 * p.A0 * (1.0 - p.gamma / 3.0) + 2.0 * p.K * p.q0 * p.q0);
   o.f4c = (T)(0.25 * A0g); o.K8 = (T)(0.125 * p.K);
   o.xi2 = (T)(2.0 * p.xi); o.nt = (T)(-2.0 * p.xi / 3.0); o.nK4 = (T)(-0.25 * p.K);
   o.up = (T)(1.0 - p.xi); o.dn = (T)(-(1.0 + p.xi)); o.di = (T)(-2.0 * p.xi);
   o.Gamma = (T)p.Gamma; o.g0 = (T)(0.5 * p.xi); o.g1 = (T)(0.25 * (p.xi + 1.0)); o.g2 = (T)(0.25 * (p.xi - 1.0));
-  o.A2 = (T)(2.0 * A0g); o.nA2 = (T)(-2.0 * A0g);
-  o.two = (T)2; o.ntwo = (T)-2; o.third = (T)(1.0 / 3.0); o.nthird = (T)(-1.0 / 3.0); o.nsix = (T)-6; o.nhalf = (T)-0.5;
+  o.two = (T)2; o.ntwo = (T)-2; o.third = (T)(1.0 / 3.0); o.nthird = (T)(-1.0 / 3.0); o.nhalf = (T)-0.5;
 }
 
 // Allocate and initialise one box inside group g.
@@ -461,7 +462,6 @@ int make_box(Group* g, const lc_grid* G, const lc_params* p, lc_lb* h) {
   B.p.flow_on = p->flow_enabled ? 1 : 0;
   fill_phys(B.pf, B.p);
   fill_phys(B.pd, B.p);
-  fill_lck(B.kf, B.p);
   fill_lck(B.kd, B.p);
   for (int k = 0; k < 2; ++k) {
     B.f[k] = galloc(g, NQ * N * ts);

@@ -44,26 +44,23 @@ struct DevParams {
 // never convert from FP64 per node).
 template <typename T>
 struct PhysT {
-  T rho0, omega, ptau;  // rho0, 1/tau, (1 - 1/(2 tau)) tau = tau - 1/2
-  T K, S0, S0l;  // S0l: the part of S0 that FP32 drops
+  T rho0, omega, pref, ptau;  // rho0, 1/tau, 1 - 1/(2 tau), (1 - 1/(2 tau)) tau = tau - 1/2
+  T A0, gamma, K, q0, xi, Gamma;
+  T S0, S0l;  // S0l: the part of S0 that FP32 drops
   T g[3];
 };
 
-// Constants of the liquid-crystal algebra, every combination that the node
-// functions multiply by formed once per box (C the model's constants, in
-// FP64).  The two-node kernels keep a copy with each value twice in shared
-// memory (LcK<f2>), one 8-byte load per packed operand.
+// Constants of the FP64 liquid-crystal algebra, every combination that the node
+// functions multiply by formed once per box.
 template <typename T>
 struct LcK {
-  T A0g, nA0g, nA3, c_lin, c_lo;   // A0 g, its negative, -A0 g / 3, H: Q beyond -A0 g Tr(Q^2), the same - 6 K
+  T A0g, nA0g, nA3, c_lin;         // A0 g, its negative, -A0 g / 3, H: Q beyond -A0 g Tr(Q^2)
   T K, nKq0, n2Kq0, Kq0;           // K, -K q0, -2 K q0, K q0
   T f2c, f4c, K8;                  // f': Tr Q^2, (Tr Q^2)^2, K / 8
   T xi2, nt, nK4, up, dn, di;      // 2 xi, -2 xi / 3, -K / 4, 1 - xi, -(1 + xi), -2 xi
   T Gamma, g0, g1, g2;             // xi / 2, (xi + 1) / 4, (xi - 1) / 4
-  T A2, nA2;                       // 2 A0 g, -2 A0 g
-  T two, ntwo, third, nthird, nsix, nhalf;
+  T two, ntwo, third, nthird, nhalf;
 };
-constexpr int LCK_N = sizeof(LcK<float>) / sizeof(float);
 
 // One colloid.  X, V, W: current state.  Xb, Vb, Wb: the state used when the
 // post-collision populations now in memory were produced; the bounce-back of
@@ -133,8 +130,9 @@ struct DevBox {
   DevState* st;
   int* gerr;            // error words of the box's group: [0] wait gave up, [1] contact in some box
   int* nlinks;          // device count of boundary links
-  // fluid nodes next to a solid or wall (mask bit NEAR), in no particular order:
-  // device count, capacity (a bound on the count over the box's motion)
+  // fluid nodes next to a solid or wall (mask bit NEAR) and the other nodes of
+  // their pairs (near_member), in no particular order: device count, capacity
+  // (a bound on the count over the box's motion)
   int* nnear;
   int* near_node;
   int near_cap;
@@ -145,7 +143,6 @@ struct DevBox {
   DevParams p;
   PhysT<float> pf;
   PhysT<double> pd;
-  LcK<float> kf;
   LcK<double> kd;
 };
 
@@ -162,13 +159,6 @@ template <>
 __device__ __forceinline__ const PhysT<float>& phys<float>(const DevBox& B) { return B.pf; }
 template <>
 __device__ __forceinline__ const PhysT<double>& phys<double>(const DevBox& B) { return B.pd; }
-
-template <typename T>
-__device__ __forceinline__ const LcK<T>& lck(const DevBox& B);
-template <>
-__device__ __forceinline__ const LcK<float>& lck<float>(const DevBox& B) { return B.kf; }
-template <>
-__device__ __forceinline__ const LcK<double>& lck<double>(const DevBox& B) { return B.kd; }
 
 // ---------------------------------------------------------------------------
 // Small helpers
@@ -787,13 +777,12 @@ __device__ __forceinline__ void derivatives(const T qi[5], const T qn[6][5], T d
 // The algebra is written out in the five stored components with what
 // tracelessness gives (off-diagonal Q.Q from two products each, H_zz from H_xx
 // and H_yy, the commutator and anticommutator of Q and H from the nine entries
-// of Q H): about 290 operations a node against 470 for the 3x3 loops it
-// replaces, which matters where FP64 issue bounds the step (k_stress FP64,
+// of Q H): about 290 operations a node against 470 for the 3x3 loops of
+// lc_node_f32, which matters where FP64 issue bounds the step (k_stress FP64,
 // 64^3: 84-87 % of the FP64 pipe).  The chiral stress term is skipped when
-// q0 = 0 (uniform over a box).  Products are added, never subtracted, with the
-// sign on a factor that is reused: the packed f2 form has no negated multiply.
-// T is the arithmetic type (float, double, or f2: two nodes at once); chiral:
-// q0 != 0; NEED_P false: the molecular field alone.
+// q0 = 0 (uniform over a box).  FP64 storage only (T = double): FP32 keeps the
+// order of lc_node_f32.  chiral: q0 != 0; NEED_P false: the molecular field
+// alone.
 template <typename T, bool NEED_P = true>
 __device__ __forceinline__ void lc_node_d(const LcK<T>& P, bool chiral, const T qi[5], const T dq[3][5],
                                           const T lap[5], T h[5], T p[9], T* fprime) {
@@ -870,32 +859,148 @@ __device__ __forceinline__ void lc_node_d(const LcK<T>& P, bool chiral, const T 
   *fprime = fp;
 }
 
+// The same in FP32 (dq2: the doubled first derivatives): H, f' and P by sums
+// over the 3x3 matrices, in an order that stays as it is (see lclb_pair.cuh,
+// which evaluates two nodes at once in the same order).
+template <bool NEED_P>
+__device__ __forceinline__ void lc_node_f32(const PhysT<float>& P, const float qi[5], const float dq2[3][5],
+                                            const float lap[5], float h[5], float p[9], float* fprime) {
+  const float A0 = P.A0, g = P.gamma, K = P.K, q0 = P.q0, xi = P.xi;
+  const float third = float(1) / float(3);
+  const float A0g = A0 * g, twoKq0 = float(2) * K * q0;
+  const float c_lin = -A0 * (float(1) - g * third) - float(4) * K * q0 * q0;  // H: coefficient of Q beyond -A0 g Tr(Q^2)
+  const float A0g3 = A0g * third;
+  float dq[3][5];
+#pragma unroll
+  for (int a = 0; a < 3; ++a)
+#pragma unroll
+    for (int k = 0; k < 5; ++k) dq[a][k] = 0.5f * dq2[a][k];
+  // Q (3x3), D[g] = d_g Q (3x3 each) from the 5 stored components
+  float Q[3][3], D[3][3][3], S2[3][3], Cm[3][3];
+#pragma unroll
+  for (int a = 0; a < 3; ++a)
+#pragma unroll
+    for (int b = 0; b < 3; ++b) {
+      Q[a][b] = qab(qi, a, b);
+#pragma unroll
+      for (int gg = 0; gg < 3; ++gg) D[gg][a][b] = qab(dq[gg], a, b);
+    }
+#pragma unroll
+  for (int a = 0; a < 3; ++a)
+#pragma unroll
+    for (int b = a; b < 3; ++b) {
+      S2[a][b] = Q[a][0] * Q[0][b] + Q[a][1] * Q[1][b] + Q[a][2] * Q[2][b];
+      S2[b][a] = S2[a][b];
+    }
+#pragma unroll
+  for (int a = 0; a < 3; ++a)
+#pragma unroll
+    for (int b = 0; b < 3; ++b) Cm[a][b] = D[(a + 1) % 3][(a + 2) % 3][b] - D[(a + 2) % 3][(a + 1) % 3][b];
+  const float trq2 = S2[0][0] + S2[1][1] + S2[2][2];
+  const float cb = c_lin - A0g * trq2;
+  const float tq3 = A0g3 * trq2;
+  float H[3][3];
+#pragma unroll
+  for (int a = 0; a < 3; ++a)
+#pragma unroll
+    for (int b = a; b < 3; ++b) {
+      const int k = a == 0 ? b : (a == 1 ? 2 + b : 5);
+      const float lp = k < 5 ? lap[k] : -(lap[0] + lap[3]);
+      float v = cb * Q[a][b] + A0g * S2[a][b] + K * lp - twoKq0 * (Cm[a][b] + Cm[b][a]);
+      if (a == b) v = v - tq3;
+      H[a][b] = v;
+      H[b][a] = v;
+    }
+  h[0] = H[0][0]; h[1] = H[0][1]; h[2] = H[0][2]; h[3] = H[1][1]; h[4] = H[1][2];
+  if (!NEED_P) return;
+  // E_ab = K d_aQ : d_bQ; both factors are symmetric and traceless, so the
+  // double contraction over the 5 stored components is
+  // A_xx B_xx + A_yy B_yy + A_zz B_zz + 2 (A_xy B_xy + A_xz B_xz + A_yz B_yz)
+  // with A_zz = -(A_xx + A_yy)
+  float E[3][3], tz[3];
+#pragma unroll
+  for (int a = 0; a < 3; ++a) tz[a] = dq[a][0] + dq[a][3];
+  const float twoK = float(2) * K;
+#pragma unroll
+  for (int a = 0; a < 3; ++a)
+#pragma unroll
+    for (int b = a; b < 3; ++b) {
+      const float e = K * (dq[a][0] * dq[b][0] + dq[a][3] * dq[b][3] + tz[a] * tz[b]) +
+                  twoK * (dq[a][1] * dq[b][1] + dq[a][2] * dq[b][2] + dq[a][4] * dq[b][4]);
+      E[a][b] = e;
+      E[b][a] = e;
+    }
+  const float Kgrad2 = E[0][0] + E[1][1] + E[2][2];  // K |grad Q|^2
+#pragma unroll
+  for (int a = 0; a < 3; ++a)
+#pragma unroll
+    for (int b = 0; b < 3; ++b) {
+      // the chiral part: sum over g != b of eps(m, b, g) d_a Q_g. . Q_m. (m = 3 - b - g);
+      // eps(m, b, g) = +1 for g = b + 1, m = b + 2 and -1 for g = b + 2, m = b + 1 (mod 3)
+      const int g1 = (b + 1) % 3, g2 = (b + 2) % 3;
+      const float e2 = (D[a][g1][0] * Q[g2][0] + D[a][g1][1] * Q[g2][1] + D[a][g1][2] * Q[g2][2]) -
+                   (D[a][g2][0] * Q[g1][0] + D[a][g2][1] * Q[g1][1] + D[a][g2][2] * Q[g1][2]);
+      E[a][b] = E[a][b] + twoKq0 * e2;
+    }
+  float trq3 = float(0), qc = float(0);
+#pragma unroll
+  for (int a = 0; a < 3; ++a)
+#pragma unroll
+    for (int b = 0; b < 3; ++b) {
+      trq3 = trq3 + Q[a][b] * S2[a][b];
+      qc = qc + Q[a][b] * Cm[a][b];
+    }
+  const float fb2 = float(0.5) * A0 * (float(1) - g * third), fb4 = float(0.25) * A0g;
+  const float fp = (fb2 * trq2 - A0g3 * trq3) + fb4 * (trq2 * trq2) + float(0.5) * Kgrad2 + twoKq0 * qc +
+               (float(2) * K * q0 * q0) * trq2;
+  float Am[3][3];
+#pragma unroll
+  for (int a = 0; a < 3; ++a)
+#pragma unroll
+    for (int b = 0; b < 3; ++b) Am[a][b] = Q[a][0] * H[0][b] + Q[a][1] * H[1][b] + Q[a][2] * H[2][b];
+  const float qh = Am[0][0] + Am[1][1] + Am[2][2];
+  const float twoxi = float(2) * xi, twoxi3 = twoxi * third;
+  const float qh2 = twoxi * qh;
+#pragma unroll
+  for (int a = 0; a < 3; ++a)
+#pragma unroll
+    for (int b = 0; b < 3; ++b) {
+      // 2 xi (Q + I/3) Q:H - xi (A + A^T) - (2 xi/3) H - E + A - A^T, plus f' on the diagonal
+      float v = qh2 * Q[a][b] - xi * (Am[a][b] + Am[b][a]) - twoxi3 * H[a][b] - E[a][b] + (Am[a][b] - Am[b][a]);
+      if (a == b) v = v + (fp + third * qh2);
+      p[3 * a + b] = v;
+    }
+  *fprime = fp;
+}
+
+// One node in the storage's arithmetic, from its derivatives or its face
+// neighbours.
+template <typename T, bool NEED_P = true>
+__device__ __forceinline__ void lc_node_dq(const DevBox& B, const T qi[5], const T dq[3][5], const T lap[5], T h[5],
+                                           T p[9], T* fprime) {
+  if constexpr (sizeof(T) == 4) lc_node_f32<NEED_P>(B.pf, qi, dq, lap, h, p, fprime);
+  else lc_node_d<T, NEED_P>(B.kd, B.p.q0 != 0.0, qi, dq, lap, h, p, fprime);
+}
 template <typename T, bool NEED_P = true>
 __device__ __forceinline__ void lc_node(const DevBox& B, const T qi[5], const T qn[6][5], T h[5], T p[9],
                                         T* fprime) {
   T dq[3][5], lap[5];
   derivatives(qi, qn, dq, lap);
-  lc_node_d<T, NEED_P>(lck<T>(B), B.p.q0 != 0.0, qi, dq, lap, h, p, fprime);
+  lc_node_dq<T, NEED_P>(B, qi, dq, lap, h, p, fprime);
 }
 
-// Per-node choice ca ? a : b (f2: per lane value).
 template <typename T>
 __device__ __forceinline__ T pos_part(T v) {
   return v > T(0) ? v : T(0);
 }
 
-// Increment of Q in one step (Eq. 2) at one node (or, T = f2, two):
+// Increment of Q in one step (Eq. 2) at one node, FP64 storage:
 //   co-rotation S = X + X^T - 2 xi (Q + I/3) Tr(QW), X = G (Q + I/3),
 //     G = xi D + Omega: 27 products for X instead of 72 for its four factors;
 //   upwind fluxes: with the positive and negative parts of the face velocity
 //     the six fluxes are one product per neighbour and component plus one
 //     with the node's own Q, adv = (self Q_i + sum_d cd[d] Q_d) / 2 (35
-//     multiply-adds and 6 selects instead of 30 and 30);
-//   FP32 storage (COMP): H was evaluated at hi, the stored Q is hi + lo: the
-//     local part of H(hi + lo) - H(hi) to first order (the bulk terms'
-//     derivative at hi applied to lo, and lo's own term -6 K lo of the
-//     Laplacian; the neighbours' lo enter at the ~1e-9 level).  Without it the
-//     relaxation stalls where A0 lo ~ the residual.
+//     multiply-adds and 6 selects instead of 30 and 30).
 // flow_terms: G (row-major), cd and self from the velocities ui and un of the
 // node and its six face neighbours; open[d] = false closes face d (solid or
 // wall) to the flux.
@@ -941,35 +1046,16 @@ __device__ __forceinline__ T advect(const T cd[6], T self, T q, const T n[6]) {
 }
 
 // FLOW = false: the flow is frozen (u = 0), G and adv are not read.
-template <bool COMP, bool FLOW, typename T>
+template <bool FLOW, typename T>
 __device__ __forceinline__ void q_increment(const LcK<T>& P, const T qi[5], const T adv[5], const T G[9],
-                                            const T hin[5], const T lo[5], T d5[5]) {
-  const T a = qi[0], b = qi[1], c = qi[2], d = qi[3], e = qi[4];
-  const T f = -a - d;
-  T h[5];
-#pragma unroll
-  for (int k = 0; k < 5; ++k) h[k] = hin[k];
-  if constexpr (COMP) {
-    const T A0g = P.A0g;
-    const T la = lo[0], lb = lo[1], lc = lo[2], ld = lo[3], le = lo[4];
-    const T lf = -la - ld;
-    const T ta = a * la, tb = b * lb, tc = c * lc, td = d * ld, te = e * le;
-    const T trl = (ta + td + f * lf) + P.two * (tb + tc + te);
-    const T trq2 = (a * a + (d * d + f * f)) + P.two * T(b * b + (c * c + e * e));
-    const T cb = P.c_lo + P.nA0g * trq2;
-    const T m = P.nA2 * trl;
-    const T nf = a + d, nd = -d, na = -a, l3 = P.nthird * trl, A2 = P.A2;
-    h[0] = h[0] + (cb * la + (A2 * (ta + tb + tc + l3) + m * a));
-    h[3] = h[3] + (cb * ld + (A2 * (tb + td + te + l3) + m * d));
-    h[1] = h[1] + (cb * lb + (A0g * T(nf * lb + (b * (la + ld) + (c * le + e * lc))) + m * b));
-    h[2] = h[2] + (cb * lc + (A0g * T(nd * lc + (b * le + (e * lb + c * (la + lf)))) + m * c));
-    h[4] = h[4] + (cb * le + (A0g * T(na * le + (b * lc + (c * lb + e * (ld + lf)))) + m * e));
-  }
+                                            const T h[5], T d5[5]) {
   if constexpr (!FLOW) {
 #pragma unroll
     for (int k = 0; k < 5; ++k) d5[k] = P.Gamma * h[k];
     return;
   }
+  const T a = qi[0], b = qi[1], c = qi[2], d = qi[3], e = qi[4];
+  const T f = -a - d;
   const T at = a + P.third, dt = d + P.third, ft = f + P.third;
   const T tm = P.ntwo * T(a * G[0] + (d * G[4] + (f * G[8] + (b * (G[1] + G[3]) + (c * (G[2] + G[6]) + e * (G[5] + G[7]))))));
   const T x00 = G[0] * at + (G[1] * b + G[2] * c), x11 = G[3] * b + (G[4] * dt + G[5] * e);
@@ -986,6 +1072,118 @@ __device__ __forceinline__ void q_increment(const LcK<T>& P, const T qi[5], cons
   S[3] = S[3] + tr3;
 #pragma unroll
   for (int k = 0; k < 5; ++k) d5[k] = S[k] + (P.Gamma * h[k] + P.nhalf * adv[k]);
+}
+
+// FP32 storage: H was evaluated at hi, the stored Q is hi + lo.  Adds the local
+// part of H(hi + lo) - H(hi) to first order: the bulk terms' derivative at hi
+// applied to lo, and lo's own term -6 K lo of the Laplacian (the neighbours' lo
+// enter K lap and the gradient terms at the ~1e-9 level).  Without it the
+// relaxation stalls where A0 lo ~ the residual.
+__device__ __forceinline__ void comp_h_f32(const PhysT<float>& P, const float qi[5], const float lo[5], float h[5]) {
+  const int ia[5] = {0, 0, 0, 1, 1}, ib[5] = {0, 1, 2, 1, 2};
+  const float A0 = P.A0, g = P.gamma, K = P.K, q0 = P.q0;
+  float Qm[3][3], Lm[3][3];
+#pragma unroll
+  for (int a = 0; a < 3; ++a)
+#pragma unroll
+    for (int b = 0; b < 3; ++b) {
+      Qm[a][b] = qab(qi, a, b);
+      Lm[a][b] = qab(lo, a, b);
+    }
+  float trq2 = float(0), trql = float(0);
+#pragma unroll
+  for (int a = 0; a < 3; ++a)
+#pragma unroll
+    for (int b = 0; b < 3; ++b) {
+      trq2 += Qm[a][b] * Qm[a][b];
+      trql += Qm[a][b] * Lm[a][b];
+    }
+  const float cb = -A0 * (float(1) - g / float(3)) - A0 * g * trq2 - float(4) * K * q0 * q0 - float(6) * K;
+  const float A0g = A0 * g;
+#pragma unroll
+  for (int k = 0; k < 5; ++k) {
+    const int a = ia[k], b = ib[k];
+    float ql = float(0);
+#pragma unroll
+    for (int c = 0; c < 3; ++c) ql += Qm[a][c] * Lm[c][b] + Lm[a][c] * Qm[c][b];
+    if (a == b) ql -= float(2) / float(3) * trql;
+    h[k] += cb * lo[k] + A0g * ql - float(2) * A0g * trql * qi[k];
+  }
+}
+
+// Increment of Q of one node, FP32 storage (h receives the compensation; fl[d]
+// false closes face d).  The order of the sums stays as it is (see
+// lclb_pair.cuh).  FLOW false: the flow is frozen (u = 0).
+template <bool FLOW>
+__device__ __forceinline__ void q_increment_f32(const PhysT<float>& P, const float qi[5], const float qn[6][5],
+                                                const float ui[3], const float un[6][3], const bool fl[6], float h[5],
+                                                const float lo[5], float d5[5]) {
+  const float Gam = P.Gamma, xi = P.xi;
+  if constexpr (!FLOW) {
+    comp_h_f32(P, qi, lo, h);
+#pragma unroll
+    for (int k = 0; k < 5; ++k) d5[k] = Gam * h[k];
+    return;
+  }
+  // velocity gradient W_ab = d_b u_a
+  float W[3][3];
+#pragma unroll
+  for (int a = 0; a < 3; ++a)
+#pragma unroll
+    for (int b = 0; b < 3; ++b) W[a][b] = float(0.5) * (un[2 * b][a] - un[2 * b + 1][a]);
+  // advective fluxes through the six faces (zero across solid faces)
+  float adv[5] = {float(0), float(0), float(0), float(0), float(0)};
+#pragma unroll
+  for (int d = 0; d < 6; ++d) {
+    if (!fl[d]) continue;
+    const int ax = d >> 1;
+    const float uf = float(0.5) * (ui[ax] + un[d][ax]);
+    const bool plus = (d & 1) == 0;
+    // + face: upwind is i when uf > 0; - face: upwind is the neighbour when uf > 0
+    const bool take_i = plus ? (uf > float(0)) : !(uf > float(0));
+#pragma unroll
+    for (int k = 0; k < 5; ++k) {
+      const float fl_ = uf * (take_i ? qi[k] : qn[d][k]);
+      adv[k] += plus ? fl_ : -fl_;
+    }
+  }
+  // co-rotation S = xi (D Qt + Qt D) + (Om Q - Q Om) - 2 xi Qt Tr(Q W), Qt = Q + I/3
+  float D[3][3], Om[3][3];
+#pragma unroll
+  for (int a = 0; a < 3; ++a)
+#pragma unroll
+    for (int b = 0; b < 3; ++b) {
+      D[a][b] = float(0.5) * (W[a][b] + W[b][a]);
+      Om[a][b] = float(0.5) * (W[a][b] - W[b][a]);
+    }
+  float trQW = float(0);
+#pragma unroll
+  for (int a = 0; a < 3; ++a)
+#pragma unroll
+    for (int b = 0; b < 3; ++b) trQW += qab(qi, a, b) * D[a][b];
+  float dQ[3][3];
+#pragma unroll
+  for (int a = 0; a < 3; ++a)
+#pragma unroll
+    for (int b = 0; b < 3; ++b) {
+      float s = float(0);
+#pragma unroll
+      for (int c = 0; c < 3; ++c)
+        s += xi * (D[a][c] * qab(qi, c, b) + qab(qi, a, c) * D[c][b]) + Om[a][c] * qab(qi, c, b) -
+             qab(qi, a, c) * Om[c][b];
+      s += xi * float(2) / float(3) * D[a][b];
+      s -= float(2) * xi * (qab(qi, a, b) + (a == b ? float(1) / float(3) : float(0))) * trQW;
+      dQ[a][b] = s;
+    }
+  const float tr = dQ[0][0] + dQ[1][1] + dQ[2][2];
+  comp_h_f32(P, qi, lo, h);
+  const int ia[5] = {0, 0, 0, 1, 1}, ib[5] = {0, 1, 2, 1, 2};
+#pragma unroll
+  for (int k = 0; k < 5; ++k) {
+    float v = Gam * h[k] + dQ[ia[k]][ib[k]] - adv[k];
+    if (ia[k] == ib[k]) v -= tr / float(3);
+    d5[k] = v;
+  }
 }
 
 }  // namespace lclb

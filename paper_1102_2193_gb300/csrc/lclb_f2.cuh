@@ -58,5 +58,6 @@ __device__ __forceinline__ f2 operator-(f2mul m, float c) { return m - f2(c); }
 __device__ __forceinline__ f2 operator-(float c, f2mul m) { return f2(c) - m; }
 
 __device__ __forceinline__ f2 pos_part(f2 v) { return f2(fmaxf(v.v.x, 0.f), fmaxf(v.v.y, 0.f)); }
+__device__ __forceinline__ f2 neg_part(f2 v) { return f2(fminf(v.v.x, 0.f), fminf(v.v.y, 0.f)); }
 
 }  // namespace lclb
