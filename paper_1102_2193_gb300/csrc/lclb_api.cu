@@ -1194,7 +1194,7 @@ int enqueue_step(Group* g) {
     return LC_OK;
   }
   if (int rc = enqueue_force_lb(g)) return rc;
-  CK(launch_phase(g, 2, LC_RESID | LC_COMMIT), &g->err);
+  CK(launch_phase(g, 2, LC_RESID | LC_FLC | LC_COMMIT), &g->err);
   if (g->nmob > 0)
     CK(launch_rediscretise(g->prec, g->d_boxes, (int)g->boxes.size(), g->d_mob, g->nmob, g->nsm,
                            reinterpret_cast<unsigned*>(g->d_err) + 2, g->d_err, spin_limit(), g->stream), &g->err);
@@ -1309,7 +1309,7 @@ int group_profile(Group* g, int n, double* ms) {
     CK(cudaEventRecord(ev[5], g->stream), &g->err);
     if (k2 >= 0 && !g->frozen) CK(launch_phase(g, k2, 0), &g->err);
     CK(cudaEventRecord(ev[1], g->stream), &g->err);
-    CK(launch_phase(g, 2, LC_RESID), &g->err);
+    CK(launch_phase(g, 2, LC_RESID | LC_FLC), &g->err);
     CK(cudaEventRecord(ev[2], g->stream), &g->err);
     CK(launch_links(g->prec, g->d_boxes, g->d_chunks, g->nchunks, g->nchunks, g->stream), &g->err);
     CK(cudaEventRecord(ev[3], g->stream), &g->err);

@@ -13,6 +13,7 @@ constexpr int FORCE_FE = 2;   // write free-energy partials (one double per tile
 constexpr int FORCE_P = 4;    // k_stress: store the stress also with the flow frozen (exports read it)
 constexpr int LB_MOM = 1;     // write mass/momentum partials (4 doubles per tile)
 constexpr int LC_RESID = 1;   // write residual partials (sum of squares, max; 2 doubles per tile)
+constexpr int LC_FLC = 4;     // k_relax: accumulate colloid LC force (a step; not set while tuning)
 constexpr int LC_COMMIT = 2;  // k_lc also runs the link exchange and, when a box is done, its colloid update and parity flip
 
 // boundary links per link-exchange work unit

@@ -2588,7 +2588,7 @@ __global__ void __launch_bounds__(TX * TY, (sizeof(T) == 4 ? 640 : 256) / (TX * 
     if (B.p.lc_on) {
       if (t < nn) {
         near_group<TY>(B, L.groups, t, [&](int j) {
-          near_stress<T, true>(B, j, commit ? FORCE_ACC : 0, reinterpret_cast<NearScratch<T>*>(ring)[wy], rs);
+          near_stress<T, true>(B, j, (mode & LC_FLC) ? FORCE_ACC : 0, reinterpret_cast<NearScratch<T>*>(ring)[wy], rs);
         });
         __syncthreads();
       } else {
