@@ -684,6 +684,13 @@ __device__ __forceinline__ void surface_q0_near(const DevBox& B, int c, int sx, 
   q0[4] = S0 * n[1] * n[2];
 }
 
+// a - b rounded, and its rounding error (Knuth's two-sum).
+__device__ __forceinline__ float two_diff(float a, float b, float& e) {
+  const float t = __fsub_rn(a, b), bb = __fsub_rn(a, t);
+  e = __fadd_rn(__fsub_rn(a, __fadd_rn(t, bb)), __fsub_rn(bb, b));
+  return t;
+}
+
 // w (Q0 - Q) for a homeotropic solid face in FP32 storage, in sums of two
 // floats (48 bits; every step below keeps the error of the FP32 operation
 // before it): n0 = d / |d| from the split position of the colloid, 1/|d| by one
@@ -697,16 +704,22 @@ __device__ __forceinline__ void surface_dn_normal(const DevBox& B, const DevColl
 #pragma unroll
   for (int a = 0; a < 3; ++a) {
     const int L = a == 0 ? B.nx : (a == 1 ? B.ny : B.nz);
-    // integer minus X: exact in the high part; the minimum image decided on both parts
-    float t = (float)s[a] - C.Xs[a][0];
-    const float xl = C.Xs[a][1];
+    // node minus X: the minimum image is taken on the integer (exact in FP32),
+    // decided on both parts of the difference, then the difference to the high
+    // part with its rounding error, which is no zero where X is small beside it
+    // (a colloid at a low face of the box)
+    const float xh = C.Xs[a][0], xl = C.Xs[a][1];
+    int si = s[a];
+    float e, t = two_diff((float)si, xh, e);
     if (a < 2 || !B.wall_z) {
       const float h = 0.5f * (float)L;
-      if (t - h >= xl) t -= (float)L;
-      else if (t + h < xl) t += (float)L;
+      if (t - h >= xl - e) si -= L;
+      else if (t + h < xl - e) si += L;
     }
-    dh[a] = t - xl;
-    dl[a] = (t - dh[a]) - xl;
+    t = two_diff((float)si, xh, e);
+    const float low = e - xl;
+    dh[a] = t + low;
+    dl[a] = (t - dh[a]) + low;
   }
   // |d|^2 = rh + rl
   float ph[3], rl = 0.f;

@@ -810,7 +810,7 @@ __device__ __noinline__ void near_stress(const DevBox& B, int i, int mode, NearS
     const int t = t0 + lane;
     int own, d, c, s[3];
     face_of(t, own, d, c, s);
-    // (node coordinates are exact in FP32 up to 2^24)
+    // (node coordinates, one box further for an image, are exact in FP32)
     const bool normal = comp && c >= 0 && B.col[c].anchoring == 0 && max(nx, max(ny, B.nz)) < (1 << 22);
     if constexpr (comp) {
       if (__ballot_sync(full, t < nface && normal)) {

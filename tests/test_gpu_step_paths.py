@@ -32,3 +32,30 @@ def test_profile_advances_as_step(prec, flow):
     assert np.abs(np.asarray(a["V"]) - b["V"]).max() <= tol * np.abs(a["V"]).max()
     assert np.abs(np.asarray(a["X"]) - b["X"]).max() <= 1e-12 * 24
     assert np.abs(qa - qb).max() <= tol
+
+
+@pytest.mark.parametrize("axis", [0, 1, 2])
+@pytest.mark.parametrize("w", [0.02, float("inf")])
+def test_normal_surface_values_at_low_face(axis, w):
+    """FP32 surface values of a colloid across the low periodic face of a long box: its LC force and torque are those
+    of the same colloid and field shifted by half the box.  Both differ by the sum of FP64 atomics and by the last bit
+    of few surface values only (1e-6; an error of 4e-6 in the normal, a rounding at the size of the box, shows at 1e-5)."""
+    import paper_1102_2193_gb300 as P
+    L, X = [20, 22, 24], np.array([9.3, 10.6, 12.4])
+    L[axis] = 256
+    X[axis] = np.round(0.4 * 2.0**40) / 2.0**40
+    prm = dict(synth.NEMATIC, q0=2 * np.pi / 17)
+    q = synth.random_q((L[2], L[1], L[0]), 9, amp=0.05, base=(0.2, 0.05, 0.02, -0.1, 0.03))
+    out = []
+    for shift in (0, 128):
+        s = P.Solver(*L, precision=P.LC_FP32, **prm)
+        s.set_Q(np.roll(q, shift, axis=3 - axis))
+        Y = X.copy()
+        Y[axis] += shift
+        s.add_colloid(Y, 6.3, P.LC_NORMAL, w)
+        s.step(1)
+        out.append(s.colloid(0))
+    a, b = out
+    F = np.abs(a["F_lc"]).max()
+    assert F > 0 and np.abs(a["F_lc"] - b["F_lc"]).max() <= 1e-6 * F
+    assert np.abs(a["T_lc"] - b["T_lc"]).max() <= 1e-6 * 6.3 * F
