@@ -18,6 +18,7 @@
 
 #include "lclb_pair.cuh"
 #include "lclb_internal.h"
+#include "lclb_barrier.h"
 
 namespace lclb {
 
@@ -3433,25 +3434,31 @@ __device__ void rd_finish(DevBox* __restrict__ boxes, int b) {
   if (ld_state(B.nlinks) > B.nlinks_cap || ld_state(B.nnear) > B.near_cap) atomicOr(&st->err, 1);
 }
 
-// Grid barrier: every block arrives on a counter that only grows and waits for
-// the multiple of the grid size that its arrival belongs to.  Bounded: after
-// spin_limit polls the error word is set and the block gives up.
+// The words of the launch's barrier: bar[0] arrivals, bar[1] generation.
+struct GridWords {
+  unsigned* bar;
+  int* err;
+  __device__ unsigned generation() const { return ld_acquire_u32(bar + 1); }
+  __device__ unsigned arrive() const {
+    __threadfence();
+    return atomicAdd(bar, 1u);
+  }
+  __device__ void clear_arrivals() const { atomicExch(bar, 0u); }
+  __device__ void advance() const {
+    __threadfence();
+    atomicAdd(bar + 1, 1u);
+  }
+  __device__ bool failed() const { return ld_acquire_u32(reinterpret_cast<const unsigned*>(err)) != 0u; }
+  __device__ void fail() const { atomicOr(err, 1); }
+  __device__ void pause() const { __nanosleep(40); }
+};
+
 __device__ bool grid_barrier(unsigned* bar, int* err, int spin_limit) {
   __shared__ int s_ok;
   __syncthreads();
   if (threadIdx.x == 0) {
-    __threadfence();
-    const unsigned n = gridDim.x, target = (atomicAdd(bar, 1u) / n + 1u) * n;
-    int ok = 0;
-    for (int spin = 0; spin <= spin_limit; ++spin) {
-      if ((int)(ld_acquire_u32(bar) - target) >= 0) {
-        ok = 1;
-        break;
-      }
-      __nanosleep(40);
-    }
-    if (!ok) atomicOr(err, 1);
-    s_ok = ok;
+    GridWords w{bar, err};
+    s_ok = barrier_wait(w, gridDim.x, spin_limit);
     __threadfence();
   }
   __syncthreads();
@@ -3462,8 +3469,11 @@ template <typename T>
 __global__ void __launch_bounds__(256) k_rediscretise(DevBox* __restrict__ boxes, int nboxes,
                                                       const int2* __restrict__ mob, int nmob, unsigned* bar, int* err,
                                                       int spin_limit) {
+  // (a wait that gave up in an earlier step: the state is invalid until the host
+  // has reported it)
   bool any = false;
-  for (int b = threadIdx.x; b < nboxes; b += blockDim.x) any = any || (boxes[b].nmobile && boxes[b].st->scan);
+  if (*err == 0)
+    for (int b = threadIdx.x; b < nboxes; b += blockDim.x) any = any || (boxes[b].nmobile && boxes[b].st->scan);
   if (!__syncthreads_or(any)) return;
   rd_find(boxes, mob, nmob);
   if (!grid_barrier(bar, err, spin_limit)) return;
