@@ -292,9 +292,12 @@ int build_chunks(Group* g) {
   return LC_OK;
 }
 
-// Groups of 32 near nodes covering every box's near-list capacity.
+// Groups of 32 near nodes covering every box's near-list capacity.  Where a box's
+// groups move, the residual records of the last step move with them (the
+// diagnostics of a box may be read after another box of the batch has changed).
 int build_groups(Group* g) {
   std::vector<int2> gr;
+  const std::vector<int> old_start = g->gstart, old_count = g->gcount;
   g->gstart.assign(g->boxes.size(), 0);
   g->gcount.assign(g->boxes.size(), 0);
   for (size_t b = 0; b < g->boxes.size(); ++b) {
@@ -303,14 +306,21 @@ int build_groups(Group* g) {
     g->gcount[b] = n;
     for (int k = 0; k < n; ++k) gr.push_back(make_int2((int)b, 32 * k));
   }
-  if ((int)gr.size() > g->group_cap) {
+  bool moved = (int)gr.size() > g->group_cap;
+  for (size_t b = 0; b < old_start.size(); ++b) moved = moved || (old_count[b] > 0 && old_start[b] != g->gstart[b]);
+  if (moved) {
+    double* const old_part = g->d_npart;
     if (g->d_groups) g->mem.put(g->d_groups, g->al);
-    if (g->d_npart) g->mem.put(g->d_npart, g->al);
     g->group_cap = (int)gr.size() + 64;
     g->d_groups = (int2*)galloc(g, sizeof(int2) * g->group_cap);
     g->d_npart = (double*)galloc(g, sizeof(double) * 3 * g->group_cap);
     if (!g->d_groups || !g->d_npart) return fail(&g->err, LC_ERR_OOM, "near group allocation failed");
     CK(cudaMemsetAsync(g->d_npart, 0, sizeof(double) * 2 * g->group_cap, g->stream), &g->err);
+    for (size_t b = 0; old_part && b < old_start.size(); ++b)
+      if (old_count[b] > 0)
+        CK(cudaMemcpyAsync(g->d_npart + 2 * (size_t)g->gstart[b], old_part + 2 * (size_t)old_start[b],
+                           2 * sizeof(double) * old_count[b], cudaMemcpyDeviceToDevice, g->stream), &g->err);
+    if (old_part) g->mem.put(old_part, g->al);
   }
   g->ngroups = (int)gr.size();
   if (!gr.empty())

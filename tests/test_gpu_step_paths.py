@@ -59,3 +59,23 @@ def test_normal_surface_values_at_low_face(axis, w):
     F = np.abs(a["F_lc"]).max()
     assert F > 0 and np.abs(a["F_lc"] - b["F_lc"]).max() <= 1e-6 * F
     assert np.abs(a["T_lc"] - b["T_lc"]).max() <= 1e-6 * 6.3 * F
+
+
+@pytest.mark.parametrize("prec", ["f32", "f64"])
+@pytest.mark.parametrize("radius", [3.0, 8.5])
+def test_residual_of_other_boxes_after_add_colloid(prec, radius):
+    """The last step's residual of a box of a batch is the same after a colloid was added to the box before it (one
+    whose near nodes fit the allocated groups, and one that takes more)."""
+    import paper_1102_2193_gb300 as P
+    prm = dict(synth.NEMATIC, q0=0.0)
+    L = ((22, 24, 26), (26, 20, 18), (18, 18, 18))
+    B = P.Batch([dict(grid=g, params=prm) for g in L], precision=P.LC_FP32 if prec == "f32" else P.LC_FP64)
+    for k, s in enumerate(B.boxes):
+        s.set_Q(synth.random_q(L[k][::-1], k, amp=0.05, base=(0.2, 0.05, 0.02, -0.1, 0.03)))
+        s.add_colloid((9.3, 8.6, 9.1), 3.1, P.LC_NORMAL, 0.02)
+    B.step(3)
+    before = [s.diag() for s in B.boxes]
+    B.boxes[0].add_colloid((19.6 if radius < 5 else 20.9, 20.4, 21.2), radius, P.LC_NORMAL, 0.02)
+    for s, d in list(zip(B.boxes, before))[1:]:
+        after = s.diag()
+        assert after["resid_rms"] == d["resid_rms"] and after["resid_max"] == d["resid_max"]
