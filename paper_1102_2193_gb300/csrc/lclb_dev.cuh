@@ -372,14 +372,58 @@ __device__ __forceinline__ void rigid_velocity(const double* V, const double* W,
 // matrix (Smith, CACM 1961) and a cross product of two rows of (A - l I).
 // FP64: the eigenvalue of the FP32 evaluation refined by two Newton steps on
 // the characteristic polynomial det(A - l I) = -l^3 + (Tr A^2 / 2) l + det A
-// (no FP64 transcendental functions; the slope in FP32, whose 1e-7 leaves the
-// steps 1e-7 -> 1e-14 -> rounding), then the FP64 cross products.  One warp
-// runs this chain per 32 nodes next to a planar colloid, and in a small box
-// the step waits for it, so FP64 divisions and square roots are kept out.
+// (no FP64 transcendental functions, the slope in FP32), then the FP64 cross
+// products.  One warp runs this chain per 32 nodes next to a planar colloid, and
+// in a small box the step waits for it, so FP64 divisions and square roots are
+// kept out.  The seed is 6e-8 / g off for a relative gap g to the second
+// eigenvalue, and a step leaves the square of the error over g: to rounding
+// for g > 0.05 (measured 1e-15), but two steps overshoot at g ~ 1e-3 and below.
+// Where the slope, 3 l^2 - Tr A^2 / 2 ~ g, is small (a texture that is nearly
+// uniaxial with negative order, as in defect cores), or A is so small or large
+// that FP32 loses it, Jacobi rotations give the direction (1e-16 / g off).
 template <typename T>
 __device__ void principal_dir(const T* q, T n[3]);
 
-__device__ __forceinline__ double principal_lambda_f64(const double* q) {
+// One rotation of the cyclic Jacobi method (Golub and Van Loan) that zeroes
+// a_pq of a symmetric 3x3 matrix: r the third index, u and v columns p and q of
+// the eigenvectors.
+__device__ __forceinline__ void jacobi_rotate(double& app, double& aqq, double& apq, double& arp, double& arq,
+                                              double u[3], double v[3]) {
+  if (apq == 0.0) return;
+  const double th = (aqq - app) / (2.0 * apq);
+  const double t = copysign(1.0, th) / (fabs(th) + sqrt(th * th + 1.0));
+  const double c = rsqrt(t * t + 1.0), s = t * c;
+  app -= t * apq;
+  aqq += t * apq;
+  apq = 0.0;
+  const double x = arp, y = arq;
+  arp = c * x - s * y;
+  arq = s * x + c * y;
+  for (int k = 0; k < 3; ++k) {
+    const double p = u[k], q = v[k];
+    u[k] = c * p - s * q;
+    v[k] = s * p + c * q;
+  }
+}
+
+// Principal direction by Jacobi rotations (the matrix scaled to size 1).
+inline __device__ __noinline__ void principal_dir_jacobi(const double* q, double n[3]) {
+  double m = 0.0;
+  for (int k = 0; k < 5; ++k) m = fmax(m, fabs(q[k]));
+  const double sc = 1.0 / m;
+  double a00 = q[0] * sc, a01 = q[1] * sc, a02 = q[2] * sc, a11 = q[3] * sc, a12 = q[4] * sc, a22 = -a00 - a11;
+  double u[3] = {1.0, 0.0, 0.0}, v[3] = {0.0, 1.0, 0.0}, w[3] = {0.0, 0.0, 1.0};
+  for (int sweep = 0; sweep < 8 && fabs(a01) + fabs(a02) + fabs(a12) > 1e-18; ++sweep) {
+    jacobi_rotate(a00, a11, a01, a02, a12, u, v);
+    jacobi_rotate(a00, a22, a02, a01, a12, u, w);
+    jacobi_rotate(a11, a22, a12, a01, a02, v, w);
+  }
+  const double* e = a00 >= a11 ? (a00 >= a22 ? u : w) : (a11 >= a22 ? v : w);
+  for (int k = 0; k < 3; ++k) n[k] = e[k];
+}
+
+// False: the two largest eigenvalues are too close for the Newton steps.
+__device__ __forceinline__ bool principal_lambda_f64(const double* q, double& lam) {
   const double a00 = q[0], a01 = q[1], a02 = q[2], a11 = q[3], a12 = q[4], a22 = -q[0] - q[3];
   // FP32 seed: the largest eigenvalue by the trigonometric formula
   const float f00 = (float)q[0], f01 = (float)q[1], f02 = (float)q[2], f11 = (float)q[3], f12 = (float)q[4];
@@ -396,14 +440,16 @@ __device__ __forceinline__ double principal_lambda_f64(const double* q) {
   }
   const double t2 = 0.5 * (a00 * a00 + a11 * a11 + a22 * a22 + 2.0 * (a01 * a01 + a02 * a02 + a12 * a12));
   const double det = a00 * (a11 * a22 - a12 * a12) - a01 * (a01 * a22 - a12 * a02) + a02 * (a01 * a12 - a11 * a02);
-  double lam = f32_to_f64(lam32);
+  lam = f32_to_f64(lam32);
+  const float t2f = (float)t2;
 #pragma unroll
   for (int it = 0; it < 2; ++it) {
     const double f = (t2 - lam * lam) * lam + det;
     const float df = (float)(t2 - 3.0 * lam * lam);
-    if (df != 0.f) lam -= f * f32_to_f64(1.f / df);
+    if (it == 0 && !(df < -0.06f * t2f && t2f > 1e-30f && t2f < 1e30f)) return false;
+    lam -= f * f32_to_f64(1.f / df);
   }
-  return lam;
+  return true;
 }
 
 // 1/sqrt(v) in FP64 from the FP32 estimate and Newton steps (FP32 storage:
@@ -427,7 +473,10 @@ __device__ void principal_dir(const T* q, T n[3]) {
   }
   T lam;
   if constexpr (sizeof(T) == 8) {
-    lam = principal_lambda_f64(q);
+    if (!principal_lambda_f64(q, lam)) {
+      principal_dir_jacobi(q, n);
+      return;
+    }
   } else {
     T p = sqrt(p2 / T(6));
     T b00 = a00 / p, b01 = a01 / p, b02 = a02 / p, b11 = a11 / p, b12 = a12 / p, b22 = a22 / p;

@@ -79,3 +79,29 @@ def test_residual_of_other_boxes_after_add_colloid(prec, radius):
     for s, d in list(zip(B.boxes, before))[1:]:
         after = s.diag()
         assert after["resid_rms"] == d["resid_rms"] and after["resid_max"] == d["resid_max"]
+
+
+@pytest.mark.parametrize("prec", ["f32", "f64"])
+@pytest.mark.parametrize("size,gap", [(1.0, 1e-1), (1.0, 1e-2), (1.0, 3e-3), (1.0, 3e-4), (1.0, 1e-4), (1.0, 1e-5),
+                                      (1.0, 1e-6), (1e-20, 0.3), (1e-22, 0.3), (1e-6, 0.1)])
+def test_planar_faces_of_close_eigenvalues(prec, size, gap):
+    """Planar surface values where the two largest eigenvalues of Q are ``gap`` apart (size 1: 0.16 + g/2, 0.16 - g/2,
+    -0.32), and of a Q that FP32 products lose: the colloid's LC force after one step against the oracle (Jacobi).
+    Tolerance: the angle of the director in FP64, 1e-17 / gap^2 (relative), ten times over, the rounding of Q as it is
+    stored (FP32 and a BF16 remainder: 4e-10 / gap at most) and of the FP32 force (2e-5)."""
+    import paper_1102_2193_gb300 as P
+    L, X, prm = (20, 18, 16), (9.4, 8.3, 7.7), dict(synth.NEMATIC, q0=0.0)
+    R = np.linalg.qr(np.random.default_rng(4).standard_normal((3, 3)))[0]
+    A = size * (R * [0.16 + gap / 2, 0.16 - gap / 2, -0.32]) @ R.T
+    q = np.tile(np.array([A[0, 0], A[0, 1], A[0, 2], A[1, 1], A[1, 2]]).reshape(5, 1, 1, 1), (1, L[2], L[1], L[0]))
+    s, o = P.Solver(*L, precision=P.LC_FP32 if prec == "f32" else P.LC_FP64, **prm), oracle.Oracle(*L, **prm)
+    for k in (s, o):
+        k.set_Q(q)
+        k.add_colloid(X, 4.6, 1, 0.03)
+        k.step(1)
+    a, b = s.colloid(0), o.colloid(0)
+    F = np.abs(b["T_lc"]).max() / 4.6 + np.abs(b["F_lc"]).max()
+    g = gap / 0.16
+    tol = 1e-9 + 1e-16 / g**2 + (2e-5 + 4e-9 / g if prec == "f32" else 0.0)
+    assert np.abs(a["F_lc"] - b["F_lc"]).max() <= tol * F
+    assert np.abs(a["T_lc"] - b["T_lc"]).max() <= 4 * tol * 4.6 * F
