@@ -1482,6 +1482,16 @@ int rebuild_geometry(lc_lb* h) {
   return LC_OK;
 }
 
+// Whether p is device memory of device dev.
+bool on_device(const void* p, int dev) {
+  cudaPointerAttributes a{};
+  if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  return a.type == cudaMemoryTypeDevice && a.device == dev;
+}
+
 int h_check(lc_lb* h) {
   if (!h) return fail(nullptr, LC_ERR_ARG, "null handle");
   return LC_OK;
@@ -1751,8 +1761,9 @@ int lc_lb_get_fields(lc_lb* h, int which, void* dst, size_t bytes, int dst_is_de
     default: return fail(&h->err, LC_ERR_ARG, "unknown field %d", which);
   }
   if (!dst || bytes < nc * N * sizeof(double)) return fail(&h->err, LC_ERR_ARG, "destination too small");
-  // a device destination is written by the export itself, a host one through scratch
-  const bool direct = dst_is_device && (reinterpret_cast<uintptr_t>(dst) & 7) == 0;
+  // memory of this GPU is written by the export itself, any other (host, or that
+  // of another GPU, which a kernel may have no access to) by a copy from scratch
+  const bool direct = dst_is_device && (reinterpret_cast<uintptr_t>(dst) & 7) == 0 && on_device(dst, g->dev);
   if (!direct)
     if (int rc = ensure_scratch(g, nc * N)) return rc;
   double* out = direct ? static_cast<double*>(dst) : g->d_scratch;

@@ -105,3 +105,29 @@ def test_planar_faces_of_close_eigenvalues(prec, size, gap):
     tol = 1e-9 + 1e-16 / g**2 + (2e-5 + 4e-9 / g if prec == "f32" else 0.0)
     assert np.abs(a["F_lc"] - b["F_lc"]).max() <= tol * F
     assert np.abs(a["T_lc"] - b["T_lc"]).max() <= 4 * tol * 4.6 * F
+
+
+@pytest.mark.parametrize("prec", ["f32", "f64"])
+def test_export_destinations(prec):
+    """Fields read into device memory, aligned to 16 bytes and to 8: the values that a host destination receives, and
+    nothing beside them."""
+    import ctypes as C
+
+    import torch
+
+    import paper_1102_2193_gb300 as P
+    L, prm = (22, 9, 7), dict(synth.NEMATIC, q0=0.2)
+    s = P.Solver(*L, precision=P.LC_FP32 if prec == "f32" else P.LC_FP64, **prm)
+    s.set_Q(synth.random_q(L[::-1], 3, amp=0.05, base=(0.2, 0.05, 0.02, -0.1, 0.03)))
+    s.add_colloid((9.3, 4.2, 3.1), 2.3, P.LC_NORMAL, 0.02)
+    s.step(2)
+    N = L[0] * L[1] * L[2]
+    for which, nc in ((P.LC_Q, 5), (P.LC_U, 3), (P.LC_RHO, 1)):
+        ref = np.empty(nc * N)
+        dp = ref.ctypes.data_as(C.c_void_p)
+        assert s.L.lc_lb_get_fields(s.h, which, dp, ref.nbytes, 0) == 0
+        for off in (0, 1):
+            out = torch.full((nc * N + 2,), 7.0, dtype=torch.float64, device="cuda")
+            assert s.L.lc_lb_get_fields(s.h, which, C.c_void_p(out.data_ptr() + 8 * off), ref.nbytes, 1) == 0
+            assert (out[off:off + nc * N].cpu().numpy() == ref).all()
+            assert (out[:off] == 7.0).all() and (out[off + nc * N:] == 7.0).all()
