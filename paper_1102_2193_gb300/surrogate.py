@@ -56,7 +56,8 @@ class UNet:
         self.params = {}
         # parameters, gradients and moments of all layers lie in one buffer each
         # (segments of whole 64-element blocks), so that clearing the gradients
-        # and the Adam step are one launch, not one per layer and tensor
+        # and the Adam step are one launch, not one per layer and tensor (while
+        # the entries of params are these views: _views)
         size = lambda n: (n + 63) // 64 * 64  # noqa: E731
         total = sum(size(cout * taps * cin) + size(cout) for _, cin, cout, taps, _, _ in LAYERS)
         self.flat = {k: torch.zeros(total, device=self.dev) for k in ("", "g", "m", "v")}
@@ -80,6 +81,7 @@ class UNet:
             P["wt"] = torch.empty(P["w"].numel(), dtype=torch.bfloat16, device=self.dev)
             self.params[name] = P
             self._cast(P["w"], P["w16"])
+        self.at = {(n, k): self._addresses(n, k) for n in self.params for k in ("w", "b")}
         self.step_count = 0
         self._alloc()
 
@@ -105,6 +107,15 @@ class UNet:
         nwp = max(self.L.lc_nn_wgrad_partial_floats(S >> lvl, S >> lvl, S >> lvl, cin, cout, taps)
                   for _, cin, cout, taps, _, lvl in LAYERS)
         self.wpart = t.empty(nwp, dtype=t.float32, device=self.dev)
+
+    def _addresses(self, name, k):
+        P = self.params[name]
+        return tuple(P[x].data_ptr() for x in (k, "g" + k, "m" + k, "v" + k) + (("w16",) if k == "w" else ()))
+
+    def _views(self) -> bool:
+        """Whether every parameter, gradient and moment is still its part of the common buffers (an entry of ``params``
+        may be replaced by a tensor of the caller's, which is then updated on its own)."""
+        return all(self._addresses(n, k) == a for (n, k), a in self.at.items())
 
     def _cast(self, a, b):
         _ok(self.L.lc_nn_cast_bf16(_p(a), _p(b), a.numel(), self.sp), "cast")
@@ -195,7 +206,12 @@ class UNet:
 
     def backward(self):
         t, S, a, L, sp = self.torch, self.S, self.a, self.L, self.sp
-        self.flat["g"].zero_()
+        if self._views():
+            self.flat["g"].zero_()
+        else:
+            for P in self.params.values():
+                P["gw"].zero_()
+                P["gb"].zero_()
         n0, n1, n2 = S**3, (S // 2)**3, (S // 4)**3
         new = lambda n, c: t.empty((n, c), dtype=t.float32, device=self.dev)  # noqa: E731
         d_c4 = new(n0, 16)
@@ -229,8 +245,12 @@ class UNet:
     def adam(self, lr=1e-3, b1=0.9, b2=0.999, eps=1e-8):
         self.step_count += 1
         f = self.flat
-        _ok(self.L.lc_nn_adam(_p(f[""]), _p(f["g"]), _p(f["m"]), _p(f["v"]), _p(self.flat16), f[""].numel(), lr, b1,
-                              b2, eps, self.step_count, self.sp), "adam")
+        parts = [(f[""], f["g"], f["m"], f["v"], self.flat16)] if self._views() else \
+            [(P[k], P["g" + k], P["m" + k], P["v" + k], P["w16"] if k == "w" else None)
+             for P in self.params.values() for k in ("w", "b")]
+        for p, g, m, v, p16 in parts:
+            _ok(self.L.lc_nn_adam(_p(p), _p(g), _p(m), _p(v), None if p16 is None else _p(p16), p.numel(), lr, b1, b2,
+                                  eps, self.step_count, self.sp), "adam")
 
     def predict_soa(self):
         """Q = Q_init + y[:, :5] as a [5][S^3] FP64 device tensor."""
