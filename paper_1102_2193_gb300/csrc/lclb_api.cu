@@ -588,7 +588,7 @@ void free_group(Group* g) {
 }
 
 // ---- autotuning -------------------------------------------------------------
-using TuneKey = std::tuple<long long, int>;  // (sum of box signature, precision)
+using TuneKey = std::tuple<long long, int>;  // (sum of box signature, precision + 2 with the flow frozen)
 std::map<TuneKey, std::vector<TileCfg>> g_tune_cache;
 
 TuneKey tune_key(Group* g) {
@@ -599,11 +599,12 @@ TuneKey tune_key(Group* g) {
     sig = sig * 1099511628211LL + h->grid.nz;
     sig = sig * 1099511628211LL + h->grid.wall_z;
   }
-  return TuneKey(sig, g->prec);
+  // (a frozen step is another kernel, with tile shapes and a variant of its own)
+  return TuneKey(sig, g->prec + (g->frozen ? 2 : 0));
 }
 
 // Optional file cache (LCLB_TUNE_CACHE): one line per entry,
-// "signature precision" and NCFG triples "ty zc persistent" (fused, lc,
+// the key (see TuneKey) and NCFG triples "ty zc persistent" (fused, lc,
 // force, lb, (variant, slab, 0), stress, lb-from-stress, dataflow step);
 // lines of another length are skipped.
 constexpr int NCFG = 8;
@@ -734,8 +735,12 @@ int autotune_group_inner(Group* g, std::string* desc) {
   // the fused and split variants are not candidates there (LCLB_VARIANT still
   // forces them)
   const bool fp32 = g->prec == LC_FP32;
+  const char* forced = getenv("LCLB_VARIANT");
   for (int k : {3, 2, 0, 1, 4, 5}) {
-    if (fp32 && (k == 3 || k == 1)) continue;
+    // FP32 boxes take k_force in a forced split variant only; with the flow
+    // frozen a step is k_relax (phase 2), and exports take the stress kernel
+    if (fp32 && (k == 3 || k == 1 || (k == 0 && !(forced && !strcmp(forced, "split"))))) continue;
+    if (g->frozen && k != 2 && k != 4) continue;
     TileCfg best = g->ph[k].cfg;
     const std::vector<int> tys = k == 3 ? std::vector<int>{4, 6, 8} : std::vector<int>{2, 4, 8};
     const std::vector<int> zcs =
@@ -770,7 +775,7 @@ int autotune_group_inner(Group* g, std::string* desc) {
   while (l % b) l += a;
   float best_split = 1e30f;
   int best_slab = 0;
-  for (int m = 1; !fp32 && l * m <= maxnz; m *= 2) {
+  for (int m = 1; !fp32 && !g->frozen && l * m <= maxnz; m *= 2) {
     g->slab = l * m;
     if ((rc = build_chunks_slab(g))) return rc;
     const float ms = time_ms(g, e0, e1, 3, tune_split_fn, nullptr, &rc);
@@ -783,7 +788,7 @@ int autotune_group_inner(Group* g, std::string* desc) {
   }
   g->slab = best_slab;
   if ((rc = build_chunks_slab(g))) return rc;
-  const float stored = time_ms(g, e0, e1, 3, tune_stored_fn, nullptr, &rc);
+  const float stored = g->frozen ? 0.f : time_ms(g, e0, e1, 3, tune_stored_fn, nullptr, &rc);
   if (rc) return rc;
   if (verbose) fprintf(stderr, "lclb tune stored %.1f us\n", 1000.f * stored);
   g->variant = 0;
@@ -792,12 +797,13 @@ int autotune_group_inner(Group* g, std::string* desc) {
     g->variant = 1;
     best_var = best_split;
   }
-  if (stored < best_var || fp32) {
+  if (stored < best_var || fp32) {  // (frozen: all three are the same launch)
     g->variant = 2;
     best_var = stored;
   }
   // dataflow: the whole step as one launch, timed without committing it
-  // (against the force + LB part plus the Q update of the classic variants)
+  // (against the force + LB part, none with the flow frozen, plus the Q update
+  // of the classic variants)
   const float classic = best_var + best_phase[2];
   const TileCfg lc_cfg = g->ph[2].cfg;
   float best_df = 1e30f;

@@ -131,3 +131,19 @@ def test_export_destinations(prec):
             assert s.L.lc_lb_get_fields(s.h, which, C.c_void_p(out.data_ptr() + 8 * off), ref.nbytes, 1) == 0
             assert (out[off:off + nc * N].cpu().numpy() == ref).all()
             assert (out[:off] == 7.0).all() and (out[off + nc * N:] == 7.0).all()
+
+
+@pytest.mark.parametrize("prec", ["f32", "f64"])
+def test_tuned_shapes_of_frozen_and_coupled_boxes(prec, tmp_path, monkeypatch):
+    """A box relaxed with the flow frozen and a coupled box of the same size are tuned apart (their steps are different
+    kernels), each once; the results do not depend on the order."""
+    import paper_1102_2193_gb300 as P
+    L = (23, 17, 21) if prec == "f32" else (21, 17, 23)
+    cache = tmp_path / "tune.txt"
+    monkeypatch.setenv("LCLB_TUNE_CACHE", str(cache))
+    for flow in (False, True, False, True):
+        s = P.Solver(*L, precision=P.LC_FP32 if prec == "f32" else P.LC_FP64, flow=flow, **dict(synth.NEMATIC, q0=0.2))
+        s.set_Q(synth.random_q(L[::-1], 3, amp=0.05, base=(0.2, 0.05, 0.02, -0.1, 0.03)))
+        s.step(2)
+    keys = [tuple(r.split()[:2]) for r in cache.read_text().splitlines()]
+    assert len(keys) == 2 and len(set(keys)) == 2
