@@ -384,8 +384,7 @@ int build_near(lc_lb* h, int n) {
     B.near_cap = need;
     int rc = upload_box(g, h);
     if (rc) return rc;
-    CK(cudaMemsetAsync(B.nnear, 0, sizeof(int), s), &h->err);
-    CK(launch_near_list(g->d_boxes, h->index, B.N, s), &h->err);
+    CK(launch_near_list(g->d_boxes, h->index, B.N, g->d_iwork, B.nnear, s), &h->err);
     if ((rc = build_groups(g))) return rc;
   }
   return LC_OK;
@@ -491,8 +490,9 @@ int make_box(Group* g, const lc_grid* G, const lc_params* p, lc_lb* h) {
   B.gerr = g->d_err;
   B.nlinks = (int*)galloc(g, sizeof(int));
   B.nnear = (int*)galloc(g, sizeof(int));
+  B.near_cnt = (int*)galloc(g, sizeof(int) * g->nsm);
   if (!B.f[0] || !B.f[1] || !B.Q[0] || !B.Q[1] || !B.u || !B.F || !B.H || !B.P || !B.mask || !B.col || !B.st ||
-      !B.nlinks || !B.nnear)
+      !B.nlinks || !B.nnear || !B.near_cnt)
     return fail(&h->err, LC_ERR_OOM, "device allocation failed for a %dx%dx%d box", G->nx, G->ny, G->nz);
   cudaStream_t s = g->stream;
   for (int k = 0; k < 2; ++k) {
@@ -1446,7 +1446,7 @@ int rebuild_geometry(lc_lb* h) {
   int total = 0, nnear = 0;
   CK(cudaMemsetAsync(h->hb.nnear, 0, sizeof(int), s), &h->err);
   if (!h->col.empty() || h->hb.wall_z) {
-    CK(launch_near_list(g->d_boxes, h->index, h->hb.N, s), &h->err);
+    CK(launch_near_list(g->d_boxes, h->index, h->hb.N, g->d_iwork, h->hb.nnear, s), &h->err);
     CK(cudaMemcpyAsync(&nnear, h->hb.nnear, sizeof(int), cudaMemcpyDeviceToHost, s), &h->err);
     if (h->col.empty()) CK(cudaStreamSynchronize(s), &h->err);  // else the link counts below wait
   }

@@ -131,10 +131,11 @@ struct DevBox {
   int* gerr;            // error words of the box's group: [0] wait gave up, [1] contact in some box
   int* nlinks;          // device count of boundary links
   // fluid nodes next to a solid or wall (mask bit NEAR) and the other nodes of
-  // their pairs (near_member), in no particular order: device count, capacity
-  // (a bound on the count over the box's motion)
+  // their pairs (near_member), in node order: device count, capacity (a bound on
+  // the count over the box's motion), counts per block of k_rediscretise
   int* nnear;
   int* near_node;
+  int* near_cnt;
   int near_cap;
   int pad1;
   int* link_node;       // boundary links of this box, sorted by (colloid, node, dir)

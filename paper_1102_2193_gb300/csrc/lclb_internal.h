@@ -82,9 +82,9 @@ int step_blocks_per_sm(int prec, int ty);
 // err the group's error words.
 cudaError_t launch_rediscretise(int prec, DevBox* boxes, int nboxes, const int2* mob, int nmob, int nsm,
                                 unsigned* bar, int* err, int spin_limit, cudaStream_t s);
-// Fills box b's list of near nodes (up to its capacity) and its count, which
-// the caller has zeroed.
-cudaError_t launch_near_list(DevBox* boxes, int b, int N, cudaStream_t s);
+// Fills box b's list of near nodes (up to its capacity) in node order; their
+// number -> *total (device), blocksum: N/256 + 1 ints.
+cudaError_t launch_near_list(DevBox* boxes, int b, int N, int* blocksum, int* total, cudaStream_t s);
 cudaError_t launch_geometry(DevBox* boxes, int b, int N, cudaStream_t s);
 cudaError_t launch_link_build(DevBox* boxes, int b, int N, int c, int* blocksum, int base, int* total,
                               cudaStream_t s);

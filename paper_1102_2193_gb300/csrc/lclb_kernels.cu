@@ -2764,22 +2764,35 @@ __device__ __forceinline__ bool near_member(const DevBox& B, int i) {
   return (m & NEAR) || (pair_box(B) && (B.mask[i ^ 1] & NEAR));
 }
 
-// Appends the listed nodes of a warp's 32 nodes to the box's list (all lanes call it).
-__device__ __forceinline__ void near_append(const DevBox& B, int i, bool near) {
+// The list is in node order, so that a box's residual, which is summed over it in
+// FP32, is the same for every handle with the same state: nodes counted per
+// block, the counts scanned, and each block's nodes written behind those of the
+// blocks before it.
+// Rank of a listed node among those of the block's 256 nodes (all threads call
+// it; s: 8 ints of shared memory).
+__device__ __forceinline__ int near_rank(bool near, int* s) {
   const unsigned m = __ballot_sync(0xffffffffu, near);
-  if (!m) return;
-  const int lane = threadIdx.x & 31, leader = __ffs(m) - 1;
-  int at = 0;
-  if (lane == leader) at = atomicAdd(B.nnear, __popc(m));
-  at = __shfl_sync(0xffffffffu, at, leader) + __popc(m & ((1u << lane) - 1u));
-  if (!near) return;
-  if (at < B.near_cap) B.near_node[at] = i;
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  __syncthreads();
+  if (lane == 0) s[wid] = __popc(m);
+  __syncthreads();
+  int r = __popc(m & ((1u << lane) - 1u));
+  for (int k = 0; k < wid; ++k) r += s[k];
+  return r;
 }
 
-__global__ void __launch_bounds__(256) k_near_list(const DevBox* __restrict__ boxes, int b) {
+__global__ void __launch_bounds__(256) k_near_count(const DevBox* __restrict__ boxes, int b, int* blocksum) {
+  const int n = __syncthreads_count(near_member(boxes[b], blockIdx.x * blockDim.x + threadIdx.x));
+  if (threadIdx.x == 0) blocksum[blockIdx.x] = n;
+}
+
+__global__ void __launch_bounds__(256) k_near_write(const DevBox* __restrict__ boxes, int b, const int* blockoff) {
+  __shared__ int s[8];
   const DevBox& B = boxes[b];
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  near_append(B, i, near_member(B, i));
+  const bool near = near_member(B, i);
+  const int at = blockoff[blockIdx.x] + near_rank(near, s);
+  if (near && at < B.near_cap) B.near_node[at] = i;
 }
 
 // Number of links from fluid node i into colloid c (bit q set in *bits).
@@ -3161,8 +3174,8 @@ __global__ void __launch_bounds__(256) k_reduce(const double* __restrict__ part,
 //             colloid; uncovered nodes take f_eq(rho_bar, u_b) and the
 //             mean Q of their fluid face neighbours (fluid before and after)
 //   rd_mask   mask bits of the changed nodes; rd_near the near flags of the
-//             region; rd_links the boundary links and near list of the box;
-//             rd_finish the box state.
+//             region; rd_count the near nodes of each block's part of the box;
+//             rd_links the boundary links and near list; rd_finish the box state.
 // As eight launches that returned at once they took 52 us of the 113 us step
 // of a 64^3 box with one mobile colloid.
 __device__ __forceinline__ int region_lo(double c, double r) { return (int)floor(c - r - 2.0); }
@@ -3376,17 +3389,56 @@ __device__ void rd_near(DevBox* __restrict__ boxes, const int2* __restrict__ mob
   }
 }
 
-// Rebuild the boundary links (unordered; lc_lb_get_links sorts them) and the
-// near-node lists of boxes whose solid set changed (their counts are zeroed
-// with the near flags).
-__device__ void rd_links(DevBox* __restrict__ boxes, int nboxes) {
+// The block's part of the nodes of box B: whole 256s, in block order.
+__device__ __forceinline__ void near_part(const DevBox& B, int& lo, int& hi) {
+  const long long per = ((B.N + 255LL) / 256 + gridDim.x - 1) / gridDim.x * 256;
+  lo = (int)min((long long)B.N, per * blockIdx.x);
+  hi = (int)min((long long)B.N, per * (blockIdx.x + 1LL));
+}
+__device__ __forceinline__ int warp_total(int v) {
+  return __reduce_add_sync(0xffffffffu, v);
+}
+
+__device__ void rd_count(DevBox* __restrict__ boxes, int nboxes) {
   for (int b = 0; b < nboxes; ++b) {
     const DevBox& B = boxes[b];
     if (ld_state(&B.st->nchg) == 0) continue;
-    const int nthr = gridDim.x * blockDim.x;
-    for (int base = blockIdx.x * blockDim.x; base < B.N; base += nthr) {
-      const int i = base + threadIdx.x;
-      near_append(B, i, near_member(B, i));
+    int lo, hi, n = 0;
+    near_part(B, lo, hi);
+    for (int base = lo; base < hi; base += 256) {
+      const int i = base + (int)threadIdx.x;
+      n += __syncthreads_count(i < hi && near_member(B, i));
+    }
+    if (threadIdx.x == 0) B.near_cnt[blockIdx.x] = n;
+  }
+}
+
+// Rebuild the boundary links (unordered; lc_lb_get_links sorts them; their count
+// is zeroed with the near flags) and the near-node lists of boxes whose solid set
+// changed.
+__device__ void rd_links(DevBox* __restrict__ boxes, int nboxes) {
+  __shared__ int s_off[8];
+  for (int b = 0; b < nboxes; ++b) {
+    const DevBox& B = boxes[b];
+    if (ld_state(&B.st->nchg) == 0) continue;
+    {  // near nodes of the block's part, behind those of the blocks before it
+      int lo, hi, before = 0;
+      near_part(B, lo, hi);
+      for (int k = threadIdx.x; k < (int)blockIdx.x; k += blockDim.x) before += __ldcg(B.near_cnt + k);
+      before = warp_total(before);
+      __syncthreads();
+      if ((threadIdx.x & 31) == 0) s_off[threadIdx.x >> 5] = before;
+      __syncthreads();
+      int at = 0;
+      for (int k = 0; k < 8; ++k) at += s_off[k];
+      for (int base = lo; base < hi; base += 256) {
+        const int i = base + (int)threadIdx.x;
+        const bool near = i < hi && near_member(B, i);
+        const int pos = at + near_rank(near, s_off);
+        if (near && pos < B.near_cap) B.near_node[pos] = i;
+        at += __syncthreads_count(near);
+      }
+      if (blockIdx.x == gridDim.x - 1 && threadIdx.x == 0) *B.nnear = at;
     }
     for (int c = 0; c < B.ncol; ++c) {
       const DevColloid& C = B.col[c];
@@ -3489,10 +3541,9 @@ __global__ void __launch_bounds__(256) k_rediscretise(DevBox* __restrict__ boxes
   rd_near(boxes, mob, nmob);
   if (blockIdx.x == 0)
     for (int b = threadIdx.x; b < nboxes; b += blockDim.x)
-      if (ld_state(&boxes[b].st->nchg) > 0) {
-        *boxes[b].nlinks = 0;
-        *boxes[b].nnear = 0;
-      }
+      if (ld_state(&boxes[b].st->nchg) > 0) *boxes[b].nlinks = 0;
+  if (!grid_barrier(bar, err, spin_limit)) return;
+  rd_count(boxes, nboxes);
   if (!grid_barrier(bar, err, spin_limit)) return;
   rd_links(boxes, nboxes);
   if (!grid_barrier(bar, err, spin_limit)) return;
@@ -3685,8 +3736,11 @@ cudaError_t launch_geometry(DevBox* boxes, int b, int N, cudaStream_t s) {
   return cudaGetLastError();
 }
 
-cudaError_t launch_near_list(DevBox* boxes, int b, int N, cudaStream_t s) {
-  k_near_list<<<nblk(N, 256), 256, 0, s>>>(boxes, b);
+cudaError_t launch_near_list(DevBox* boxes, int b, int N, int* blocksum, int* total, cudaStream_t s) {
+  const int nb = nblk(N, 256);
+  k_near_count<<<nb, 256, 0, s>>>(boxes, b, blocksum);
+  k_scan<<<1, 1024, 0, s>>>(blocksum, nb, 0, total);
+  k_near_write<<<nb, 256, 0, s>>>(boxes, b, blocksum);
   return cudaGetLastError();
 }
 

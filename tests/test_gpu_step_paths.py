@@ -147,3 +147,27 @@ def test_tuned_shapes_of_frozen_and_coupled_boxes(prec, tmp_path, monkeypatch):
         s.step(2)
     keys = [tuple(r.split()[:2]) for r in cache.read_text().splitlines()]
     assert len(keys) == 2 and len(set(keys)) == 2
+
+
+@pytest.mark.parametrize("moving", [False, True])
+@pytest.mark.parametrize("nx", [38, 37])
+def test_residual_is_the_same_for_every_handle(nx, moving):
+    """The FP32 residual of a box with many near nodes, summed over the list of them: the same bits from eight handles
+    of the same state, also after a colloid has moved from node to node (a colloid held by its own inertia: its
+    velocity is set before every step, so that sums in any order do not reach the fields)."""
+    import paper_1102_2193_gb300 as P
+    L, prm = (nx, 34, 36), dict(synth.NEMATIC, q0=0.3)
+    q = synth.random_q(L[::-1], 3, amp=0.05, base=(0.2, 0.05, 0.02, -0.1, 0.03))
+    seen = set()
+    for _ in range(8):
+        s = P.Solver(*L, wall_z=True, precision=P.LC_FP32, flow=False, **prm)
+        s.set_Q(q)
+        s.add_colloid((14.3, 16.2, 17.4), 9.6, P.LC_NORMAL, 0.02, mobile=moving)
+        if moving:
+            for _ in range(3):
+                s.set_colloid_velocity(0, (0.4, 0.3, 0.2))
+                s.step(1)
+        s.step(1)
+        d = s.diag()
+        seen.add((d["resid_rms"], d["resid_max"]))
+    assert len(seen) == 1
