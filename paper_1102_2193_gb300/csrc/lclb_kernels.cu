@@ -876,18 +876,22 @@ __device__ __noinline__ void near_stress(const DevBox& B, int i, int mode, NearS
   }
   if (fe && valid) {
     // free energy of the node, and of its weakly anchored faces (w/2)|Qs - Q0|^2
-    // with Qs - Q0 = -(1/wfac - 1)(Qs - Q)
+    // with Qs - Q0 = -(K/w)(Qs - Q), squared in FP64
     *fe += to_f64(fp);
 #pragma unroll
     for (int d = 0; d < 6; ++d) {
       if (!((solid >> d) & 1u) || nb[d] < 0) continue;
       const DevColloid& C = B.col[cf[d] - 1];
       if (C.strong) continue;
-      const T dz = dn[d][0] + dn[d][3];
-      const T s2 = dn[d][0] * dn[d][0] + dn[d][3] * dn[d][3] + dz * dz +
-                   T(2) * (dn[d][1] * dn[d][1] + dn[d][2] * dn[d][2] + dn[d][4] * dn[d][4]);
-      const double r = 1.0 / C.wfac - 1.0;
-      *fe += 0.5 * C.w * r * r * to_f64(s2);
+      const double r = B.p.K / C.w;
+      double e[5], s2 = 0.0;
+#pragma unroll
+      for (int k = 0; k < 5; ++k) {
+        e[k] = r * to_f64(dn[d][k]);
+        s2 += (k == 0 || k == 3 ? 1.0 : 2.0) * e[k] * e[k];
+      }
+      s2 += (e[0] + e[3]) * (e[0] + e[3]);
+      *fe += 0.5 * C.w * s2;
     }
   }
   if (!(mode & FORCE_ACC)) return;

@@ -171,3 +171,19 @@ def test_residual_is_the_same_for_every_handle(nx, moving):
         d = s.diag()
         seen.add((d["resid_rms"], d["resid_max"]))
     assert len(seen) == 1
+
+
+@pytest.mark.parametrize("w", [1e-3, 1e-12, 1e-22, 1e3])
+@pytest.mark.parametrize("prec", ["f32", "f64"])
+def test_surface_energy(w, prec):
+    """Free energy of weakly anchored faces alone (no bulk term, a uniform Q): (w/2)|Qs - Q0|^2 of every face against the
+    oracle, over the range of w in which squares of Qs - Q leave FP32.  Tolerance: FP32 surface values (1e-6)."""
+    import paper_1102_2193_gb300 as P
+    L, prm = (20, 18, 16), dict(synth.NEMATIC, q0=0.0, A0=0.0)
+    q = np.tile(np.array([0.2, 0.05, 0.02, -0.1, 0.03]).reshape(5, 1, 1, 1), (1, L[2], L[1], L[0]))
+    s, o = P.Solver(*L, precision=P.LC_FP32 if prec == "f32" else P.LC_FP64, **prm), oracle.Oracle(*L, **prm)
+    for k in (s, o):
+        k.set_Q(q)
+        k.add_colloid((9.4, 8.3, 7.7), 4.6, 0, w)
+    a, b = s.diag()["free_energy"], o.diag()["free_energy"]
+    assert b > 0 and abs(a - b) <= (1e-6 if prec == "f32" else 1e-11) * b
