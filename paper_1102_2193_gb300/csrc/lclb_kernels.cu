@@ -3558,6 +3558,13 @@ __global__ void __launch_bounds__(256) k_rediscretise(DevBox* __restrict__ boxes
 // ---------------------------------------------------------------------------
 // host launchers
 // ---------------------------------------------------------------------------
+// An error that is returned to the caller is taken from the runtime, so that the
+// next launch does not report it again.
+static cudaError_t taken(cudaError_t e) {
+  cudaGetLastError();
+  return e;
+}
+
 template <typename T, int TY>
 static cudaError_t launch_force_t(const Launch& L, int mode, double* part) {
   constexpr int HP = (TX + 2) * (TY + 2);
@@ -3599,7 +3606,7 @@ static cudaError_t launch_stress_t(const Launch& L, int mode, double* part) {
   constexpr size_t ring = ring_bytes<T, 5, TY>(), near = sizeof(NearScratch<T>) * TY, smem = ring > near ? ring : near;
   auto* fn = (mode & FORCE_FE) ? k_stress<T, TY, true> : k_stress<T, TY, false>;
   cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (e != cudaSuccess) return e;
+  if (e != cudaSuccess) return taken(e);
   fn<<<L.grid, dim3(TX, TY), smem, L.stream>>>(L, mode, part);
   return cudaGetLastError();
 }
@@ -3615,7 +3622,7 @@ static cudaError_t launch_lc_t(const Launch& L, int mode, double* part) {
   constexpr size_t smem = ring_bytes<T, 8, TY>();
   if (smem > 0) {
     cudaError_t e = cudaFuncSetAttribute(k_lc<T, TY>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
+    if (e != cudaSuccess) return taken(e);
   }
   k_lc<T, TY><<<L.grid, dim3(TX, TY), smem, L.stream>>>(L, mode, part);
   return cudaGetLastError();
@@ -3625,7 +3632,7 @@ template <typename T, int TY>
 static cudaError_t launch_relax_t(const Launch& L, int mode, double* part) {
   constexpr size_t ring = ring_bytes<T, 5, TY>(), near = sizeof(NearScratch<T>) * TY, smem = ring > near ? ring : near;
   cudaError_t e = cudaFuncSetAttribute(k_relax<T, TY>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (e != cudaSuccess) return e;
+  if (e != cudaSuccess) return taken(e);
   k_relax<T, TY><<<L.grid, dim3(TX, TY), smem, L.stream>>>(L, mode, part);
   return cudaGetLastError();
 }
@@ -3696,7 +3703,7 @@ static cudaError_t launch_step_t(DevBox* boxes, const StepItem* items, int nitem
                                  double* part, int spin_limit, int commit, int* err, int grid, cudaStream_t s) {
   constexpr size_t smem = sizeof(NearScratch<T>) * TY;
   cudaError_t e = cudaFuncSetAttribute(k_step<T, TY>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (e != cudaSuccess) return e;
+  if (e != cudaSuccess) return taken(e);
   k_step<T, TY><<<grid, dim3(TX, TY), smem, s>>>(boxes, items, nitems, zc, sync, part, spin_limit, commit, err);
   return cudaGetLastError();
 }
@@ -3793,7 +3800,7 @@ cudaError_t launch_rediscretise(int prec, DevBox* boxes, int nboxes, const int2*
   void* args[] = {&boxes, &nboxes, &mob, &nmob, &bar, &err, &spin_limit};
   const void* fn = prec == 0 ? (const void*)k_rediscretise<float> : (const void*)k_rediscretise<double>;
   cudaError_t e = cudaLaunchCooperativeKernel(fn, dim3(nsm), dim3(256), args, 0, s);
-  if (e != cudaSuccess) return e;
+  if (e != cudaSuccess) return taken(e);
   return cudaGetLastError();
 }
 

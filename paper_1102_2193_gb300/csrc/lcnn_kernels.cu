@@ -888,6 +888,14 @@ static inline int grid_for(size_t n, int bs = 256) {
   return (int)(g > 65535 * 8 ? 65535 * 8 : (g < 1 ? 1 : g));
 }
 
+// The status of a runtime call that may have failed; its error is taken, so that
+// the next call does not report it again.
+static inline int taken(cudaError_t e) {
+  if (e == cudaSuccess) return LC_NN_OK;
+  cudaGetLastError();
+  return LC_NN_ERR_CUDA;
+}
+
 static inline bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15) == 0; }
 
 template <int NT, int MT, int NW, int TX, int TY, int TZ>
@@ -895,7 +903,7 @@ static int launch_conv_tile(const __nv_bfloat16* in, const __nv_bfloat16* w, con
                             __nv_bfloat16* out16, int W, int H, int D, int cin, int cout, int relu, cudaStream_t s) {
   constexpr int smem = ((TX + 2) * (TY + 2) * (TZ + 2) + 27 * NT * 8) * 32;
   auto* fn = k_conv_tile<NT, MT, NW, TX, TY, TZ>;
-  if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess) return LC_NN_ERR_CUDA;
+  if (taken(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem)) != LC_NN_OK) return LC_NN_ERR_CUDA;
   const int ntx = (W + TX - 1) / TX, nty = (H + TY - 1) / TY, ntz = (D + TZ - 1) / TZ;
   fn<<<dim3((unsigned)ntx * nty * ntz, cout / (NT * 8)), 32 * NW, smem, s>>>(in, w, bias, out32, out16, W, H, D, cin,
                                                                             cout, relu, ntx, nty);
@@ -932,7 +940,7 @@ static int conv_tiled(const __nv_bfloat16* in, const __nv_bfloat16* w, const flo
 
 static int launch_bias_grad(const float* dout, float* db, int npos, int c, cudaStream_t s) {
   auto* fn = c % 4 == 0 && aligned16(dout) ? k_bias_grad<4> : k_bias_grad<1>;
-  if (cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) return LC_NN_ERR_CUDA;
+  if (taken(cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1)) != LC_NN_OK) return LC_NN_ERR_CUDA;
   cudaLaunchConfig_t cfg{};
   cudaLaunchAttribute at{};
   cfg.gridDim = dim3((c + 15) / 16 * BIAS_CLUSTER);
@@ -943,7 +951,7 @@ static int launch_bias_grad(const float* dout, float* db, int npos, int c, cudaS
   at.val.clusterDim.y = at.val.clusterDim.z = 1;
   cfg.attrs = &at;
   cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, fn, dout, db, npos, c) == cudaSuccess ? LC_NN_OK : LC_NN_ERR_CUDA;
+  return taken(cudaLaunchKernelEx(&cfg, fn, dout, db, npos, c));
 }
 
 template <int TPW, int TY, int TZ>
@@ -951,7 +959,7 @@ static int launch_wgrad_tile(const __nv_bfloat16* dout, const __nv_bfloat16* in,
                              int cin, int cout, int nchunk, cudaStream_t s) {
   constexpr int smem = (18 * (TY + 2) * (TZ + 2) + 1 + 16 * TY * TZ) * 32;
   auto* fn = k_wgrad_tile<TPW, TY, TZ>;
-  if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess) return LC_NN_ERR_CUDA;
+  if (taken(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem)) != LC_NN_OK) return LC_NN_ERR_CUDA;
   fn<<<dim3(nchunk, (cout / 16) * (cin / 16), 3 / TPW), 288, smem, s>>>(
       dout, in, part, W, H, D, cin, cout, (W + 15) / 16, (H + TY - 1) / TY, (D + TZ - 1) / TZ, nchunk);
   return cudaGetLastError() == cudaSuccess ? LC_NN_OK : LC_NN_ERR_CUDA;
