@@ -1027,6 +1027,7 @@ int lc_nn_conv3d_wgrad(const void* dout, const void* in, float* dw, float* parti
   if (!dout || !in || !dw || !partial || cout % 16 || cin % 8 || cin > 80) return LC_NN_ERR_ARG;
   const int npos = W * H * D;
   if (npos <= 0) return LC_NN_ERR_ARG;
+  if (cin != 8 && cin != 16 && cin != 32 && cin != 48 && cin != 80) return LC_NN_ERR_ARG;  // the same for every path
   const int chunk = wgrad_chunk(npos);
   const int nchunk = (npos + chunk - 1) / chunk;
   const dim3 grid(nchunk, taps, cout / 16);

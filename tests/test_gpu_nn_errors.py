@@ -20,3 +20,20 @@ def test_refused_bias_gradient_leaves_no_error():
     assert L.lc_nn_bias_grad(a, b, 64, 16, None) == 0
     torch.cuda.synchronize()
     assert (db == 64.0).all()
+
+
+@pytest.mark.parametrize("cin", [24, 40, 56, 64, 72, 0])
+@pytest.mark.parametrize("taps", [1, 27])
+def test_weight_gradient_refuses_other_channel_counts(cin, taps):
+    """Input-channel counts that no layer kernel is made for are refused whichever path the tensors' alignment takes."""
+    import ctypes as C
+
+    import paper_1102_2193_gb300 as P
+    L = P.lib()
+    z = torch.zeros(64 * 80 + 8, dtype=torch.bfloat16, device="cuda")
+    w = torch.zeros(16 * 27 * 80, dtype=torch.float32, device="cuda")
+    part = torch.zeros(16 * 27 * 80, dtype=torch.float32, device="cuda")
+    for off in (0, 2):
+        p = C.c_void_p(z.data_ptr() + 2 * off)
+        assert L.lc_nn_conv3d_wgrad(p, p, C.c_void_p(w.data_ptr()), C.c_void_p(part.data_ptr()), 4, 4, 4, cin, 16, taps,
+                                    None) == -1
