@@ -63,7 +63,7 @@ KERNEL_DESC = {
     "k_stress": "H and P stored once per fluid node, colloid LC force (stored variant)",
     "k_lbp": "body force from stored P + pull collide-stream (stored variant)",
 }
-KERNEL_SOURCES = ("paper_1102_2193_gb300/csrc/lclb_kernels.cu", "paper_1102_2193_gb300/csrc/lclb_dev.cuh")
+KERNEL_SOURCES = tuple("paper_1102_2193_gb300/csrc/" + f for f in ("lclb_kernels.cu", "lclb_dev.cuh", "lclb_pair.cuh"))
 
 
 def kernel_hash() -> str:

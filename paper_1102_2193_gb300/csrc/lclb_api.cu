@@ -2041,8 +2041,9 @@ int lc_lb_batch_profile(lc_lb_batch* b, int nsteps, double ms_out[5]) {
 }  // extern "C"
 
 // ---- diagnostics without allocation ------------------------------------------
-// Scratch of lc_lb_diagnostics_noalloc: one record of 6 doubles per block of
-// 256 nodes for up to 8192 blocks (2,097,152 nodes), then 8 doubles for the
+// Scratch of lc_lb_diagnostics_noalloc: 8192 records of 6 doubles, one per 256
+// nodes of the largest box (2,097,152 nodes; a block writes one record for every
+// 1024), then 8 doubles for the
 // reduced values: 384 KiB + 64 B on every device that loads the library.
 namespace {
 constexpr int NOALLOC_MAX_BLOCKS = 8192;

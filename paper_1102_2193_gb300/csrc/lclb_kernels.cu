@@ -963,7 +963,7 @@ __device__ __forceinline__ void stress_node(const DevBox& B, const PhysT<T>& PP,
   }
 }
 
-// k_stress: H and P stored once per fluid node.  A warp evaluates its row's
+// Stress tile of k_step: H and P stored once per fluid node.  A warp evaluates its row's
 // nodes away from solids and walls together; nodes next to a solid or wall
 // (surface values, colloid faces) are queued per warp and evaluated 32 at a
 // time, so a row that crosses a colloid does not run the surface path with
@@ -1071,7 +1071,7 @@ __device__ __forceinline__ void queue_push(int (*sq)[2 * TX], int wy, int lane, 
   }
 }
 
-// Stored-stress kernel, two nodes per lane: H and P of the pair from packed
+// Stress tile of k_step, two nodes per lane: H and P of the pair from packed
 // derivatives (the z-neighbours rolled down the column as in stress_tile).
 // The loads of the next plane (mask, the column's z + 1 and the rows y +- 1)
 // are issued before the current plane is evaluated, so their latency is
@@ -1211,8 +1211,9 @@ __device__ __forceinline__ void cp_async16(float* dst, const float* src) {
 // kept from plane to plane.  (Each lane copying its own pair, its row's edges
 // and, by turns, the rows above and below took 24 copies a plane and warp for
 // 5 components and 43 for 8, with their addresses a quarter of the kernels'
-// instructions.  128^3: k_stress 59 -> 44 us, k_lc 71 -> 53; 256 x 192 x 160:
-// 167 -> 126 and 207 -> 162; a step of k_relax at 96^3 26.5 -> 22.2.)
+// instructions.  When that was changed, 128^3: k_stress 59 -> 44 us, k_lc 71 -> 53;
+// 256 x 192 x 160: 167 -> 126 and 207 -> 162; a step of k_relax at 96^3 26.5 ->
+// 22.2.)
 struct RingLane {
   int x, y, row;   // node column, row start of y (node index)
   int li, ri;      // ring columns of x - 1 and x + 2
@@ -1412,14 +1413,16 @@ __device__ __forceinline__ void block_fe(double fe, double* out) {
 // nodes.  FE (diagnostics): the free energy of each tile into part and of each
 // block of near groups into L.fepart.
 // FP32 tiles of even width: two nodes per lane from the ring, packed arithmetic,
-// 597 instructions a pair and warp, 16 warps per SM at 128 registers; bound by
-// issue and by the FP32 pipe, which a packed instruction holds for two cycles
+// about 600 instructions a pair and warp, 16 warps per SM at 128 registers; bound
+// by issue and by the FP32 pipe, which a packed instruction holds for two cycles
 // (76 bytes a node: 23 us at 128^3).  One or two rows of a tile per thread, and 168
 // registers with fewer warps, measured the same or slower.  FP64: bound by the
 // FP64 pipe (84 % busy).  Near groups: a chain of FP64 surface values, 64 cycles
 // an instruction and warp, spread over all SMs.  128^3 with one
 // colloid: near nodes queued by tiles and Q by shuffles and loads 75 us, near
-// groups and the ring 58, its copies in 16-byte pieces 44.
+// groups and the ring 58, its copies in 16-byte pieces 44, the tiles of chiral and
+// other boxes compiled apart 41 (one code with branches on q0: 52); 256 x 192 x
+// 160, nematic: 117.
 template <typename T, int TY, bool FE>
 __global__ void __launch_bounds__(TX * TY, (sizeof(T) == 4 ? 512 : 256) / (TX * TY)) k_stress(Launch L, int mode,
                                                                                              double* __restrict__ part) {
@@ -1515,7 +1518,7 @@ __device__ __forceinline__ void lbp_node(const DevBox& B, const PhysT<T>& PP, co
   collide_store(PP, fout, ub, B.N, i, df, Fx, Fy, Fz);
 }
 
-// k_lbp: like k_stress, a warp collides the plain fluid nodes of its row
+// LB tile of k_step: as there, a warp collides the plain fluid nodes of its row
 // together and queues the nodes next to a solid or wall (bounce-back links,
 // solid faces of the force) in shared memory, 32 at a time.
 template <typename T, int TY, bool CG>
@@ -1598,10 +1601,12 @@ __device__ __forceinline__ void near_lbp(const DevBox& B, int j) {
 
 // Bound by the memory system: 38 population streams of 4 bytes a node, 18
 // stress values and 3 velocities: 159 MB of populations read and written and 75
-// MB of stress at 128^3 (70 us under the profiler, 5.0 TB/s; 79 in the step).  What hides the
+// MB of stress at 128^3 (70 us under the profiler, 5.0 TB/s; 76 in the step, 280
+// at 256 x 192 x 160).  What hides the
 // latency is warps: 64 registers for 32 warps per SM 77 us, 80 registers 87, 48
 // registers 88.  The rows of the next plane staged in shared memory by 16-byte
-// asynchronous copies, which leaves 20 warps per SM: 94.
+// asynchronous copies, which leaves 20 warps per SM: 94.  (Opposite directions
+// collided together, in a sum of another order, saved 2 us.)
 template <typename T, int TY>
 __global__ void __launch_bounds__(TX * TY, (sizeof(T) == 4 ? 1024 : 384) / (TX * TY)) k_lbp(Launch L) {
   __shared__ DevBox B;
@@ -1792,7 +1797,7 @@ __device__ __forceinline__ void lc_update_node(const DevBox& B, const PhysT<T>& 
   add_residual(d5, rsum, rmax);
 }
 
-// k_lc: Beris-Edwards update; plain nodes of a warp's row together, nodes
+// Q-update tile of k_step: plain nodes of a warp's row together, nodes
 // next to a solid or wall queued and updated 32 at a time.  part (if non-null)
 // receives the tile's residual partials (sum of squares, max), one record per
 // warp (TY records per tile).
@@ -1854,7 +1859,7 @@ __device__ __forceinline__ void lc_tile(const DevBox& B, const int4 td, int zc, 
   if (part) warp_residual<T>(part, wy, lane, rsum, rmax);
 }
 
-// Q update, two nodes per lane (FP32 boxes of even width; tiles 64 wide): the
+// Q-update tile of k_step, two nodes per lane (FP32 boxes of even width; tiles 64 wide): the
 // Beris-Edwards update of lc_update_node for the nodes x, x + 1 at once, in
 // packed FP32x2 arithmetic, with Q, u, H and the BF16 remainder of Q moved as
 // pairs.
@@ -2416,8 +2421,8 @@ __device__ __forceinline__ void lc_commit(const Launch& L, int b, unsigned n) {
 // width: as k_stress, Q and u from the ring (8 components), H and the remainder
 // of Q loaded per pair ahead of the plane's barrier; 128 registers, one
 // component's neighbours read at a time (all at once spill).  Bound by issue:
-// 128^3 67 + 16 us (links) + 6 (colloid) at the start, 53 us for all of it now;
-// 256 x 192 x 160 162 us.
+// 128^3 67 + 16 us (links) + 6 (colloid) as three launches, 60 us for all of it now
+// (55 with shorter sums in another order, see lclb_pair.cuh); 256 x 192 x 160 186 us.
 template <typename T, int TY>
 __global__ void __launch_bounds__(TX * TY, (sizeof(T) == 4 ? 512 : 256) / (TX * TY)) k_lc(Launch L, int mode,
                                                                                          double* __restrict__ part) {
@@ -2474,7 +2479,7 @@ __global__ void __launch_bounds__(TX * TY, (sizeof(T) == 4 ? 512 : 256) / (TX * 
 // flux, so H is used where it is formed and each node moves its Q twice (60
 // bytes with the remainder) instead of the 190 of the separate stress and Q
 // update.  Near nodes still take their stress for the colloid's LC force.
-// Bound by issue of the molecular field (about 130 packed operations a pair);
+// Bound by issue of the molecular field (about 140 packed operations a pair);
 // 96^3: 105 us for the launches of the general step, 69 without its stores and
 // loads, 30 as one launch, 22 with the ring copied in 16-byte pieces.
 template <int TY, bool CHIRAL>
