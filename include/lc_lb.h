@@ -287,7 +287,7 @@ const char* lc_lb_batch_last_error(const lc_lb_batch* b);
 
 /* Autotuner: time the candidate tile shapes of each phase kernel on a
  * scratch box of the given size and precision, and keep the fastest (cached
- * per size and precision for the process; LCLB_TUNE_CACHE names a file to
+ * per size, precision and frozen or coupled flow for the process; LCLB_TUNE_CACHE names a file to
  * persist it).  Called automatically on first use of a size; exposed to
  * force a retune.  out_desc (may be NULL) receives a short text of the
  * choice. */
