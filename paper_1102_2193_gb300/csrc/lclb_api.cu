@@ -1158,7 +1158,7 @@ int check_step_err(Group* g, std::string* err) {
   CK(cudaStreamSynchronize(g->stream), err);
   if (hv[0] == 0 && hv[1] == 0) return LC_OK;
   const bool timeout = hv[0] != 0;
-  CK(cudaMemsetAsync(g->d_err, 0, (timeout ? 4 : 2) * sizeof(int), g->stream), err);  // [2], [3]: grid barrier of k_rediscretise
+  CK(cudaMemsetAsync(g->d_err, 0, (timeout ? 4 : 2) * sizeof(int), g->stream), err);  // [2]: grid barrier of k_rediscretise
   long long cstep = -1;
   int cbox = -1, ccol = -1, cpartner = -2;
   for (size_t b = 0; b < g->boxes.size(); ++b) {

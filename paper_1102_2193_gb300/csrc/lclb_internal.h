@@ -78,8 +78,8 @@ cudaError_t launch_step(int prec, int ty, DevBox* boxes, const StepItem* items, 
                         double* part, int spin_limit, int commit, int* err, int grid, cudaStream_t s);
 int step_blocks_per_sm(int prec, int ty);
 // Re-discretisation after the colloid update; mob lists (box, colloid) of
-// mobile colloids, bar the grid barrier's two words (reset after an error only),
-// err the group's error words.
+// mobile colloids, bar the grid barrier's word (reset after an error only), err
+// the group's error words.
 cudaError_t launch_rediscretise(int prec, DevBox* boxes, int nboxes, const int2* mob, int nmob, int nsm,
                                 unsigned* bar, int* err, int spin_limit, cudaStream_t s);
 // Fills box b's list of near nodes (up to its capacity) in node order; their

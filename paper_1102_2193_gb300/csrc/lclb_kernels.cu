@@ -3495,19 +3495,14 @@ __device__ void rd_finish(DevBox* __restrict__ boxes, int b) {
   if (ld_state(B.nlinks) > B.nlinks_cap || ld_state(B.nnear) > B.near_cap) atomicOr(&st->err, 1);
 }
 
-// The words of the launch's barrier: bar[0] arrivals, bar[1] generation.
+// The word of the launch's barrier and the group's error word.
 struct GridWords {
   unsigned* bar;
   int* err;
-  __device__ unsigned generation() const { return ld_acquire_u32(bar + 1); }
-  __device__ unsigned arrive() const {
+  __device__ unsigned word() const { return ld_acquire_u32(bar); }
+  __device__ unsigned arrive(unsigned add) const {
     __threadfence();
-    return atomicAdd(bar, 1u);
-  }
-  __device__ void clear_arrivals() const { atomicExch(bar, 0u); }
-  __device__ void advance() const {
-    __threadfence();
-    atomicAdd(bar + 1, 1u);
+    return atomicAdd(bar, add);
   }
   __device__ bool failed() const { return ld_acquire_u32(reinterpret_cast<const unsigned*>(err)) != 0u; }
   __device__ void fail() const { atomicOr(err, 1); }
@@ -3519,7 +3514,7 @@ __device__ bool grid_barrier(unsigned* bar, int* err, int spin_limit) {
   __syncthreads();
   if (threadIdx.x == 0) {
     GridWords w{bar, err};
-    s_ok = barrier_wait(w, gridDim.x, spin_limit);
+    s_ok = barrier_wait(w, gridDim.x, blockIdx.x == 0, spin_limit);
     __threadfence();
   }
   __syncthreads();

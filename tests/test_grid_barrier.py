@@ -1,5 +1,5 @@
-"""The barrier of the re-discretisation launch, compiled for the host: threads in the place of blocks, the generation
-word started just below its wrap at 2^32."""
+"""The barrier of the re-discretisation launch, compiled for the host: threads in the place of blocks, across both sides
+of its word (the top bit) and the wrap at 2^32."""
 import os
 import shutil
 import subprocess
@@ -14,43 +14,40 @@ SRC = r"""
 #include <vector>
 #include "lclb_barrier.h"
 struct Words {
-  std::atomic<unsigned> count{0}, gen{0};
+  std::atomic<unsigned> bar{0};
   std::atomic<int> err{0};
-  unsigned generation() { return gen.load(std::memory_order_acquire); }
-  unsigned arrive() { return count.fetch_add(1, std::memory_order_acq_rel); }
-  void clear_arrivals() { count.store(0, std::memory_order_relaxed); }
-  void advance() { gen.fetch_add(1, std::memory_order_acq_rel); }
+  unsigned word() { return bar.load(std::memory_order_acquire); }
+  unsigned arrive(unsigned add) { return bar.fetch_add(add, std::memory_order_acq_rel); }
   bool failed() { return err.load() != 0; }
   void fail() { err.fetch_or(1); }
   void pause() { std::this_thread::yield(); }
 };
 int main() {
-  // n threads, barriers from 6 below the wrap to 6 above it: between two barriers every thread must have passed the first
+  // n threads, 13 barriers: between two of them every thread must have passed the first
   for (unsigned n : {1u, 3u, 5u}) {
     Words w;
-    w.gen = 0u - 6u;
     std::vector<std::atomic<int>> at(n);
     for (auto& a : at) a = 0;
     std::atomic<int> bad{0};
     std::vector<std::thread> th;
     for (unsigned t = 0; t < n; ++t)
       th.emplace_back([&, t] {
-        for (int r = 1; r <= 12; ++r) {
+        for (int r = 1; r <= 13; ++r) {
           at[t] = r;
-          if (!lclb::barrier_wait(w, n, 1 << 30)) bad = 1;
+          if (!lclb::barrier_wait(w, n, t == n - 1, 1 << 30)) bad = 1;
           for (unsigned k = 0; k < n; ++k)
             if (at[k] < r || at[k] > r + 1) bad = 1;
         }
       });
     for (auto& t : th) t.join();
-    if (bad || w.gen != 6u || w.count != 0u || w.err) { std::printf("n = %u: broken\n", n); return 1; }
+    if (bad || w.bar != 0x80000000u || w.err) { std::printf("n = %u: broken\n", n); return 1; }
   }
   // a missing arrival ends the wait with the error set; a set error ends other waits early
   Words w;
-  if (lclb::barrier_wait(w, 2, 1000) || !w.err) { std::printf("no error\n"); return 1; }
+  if (lclb::barrier_wait(w, 2, true, 1000) || !w.err) { std::printf("no error\n"); return 1; }
   Words v;
   v.err = 1;
-  if (lclb::barrier_wait(v, 2, 2000000000)) { std::printf("waited\n"); return 1; }
+  if (lclb::barrier_wait(v, 2, false, 2000000000)) { std::printf("waited\n"); return 1; }
   return 0;
 }
 """
