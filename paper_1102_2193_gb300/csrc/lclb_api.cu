@@ -268,6 +268,7 @@ Launch phase_launch(Group* g, int k, int mode, int box = -1) {
 
 int upload_box(Group* g, lc_lb* h) {
   CK(cudaMemcpyAsync(g->d_boxes + h->index, &h->hb, sizeof(DevBox), cudaMemcpyHostToDevice, g->stream), &h->err);
+  CK(launch_pair_constants(g->d_boxes, h->index, g->stream), &h->err);
   g->dirty = true;
   return LC_OK;
 }

@@ -50,6 +50,41 @@ struct PhysT {
   T g[3];
 };
 
+// Constants of the packed FP32 functions (lclb_pair.cuh): one per field in the
+// box's record, twice in the kernels' shared copy (T = f2).
+template <typename T>
+struct LcPairT {
+  T A0g, nA0g, c_lin, A0g3, nA0g3;   // A0 g, H: Q beyond -A0 g Tr(Q^2), A0 g / 3
+  T K, nK, K4, tK4;                  // K, K / 4, 2 K / 4
+  T Kq, nKq, n2Kq, Kqq;              // K q0 (half of 2 K q0), 2 K q0^2
+  T fb2, fb4, half, third;
+  T twoxi, ntwoxi, nxi, ntwoxi3;     // 2 xi, -xi, -2 xi / 3
+  T nsix;
+  T xi, xi23, Gam4, ntwo;            // increment of Q (scaled by four)
+  T c_lo, A2, nq23, Gam;
+};
+constexpr int LCPAIR_N = sizeof(LcPairT<float>) / sizeof(float);
+
+// Formed on the device, once per upload of the record, by the expressions of the
+// one-node functions (so that both round alike).
+__device__ __forceinline__ void lc_pair_constants(LcPairT<float>& C, const PhysT<float>& P) {
+  const float A0 = P.A0, g = P.gamma, K = P.K, q0 = P.q0, xi = P.xi;
+  const float third = 1.f / 3.f;
+  const float A0g = A0 * g, twoKq0 = 2.f * K * q0;
+  const float c_lin = -A0 * (1.f - g * third) - 4.f * K * q0 * q0;
+  const float A0g3 = A0g * third;
+  C.A0g = A0g; C.nA0g = -A0g; C.c_lin = c_lin; C.A0g3 = A0g3; C.nA0g3 = -A0g3;
+  C.K = K; C.nK = -K; C.K4 = 0.25f * K; C.tK4 = 0.5f * K;
+  C.Kq = 0.5f * twoKq0; C.nKq = -0.5f * twoKq0; C.n2Kq = -twoKq0; C.Kqq = 2.f * K * q0 * q0;
+  C.fb2 = 0.5f * A0 * (1.f - g * third); C.fb4 = 0.25f * A0g; C.half = 0.5f; C.third = third;
+  const float twoxi = 2.f * xi, twoxi3 = twoxi * third;
+  C.twoxi = twoxi; C.ntwoxi = -twoxi; C.nxi = -xi; C.ntwoxi3 = -twoxi3;
+  C.nsix = -6.f;
+  C.xi = xi; C.xi23 = 2.f * xi / 3.f; C.Gam4 = 4.f * P.Gamma; C.ntwo = -2.f;
+  C.c_lo = -A0 * (1.f - g / 3.f) - 4.f * K * q0 * q0 - 6.f * K;
+  C.A2 = 2.f * A0g; C.nq23 = -(2.f / 3.f); C.Gam = P.Gamma;
+}
+
 // Constants of the FP64 liquid-crystal algebra, every combination that the node
 // functions multiply by formed once per box.
 template <typename T>
@@ -145,6 +180,7 @@ struct DevBox {
   PhysT<float> pf;
   PhysT<double> pd;
   LcK<double> kd;
+  LcPairT<float> kp;    // written on the device (k_pair_constants)
 };
 
 // FP32 boxes of even width run the two-node paths of the stress kernel and

@@ -85,6 +85,7 @@ cudaError_t launch_rediscretise(int prec, DevBox* boxes, int nboxes, const int2*
 // Fills box b's list of near nodes (up to its capacity) in node order; their
 // number -> *total (device), blocksum: N/256 + 1 ints.
 cudaError_t launch_near_list(DevBox* boxes, int b, int N, int* blocksum, int* total, cudaStream_t s);
+cudaError_t launch_pair_constants(DevBox* boxes, int b, cudaStream_t s);  // DevBox::kp, after an upload
 cudaError_t launch_geometry(DevBox* boxes, int b, int N, cudaStream_t s);
 cudaError_t launch_link_build(DevBox* boxes, int b, int N, int c, int* blocksum, int base, int* total,
                               cudaStream_t s);

@@ -177,7 +177,10 @@ __device__ __forceinline__ void load_box(DevBox& sb, const DevBox* boxes, int b)
 
 // The constants of the two-node paths from the shared record.
 __device__ __forceinline__ void load_k2(LcPair& k2, const DevBox& B) {
-  if (threadIdx.x + threadIdx.y == 0) lc_pair_constants(k2, B.pf);
+  const float* src = reinterpret_cast<const float*>(&B.kp);
+  f2* dst = reinterpret_cast<f2*>(&k2);
+  const int nthr = blockDim.x * blockDim.y;
+  for (int k = threadIdx.x + blockDim.x * threadIdx.y; k < LCPAIR_N; k += nthr) dst[k] = f2(src[k]);
   __syncthreads();
 }
 
@@ -188,10 +191,11 @@ __device__ __forceinline__ void load_box(DevBox& sb, const DevBox* boxes, int b,
   load_box(sb, boxes, b);
   cur = b;
 }
+template <typename T>
 __device__ __forceinline__ void load_box(DevBox& sb, LcPair& k2, const DevBox* boxes, int b, int& cur) {
   if (b == cur) return;
   load_box(sb, boxes, b);
-  load_k2(k2, sb);
+  if constexpr (sizeof(T) == 4) load_k2(k2, sb);
   cur = b;
 }
 
@@ -1433,7 +1437,7 @@ __global__ void __launch_bounds__(TX * TY, (sizeof(T) == 4 ? 512 : 256) / (TX * 
   const int nn = L.ngroups / TY, units = nn + L.ntiles;
   for (int t = blockIdx.x; t < units; t += gridDim.x) {
     const int4 td = t < nn ? make_int4(L.groups[t * TY].x, 0, 0, 0) : L.tiles[t - nn];
-    load_box(B, K2, L.boxes, td.x, cur_box);
+    load_box<T>(B, K2, L.boxes, td.x, cur_box);
     double fe = 0.0;
     if (t < nn) {
       if (B.p.lc_on)
@@ -2445,7 +2449,7 @@ __global__ void __launch_bounds__(TX * TY, (sizeof(T) == 4 ? 512 : 256) / (TX * 
       run_n = 0;
     }
     ++run_n;
-    load_box(B, K2, L.boxes, td.x, cur_box);
+    load_box<T>(B, K2, L.boxes, td.x, cur_box);
     T rsum = T(0), rmax = T(0);  // per-thread residual (sum of squares, max), in T
     if (t < nn) {
       if (B.p.lc_on)
@@ -2593,7 +2597,7 @@ __global__ void __launch_bounds__(TX * TY, (sizeof(T) == 4 ? 640 : 256) / (TX * 
       run_n = 0;
     }
     ++run_n;
-    load_box(B, K2, L.boxes, td.x, cur_box);
+    load_box<T>(B, K2, L.boxes, td.x, cur_box);
     T rs[2] = {T(0), T(0)};
     if (B.p.lc_on) {
       if (t < nn) {
@@ -2687,7 +2691,7 @@ __global__ void __launch_bounds__(TX * TY, (sizeof(T) == 4 ? 512 : 256) / (TX * 
     }
     __syncthreads();
     if (s_ok) {
-      load_box(B, K2, boxes, I.box, cur_box);
+      load_box<T>(B, K2, boxes, I.box, cur_box);
       const int4 td = make_int4(I.box, I.x0, I.y0, I.z0);
       switch (I.kind) {
         case ITEM_STRESS:
@@ -2725,6 +2729,8 @@ __global__ void __launch_bounds__(TX * TY, (sizeof(T) == 4 ? 512 : 256) / (TX * 
 // ---------------------------------------------------------------------------
 // geometry: solid mask, near flags, boundary links (cold path)
 // ---------------------------------------------------------------------------
+__global__ void k_pair_constants(DevBox* __restrict__ boxes, int b) { lc_pair_constants(boxes[b].kp, boxes[b].pf); }
+
 __global__ void k_mask(DevBox* __restrict__ boxes, int b) {
   const DevBox& B = boxes[b];
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
@@ -3740,6 +3746,11 @@ int step_blocks_per_sm(int prec, int ty) {
 }
 
 static inline int nblk(int N, int bs) { return (N + bs - 1) / bs; }
+
+cudaError_t launch_pair_constants(DevBox* boxes, int b, cudaStream_t s) {
+  k_pair_constants<<<1, 1, 0, s>>>(boxes, b);
+  return cudaGetLastError();
+}
 
 cudaError_t launch_geometry(DevBox* boxes, int b, int N, cudaStream_t s) {
   k_mask<<<nblk(N, 256), 256, 0, s>>>(boxes, b);

@@ -15,36 +15,7 @@
 
 namespace lclb {
 
-// Constants of the two functions, each value twice (one 8-byte load per packed
-// operand), formed in FP32 as the one-node functions form them.
-struct LcPair {
-  f2 A0g, nA0g, c_lin, A0g3, nA0g3;   // A0 g, H: Q beyond -A0 g Tr(Q^2), A0 g / 3
-  f2 K, nK, K4, tK4;                  // K, K / 4, 2 K / 4
-  f2 Kq, nKq, n2Kq, Kqq;              // K q0 (half of 2 K q0), 2 K q0^2
-  f2 fb2, fb4, half, third;
-  f2 twoxi, ntwoxi, nxi, ntwoxi3;     // 2 xi, -xi, -2 xi / 3
-  f2 nsix;
-  f2 xi, xi23, Gam4, ntwo;    // increment of Q (scaled by four)
-  f2 c_lo, A2, nq23, Gam;
-};
-
-__device__ __forceinline__ void lc_pair_constants(LcPair& C, const PhysT<float>& P) {
-  const float A0 = P.A0, g = P.gamma, K = P.K, q0 = P.q0, xi = P.xi;
-  const float third = 1.f / 3.f;
-  const float A0g = A0 * g, twoKq0 = 2.f * K * q0;
-  const float c_lin = -A0 * (1.f - g * third) - 4.f * K * q0 * q0;
-  const float A0g3 = A0g * third;
-  C.A0g = f2(A0g); C.nA0g = f2(-A0g); C.c_lin = f2(c_lin); C.A0g3 = f2(A0g3); C.nA0g3 = f2(-A0g3);
-  C.K = f2(K); C.nK = f2(-K); C.K4 = f2(0.25f * K); C.tK4 = f2(0.5f * K);
-  C.Kq = f2(0.5f * twoKq0); C.nKq = f2(-0.5f * twoKq0); C.n2Kq = f2(-twoKq0); C.Kqq = f2(2.f * K * q0 * q0);
-  C.fb2 = f2(0.5f * A0 * (1.f - g * third)); C.fb4 = f2(0.25f * A0g); C.half = f2(0.5f); C.third = f2(third);
-  const float twoxi = 2.f * xi, twoxi3 = twoxi * third;
-  C.twoxi = f2(twoxi); C.ntwoxi = f2(-twoxi); C.nxi = f2(-xi); C.ntwoxi3 = f2(-twoxi3);
-  C.nsix = f2(-6.f);
-  C.xi = f2(xi); C.xi23 = f2(2.f * xi / 3.f); C.Gam4 = f2(4.f * P.Gamma); C.ntwo = f2(-2.f);
-  C.c_lo = f2(-A0 * (1.f - g / 3.f) - 4.f * K * q0 * q0 - 6.f * K);
-  C.A2 = f2(2.f * A0g); C.nq23 = f2(-(2.f / 3.f)); C.Gam = f2(P.Gamma);
-}
+using LcPair = LcPairT<f2>;  // each value twice: one 8-byte load per packed operand
 
 // lc_node_f32 of two nodes.  dq: the doubled first derivatives; CHIRAL: q0 != 0.
 template <bool CHIRAL, bool NEED_P>
